@@ -1,0 +1,329 @@
+"""The calls whose speed matters to a program that uses this package, as cases that can be timed and compared.
+
+A case is one unit of work of such a program, through the package's public classes:
+
+``layers``   one request through the attention blocks of ``layers`` decoder layers (LocretLayer, LayerStack): reset, the
+             prompt of ``tokens`` tokens in chunks of ``chunk``, then ``turns`` times a short input of ``turn`` tokens and
+             ``decode`` single tokens appended without eviction (the last ones of a prompt, a question, an answer).
+``blocks``   the same through whole decoder layers (LocretBlock), the output of one being the input of the next.
+``token``    one token through layers whose caches are full, each of which evicts one unit: a stream without an end.
+``train``    one optimiser step of a layer's retaining head on one sequence: labels, loss and gradients, AdamW on W1 and W2.
+``labels``   the training labels alone, of a long prompt.
+
+A prompt is at most one chunk longer than the budget, so that the last chunk is the one that evicts.  Units at the cut of an
+eviction are less far apart in score than the bf16 rounding of two correct implementations, and a unit decided the other way
+re-assigns the positions of the others; nothing computed after such a cut could be compared.  (``token`` evicts the one
+lowest unit of a cache, which is far enough from the next.)
+
+Shapes, budgets and chunk sizes are those of workloads/configs.py (its small case and its two 7-8B-class shapes); hidden
+states and weights have the distributions given there.
+"""
+
+from __future__ import annotations
+
+import math
+from types import SimpleNamespace
+
+import torch
+
+import paper_2410_01805_b200 as locret
+
+# widths of the decoder layers; hidden: how the hidden states are distributed
+SHAPES = {
+    "small": dict(d_model=512, n_q_heads=8, n_kv_heads=2, head_dim=64, d_retain=256, rope_theta=10000.0, d_ff=1536,
+                  hidden="normal"),
+    "llama": dict(d_model=4096, n_q_heads=32, n_kv_heads=8, head_dim=128, d_retain=1024, rope_theta=500000.0,
+                  d_ff=14336, hidden="outlier"),
+    "phi3": dict(d_model=3072, n_q_heads=32, n_kv_heads=32, head_dim=96, d_retain=1024, rope_theta=10000.0, d_ff=8192,
+                 hidden="topics"),
+}
+
+
+def listed():
+    return [
+        # the smallest call: one token of a small model's stream, one layer, evicting; latency is all of it
+        dict(name="small_token", kind="token", shape="small", layers=1, budget=1024, n_stab=64, int4=False),
+        # a short prompt through a small layer: three chunks, the last one ragged and evicting
+        dict(name="small_prefill", kind="layers", shape="small", layers=1, tokens=1400, chunk=512, budget=1024, n_stab=64,
+             turns=0, turn=0, decode=0, int4=False),
+        # long prompts of the grouped-query 8B shape, bf16 cache: filling the cache and the first eviction
+        dict(name="llama_prefill", kind="layers", shape="llama", layers=4, tokens=9144, chunk=3072, budget=6144, n_stab=2500,
+             turns=0, turn=0, decode=0, int4=False),
+        # the same with the cache kept in 4 bits
+        dict(name="llama_prefill_int4", kind="layers", shape="llama", layers=4, tokens=9216, chunk=3072, budget=6144,
+             n_stab=2500, turns=0, turn=0, decode=0, int4=True),
+        # the multi-head shape (32 KV heads of 96) with its large budget and small chunks
+        dict(name="phi3_prefill", kind="layers", shape="phi3", layers=1, tokens=17000, chunk=1024, budget=16384, n_stab=1024,
+             turns=0, turn=0, decode=0, int4=False),
+        # an answer of 256 tokens after a prompt that fills the budget
+        dict(name="llama_decode", kind="layers", shape="llama", layers=4, tokens=6000, chunk=3072, budget=6000, n_stab=2500,
+             turns=1, turn=0, decode=256, int4=False),
+        dict(name="llama_decode_int4", kind="layers", shape="llama", layers=4, tokens=6000, chunk=3072, budget=6000,
+             n_stab=2500, turns=1, turn=0, decode=256, int4=True),
+        # a conversation: short questions (odd sizes below one query tile) and short answers over a cached prompt
+        dict(name="llama_chat", kind="layers", shape="llama", layers=4, tokens=4500, chunk=3072, budget=6000, n_stab=128,
+             turns=4, turn=45, decode=8, int4=False),
+        # whole decoder layers: a long prompt, and a conversation
+        dict(name="llama_block_prefill", kind="blocks", shape="llama", layers=2, tokens=9216, chunk=3072, budget=6144,
+             n_stab=2500, turns=0, turn=0, decode=0, int4=False),
+        dict(name="llama_block_chat", kind="blocks", shape="llama", layers=2, tokens=1000, chunk=1024, budget=2048,
+             n_stab=128, turns=2, turn=20, decode=48, int4=False),
+        # training of the retaining heads: a step on a sequence of the length the method trains on, and the labels of a
+        # long prompt against a long answer
+        dict(name="llama_train", kind="train", shape="llama", tokens=10240, answer=512),
+        dict(name="llama_labels_128k", kind="labels", shape="llama", tokens=131072, answer=1024),
+    ]
+
+
+def _log(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def _draw_once(rng):
+    kind = rng.choice(("token", "layers", "layers", "layers", "layers", "blocks", "blocks", "train", "labels"))
+    shape = rng.choice(("small", "llama", "llama", "phi3"))
+    if kind == "labels":
+        return dict(kind=kind, shape=shape, tokens=_log(rng, 500, 131072), answer=_log(rng, 16, 1024))
+    if kind == "train":
+        return dict(kind=kind, shape=shape, tokens=64 * _log(rng, 4, 160), answer=_log(rng, 16, 1024))
+    layers = rng.randint(1, 4 if kind != "blocks" else 2)
+    int4 = kind != "blocks" and rng.random() < 0.25
+    if kind == "token":
+        budget = _log(rng, 256, 8192)
+        return dict(kind=kind, shape=shape, layers=layers, budget=budget, n_stab=rng.randint(0, budget // 2), int4=int4)
+    case = dict(kind=kind, shape=shape, layers=layers, int4=int4)
+    chunk = _log(rng, 200, 3072)
+    if rng.random() < 0.5:  # a prompt that ends in an eviction
+        full = rng.randint(1, max(1, min(8, 16384 // chunk)))
+        budget = full * chunk + rng.randint(0, chunk // 2)
+        last = rng.randint(budget - full * chunk + 1, chunk) if budget - full * chunk < chunk else chunk
+        case.update(tokens=full * chunk + last, chunk=chunk, budget=budget, n_stab=rng.randint(0, budget // 2), turns=0,
+                    turn=0, decode=0)
+    else:                   # a prompt that fits, and a conversation
+        tokens = _log(rng, 100, 6000)
+        budget = tokens + rng.randint(0, 2000)
+        turns = rng.randint(1, 4)
+        case.update(tokens=tokens, chunk=max(chunk, 256), budget=budget, n_stab=rng.randint(0, budget // 2), turns=turns,
+                    turn=rng.choice((0, _log(rng, 2, 200))), decode=_log(rng, 1, 128 // turns))
+    return case
+
+
+def _seconds(case):
+    """A rough time, to keep drawn cases below the largest listed one."""
+    w = work(case)
+    return w["flops"] / 1e15 + w["bytes"] / 4e12
+
+
+def draw(rng):
+    most = max(_seconds(c) for c in listed())
+    while True:
+        case = _draw_once(rng)
+        if _seconds(case) <= most:
+            return case
+
+
+# ------------------------------------------------------------------------------------------------ inputs
+
+def _shape(case):
+    s = dict(SHAPES[case["shape"]])
+    hidden = s.pop("hidden")
+    ns = SimpleNamespace(act=0, rh_input=0, kv_dtype=1 if case.get("int4") else 0, **s)
+    ns.d_in = (ns.n_q_heads + 2 * ns.n_kv_heads) * ns.head_dim
+    return ns, hidden
+
+
+def _hidden(kind, n, width, gen):
+    x = torch.randn(n, width, generator=gen, device="cuda")
+    if kind == "outlier":    # a token in a thousand has 20 times the norm
+        x *= torch.where(torch.rand(n, 1, generator=gen, device="cuda") < 1e-3, 20.0, 1.0)
+    elif kind == "topics":   # segments of about 512 tokens around one of 64 means
+        means = torch.randn(64, width, generator=gen, device="cuda")
+        border = torch.rand(n, generator=gen, device="cuda") < 1 / 512
+        ids = torch.randint(0, 64, (n + 1,), generator=gen, device="cuda")[torch.cumsum(border.int(), 0)]
+        x = math.sqrt(0.5) * (x + means[ids])
+    return x.bfloat16()
+
+
+def _matrix(rows, cols, gen):
+    return (torch.randn(rows, cols, generator=gen, device="cuda") / math.sqrt(rows)).bfloat16()
+
+
+def _chunks(case):
+    return [(t, min(t + case["chunk"], case["tokens"])) for t in range(0, case["tokens"], case["chunk"])]
+
+
+def _request_tokens(case):
+    return case["tokens"] + case["turns"] * (case["turn"] + case["decode"])
+
+
+def prepare(case, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(int(seed))
+    s, hidden = _shape(case)
+    if case["kind"] in ("train", "labels"):
+        state = dict(case=case,
+                     q=torch.randn(case["answer"], s.n_q_heads, s.head_dim, generator=gen, device="cuda").bfloat16(),
+                     k=torch.randn(case["tokens"], s.n_kv_heads, s.head_dim, generator=gen, device="cuda").bfloat16())
+        if case["kind"] == "train":
+            state["z"] = torch.randn(case["tokens"], s.d_in, generator=gen, device="cuda").bfloat16()
+            params = []
+            for w in (_matrix(s.d_in, s.d_retain, gen), _matrix(s.d_retain, s.n_kv_heads, gen)):
+                p = w.float()
+                params.append(dict(p=p, bf16=w, m=torch.zeros_like(p), v=torch.zeros_like(p)))
+            state.update(params=params, step=0)
+        return state
+
+    token = case["kind"] == "token"
+    budget = case["budget"]
+    chunk = case["chunk"] if not token else min(budget, 1024)
+    tokens = _request_tokens(case) if not token else 1
+    reserve = tokens - case["tokens"] if not token else 0
+    layers = []
+    for _ in range(case["layers"]):
+        w = [_matrix(s.d_model, s.d_in, gen), _matrix(s.d_in, s.d_retain, gen), _matrix(s.d_retain, s.n_kv_heads, gen)]
+        if case["kind"] == "blocks":
+            hd = s.n_q_heads * s.head_dim
+            w += [_matrix(hd, s.d_model, gen), _matrix(s.d_model, s.d_ff, gen), _matrix(s.d_model, s.d_ff, gen),
+                  _matrix(s.d_ff, s.d_model, gen)]
+            w += [(1 + 0.1 * torch.randn(s.d_model, generator=gen, device="cuda")).bfloat16() for _ in range(2)]
+            layers.append(locret.LocretBlock(s, *w, budget, chunk, case["n_stab"], reserve=reserve))
+        else:
+            layers.append(locret.LocretLayer(s, *w, budget, chunk, case["n_stab"], reserve=reserve))
+    width = s.d_model if case["kind"] == "blocks" else s.n_q_heads * s.head_dim
+    out = torch.zeros(*([tokens] if case["kind"] == "blocks" else [len(layers), tokens]), width, dtype=torch.bfloat16,
+                      device="cuda")
+    state = dict(case=case, layers=layers, x=_hidden(hidden, tokens, s.d_model, gen), out=out)
+    if case["kind"] == "layers":
+        state["stack"] = locret.LayerStack(layers)
+    if token:  # the caches are full when the measured tokens arrive
+        fill = _hidden(hidden, budget, s.d_model, gen)
+        trash = torch.empty(chunk, width, dtype=torch.bfloat16, device="cuda")
+        for t in range(0, budget, chunk):
+            part = fill[t:t + chunk]
+            for layer in layers:
+                layer.prefill_chunk(part, trash, 0)
+    return state
+
+
+# ------------------------------------------------------------------------------------------------ one pass
+
+def _run_layers(state):
+    case, x, out = state["case"], state["x"], state["out"]
+    for layer in state["layers"]:
+        layer.reset()
+    for t0, t1 in _chunks(case):
+        for layer, o in zip(state["layers"], out):
+            layer.prefill_chunk(x[t0:t1], o[t0:t1], 0)
+    t = case["tokens"]
+    for _ in range(case["turns"]):
+        if case["turn"]:
+            for layer, o in zip(state["layers"], out):
+                layer.prefill_chunk(x[t:t + case["turn"]], o[t:t + case["turn"]], locret.NO_EVICT)
+            t += case["turn"]
+        for t in range(t, t + case["decode"]):
+            state["stack"].decode_step(x[t], out[0, t], out.stride(0))
+        t += 1
+    return out
+
+
+def _run_blocks(state):
+    case, x, y = state["case"], state["x"], state["out"]
+    blocks = state["layers"]
+    for b in blocks:
+        b.attn.reset()
+
+    def through(t0, t1, flags):
+        src = x[t0:t1]
+        for b in blocks:
+            b.prefill_chunk(src, y[t0:t1], flags)
+            src = y[t0:t1]
+
+    for t0, t1 in _chunks(case):
+        through(t0, t1, 0)
+    t = case["tokens"]
+    for _ in range(case["turns"]):
+        if case["turn"]:
+            through(t, t + case["turn"], locret.NO_EVICT)
+            t += case["turn"]
+        for t in range(t, t + case["decode"]):
+            through(t, t + 1, locret.NO_EVICT)
+        t += 1
+    return y
+
+
+def run(state):
+    kind = state["case"]["kind"]
+    if kind == "layers":
+        return _run_layers(state)
+    if kind == "blocks":
+        return _run_blocks(state)
+    if kind == "token":
+        for layer, o in zip(state["layers"], state["out"]):
+            layer.prefill_chunk(state["x"], o, 0)
+        return state["out"]
+    labels = locret.cis_labels(state["q"], state["k"])
+    if kind == "labels":
+        return labels
+    w1, w2 = state["params"]
+    loss, d_w1, d_w2 = locret.rh_loss_grad(state["z"], labels, w1["bf16"], w2["bf16"])
+    state["step"] += 1
+    for w, g in ((w1, d_w1), (w2, d_w2)):
+        locret.adamw_step(w["p"], g, w["m"], w["v"], state["step"], 5e-4, param_bf16=w["bf16"])
+    return dict(labels=labels, loss=loss, d_w1=d_w1, d_w2=d_w2, w1=w1["p"], w2=w2["p"], w1_bf16=w1["bf16"],
+                w2_bf16=w2["bf16"], m1=w1["m"], v1=w1["v"])
+
+
+# ------------------------------------------------------------------------------------------------ what a pass cannot do without
+
+def work(case):
+    s, _ = _shape(case)
+    h, hk, d, D, R = s.n_q_heads, s.n_kv_heads, s.head_dim, s.d_model, s.d_retain
+    nbytes = flops = 0.0
+    if case["kind"] in ("train", "labels"):
+        n, na = case["tokens"], case["answer"]
+        flops += 2.0 * n * na * h * d
+        nbytes += 2.0 * d * (na * h + n * hk) + 4.0 * hk * n
+        if case["kind"] == "train":
+            flops += 4.0 * n * s.d_in * R + 6.0 * n * R * hk
+            params = s.d_in * R + R * hk
+            # z, labels, weights in; gradients out; AdamW: gradient, parameter and moments in, the latter and bf16 out
+            nbytes += 2.0 * n * s.d_in + 4.0 * hk * n + params * (2 + 4 + 16 + 12 + 2)
+        return dict(bytes=nbytes, flops=flops)
+
+    calls, have = [], 0   # (tokens, retained units before, whether it evicts)
+    if case["kind"] == "token":
+        calls.append((1, case["budget"], True))
+    else:
+        for t0, t1 in _chunks(case):
+            calls.append((t1 - t0, have, have + t1 - t0 > case["budget"]))
+            have = min(case["budget"], have + t1 - t0)
+        for _ in range(case["turns"]):
+            for n in ([case["turn"]] if case["turn"] else []) + [1] * case["decode"]:
+                calls.append((n, have, False))
+                have += n
+    unit = 2.0 * (d / 2 + 2) if case["int4"] else 4.0 * d   # K and V of one unit of one head
+    block = case["kind"] == "blocks"
+    for n, ln, evicts in calls:
+        flops += 2.0 * n * (D * s.d_in + s.d_in * R + R * hk) + 4.0 * h * d * (n * ln + n * (n + 1) / 2)
+        nbytes += 2.0 * (D * s.d_in + s.d_in * R + R * hk) + hk * unit * (ln + n) + 2.0 * n * D
+        nbytes += 4.0 * hk * (n + (ln if evicts else 0))     # scores
+        if block:
+            flops += 2.0 * n * (h * d * D + 3 * D * s.d_ff)
+            nbytes += 2.0 * (h * d * D + 3 * D * s.d_ff) + 2.0 * n * D
+        else:
+            nbytes += 2.0 * n * h * d
+    return dict(bytes=nbytes * case["layers"], flops=flops * case["layers"])
+
+
+def tolerance(case):
+    """About four times what was seen: the default kernels against the mma.sync kernels (LOCRET_LEGACY_MMA=1: other tiles,
+    other order of the sums) gave rel up to 2.6e-3 and max up to 0.12 (0.24 with the 4-bit cache) through layers, 3.3e-3
+    and 0.03 through blocks; labels, loss, gradients and updated weights against 64 bits 1.3e-7 for the labels and up to
+    1.9e-3 / 0.08 for the rest (the contraction for W1 takes bf16 operands, and AdamW's first steps have the gradient's sign)."""
+    if case["kind"] == "labels":
+        return {"rel": 1e-6, "max": 1e-5}
+    if case["kind"] == "blocks":
+        return {"rel": 1.3e-2, "max": 0.2}
+    if case["kind"] == "train":
+        return {"rel": 8e-3, "max": 0.35}
+    return {"rel": 1e-2, "max": 0.95 if case["int4"] else 0.5}
