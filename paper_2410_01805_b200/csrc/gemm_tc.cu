@@ -61,6 +61,39 @@ bool tmap_encode_3d_bf16(CUtensorMap *map, const void *base, uint64_t d0, uint64
 }
 
 namespace {
+struct MapCache {
+  const void *base = nullptr;
+  uint64_t inner = 0, outer = 0, stride = 0;
+  uint32_t box_outer = 0;
+  CUtensorMap map;
+};
+}  // namespace
+
+// Small per-thread cache of encoded maps (weights and staging buffers repeat every call).  The map is
+// copied out: a pointer into the cache would not survive the next miss, which may reuse its slot.
+bool cached_map_k64(CUtensorMap *out, const void *base, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
+                    uint32_t box_outer) {
+  constexpr int SLOTS = 256;
+  static thread_local MapCache cache[SLOTS];
+  static thread_local int next = 0;
+  for (int i = 0; i < SLOTS; i++) {
+    MapCache &c = cache[i];
+    if (c.base == base && c.inner == inner && c.outer == outer && c.stride == stride_bytes &&
+        c.box_outer == box_outer) {
+      *out = c.map;
+      return true;
+    }
+  }
+  MapCache &c = cache[next];
+  next = (next + 1) % SLOTS;
+  c.base = nullptr;
+  if (!tmap_encode_2d_bf16(&c.map, base, inner, outer, stride_bytes, 64, box_outer)) return false;
+  c.base = base; c.inner = inner; c.outer = outer; c.stride = stride_bytes; c.box_outer = box_outer;
+  *out = c.map;
+  return true;
+}
+
+namespace {
 
 using namespace tc;
 
@@ -525,35 +558,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   }
 }
 
-struct MapCache {
-  const void *base = nullptr;
-  uint64_t inner = 0, outer = 0, stride = 0;
-  uint32_t box_outer = 0;
-  CUtensorMap map;
-};
-
-// Small per-thread cache of encoded maps (weights and staging buffers repeat every call).
-const CUtensorMap *cached_map(const void *base, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
-                              uint32_t box_outer) {
-  constexpr int SLOTS = 256;
-  static thread_local MapCache cache[SLOTS];
-  static thread_local int next = 0;
-  for (int i = 0; i < SLOTS; i++) {
-    MapCache &c = cache[i];
-    if (c.base == base && c.inner == inner && c.outer == outer && c.stride == stride_bytes &&
-        c.box_outer == box_outer)
-      return &c.map;
-  }
-  MapCache &c = cache[next];
-  next = (next + 1) % SLOTS;
-  if (!tmap_encode_2d_bf16(&c.map, base, inner, outer, stride_bytes, BK, box_outer)) {
-    c.base = nullptr;
-    return nullptr;
-  }
-  c.base = base; c.inner = inner; c.outer = outer; c.stride = stride_bytes; c.box_outer = box_outer;
-  return &c.map;
-}
-
 template <int BN, int MODE, int HD = 0>
 cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M, int N,
                      int K, const float *W2, float *partial, int h_kv, int act, const RopeAppendArgs &ra,
@@ -563,9 +567,9 @@ cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, i
   if (cudaError_t e = allow_dynamic_smem(gemm_tc_kernel<BN, MODE, HD>, Cfg::smem_bytes(MODE), attr_set);
       e != cudaSuccess)
     return e;
-  const CUtensorMap *ma = cached_map(A, K, M, (uint64_t)lda * 2, BM);
-  const CUtensorMap *mb = cached_map(Bt, K, N, (uint64_t)ldb * 2, BN);
-  if (!ma || !mb) return cudaErrorInvalidValue;
+  CUtensorMap ma, mb;
+  if (!cached_map_k64(&ma, A, K, M, (uint64_t)lda * 2, BM) || !cached_map_k64(&mb, Bt, K, N, (uint64_t)ldb * 2, BN))
+    return cudaErrorInvalidValue;
   const int num_sms = sm_count_of_current_device();
   const int total = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
   const int grid = total < num_sms ? total : num_sms;
@@ -575,7 +579,7 @@ cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, i
   const size_t a_bytes = (size_t)M * K * 2, b_bytes = (size_t)N * K * 2;
   const int n_major = MODE != 1 && b_bytes > a_bytes;  // (MODE 1 indexes its partial sums by column tile either way)
   gemm_tc_kernel<BN, MODE, HD><<<grid, GT_THREADS, Cfg::smem_bytes(MODE), st>>>(
-      *ma, *mb, C, ldc, M, N, K, W2, partial, h_kv, act, ra, resid, ldr, n_major, status);
+      ma, mb, C, ldc, M, N, K, W2, partial, h_kv, act, ra, resid, ldr, n_major, status);
   return cudaGetLastError();
 }
 

@@ -253,7 +253,10 @@ bool tmap_encode_2d_bf16(CUtensorMap *map, const void *base, uint64_t inner, uin
 bool tmap_encode_3d_bf16(CUtensorMap *map, const void *base, uint64_t d0, uint64_t d1, uint64_t d2,
                          uint64_t stride1_bytes, uint64_t stride2_bytes, uint32_t b0, uint32_t b1,
                          uint32_t b2);
-
+// Map of a [outer x inner] bf16 matrix in boxes of 64 x box_outer elements, from a small per-thread cache
+// (a map is a function of its arguments alone); false if it cannot be encoded.
+bool cached_map_k64(CUtensorMap *out, const void *base, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
+                    uint32_t box_outer);
 
 // Eq. 1 on tcgen05 (attn_tc.cu).  map_k / map_v: 3-D maps {d, cap, h_kv}, box {64, 128, 1};
 // map_q: 2-D map {h*d, rows}, box {64, 128}.
