@@ -2,6 +2,8 @@
 // SiLU FFN with its residual.  The three projections run on the tcgen05 GEMM (residual add and
 // silu(gate) * up in its epilogues); shapes that GEMM does not take fall back to the mma.sync
 // GEMM plus element-wise kernels.
+#include <stdlib.h>
+
 #include <map>
 #include <mutex>
 #include <new>
@@ -47,6 +49,59 @@ __global__ void rmsnorm_kernel(const bf16 *__restrict__ x, const bf16 *__restric
     }
     dst[v] = make_uint4(o[0], o[1], o[2], o[3]);
   }
+}
+
+// ---- the same for few rows: one block per row (a warp alone takes 7.6 us for a row of 4096)
+__global__ void __launch_bounds__(256)
+rmsnorm_row_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ gain, bf16 *__restrict__ y, int D, float eps) {
+  __shared__ float part[8];
+  const int row = blockIdx.x, tid = threadIdx.x;
+  const uint4 *gv = reinterpret_cast<const uint4 *>(gain);
+  uint4 g0 = make_uint4(0, 0, 0, 0);
+  if (tid < D / 8) g0 = gv[tid];   // (the gain depends on nothing before this kernel)
+  pdl_wait();
+  pdl_launch_dependents();
+  const uint4 *src = reinterpret_cast<const uint4 *>(x + (size_t)row * D);
+  uint4 *dst = reinterpret_cast<uint4 *>(y + (size_t)row * D);
+  float ss = 0.f;
+  for (int v = tid; v < D / 8; v += 256) {
+    const uint4 q = src[v];
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      const float a = __uint_as_float(w[e] << 16), b = __uint_as_float(w[e] & 0xffff0000u);
+      ss = fmaf(a, a, ss);
+      ss = fmaf(b, b, ss);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if ((tid & 31) == 0) part[tid >> 5] = ss;
+  __syncthreads();
+  float t = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; i++) t += part[i];
+  const float inv = rsqrtf(t / (float)D + eps);
+  for (int v = tid; v < D / 8; v += 256) {
+    const uint4 q = src[v], g = v == tid ? g0 : gv[v];
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w}, gw[4] = {g.x, g.y, g.z, g.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      const float a = __uint_as_float(w[e] << 16) * inv * __uint_as_float(gw[e] << 16);
+      const float b = __uint_as_float(w[e] & 0xffff0000u) * inv * __uint_as_float(gw[e] & 0xffff0000u);
+      o[e] = pack_bf16(a, b);
+    }
+    dst[v] = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+}
+
+cudaError_t launch_rmsnorm(const bf16 *x, const bf16 *gain, bf16 *y, int rows, int D, float eps, cudaStream_t st,
+                           bool pdl) {
+  if (rows <= 512)
+    return launch_kernel(rmsnorm_row_kernel, dim3(rows), dim3(256), 0, st, pdl, x, gain, y, D, eps);
+  rmsnorm_kernel<<<(rows + 7) / 8, 256, 0, st>>>(x, gain, y, rows, D, eps);
+  return cudaGetLastError();
 }
 
 // ---- fallbacks for shapes the tcgen05 GEMM does not take
@@ -136,6 +191,7 @@ struct locret_block {
   int *d_status;
   BlockScratch *pool;
   int device;
+  bool use_pdl;  // (LOCRET_NO_PDL=1 disables, as for a layer)
 };
 
 #define BCK(call)                                                            \
@@ -177,6 +233,8 @@ int locret_block_create(const locret_block_cfg *cfg, int32_t budget, int32_t chu
   B->st = (cudaStream_t)cfg->attn.stream;
   B->D = cfg->attn.d_model; B->hd = cfg->attn.n_q_heads * cfg->attn.head_dim; B->F = cfg->d_ff;
   B->chunk = chunk;
+  const char *np = getenv("LOCRET_NO_PDL");
+  B->use_pdl = !(np && np[0] == '1');
   B->eps = cfg->rms_eps > 0.f ? cfg->rms_eps : 1e-5f;
   const int D = B->D, hd = B->hd, F = B->F;
   bool ok = cudaMalloc(&B->wo_t, (size_t)D * hd * sizeof(bf16)) == cudaSuccess;
@@ -229,29 +287,32 @@ int locret_block_prefill_chunk(locret_block *B, const void *x_in, int32_t n_tok,
   const int D = B->D, hd = B->hd, F = B->F;
   const bf16 *x = (const bf16 *)x_in;
   bf16 *y = (bf16 *)y_out;
-  const int rows_per_blk = 8;
-  const dim3 nblk((n_tok + rows_per_blk - 1) / rows_per_blk);
+  // every kernel of a step of few tokens may start while the one before it drains (each waits for it before it
+  // touches what that one writes or reads), so the weight stream does not stop between them
+  const bool pdl = n_tok <= 256 && B->use_pdl;
   // h1 = RMSNorm(x; g1)
-  rmsnorm_kernel<<<nblk, rows_per_blk * 32, 0, B->st>>>(x, B->g1, P->h, n_tok, D, B->eps);
-  BCK(cudaGetLastError());
+  BCK(launch_rmsnorm(x, B->g1, P->h, n_tok, D, B->eps, B->st, pdl));
   // the attention block (projection, RoPE, attention, retaining head, eviction)
   int rc = locret_prefill_chunk(B->attn, P->h, n_tok, flags, P->att);
   if (rc != LOCRET_OK) return rc;
   // x1 = x + attn_out W_o
   const bool tc = n_tok >= 32;
-  if (tc && gemm_tc_supported(n_tok, D, hd, hd, hd)) {
+  if (skinny_use(n_tok, D, hd, hd, hd)) {
+    BCK(launch_skinny_gemm(P->att, hd, B->wo_t, hd, P->x1, D, n_tok, D, hd, x, D, B->d_status, B->st, pdl));
+  } else if (tc && gemm_tc_supported(n_tok, D, hd, hd, hd)) {
     BCK(launch_gemm_tc_resid(P->att, hd, B->wo_t, hd, P->x1, D, n_tok, D, hd, x, D, B->d_status, B->st));
-  } else if (n_tok == 1 && hd % 8 == 0) {  // one token: bandwidth-bound GEMV
+  } else if (n_tok == 1 && hd % 8 == 0) {  // one token, K not a multiple of 64
     BCK(launch_gemv_resid(P->att, B->wo_t, D, hd, x, P->x1, B->st));
   } else {
     gemm_resid_naive_kernel<<<dim3((D + 127) / 128, n_tok), 128, 0, B->st>>>(P->att, B->wo_t, x, P->x1, n_tok, D, hd);
     BCK(cudaGetLastError());
   }
   // h2 = RMSNorm(x1; g2)
-  rmsnorm_kernel<<<nblk, rows_per_blk * 32, 0, B->st>>>(P->x1, B->g2, P->h, n_tok, D, B->eps);
-  BCK(cudaGetLastError());
+  BCK(launch_rmsnorm(P->x1, B->g2, P->h, n_tok, D, B->eps, B->st, pdl));
   // act = silu(h2 W_gate) * (h2 W_up)
-  if (tc && gemm_tc_gated_supported(n_tok, 2 * F, D, D, D)) {
+  if (skinny_use(n_tok, 2 * F, D, D, D)) {
+    BCK(launch_skinny_gated(P->h, D, B->wgu_t, D, P->act, n_tok, F, D, B->d_status, B->st, pdl));
+  } else if (tc && gemm_tc_gated_supported(n_tok, 2 * F, D, D, D)) {
     BCK(launch_gemm_tc_gated(P->h, D, B->wgu_t, D, P->act, F, n_tok, 2 * F, D, B->d_status, B->st));
   } else if (n_tok == 1) {
     BCK(launch_gemv_gated(P->h, B->wgu_t, F, D, P->act, B->st));
@@ -266,8 +327,10 @@ int locret_block_prefill_chunk(locret_block *B, const void *x_in, int32_t n_tok,
     swiglu_kernel<<<(unsigned)((n + 255) / 256), 256, 0, B->st>>>(P->gu, P->act, n_tok, F);
     BCK(cudaGetLastError());
   }
-  // y = x1 + act W_down
-  if (tc && gemm_tc_supported(n_tok, D, F, F, F)) {
+  // y = x1 + act W_down  (d_ff is a multiple of 128, so the fallbacks of W_o are not needed)
+  if (skinny_use(n_tok, D, F, F, F)) {
+    BCK(launch_skinny_gemm(P->act, F, B->wd_t, F, y, D, n_tok, D, F, P->x1, D, B->d_status, B->st, pdl));
+  } else if (tc && gemm_tc_supported(n_tok, D, F, F, F)) {
     BCK(launch_gemm_tc_resid(P->act, F, B->wd_t, F, y, D, n_tok, D, F, P->x1, D, B->d_status, B->st));
   } else if (n_tok == 1) {
     BCK(launch_gemv_resid(P->act, B->wd_t, D, F, P->x1, y, B->st));

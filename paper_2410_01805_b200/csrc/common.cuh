@@ -184,6 +184,20 @@ cudaError_t launch_rh_gemm_tc(const bf16 *A, int lda, const bf16 *W1t, const flo
                               cudaStream_t st);
 int rh_tc_num_tiles(int d_R);
 
+// Projections of a few tokens (skinny.cu): the weights stream once, the tokens are the narrow side.
+//   gemm:  Y [n_tok x N] = X Wt^T (+ R, added before the one rounding; R may be null)
+//   gated: act [n_tok x F] = silu(X Wg) * (X Wu), Wt [2F x K] in the interleaved layout of launch_gemm_tc_gated
+//   rh:    partial[tile][n_tok][h_kv], as launch_rh_gemm_tc, in tiles of 128 rows of W1t
+// use: the rule by which a call takes this path and not the GEMM of gemm_tc.cu
+bool skinny_use(int n_tok, int N, int K, int ldx, int ldw);
+bool skinny_supported(int n_tok, int N, int K, int ldx, int ldw);
+cudaError_t launch_skinny_gemm(const bf16 *X, int ldx, const bf16 *Wt, int ldw, bf16 *Y, int ldy, int n_tok, int N, int K,
+                               const bf16 *R, int ldr, int *status, cudaStream_t st, bool pdl = false);
+cudaError_t launch_skinny_gated(const bf16 *X, int ldx, const bf16 *Wt, int ldw, bf16 *act, int n_tok, int F, int K,
+                                int *status, cudaStream_t st, bool pdl = false);
+cudaError_t launch_skinny_rh(const bf16 *Z, int ldz, const bf16 *W1t, const float *W2, float *partial, int n_tok, int d_R,
+                             int K, int h_kv, int act, int *n_tiles, int *status, cudaStream_t st);
+
 // scores[m][slot0 + t] = sum_nt partial[nt][t][m]
 cudaError_t launch_rh_reduce(const float *partial, int n_tiles, int M, int h_kv, float *scores,
                              int score_stride, int slot0, cudaStream_t st, const PerHead *slot0_m = nullptr);

@@ -603,7 +603,9 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   ra.per_head = L->per_head ? 1 : 0;
   ra.len_m = L->len_m;
   // with a tensor-core projection whose width is a whole number of tiles the epilogue of the GEMM does the RoPE pass
-  const bool fused_rope = !decode && !L->per_head && L->fuse_rope && L->use_tc && n_tok >= 32 &&
+  // (few tokens: the projection that divides K over a cluster, and the RoPE pass)
+  const bool skinny = !decode && L->use_tc && skinny_use(n_tok, L->d_in, L->D, L->D, L->D);
+  const bool fused_rope = !decode && !skinny && !L->per_head && L->fuse_rope && L->use_tc && n_tok >= 32 &&
                           qkv_rope_tc_supported(n_tok, L->d_in, L->D, L->D, L->D, L->d);
   const bool deq = L->int4 && L->len > 0 && !decode;
   if (deq) {
@@ -623,6 +625,9 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
     Timed t(L, LOCRET_K_QKV);
     if (decode)  // projection, positions, RoPE and append of the one token in one kernel
       CK(launch_gemv_rope((const bf16 *)hidden_in, L->wqkv_t, L->D, staging, ra, L->st, pdl));
+    else if (skinny)
+      CK(launch_skinny_gemm((const bf16 *)hidden_in, L->D, L->wqkv_t, L->D, staging, L->d_in, n_tok, L->d_in, L->D,
+                            nullptr, 0, L->d_status + 1, L->st));
     else if (fused_rope)
       CK(launch_qkv_rope_tc((const bf16 *)hidden_in, L->D, L->wqkv_t, L->D, staging, n_tok, L->d_in, L->D,
                             ra, L->d_status + 1, L->st));
@@ -742,6 +747,9 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
     if (decode)
       CK(launch_rh_gemv(z, L->w1_t, L->w2f, P->partial, L->d_R, L->d_in, L->h_kv, L->cfg.act, P->dec_cnt,
                         L->s + L->len, L->cap, S, pdl));
+    else if (L->use_tc && skinny_use(n_tok, L->d_R, L->d_in, L->d_in, L->d_in))
+      CK(launch_skinny_rh(z, L->d_in, L->w1_t, L->w2f, P->partial, n_tok, L->d_R, L->d_in, L->h_kv, L->cfg.act, &n_tiles,
+                          L->d_status + 3, S));
     else if (L->use_tc && n_tok >= 32 && gemm_tc_supported(n_tok, L->d_R, L->d_in, L->d_in, L->d_in))
       CK(launch_rh_gemm_tc(z, L->d_in, L->w1_t, L->w2f, P->partial, n_tok, L->d_R, L->d_in, L->h_kv,
                            L->cfg.act, &n_tiles, L->d_status + 3, S));
