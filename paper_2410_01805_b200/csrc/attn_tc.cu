@@ -36,6 +36,7 @@ constexpr int TILE = 128;               // query rows per tile and keys per tile
 constexpr int HD = 128;                 // column pitch of a head in shared and tensor memory
 constexpr int HALF_BYTES = TILE * 128;  // one 64-column swizzled box of 128 rows: 16 KB
 constexpr int TILE_BYTES = 2 * HALF_BYTES;
+constexpr int MAX_SPLIT = 8;            // portable cluster size
 constexpr int AT_SMEM = 1024 + 6 * TILE_BYTES + 256 + 2048;  // Q0,Q1,K0,K1,V0,V1 + barriers + softmax exchange
 // The accumulator is rescaled only when a row's maximum has grown by more than 2^100 since the
 // scale in use was fixed.  P is stored as bf16 and O, l accumulate in fp32, both with an 8-bit
@@ -44,6 +45,7 @@ constexpr int AT_SMEM = 1024 + 6 * TILE_BYTES + 256 + 2048;  // Q0,Q1,K0,K1,V0,V
 // trigger a rescale (a TMEM round trip on the critical path) at almost every tile that holds one
 // of the workload's 20x-norm outlier keys.
 constexpr float RESCALE_LOG2 = 100.0f;
+constexpr float NO_KEY = -1e30f;  // SPLIT: maximum of a row that has not seen a key yet
 constexpr int PF = 6;       // key tiles prefetched into L2 ahead of the shared-memory pipeline
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -85,9 +87,16 @@ struct AttnParams {
   int *status;
   int per_head;   // a budget per head: KV head m holds len_m.v[m] retained units
   PerHead len_m;
+  int n_split;    // SPLIT: CTAs of a cluster, each with its share of the key tiles
 };
 
-template <int D>
+// SPLIT: a cluster of n_split CTAs shares one pair of query tiles and divides its key tiles in
+// contiguous ranges, for calls with too few query tiles to fill the GPU.  Each CTA leaves its
+// unnormalised accumulator (as [column][row]), row maxima and row sums in its shared memory, and
+// rank r combines its share of the columns over all ranks in rank order.  Bound by latency, not by the key tiles:
+// 45 tokens over 4500 cached keys of the Llama shape take 29 us in 16 clusters of eight (five key tiles each);
+// the mma.sync kernel that took fewer than 64 tokens before needs 124 us (32 CTAs, all keys in sequence).
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
@@ -116,29 +125,35 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
 
   // which two query tiles; longest key ranges first
   int row0[2], head[2];
+  const int n_split = SPLIT ? p.n_split : 1;
+  const int unit = SPLIT ? (int)blockIdx.x / n_split : (int)blockIdx.x;
+  const int rank = SPLIT ? (int)blockIdx.x - unit * n_split : 0;
   if (p.pair_heads) {
     const int hp = p.h / 2;
-    const int rb = n_rb - 1 - (int)blockIdx.x / hp;
-    const int hq = (int)blockIdx.x % hp;
+    const int rb = n_rb - 1 - unit / hp;
+    const int hq = unit % hp;
     row0[0] = row0[1] = rb * TILE;
     head[0] = 2 * hq; head[1] = 2 * hq + 1;
   } else {
     const int n_rp = (n_rb + 1) / 2;
-    const int rp = n_rp - 1 - (int)blockIdx.x / p.h;
+    const int rp = n_rp - 1 - unit / p.h;
     row0[0] = rp * 2 * TILE; row0[1] = row0[0] + TILE;
-    head[0] = head[1] = (int)blockIdx.x % p.h;
+    head[0] = head[1] = unit % p.h;
   }
   const int kvh = head[0] / g;
   const int len = p.per_head ? p.len_m.v[kvh] : p.len;   // retained units of this KV head
   const int n = len + p.n_tok;
   int NK = (len + row0[1] + TILE + TILE - 1) / TILE;
   NK = min(NK, (n + TILE - 1) / TILE);
+  const int tile_lo = SPLIT ? (int)((long long)rank * NK / n_split) : 0;  // (a share may be empty)
+  if (SPLIT) NK = (int)((long long)(rank + 1) * NK / n_split) - tile_lo;
   // The softmax is order independent, so every CTA walks the key tiles that need no mask in its
   // own rotated order: CTAs of one KV head start together, and in a common order they would all
   // ask the L2 for the same K and V lines at the same moment (measured: 1.4x slower).
-  const int NF = min(NK, (len + row0[0] + 1) / TILE);  // tiles fully visible to every row
+  // (the CTAs of a cluster are on different tiles anyway)
+  const int NF = SPLIT ? 0 : min(NK, (len + row0[0] + 1) / TILE);  // tiles fully visible to every row
   const int rot = NF > 0 ? (int)((blockIdx.x * 29u + 7u) % (unsigned)NF) : 0;
-  auto tile_of = [&](int j) { int x = j + rot; return j < NF ? (x >= NF ? x - NF : x) : j; };
+  auto tile_of = [&](int j) { int x = j + rot; return SPLIT ? tile_lo + j : (j < NF ? (x >= NF ? x - NF : x) : j); };
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
@@ -239,8 +254,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         }
       };
       bool ok = mbar_wait(q_full, 0, abort_flag, p.status);
-      ok = ok && mbar_wait(&k_full[0], 0, abort_flag, p.status);
-      if (ok) {
+      if (!SPLIT || NK > 0) ok = ok && mbar_wait(&k_full[0], 0, abort_flag, p.status);
+      if (ok && (!SPLIT || NK > 0)) {
         tc_fence_after();
         issue_s(0);
       }
@@ -265,6 +280,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         }
       }
     }
+  }
+  if (SPLIT) {  // (the softmax warps' two meetings of the cluster)
+    __syncwarp();
+    cluster_sync_all();
+    cluster_sync_all();
   }
   } else {
     // ------------------------------------------------------------ softmax: all eight warps work
@@ -323,6 +343,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         xch[(t * 2 + hf) * TILE + r] = tmax;
         pair_sync();
         tmax = fmaxf(tmax, xch[(t * 2 + (hf ^ 1)) * TILE + r]) * c;
+        if (SPLIT) tmax = fmaxf(tmax, NO_KEY);  // a share's first tile may lie wholly behind the causal boundary
 
         if (j == 0) {
           m_used[t] = tmax;
@@ -380,6 +401,73 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       }
     }
 
+    if (SPLIT) {
+      // every product of both tiles is complete and every loaded tile consumed: the stages are free
+      if (ok && NK > 0) ok = mbar_wait(&o_full[0], (NK - 1) & 1, abort_flag, p.status);
+      if (ok && NK > 0) ok = mbar_wait(&o_full[1], (NK - 1) & 1, abort_flag, p.status);
+      tc_fence_after();
+      float *so = reinterpret_cast<float *>(smem);                            // [tile][column][row]
+      float *sm = reinterpret_cast<float *>(smem + 2 * D * TILE * 4);         // [tile][row] maxima, then sums
+#pragma unroll
+      for (int t = 0; t < 2; t++) {
+        const uint32_t o_addr = tmem_base + lane_off + 2 * TILE + t * HD;
+        xch[(t * 2 + hf) * TILE + r] = l[t];
+        pair_sync();
+        if (hf == 0) {
+          sm[t * TILE + r] = m_used[t];
+          sm[(2 + t) * TILE + r] = l[t] + xch[(t * 2 + 1) * TILE + r];
+        }
+        if (ok && NK > 0) {
+#pragma unroll 1
+          for (int q = hf; q < D / 32; q += 2) {
+            uint32_t o[32];
+            tmem_ld32(o_addr + q * 32, o);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 32; i++) so[(t * D + q * 32 + i) * TILE + r] = __uint_as_float(o[i]);
+          }
+        }
+      }
+      cluster_sync_all();
+      // this rank's share of the columns, four at a time; lanes along rows
+      constexpr int G = D / 4;
+      const int g_lo = rank * G / n_split, g_hi = (rank + 1) * G / n_split;
+      const uint32_t so_a = smem_u32(so), sm_a = smem_u32(sm);
+      for (int i = threadIdx.x; i < (g_hi - g_lo) * 2 * TILE; i += 256) {
+        const int tr = i & (2 * TILE - 1), t = tr >> 7, c0 = (g_lo + i / (2 * TILE)) * 4;
+        const int row = row0[t] + (tr & (TILE - 1));
+        if (row >= p.n_tok) continue;
+        // (unrolled over the largest cluster: every remote load is in flight before the first is used)
+        float mk[MAX_SPLIT], lk[MAX_SPLIT], ok4[MAX_SPLIT][4];
+        float mx = NO_KEY;
+#pragma unroll
+        for (int k = 0; k < MAX_SPLIT; k++) {
+          mk[k] = NO_KEY;
+          if (k >= n_split) continue;
+          const uint32_t ma = cluster_map(sm_a, k) + tr * 4;
+          const uint32_t oa = cluster_map(so_a, k) + (uint32_t)((t * D + c0) * TILE + (tr & (TILE - 1))) * 4;
+          mk[k] = ld_cluster_f1(ma);
+          lk[k] = ld_cluster_f1(ma + 2 * TILE * 4);
+#pragma unroll
+          for (int e = 0; e < 4; e++) ok4[k][e] = ld_cluster_f1(oa + e * TILE * 4);
+        }
+#pragma unroll
+        for (int k = 0; k < MAX_SPLIT; k++) mx = fmaxf(mx, mk[k]);
+        float acc[4] = {0.f, 0.f, 0.f, 0.f}, ls = 0.f;
+#pragma unroll
+        for (int k = 0; k < MAX_SPLIT; k++) {
+          if (!(mk[k] > NO_KEY)) continue;  // (a share without a key for this row, or none at all)
+          const float w = exp2f(mk[k] - mx);
+          ls = fmaf(w, lk[k], ls);
+#pragma unroll
+          for (int e = 0; e < 4; e++) acc[e] = fmaf(w, ok4[k][e], acc[e]);
+        }
+        const float inv = 1.0f / ls;
+        *reinterpret_cast<uint2 *>(p.out + (size_t)row * p.h * D + (size_t)head[t] * D + c0) =
+            make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
+      }
+      cluster_sync_all();  // no CTA leaves while another may still read its share
+    } else {
 #pragma unroll
     for (int t = 0; t < 2; t++) {
       const int row = row0[t] + r;
@@ -410,6 +498,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         }
       }
     }
+    }
   }
 
   tc_fence_before();
@@ -424,18 +513,70 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
 }  // namespace
 
 bool attention_tc_supported(int n_tok, int h, int h_kv, int d) {
-  return (d == 64 || d == 96 || d == 128) && n_tok >= 64 && h % h_kv == 0;
+  return (d == 64 || d == 96 || d == 128) && n_tok >= 2 && h % h_kv == 0;
+}
+
+namespace {
+
+// Clusters of `size` CTAs of the split kernel that are resident at once on the current device (0: the size cannot be
+// launched), asked for once per device and size.
+template <int D>
+int resident_clusters(int size) {
+  static int known[MAX_DEVICES][MAX_SPLIT + 1] = {};  // 0: not asked for yet; value + 1
+  int dev = 0;
+  if (current_device_index(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
+  if (known[dev][size] == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(AT_THREADS);
+    cfg.dynamicSmemBytes = AT_SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, true>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    known[dev][size] = n + 1;
+  }
+  return known[dev][size] - 1;
 }
 
 // map_k / map_v: 3-D maps {d, cap, h_kv} with box {64, 128, 1}; map_q: 2-D {h*d, rows} box {64, 128}.
 template <int D>
-static cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, const CUtensorMap *map_v,
-                                 const AttnParams &p, int grid, cudaStream_t st) {
-  static PerDeviceFlag attr_set;
-  if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D>, AT_SMEM, attr_set); e != cudaSuccess) return e;
-  attn_tc_kernel<D><<<grid, AT_THREADS, AT_SMEM, st>>>(*map_q, *map_k, *map_v, p);
-  return cudaGetLastError();
+cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, const CUtensorMap *map_v, AttnParams &p,
+                          int grid, int len_max, cudaStream_t st) {
+  static PerDeviceFlag attr_set, attr_set_split;
+  if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, false>, AT_SMEM, attr_set); e != cudaSuccess) return e;
+  if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, true>, AT_SMEM, attr_set_split); e != cudaSuccess) return e;
+  // The key tiles are divided when that keeps all CTAs resident at once; the share then takes about two tiles' time
+  // more for the combination.  (With more than one wave of clusters it lost: 1428 tokens over 3072 cached keys of the
+  // Llama shape, 192 CTAs, took 168 us in clusters of two and 104 us undivided.)
+  const int nk = (len_max + p.n_tok + TILE - 1) / TILE;
+  int best = 1, best_cost = nk;
+  for (int s = 2; s <= MAX_SPLIT && s <= nk && grid * s <= sm_count_of_current_device(); s++) {
+    const int cost = (nk + s - 1) / s + 2;
+    if (cost < best_cost && grid <= resident_clusters<D>(s)) { best = s; best_cost = cost; }
+  }
+  p.n_split = best;
+  if (best == 1) {
+    attn_tc_kernel<D, false><<<grid, AT_THREADS, AT_SMEM, st>>>(*map_q, *map_k, *map_v, p);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid * best);
+  cfg.blockDim = dim3(AT_THREADS);
+  cfg.dynamicSmemBytes = AT_SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = best; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, true>, *map_q, *map_k, *map_v, static_cast<const AttnParams>(p));
 }
+
+}  // namespace
 
 cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map_k,
                                 const CUtensorMap *map_v, bf16 *out, int n_tok, int h, int h_kv, int d,
@@ -449,10 +590,13 @@ cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map
   p.status = status;
   const int n_rb = (n_tok + TILE - 1) / TILE;
   const int grid = p.pair_heads ? n_rb * (h / 2) : ((n_rb + 1) / 2) * h;
+  int len_max = len;
+  if (len_m)
+    for (int m = 0; m < h_kv; m++) len_max = len_m->v[m] > len_max ? len_m->v[m] : len_max;
   switch (d) {
-    case 64: return launch_attn_d<64>(map_q, map_k, map_v, p, grid, st);
-    case 96: return launch_attn_d<96>(map_q, map_k, map_v, p, grid, st);
-    case 128: return launch_attn_d<128>(map_q, map_k, map_v, p, grid, st);
+    case 64: return launch_attn_d<64>(map_q, map_k, map_v, p, grid, len_max, st);
+    case 96: return launch_attn_d<96>(map_q, map_k, map_v, p, grid, len_max, st);
+    case 128: return launch_attn_d<128>(map_q, map_k, map_v, p, grid, len_max, st);
   }
   return cudaErrorInvalidValue;
 }
