@@ -379,8 +379,8 @@ void locret_block_destroy(locret_block *block);
  * after RoPE); k_prompt: device bf16 [n_q × h_kv × d]; labels: device fp32 [h_kv × n_q]
  * (overwritten).  The passage prints the product without the 1/sqrt(d) of Eq. 1: scale = 1
  * reproduces it as printed; scale must be > 0.  head_dim 64, 96 or 128; pointers 16-byte aligned.
- * One tensor-core contraction per query head whose epilogue keeps only row maxima (the
- * n_q × n_a score matrix is never written).  Synchronises the stream before it returns.
+ * A tensor-core contraction whose epilogue keeps only row maxima (the n_q × n_a score matrix is
+ * never written).  Synchronises the stream before it returns.
  */
 int locret_cis_labels(const void *q_ans, const void *k_prompt, int32_t n_a, int32_t n_q, int32_t h,
                       int32_t h_kv, int32_t d, float scale, float *labels, void *stream);
@@ -395,12 +395,22 @@ int locret_cis_labels(const void *q_ans, const void *k_prompt, int32_t n_a, int3
  * device: loss (one fp32), d_w1 fp32 [d_in × d_R], d_w2 fp32 [d_R × h_kv] (all overwritten).
  * Requires n, d_in multiples of 64, d_R a multiple of 32, h_kv <= 32, alpha >= 0.  The two
  * large contractions take bf16 operands (dpre is rounded to bf16) and accumulate in fp32.
- * Allocates and frees its workspace (about n·(4 d_R + 2 d_in + 2 d_R) bytes) inside the call and
- * synchronises the stream before it returns.
+ * Allocates and frees its workspace (about n·6 d_R bytes) inside the call and synchronises the stream
+ * before it returns.
  */
 int locret_rh_loss_grad(const void *z, const float *labels, const void *w1, const void *w2, int32_t n,
                         int32_t d_in, int32_t d_R, int32_t h_kv, float alpha, float *loss, float *d_w1,
                         float *d_w2, void *stream);
+
+/*
+ * The same in a workspace of the caller's (device memory, 16-byte aligned, at least the bytes that
+ * locret_rh_loss_grad_workspace reports; contents need not be kept between calls): allocating and freeing it
+ * inside every call costs more than the call's kernels.  LOCRET_ERR_CAPACITY if it is too small.
+ */
+int locret_rh_loss_grad_workspace(int32_t n, int32_t d_R, int32_t h_kv, int64_t *bytes);
+int locret_rh_loss_grad_ws(const void *z, const float *labels, const void *w1, const void *w2, int32_t n,
+                           int32_t d_in, int32_t d_R, int32_t h_kv, float alpha, float *loss, float *d_w1,
+                           float *d_w2, void *workspace, int64_t workspace_bytes, void *stream);
 
 /*
  * One AdamW update of a parameter array (Appendix A: AdamW, learning rate 5e-4 with a linear

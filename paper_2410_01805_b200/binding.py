@@ -85,6 +85,9 @@ def _load():
     l.locret_block_destroy.argtypes = [P]
     l.locret_block_destroy.restype = None
     l.locret_rh_loss_grad.argtypes = [P, P, P, P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_float, P, P, P, P]
+    l.locret_rh_loss_grad_workspace.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int64)]
+    l.locret_rh_loss_grad_ws.argtypes = [P, P, P, P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_float, P, P, P, P,
+                                         C.c_int64, P]
     l.locret_adamw_step.argtypes = [P, P, P, P, P, C.c_int64, C.c_int32, C.c_float, C.c_float, C.c_float, C.c_float, C.c_float, P]
     l.locret_cis_labels.argtypes = [P, P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_float, P, P]
     return l
@@ -451,9 +454,13 @@ def rh_loss_grad(z: torch.Tensor, labels: torch.Tensor, w1: torch.Tensor, w2: to
     loss = torch.empty((), dtype=torch.float32, device=z.device)
     d_w1 = torch.empty((d_in, d_R), dtype=torch.float32, device=z.device)
     d_w2 = torch.empty((d_R, h_kv), dtype=torch.float32, device=z.device)
-    _check(lib.locret_rh_loss_grad(z.data_ptr(), labels.data_ptr(), w1.data_ptr(), w2.data_ptr(), n, d_in, d_R, h_kv,
-                                   float(alpha), loss.data_ptr(), d_w1.data_ptr(), d_w2.data_ptr(),
-                                   torch.cuda.current_stream().cuda_stream), "locret_rh_loss_grad")
+    need = C.c_int64()
+    _check(lib.locret_rh_loss_grad_workspace(n, d_R, h_kv, C.byref(need)), "locret_rh_loss_grad")
+    # (from torch's caching allocator, like the results: the call is synchronous, so the block is free again after it)
+    ws = torch.empty(need.value, dtype=torch.uint8, device=z.device)
+    _check(lib.locret_rh_loss_grad_ws(z.data_ptr(), labels.data_ptr(), w1.data_ptr(), w2.data_ptr(), n, d_in, d_R, h_kv,
+                                      float(alpha), loss.data_ptr(), d_w1.data_ptr(), d_w2.data_ptr(), ws.data_ptr(),
+                                      need.value, torch.cuda.current_stream().cuda_stream), "locret_rh_loss_grad")
     return loss, d_w1, d_w2
 
 

@@ -155,10 +155,12 @@ cudaError_t launch_gemm_tc_resid(const bf16 *A, int lda, const bf16 *Bt, int ldb
                                  int N, int K, const bf16 *R, int ldr, int *status, cudaStream_t st);
 // first half of a gated FFN: C[M x N/2] = silu(A Wg) * (A Wu); Bt [N x K] interleaves, per block of
 // 128 outputs, 128 rows of Wg^T and 128 rows of Wu^T
-// out[m] = max(out[m], scale * max_n (A Bt^T)[m][n]): row maxima merged with atomics (out fp32,
-// initialised by the caller); K % 64 == 0, lda / ldb multiples of 8, scale > 0
-cudaError_t launch_gemm_tc_rowmax(const bf16 *A, int lda, const bf16 *Bt, int ldb, float *out, int M, int N,
-                                  int K, float scale, int *status, cudaStream_t st);
+// training of the retaining head (operands as they lie, see gemm_tc.cu): pre-activations with partial scores, and A^T B
+int rh_pre_num_tiles(int d_R);
+cudaError_t launch_rh_pre_tc(const bf16 *Z, int ldz, const bf16 *W1, int ldw, float *pre, const float *W2, float *partial,
+                             int M, int d_R, int K, int h_kv, int *status, cudaStream_t st);
+cudaError_t launch_gemm_tn_f32(const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int M, int N, int K,
+                               int *status, cudaStream_t st);
 // C (fp32, leading dimension ldc in floats) = A Bt^T
 // heads divided over GPUs: this GPU's partial first product of the retaining head (fallback for
 // shapes the tensor-core GEMM does not take), and scores from the summed product

@@ -4,8 +4,8 @@
 // accumulator from TMEM and run the epilogue:
 //   MODE 0: bf16 store (the QKV projection);
 //   MODE 1: the retaining head's activation and its second, thin GEMM with W2, written as one
-//           partial score per (N-tile, row, KV head)                       (Section 3.3).
-#include <cstring>
+//           partial score per (N-tile, row, KV head)                       (Section 3.3);
+//   the other modes are described at their branches.
 #include "tc_common.cuh"
 
 namespace locret {
@@ -99,6 +99,7 @@ using namespace tc;
 
 constexpr int BM = 128, BK = 64, GT_THREADS = 192;
 constexpr int MAX_HKV = 32;
+constexpr int MN_BOX = 64 * BK * 2;           // an MN-major box: 64 rows of K, 64 columns
 constexpr int EPI_WARP_BYTES = 32 * 128 * 2;  // 32 rows of a head of up to 128 bf16
 
 // sigma of the retaining head with the fast division / exponential intrinsics (relative error
@@ -118,11 +119,13 @@ struct GemmCfg {
   static constexpr int EPI_BYTES = 4 * EPI_WARP_BYTES;  // MODE 2: one staged head of 32 rows per warp
   // 1024 for alignment slack, barriers + tmem pointer in a small tail
   static constexpr int smem_bytes(int mode) {
-    return 1024 + STAGES * STAGE_BYTES + (mode == 1 ? W2_BYTES : (mode == 2 ? EPI_BYTES : 0)) + 256;
+    return 1024 + STAGES * STAGE_BYTES + (mode == 1 || mode == 7 ? W2_BYTES : (mode == 2 ? EPI_BYTES : 0)) + 256;
   }
 };
 
-template <int BN, int MODE, int HD = 0>
+// MAJOR: bit 0, A is stored [K x M]; bit 1, B is stored [K x N] (tcgen05 reads such "MN-major" operands as they lie,
+// in swizzled boxes of 64 columns x 64 rows of K).
+template <int BN, int MODE, int HD = 0, int MAJOR = 0>
 __global__ void __launch_bounds__(GT_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                bf16 *__restrict__ C, int ldc, int M, int N, int K, const float *__restrict__ W2,
@@ -140,7 +143,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   float *sW2 = reinterpret_cast<float *>(tiles + STAGES * Cfg::STAGE_BYTES);
   unsigned char *sEpi = tiles + STAGES * Cfg::STAGE_BYTES;
   unsigned char *tail = tiles + STAGES * Cfg::STAGE_BYTES +
-                        (MODE == 1 ? Cfg::W2_BYTES : (MODE == 2 ? Cfg::EPI_BYTES : 0));
+                        (MODE == 1 || MODE == 7 ? Cfg::W2_BYTES : (MODE == 2 ? Cfg::EPI_BYTES : 0));
   uint64_t *full = reinterpret_cast<uint64_t *>(tail);
   uint64_t *empty = full + STAGES;
   uint64_t *acc_full = empty + STAGES;   // [2]
@@ -192,14 +195,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (!ok) break;
           mbar_expect_tx(&full[s], Cfg::STAGE_BYTES);
           unsigned char *a_dst = tiles + s * Cfg::STAGE_BYTES;
-          tma_load_2d(a_dst, &map_a, kb * BK, m0, &full[s]);
-          tma_load_2d(a_dst + Cfg::A_BYTES, &map_b, kb * BK, n0, &full[s]);
+          if (MAJOR & 1) {
+#pragma unroll
+            for (int i = 0; i < BM / 64; i++) tma_load_2d(a_dst + i * MN_BOX, &map_a, m0 + i * 64, kb * BK, &full[s]);
+          } else {
+            tma_load_2d(a_dst, &map_a, kb * BK, m0, &full[s]);
+          }
+          if (MAJOR & 2) {
+#pragma unroll
+            for (int i = 0; i < BN / 64; i++)
+              tma_load_2d(a_dst + Cfg::A_BYTES + i * MN_BOX, &map_b, n0 + i * 64, kb * BK, &full[s]);
+          } else {
+            tma_load_2d(a_dst + Cfg::A_BYTES, &map_b, kb * BK, n0, &full[s]);
+          }
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16(BM, BN, 0, 0);
+      constexpr uint32_t idesc = idesc_bf16(BM, BN, MAJOR & 1, MAJOR >> 1);
+      constexpr uint64_t a_step = ((MAJOR & 1) ? 16 * 128 : 32) >> 4, b_step = ((MAJOR & 2) ? 16 * 128 : 32) >> 4;
       uint32_t it = 0, lt = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, lt++) {
@@ -215,11 +230,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (!ok) break;
           tc_fence_after();
           unsigned char *a_src = tiles + s * Cfg::STAGE_BYTES;
-          const uint64_t da = desc_kmajor_sw128(a_src), db = desc_kmajor_sw128(a_src + Cfg::A_BYTES);
+          const uint64_t da = (MAJOR & 1) ? desc_mnmajor_sw128(a_src, MN_BOX) : desc_kmajor_sw128(a_src);
+          const uint64_t db = (MAJOR & 2) ? desc_mnmajor_sw128(a_src + Cfg::A_BYTES, MN_BOX)
+                                          : desc_kmajor_sw128(a_src + Cfg::A_BYTES);
 #pragma unroll
           for (int k = 0; k < BK / 16; k++) {
             if (kb == 0 && k == 0) mma_ss_first(d_tmem, da, db, idesc);
-            else mma_ss_acc(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc);
+            else mma_ss_acc(d_tmem, da + (uint64_t)k * a_step, db + (uint64_t)k * b_step, idesc);
           }
           mma_commit(&empty[s]);  // frees the stage once these MMAs have read it
         }
@@ -238,7 +255,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       tile_mn(tile, m0, n0);
       const uint32_t buf = lt & 1;
       const int row = m0 + quarter * 32 + lane;
-      if (MODE == 1) {
+      if (MODE == 1 || MODE == 7) {
         // this tile's slice of W2; the named barrier keeps the four warps together around it
         asm volatile("bar.sync 1, 128;" ::: "memory");
         for (int v = etid; v < BN * h_kv; v += 128) {
@@ -331,32 +348,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                                : "memory");
               }
             }
-          }
-        }
-      } else if (MODE == 4) {
-        // Row maximum of A B^T over the valid columns, merged into out[row] with an atomic
-        // maximum on the order-preserving integer image of the float (`partial` is the output,
-        // `act` carries the bits of the scale factor): the labels of Section 3.3.
-        if (ok) {
-          const float scale = __int_as_float(act);
-          float mx = -INFINITY;
-#pragma unroll 1
-          for (int c0 = 0; c0 < BN; c0 += 32) {
-            uint32_t r[32];
-            tmem_ld32(taddr + c0, r);
-            tmem_wait_ld();
-            if (n0 + c0 < N) {
-#pragma unroll
-              for (int i = 0; i < 32; i++)
-                if (n0 + c0 + i < N) mx = fmaxf(mx, __uint_as_float(r[i]));
-            }
-          }
-          if (row < M && mx > -INFINITY) {
-            mx *= scale;
-            if (mx == 0.f) mx = 0.f;  // -0 would order below every negative as an integer
-            float *dst = partial + row;
-            if (mx >= 0.f) atomicMax(reinterpret_cast<int *>(dst), __float_as_int(mx));
-            else atomicMin(reinterpret_cast<unsigned int *>(dst), __float_as_uint(mx));
           }
         }
       } else if (MODE == 3) {
@@ -499,8 +490,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             // activation of the 32 columns first (independent, so the special-function unit
             // pipelines them), then the thin GEMM with W2 as broadcast 16-byte loads
             float a[32];
+            if (MODE == 7) {  // training: the pre-activations are kept, and SiLU divides exactly
+              if (row < M && n0 + c0 < N) {
+                float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(C) + (size_t)row * ldc + n0 + c0);
 #pragma unroll
-            for (int i = 0; i < 32; i++) a[i] = fast_act(__uint_as_float(r[i]), act);
+                for (int v = 0; v < 8; v++)
+                  dst[v] = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
+                                       __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3]));
+              }
+#pragma unroll
+              for (int i = 0; i < 32; i++) a[i] = apply_act(__uint_as_float(r[i]), 0);
+            } else {
+#pragma unroll
+              for (int i = 0; i < 32; i++) a[i] = fast_act(__uint_as_float(r[i]), act);
+            }
             if (h_kv == 8) {
 #pragma unroll
               for (int i = 0; i < 32; i++) {
@@ -558,18 +561,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   }
 }
 
-template <int BN, int MODE, int HD = 0>
+template <int BN, int MODE, int HD = 0, int MAJOR = 0>
 cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M, int N,
                      int K, const float *W2, float *partial, int h_kv, int act, const RopeAppendArgs &ra,
                      int *status, cudaStream_t st, const bf16 *resid = nullptr, int ldr = 0) {
   using Cfg = GemmCfg<BN>;
   static PerDeviceFlag attr_set;
-  if (cudaError_t e = allow_dynamic_smem(gemm_tc_kernel<BN, MODE, HD>, Cfg::smem_bytes(MODE), attr_set);
+  if (cudaError_t e = allow_dynamic_smem(gemm_tc_kernel<BN, MODE, HD, MAJOR>, Cfg::smem_bytes(MODE), attr_set);
       e != cudaSuccess)
     return e;
   CUtensorMap ma, mb;
-  if (!cached_map_k64(&ma, A, K, M, (uint64_t)lda * 2, BM) || !cached_map_k64(&mb, Bt, K, N, (uint64_t)ldb * 2, BN))
-    return cudaErrorInvalidValue;
+  const bool a_ok = (MAJOR & 1) ? cached_map_k64(&ma, A, M, K, (uint64_t)lda * 2, BK)
+                                : cached_map_k64(&ma, A, K, M, (uint64_t)lda * 2, BM);
+  const bool b_ok = (MAJOR & 2) ? cached_map_k64(&mb, Bt, N, K, (uint64_t)ldb * 2, BK)
+                                : cached_map_k64(&mb, Bt, K, N, (uint64_t)ldb * 2, BN);
+  if (!a_ok || !b_ok) return cudaErrorInvalidValue;
   const int num_sms = sm_count_of_current_device();
   const int total = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
   const int grid = total < num_sms ? total : num_sms;
@@ -577,8 +583,8 @@ cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, i
   // from HBM once; in row-block-major order a B that exceeds the L2 is re-read for every row
   // block, and even one that fits is read about three times)
   const size_t a_bytes = (size_t)M * K * 2, b_bytes = (size_t)N * K * 2;
-  const int n_major = MODE != 1 && b_bytes > a_bytes;  // (MODE 1 indexes its partial sums by column tile either way)
-  gemm_tc_kernel<BN, MODE, HD><<<grid, GT_THREADS, Cfg::smem_bytes(MODE), st>>>(
+  const int n_major = MODE != 1 && MODE != 7 && b_bytes > a_bytes;  // (MODE 1 and 7 index their partial sums by column tile either way)
+  gemm_tc_kernel<BN, MODE, HD, MAJOR><<<grid, GT_THREADS, Cfg::smem_bytes(MODE), st>>>(
       ma, mb, C, ldc, M, N, K, W2, partial, h_kv, act, ra, resid, ldr, n_major, status);
   return cudaGetLastError();
 }
@@ -635,14 +641,23 @@ cudaError_t launch_gemm_tc_f32_add_peers(const bf16 *A, int lda, const bf16 *Bt,
   return launch_t<128, 6>(A, lda, Bt, ldb, nullptr, ldc, M, N, K, nullptr, pl, n_peers, 0, RopeAppendArgs{}, status, st);
 }
 
-// out[m] = max(out[m], scale * max_n (A Bt^T)[m][n]) for m < M (out fp32, initialised by the
-// caller, e.g. to -inf); scale > 0.  K % 8 == 0 (a last K-block that is not full is zero-filled by
-// TMA); any N.
-cudaError_t launch_gemm_tc_rowmax(const bf16 *A, int lda, const bf16 *Bt, int ldb, float *out, int M, int N,
-                                  int K, float scale, int *status, cudaStream_t st) {
-  int bits;
-  memcpy(&bits, &scale, sizeof(bits));
-  return launch_t<256, 4>(A, lda, Bt, ldb, nullptr, 0, M, N, K, nullptr, out, 0, bits, RopeAppendArgs{}, status, st);
+// Training of the retaining head: C (fp32) = A B with B [K x N] as it lies (row-major), and, per column tile,
+// the scores of each row: partial[tile][M][h_kv] = sum over the tile's columns of silu(C) W2.
+int rh_pre_num_tiles(int d_R) { return d_R >= 256 ? (d_R + 255) / 256 : (d_R + 127) / 128; }
+cudaError_t launch_rh_pre_tc(const bf16 *Z, int ldz, const bf16 *W1, int ldw, float *pre, const float *W2, float *partial,
+                             int M, int d_R, int K, int h_kv, int *status, cudaStream_t st) {
+  bf16 *C = reinterpret_cast<bf16 *>(pre);
+  if (d_R >= 256)
+    return launch_t<256, 7, 0, 2>(Z, ldz, W1, ldw, C, d_R, M, d_R, K, W2, partial, h_kv, 0, RopeAppendArgs{}, status, st);
+  return launch_t<128, 7, 0, 2>(Z, ldz, W1, ldw, C, d_R, M, d_R, K, W2, partial, h_kv, 0, RopeAppendArgs{}, status, st);
+}
+// C [M x N] (fp32) = A^T B with A [K x M] and B [K x N] as they lie (row-major)
+cudaError_t launch_gemm_tn_f32(const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int M, int N, int K,
+                               int *status, cudaStream_t st) {
+  bf16 *Cb = reinterpret_cast<bf16 *>(C);
+  if (N >= 256)
+    return launch_t<256, 5, 0, 3>(A, lda, B, ldb, Cb, ldc, M, N, K, nullptr, nullptr, 0, 0, RopeAppendArgs{}, status, st);
+  return launch_t<128, 5, 0, 3>(A, lda, B, ldb, Cb, ldc, M, N, K, nullptr, nullptr, 0, 0, RopeAppendArgs{}, status, st);
 }
 
 // QKV projection whose epilogue also assigns positions, rotates Q and K and appends K, V to the

@@ -1,6 +1,9 @@
 // Training of the retaining head (Eq. 2, Eq. 3): loss and gradients of W1, W2 for one sequence,
-// backbone frozen.  The two large contractions (z W1 and z^T dpre) run on the tcgen05 GEMM with
-// fp32 results; the rest is element-wise work around the thin W2.
+// backbone frozen.  Five launches: clear and W2 in fp32; pre = z W1 with the scores' partial sums in
+// its epilogue; loss and its derivative per score; one pass over pre that forms both dpre and dW2; dW1 = z^T dpre.
+// Both contractions run on the tcgen05 GEMM with W1, z and dpre read as they lie (no transposed
+// copies).  Llama shape, 10240 tokens: the two contractions 2 x 75 us of tensor time at the measured
+// peak, pre (42 MB, fp32) is written once and read once.
 #include "../../include/locret.h"
 #include "common.cuh"
 
@@ -10,50 +13,40 @@ namespace {
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + __expf(-x)); }
 
-// one warp per token: s[t][m] = sum_r silu(pre[t][r]) W2[r][m]
-__global__ void rh_scores_f32_kernel(const float *__restrict__ pre, const float *__restrict__ w2,
-                                     float *__restrict__ s, int n, int d_R, int h_kv) {
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (t >= n) return;
-  float acc[32];
-#pragma unroll
-  for (int m = 0; m < 32; m++) acc[m] = 0.f;
-  for (int r = lane; r < d_R; r += 32) {
-    const float p = pre[(size_t)t * d_R + r];
-    const float a = p * sigmoidf_(p);
-#pragma unroll
-    for (int m = 0; m < 32; m++)
-      if (m < h_kv) acc[m] = fmaf(a, w2[(size_t)r * h_kv + m], acc[m]);
+__global__ void rh_clear_kernel(const bf16 *__restrict__ w2, float *__restrict__ w2f, float *__restrict__ dw2, int n,
+                                float *__restrict__ loss, int *__restrict__ status) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) {
+    w2f[i] = __bfloat162float(w2[i]);
+    dw2[i] = 0.f;
   }
-#pragma unroll
-  for (int m = 0; m < 32; m++) {
-    if (m < h_kv) {
-      float v = acc[m];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) s[(size_t)t * h_kv + m] = v;
-    }
-  }
+  if (i == 0) { *loss = 0.f; *status = 0; }
 }
 
 // Eq. 3 per (token, head): Smooth-L1 (threshold 1) to the label plus alpha (s[t] - s[t+1])^2;
-// ds = its derivative; the loss is summed with one atomic per block
-__global__ void rh_loss_kernel(const float *__restrict__ s, const float *__restrict__ labels, float *__restrict__ ds,
+// ds = its derivative; the loss is summed with one atomic per block.  s = the sum of the column tiles' partial scores
+// [tile][token][head], in tile order.
+__global__ void rh_loss_kernel(const float *__restrict__ partial, int n_tiles, const float *__restrict__ labels, float *__restrict__ ds,
                                float *__restrict__ loss, int n, int h_kv, float alpha) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float l = 0.f;
+  auto s = [&](int at) {
+    float v = 0.f;
+    for (int nt = 0; nt < n_tiles; nt++) v += partial[(size_t)nt * n * h_kv + at];
+    return v;
+  };
   if (i < n * h_kv) {
     const int t = i / h_kv, m = i - t * h_kv;
-    const float v = s[i], diff = v - labels[(size_t)m * n + t];
+    const float v = s(i), diff = v - labels[(size_t)m * n + t];
     const float ad = fabsf(diff);
     l = ad < 1.0f ? 0.5f * diff * diff : ad - 0.5f;
     float g = fminf(fmaxf(diff, -1.0f), 1.0f);
     if (t + 1 < n) {
-      const float adj = v - s[i + h_kv];
+      const float adj = v - s(i + h_kv);
       l = fmaf(alpha * adj, adj, l);
       g = fmaf(2.0f * alpha, adj, g);
     }
-    if (t > 0) g -= 2.0f * alpha * (s[i - h_kv] - v);
+    if (t > 0) g -= 2.0f * alpha * (s(i - h_kv) - v);
     ds[i] = g;
   }
   __shared__ float red[32];
@@ -69,60 +62,73 @@ __global__ void rh_loss_kernel(const float *__restrict__ s, const float *__restr
   }
 }
 
-// dW2[r][m] += sum over a slab of tokens of silu(pre[t][r]) ds[t][m]; thread = r
-__global__ void rh_dw2_kernel(const float *__restrict__ pre, const float *__restrict__ ds, float *__restrict__ dw2,
-                              int n, int d_R, int h_kv, int slab) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  const int t0 = blockIdx.y * slab, t1 = min(n, t0 + slab);
-  if (r >= d_R) return;
-  float acc[32];
-#pragma unroll
-  for (int m = 0; m < 32; m++) acc[m] = 0.f;
-  for (int t = t0; t < t1; t++) {
-    const float p = pre[(size_t)t * d_R + r];
-    const float a = p * sigmoidf_(p);
-#pragma unroll
-    for (int m = 0; m < 32; m++)
-      if (m < h_kv) acc[m] = fmaf(a, ds[(size_t)t * h_kv + m], acc[m]);
-  }
-#pragma unroll
-  for (int m = 0; m < 32; m++)
-    if (m < h_kv) atomicAdd(dw2 + (size_t)r * h_kv + m, acc[m]);
-}
+// One pass over pre, thread = two neighbouring columns r, block = a slab of tokens:
+//   dpre[t][r] = bf16( (sum_m ds[t][m] W2[r][m]) * silu'(pre[t][r]) )
+//   dW2[r][m] += sum over the slab of silu(pre[t][r]) ds[t][m]
+// The columns' W2 and dW2 stay in registers, ds of the slab in shared memory (heads padded to HK with zeros).
+// Bound by the FMAs (4 HK per pre-activation pair), not by the 6 bytes per element.
+constexpr int DP_THREADS = 128, DP_SLAB = 64;
 
-// dpreT[r][t] = bf16( (sum_m ds[t][m] W2[r][m]) * silu'(pre[t][r]) ), written transposed through a
-// shared-memory tile so that the second contraction finds its K dimension (tokens) contiguous
-__global__ void rh_dpre_t_kernel(const float *__restrict__ pre, const float *__restrict__ ds,
-                                 const float *__restrict__ w2, bf16 *__restrict__ dpre_t, int n, int d_R, int h_kv) {
-  __shared__ float tile[32][33];
-  const int r = blockIdx.x * 32 + threadIdx.x;
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const int t = blockIdx.y * 32 + y;
-    float v = 0.f;
-    if (t < n && r < d_R) {
-      float da = 0.f;
-      for (int m = 0; m < h_kv; m++) da = fmaf(ds[(size_t)t * h_kv + m], w2[(size_t)r * h_kv + m], da);
-      const float p = pre[(size_t)t * d_R + r], sg = sigmoidf_(p);
-      v = da * (sg * (1.0f + p * (1.0f - sg)));
-    }
-    tile[y][threadIdx.x] = v;
+template <int HK>
+__global__ void __launch_bounds__(DP_THREADS)
+rh_dpre_dw2_kernel(const float *__restrict__ pre, const float *__restrict__ ds, const float *__restrict__ w2,
+                   bf16 *__restrict__ dpre, float *__restrict__ dw2, int n, int d_R, int h_kv) {
+  __shared__ float sds[DP_SLAB][HK];
+  const int r = (blockIdx.x * DP_THREADS + threadIdx.x) * 2;
+  const int t0 = blockIdx.y * DP_SLAB, nt = min(DP_SLAB, n - t0);
+  for (int i = threadIdx.x; i < DP_SLAB * HK; i += DP_THREADS) {
+    const int t = i / HK, m = i % HK;
+    sds[t][m] = (t < nt && m < h_kv) ? ds[(size_t)(t0 + t) * h_kv + m] : 0.f;
   }
   __syncthreads();
-  const int t = blockIdx.y * 32 + threadIdx.x;
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const int rr = blockIdx.x * 32 + y;
-    if (t < n && rr < d_R) dpre_t[(size_t)rr * n + t] = __float2bfloat16_rn(tile[threadIdx.x][y]);
+  if (r >= d_R) return;   // (d_R is even)
+  float w[2][HK], acc[2][HK];
+#pragma unroll
+  for (int e = 0; e < 2; e++)
+#pragma unroll
+    for (int m = 0; m < HK; m++) {
+      w[e][m] = m < h_kv ? w2[(size_t)(r + e) * h_kv + m] : 0.f;
+      acc[e][m] = 0.f;
+    }
+#pragma unroll 4
+  for (int t = 0; t < nt; t++) {
+    const float2 p = *reinterpret_cast<const float2 *>(pre + (size_t)(t0 + t) * d_R + r);
+    const float s0 = sigmoidf_(p.x), s1 = sigmoidf_(p.y);
+    const float a0 = p.x * s0, a1 = p.y * s1;
+    float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+    for (int m = 0; m < HK; m++) {
+      const float g = sds[t][m];
+      d0 = fmaf(g, w[0][m], d0);
+      d1 = fmaf(g, w[1][m], d1);
+      acc[0][m] = fmaf(a0, g, acc[0][m]);
+      acc[1][m] = fmaf(a1, g, acc[1][m]);
+    }
+    *reinterpret_cast<uint32_t *>(dpre + (size_t)(t0 + t) * d_R + r) =
+        pack_bf16(d0 * (s0 * (1.0f + p.x * (1.0f - s0))), d1 * (s1 * (1.0f + p.y * (1.0f - s1))));
   }
+#pragma unroll
+  for (int e = 0; e < 2; e++)
+#pragma unroll
+    for (int m = 0; m < HK; m++)
+      if (m < h_kv) atomicAdd(dw2 + (size_t)(r + e) * h_kv + m, acc[e][m]);
 }
 
 __device__ int g_train_status;
 
-// workspace from the stream-ordered allocator: after the first call the pool serves it without a
-// device synchronisation
-struct Scratch {
-  cudaStream_t st = nullptr;
-  void *p[8] = {};
-  ~Scratch() { for (void *q : p) if (q) cudaFreeAsync(q, st); }
+size_t pad256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// The call's workspace in one block: offsets of its arrays.
+struct Workspace {
+  size_t pre, dpre, w2f, partial, ds, bytes;
+  Workspace(size_t n, size_t d_R, size_t h_kv) {
+    pre = 0;
+    dpre = pre + pad256(n * d_R * sizeof(float));
+    w2f = dpre + pad256(n * d_R * sizeof(bf16));
+    partial = w2f + pad256(d_R * h_kv * sizeof(float));
+    ds = partial + pad256(rh_pre_num_tiles((int)d_R) * n * h_kv * sizeof(float));
+    bytes = ds + pad256(n * h_kv * sizeof(float));
+  }
 };
 
 }  // namespace
@@ -133,71 +139,102 @@ struct Scratch {
     if (e__ != cudaSuccess) { cudaGetLastError(); return LOCRET_ERR_CUDA; }  \
   } while (0)
 
-extern "C" int locret_rh_loss_grad(const void *z, const float *labels, const void *w1, const void *w2, int32_t n,
-                                   int32_t d_in, int32_t d_R, int32_t h_kv, float alpha, float *loss,
-                                   float *d_w1, float *d_w2, void *stream) {
-  if (!z || !labels || !w1 || !w2 || !loss || !d_w1 || !d_w2) return LOCRET_ERR_INVALID;
-  if (n < 64 || n % 64 || d_in < 64 || d_in % 64 || d_R < 32 || d_R % 32 || h_kv < 1 || h_kv > 32 || alpha < 0.f)
+static bool rh_sizes_ok(int32_t n, int32_t d_R, int32_t h_kv) {
+  return n >= 64 && n % 64 == 0 && d_R >= 32 && d_R % 32 == 0 && h_kv >= 1 && h_kv <= 32;
+}
+
+extern "C" int locret_rh_loss_grad_workspace(int32_t n, int32_t d_R, int32_t h_kv, int64_t *bytes) {
+  if (!bytes || !rh_sizes_ok(n, d_R, h_kv)) return LOCRET_ERR_INVALID;
+  *bytes = (int64_t)Workspace(n, d_R, h_kv).bytes;
+  return LOCRET_OK;
+}
+
+extern "C" int locret_rh_loss_grad_ws(const void *z, const float *labels, const void *w1, const void *w2, int32_t n,
+                                      int32_t d_in, int32_t d_R, int32_t h_kv, float alpha, float *loss, float *d_w1,
+                                      float *d_w2, void *workspace, int64_t workspace_bytes, void *stream) {
+  if (!z || !labels || !w1 || !w2 || !loss || !d_w1 || !d_w2 || !workspace) return LOCRET_ERR_INVALID;
+  if (!rh_sizes_ok(n, d_R, h_kv) || d_in < 64 || d_in % 64 || alpha < 0.f) return LOCRET_ERR_INVALID;
+  if ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(w1) | reinterpret_cast<uintptr_t>(d_w1) |
+       reinterpret_cast<uintptr_t>(workspace)) & 15u)
     return LOCRET_ERR_INVALID;
-  if ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(w1) | reinterpret_cast<uintptr_t>(d_w1)) & 15u)
-    return LOCRET_ERR_INVALID;
+  const Workspace ws(n, d_R, h_kv);
+  if (workspace_bytes < (int64_t)ws.bytes) return LOCRET_ERR_CAPACITY;
   cudaStream_t st = (cudaStream_t)stream;
-  Scratch sc;  // freed on every return path
-  sc.st = st;
-  bf16 *w1_t, *z_t, *dpre_t;
-  float *pre, *w2f, *s, *ds;
-  auto alloc = [&](int slot, void **out, size_t bytes) {
-    if (cudaMallocAsync(out, bytes, st) != cudaSuccess) { cudaGetLastError(); return false; }
-    sc.p[slot] = *out;
-    return true;
-  };
-  if (!alloc(0, (void **)&w1_t, (size_t)d_R * d_in * sizeof(bf16)) || !alloc(1, (void **)&z_t, (size_t)d_in * n * sizeof(bf16)) ||
-      !alloc(2, (void **)&dpre_t, (size_t)d_R * n * sizeof(bf16)) || !alloc(3, (void **)&pre, (size_t)n * d_R * sizeof(float)) ||
-      !alloc(4, (void **)&w2f, (size_t)d_R * h_kv * sizeof(float)) || !alloc(5, (void **)&s, (size_t)n * h_kv * sizeof(float)) ||
-      !alloc(6, (void **)&ds, (size_t)n * h_kv * sizeof(float)))
-    return LOCRET_ERR_ALLOC;
+  unsigned char *base = static_cast<unsigned char *>(workspace);
+  float *pre = (float *)(base + ws.pre), *w2f = (float *)(base + ws.w2f), *partial = (float *)(base + ws.partial),
+        *ds = (float *)(base + ws.ds);
+  bf16 *dpre = (bf16 *)(base + ws.dpre);
   int *d_status = nullptr;
   TCK(cudaGetSymbolAddress((void **)&d_status, g_train_status));
-  TCK(cudaMemsetAsync(d_status, 0, sizeof(int), st));
-  TCK(cudaMemsetAsync(loss, 0, sizeof(float), st));
-  TCK(cudaMemsetAsync(d_w2, 0, (size_t)d_R * h_kv * sizeof(float), st));
-  TCK(launch_transpose_bf16((const bf16 *)w1, w1_t, d_in, d_R, st));   // [d_in x d_R] -> [d_R x d_in]
-  TCK(launch_transpose_bf16((const bf16 *)z, z_t, n, d_in, st));       // [n x d_in]  -> [d_in x n]
-  TCK(launch_bf16_to_f32((const bf16 *)w2, w2f, d_R * h_kv, st));
-  // pre = z W1 (fp32)
-  TCK(launch_gemm_tc_f32((const bf16 *)z, d_in, w1_t, d_in, pre, d_R, n, d_R, d_in, d_status, st));
-  rh_scores_f32_kernel<<<(n + 7) / 8, 256, 0, st>>>(pre, w2f, s, n, d_R, h_kv);
+  rh_clear_kernel<<<(d_R * h_kv + 255) / 256, 256, 0, st>>>((const bf16 *)w2, w2f, d_w2, d_R * h_kv, loss, d_status);
   TCK(cudaGetLastError());
-  rh_loss_kernel<<<(n * h_kv + 255) / 256, 256, 0, st>>>(s, labels, ds, loss, n, h_kv, alpha);
+  // pre = z W1 (fp32) and the scores
+  TCK(launch_rh_pre_tc((const bf16 *)z, d_in, (const bf16 *)w1, d_R, pre, w2f, partial, n, d_R, d_in, h_kv, d_status, st));
+  rh_loss_kernel<<<(n * h_kv + 255) / 256, 256, 0, st>>>(partial, rh_pre_num_tiles(d_R), labels, ds, loss, n, h_kv, alpha);
   TCK(cudaGetLastError());
-  const int slab = 256;
-  rh_dw2_kernel<<<dim3((d_R + 127) / 128, (n + slab - 1) / slab), 128, 0, st>>>(pre, ds, d_w2, n, d_R, h_kv, slab);
+  const dim3 grid((d_R / 2 + DP_THREADS - 1) / DP_THREADS, (n + DP_SLAB - 1) / DP_SLAB);
+  if (h_kv <= 8) rh_dpre_dw2_kernel<8><<<grid, DP_THREADS, 0, st>>>(pre, ds, w2f, dpre, d_w2, n, d_R, h_kv);
+  else rh_dpre_dw2_kernel<32><<<grid, DP_THREADS, 0, st>>>(pre, ds, w2f, dpre, d_w2, n, d_R, h_kv);
   TCK(cudaGetLastError());
-  rh_dpre_t_kernel<<<dim3((d_R + 31) / 32, (n + 31) / 32), dim3(32, 8), 0, st>>>(pre, ds, w2f, dpre_t, n, d_R, h_kv);
-  TCK(cudaGetLastError());
-  // dW1 [d_in x d_R] = z^T dpre: both operands with the tokens as their contiguous K dimension
-  TCK(launch_gemm_tc_f32(z_t, n, dpre_t, n, d_w1, d_R, d_in, d_R, n, d_status, st));
+  // dW1 [d_in x d_R] = z^T dpre
+  TCK(launch_gemm_tn_f32((const bf16 *)z, d_in, dpre, d_R, d_w1, d_R, d_in, d_R, n, d_status, st));
   int status = 0;
   TCK(cudaMemcpyAsync(&status, d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   TCK(cudaStreamSynchronize(st));
   return status ? LOCRET_ERR_DEVICE_TIMEOUT : LOCRET_OK;
 }
 
+extern "C" int locret_rh_loss_grad(const void *z, const float *labels, const void *w1, const void *w2, int32_t n,
+                                   int32_t d_in, int32_t d_R, int32_t h_kv, float alpha, float *loss,
+                                   float *d_w1, float *d_w2, void *stream) {
+  if (!rh_sizes_ok(n, d_R, h_kv)) return LOCRET_ERR_INVALID;
+  // (the stream-ordered pool gives its memory back at every synchronisation: callers in a loop keep a workspace)
+  const int64_t bytes = (int64_t)Workspace(n, d_R, h_kv).bytes;
+  void *ws = nullptr;
+  if (cudaMallocAsync(&ws, (size_t)bytes, (cudaStream_t)stream) != cudaSuccess) { cudaGetLastError(); return LOCRET_ERR_ALLOC; }
+  const int rc = locret_rh_loss_grad_ws(z, labels, w1, w2, n, d_in, d_R, h_kv, alpha, loss, d_w1, d_w2, ws, bytes, stream);
+  if (cudaFreeAsync(ws, (cudaStream_t)stream) != cudaSuccess) { cudaGetLastError(); return rc ? rc : LOCRET_ERR_CUDA; }
+  return rc;
+}
+
 // ---------------------------------------------------------------- AdamW (Appendix A, training)
 namespace {
+struct AdamW { float lr, beta1, beta2, eps, wd, bc1, bc2; };
+
+__device__ __forceinline__ float adamw_one(float p, float g, float &m, float &v, const AdamW &a) {
+  m = a.beta1 * m + (1.0f - a.beta1) * g;
+  v = a.beta2 * v + (1.0f - a.beta2) * g * g;
+  return p * (1.0f - a.lr * a.wd) - a.lr * (m / a.bc1) / (sqrtf(v / a.bc2) + a.eps);
+}
+
+// Bound by memory (30 bytes per parameter with the bf16 copy): four parameters per thread with 16-byte accesses where
+// every array is aligned for them (vec), one otherwise and in the remainder.
 __global__ void adamw_kernel(float *__restrict__ p, bf16 *__restrict__ p_bf16, const float *__restrict__ g,
-                             float *__restrict__ m, float *__restrict__ v, size_t n, float lr, float beta1,
-                             float beta2, float eps, float wd, float bc1, float bc2) {
+                             float *__restrict__ m, float *__restrict__ v, size_t n, AdamW a, int vec) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = beta1 * m[i] + (1.0f - beta1) * gi;
-  const float vi = beta2 * v[i] + (1.0f - beta2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float pi = p[i] * (1.0f - lr * wd) - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-  p[i] = pi;
-  if (p_bf16) p_bf16[i] = __float2bfloat16_rn(pi);
+  if (vec && 4 * i + 4 <= n) {
+    float4 pp = reinterpret_cast<float4 *>(p)[i], mm = reinterpret_cast<float4 *>(m)[i],
+           vv = reinterpret_cast<float4 *>(v)[i];
+    const float4 gg = reinterpret_cast<const float4 *>(g)[i];
+    pp.x = adamw_one(pp.x, gg.x, mm.x, vv.x, a);
+    pp.y = adamw_one(pp.y, gg.y, mm.y, vv.y, a);
+    pp.z = adamw_one(pp.z, gg.z, mm.z, vv.z, a);
+    pp.w = adamw_one(pp.w, gg.w, mm.w, vv.w, a);
+    reinterpret_cast<float4 *>(m)[i] = mm;
+    reinterpret_cast<float4 *>(v)[i] = vv;
+    reinterpret_cast<float4 *>(p)[i] = pp;
+    if (p_bf16) reinterpret_cast<uint2 *>(p_bf16)[i] = make_uint2(pack_bf16(pp.x, pp.y), pack_bf16(pp.z, pp.w));
+    return;
+  }
+  const size_t lo = vec ? 4 * i : i, hi = vec ? n : (i < n ? i + 1 : 0);
+  for (size_t k = lo; k < hi; k++) {
+    float mk = m[k], vk = v[k];
+    const float pk = adamw_one(p[k], g[k], mk, vk, a);
+    m[k] = mk;
+    v[k] = vk;
+    p[k] = pk;
+    if (p_bf16) p_bf16[k] = __float2bfloat16_rn(pk);
+  }
 }
 }  // namespace
 
@@ -207,9 +244,13 @@ extern "C" int locret_adamw_step(float *param, void *param_bf16, const float *gr
   if (!param || !grad || !m || !v || n < 1 || step < 1) return LOCRET_ERR_INVALID;
   if (!(beta1 >= 0.f && beta1 < 1.f && beta2 >= 0.f && beta2 < 1.f) || eps <= 0.f) return LOCRET_ERR_INVALID;
   const float bc1 = 1.0f - powf(beta1, (float)step), bc2 = 1.0f - powf(beta2, (float)step);
-  adamw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(param, (bf16 *)param_bf16, grad, m, v,
-                                                                             (size_t)n, lr, beta1, beta2, eps,
-                                                                             weight_decay, bc1, bc2);
+  const AdamW a = {lr, beta1, beta2, eps, weight_decay, bc1, bc2};
+  const uintptr_t bits = reinterpret_cast<uintptr_t>(param) | reinterpret_cast<uintptr_t>(grad) |
+                         reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(v);
+  const int vec = (bits & 15u) == 0 && (reinterpret_cast<uintptr_t>(param_bf16) & 7u) == 0;
+  const size_t threads = vec ? ((size_t)n + 3) / 4 : (size_t)n;
+  adamw_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, (cudaStream_t)stream>>>(param, (bf16 *)param_bf16, grad, m, v,
+                                                                                   (size_t)n, a, vec);
   TCK(cudaGetLastError());
   return LOCRET_OK;
 }
