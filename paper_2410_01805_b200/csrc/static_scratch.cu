@@ -61,8 +61,13 @@ extern "C" int locret_rh_scores_static(const void *z, int32_t n_tok, int32_t d_i
   cudaStream_t st = (cudaStream_t)stream;
   int n_tiles = 0;
   // Every partial this call reads is written by this call first, so nothing has to be cleared.
-  if (launch_rh_gemm_tc((const bf16 *)z, d_in, (const bf16 *)w1_t, w2, partial, n_tok, d_retain, d_in,
-                        n_kv_heads, act, &n_tiles, status, st) != cudaSuccess) {
+  const cudaError_t e =
+      skinny_use(n_tok, d_retain, d_in, d_in, d_in)
+          ? launch_skinny_rh((const bf16 *)z, d_in, (const bf16 *)w1_t, w2, partial, n_tok, d_retain, d_in, n_kv_heads, act,
+                             &n_tiles, status, st)
+          : launch_rh_gemm_tc((const bf16 *)z, d_in, (const bf16 *)w1_t, w2, partial, n_tok, d_retain, d_in, n_kv_heads,
+                              act, &n_tiles, status, st);
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return LOCRET_ERR_CUDA;
   }
