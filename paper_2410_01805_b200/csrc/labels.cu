@@ -9,7 +9,8 @@
 // multiplied.  Eight warps reduce, each thread one row's maximum over half the columns, three-input maxima, all
 // query tiles of a work unit before one atomic maximum per row on the order-preserving integer image.
 // One launch for all heads (a launch of the 128 x 256 GEMM per query head before: two K-blocks per tile, the keys
-// re-read for every head).
+// re-read for every head).  131072 keys, 1024 answers, 32 query heads of 8 KV heads of 128: 0.70 ms = 1.57 PFLOP/s
+// (1.45 ms before); the measured burst peak allows 0.64 ms.
 #include "../../include/locret.h"
 #include "tc_common.cuh"
 
@@ -20,10 +21,11 @@ namespace {
 using namespace locret::tc;
 
 constexpr int LB_THREADS = 320;              // warps 0-7 reduce, 8 TMA, 9 MMA
-constexpr int LB_ROWS = 128, LB_COLS = 256, LB_STAGES = 4;
+constexpr int LB_ROWS = 128, LB_COLS = 256;
 constexpr int LB_A_BLOCK = LB_ROWS * 128;    // 64 columns of a key tile, swizzled: 16 KB
 constexpr int LB_B_BLOCK = LB_COLS * 128;    // 64 columns of a query tile: 32 KB
-constexpr int LB_SMEM = 1024 + 4 * LB_A_BLOCK + LB_STAGES * LB_B_BLOCK + 256;
+constexpr int LB_B_BLOCKS = 4;               // resident: two query tiles of d > 64, four of d = 64
+constexpr int LB_SMEM = 1024 + 4 * LB_A_BLOCK + LB_B_BLOCKS * LB_B_BLOCK + 256;
 
 struct LabelParams {
   float *labels;
@@ -36,13 +38,16 @@ struct LabelParams {
 
 __device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
 
+template <int D>
 __global__ void __launch_bounds__(LB_THREADS, 1)
 labels_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q, const LabelParams p) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   unsigned char *sA = smem, *sB = smem + 4 * LB_A_BLOCK;  // sA: [tile][64-column block]
-  uint64_t *bars = reinterpret_cast<uint64_t *>(sB + LB_STAGES * LB_B_BLOCK);
+  constexpr int KB = (D + 63) / 64, KSTEPS = D / 16;
+  constexpr int LB_STAGES = LB_B_BLOCKS / KB;  // a stage holds one query tile
+  uint64_t *bars = reinterpret_cast<uint64_t *>(sB + LB_B_BLOCKS * LB_B_BLOCK);
   uint64_t *b_full = bars, *b_empty = bars + LB_STAGES;
   uint64_t *a_full = bars + 2 * LB_STAGES, *a_empty = a_full + 2, *acc_full = a_empty + 2, *acc_empty = acc_full + 2;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
@@ -68,7 +73,6 @@ labels_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  const int kblocks = (p.d + 63) / 64, ksteps = p.d / 16;
   const int per_q = LB_COLS / p.gb;                        // answers in a query tile
   const int a_tiles = (p.n_a + per_q - 1) / per_q;         // query tiles of one set of gb heads
   const int units = p.h_kv * p.pairs * p.splits;
@@ -80,7 +84,10 @@ labels_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__
     t0 = (int)((long long)sp * p.q_tiles / p.splits);
     t1 = (int)((long long)(sp + 1) * p.q_tiles / p.splits);
   };
-  auto valid_of = [&](int t) { return min(per_q, p.n_a - (t % a_tiles) * per_q) * p.gb; };  // columns of a query tile
+  // A query tile t is answers [at * per_q, ..) of the heads of set js, t = js * a_tiles + at; the loops below step
+  // (js, at) instead of dividing: the issuing thread must not spend more than the two or three instructions that
+  // the tensor pipe queues ahead (with divisions and per-step descriptors it took 197 cycles per MMA of 128).
+  auto valid_of = [&](int at) { return min(per_q, p.n_a - at * per_q) * p.gb; };  // columns of a query tile
 
   if (warp == 8) {
     if (lane == 0) {
@@ -92,48 +99,57 @@ labels_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__
         for (int i = 0; i < 2 && ok; i++) {  // (a tile past the end is loaded as zeros and not stored)
           ok = mbar_wait(&a_empty[i], (un & 1) ^ 1, abort_flag, p.status);
           if (!ok) break;
-          mbar_expect_tx(&a_full[i], kblocks * LB_A_BLOCK);
-          for (int kb = 0; kb < kblocks; kb++)
+          mbar_expect_tx(&a_full[i], KB * LB_A_BLOCK);
+#pragma unroll
+          for (int kb = 0; kb < KB; kb++)
             tma_load_3d(sA + (i * 2 + kb) * LB_A_BLOCK, &map_k, kb * 64, m, key0 + i * LB_ROWS, &a_full[i]);
         }
-        for (int t = t0; t < t1 && ok; t++)
-          for (int kb = 0; kb < kblocks; kb++, it++) {
-            const int s = it % LB_STAGES;
-            ok = mbar_wait(&b_empty[s], ((it / LB_STAGES) & 1) ^ 1, abort_flag, p.status);
-            if (!ok) break;
-            mbar_expect_tx(&b_full[s], LB_B_BLOCK);
-            tma_load_3d(sB + s * LB_B_BLOCK, &map_q, kb * 64, m * p.g + (t / a_tiles) * p.gb, (t % a_tiles) * per_q,
-                        &b_full[s]);
-          }
+        int js = t0 / a_tiles, at = t0 - js * a_tiles;
+        for (int t = t0; t < t1 && ok; t++, it++) {
+          const int s = it % LB_STAGES;
+          ok = mbar_wait(&b_empty[s], ((it / LB_STAGES) & 1) ^ 1, abort_flag, p.status);
+          if (!ok) break;
+          mbar_expect_tx(&b_full[s], KB * LB_B_BLOCK);
+#pragma unroll
+          for (int kb = 0; kb < KB; kb++)
+            tma_load_3d(sB + (s * KB + kb) * LB_B_BLOCK, &map_q, kb * 64, m * p.g + js * p.gb, at * per_q, &b_full[s]);
+          if (++at == a_tiles) { at = 0; js++; }
+        }
       }
     }
   } else if (warp == 9) {
     if (lane == 0) {
-      uint32_t it = 0, un = 0, nt = 0;  // stages, units and query tiles seen so far
+      const uint64_t da0 = desc_kmajor_sw128(sA), db0 = desc_kmajor_sw128(sB);
+      uint32_t un = 0, nt = 0;  // units and query tiles seen so far
       bool ok = true;
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x, un++) {
         int m, key0, t0, t1;
         unit_of(u, m, key0, t0, t1);
+        int at = t0 % a_tiles;
         for (int t = t0; t < t1 && ok; t++, nt++) {
-          const uint32_t idesc = idesc_bf16(LB_ROWS, (valid_of(t) + 15) & ~15, 0, 0);
-          for (int kb = 0; kb < kblocks && ok; kb++)
-            ok = mbar_wait(&b_full[(it + kb) % LB_STAGES], ((it + kb) / LB_STAGES) & 1, abort_flag, p.status);
-          for (int i = 0; i < 2 && ok; i++) {
-            if (t == t0) ok = mbar_wait(&a_full[i], un & 1, abort_flag, p.status);
+          const uint32_t idesc = idesc_bf16(LB_ROWS, (valid_of(at) + 15) & ~15, 0, 0);
+          if (++at == a_tiles) at = 0;
+          const int s = nt % LB_STAGES;
+          const uint64_t db = db0 + (uint64_t)(s * (KB * LB_B_BLOCK >> 4));
+          ok = mbar_wait(&b_full[s], (nt / LB_STAGES) & 1, abort_flag, p.status);
+#pragma unroll
+          for (int i = 0; i < 2; i++) {
+            if (t == t0) ok = ok && mbar_wait(&a_full[i], un & 1, abort_flag, p.status);
             ok = ok && mbar_wait(&acc_empty[i], (nt & 1) ^ 1, abort_flag, p.status);
             if (!ok) break;
             tc_fence_after();
-            for (int kk = 0; kk < ksteps; kk++) {
-              const uint64_t da = desc_kmajor_sw128(sA + (i * 2 + (kk >> 2)) * LB_A_BLOCK) + (uint64_t)((kk & 3) * 2);
-              const uint64_t db =
-                  desc_kmajor_sw128(sB + ((it + (kk >> 2)) % LB_STAGES) * LB_B_BLOCK) + (uint64_t)((kk & 3) * 2);
-              mma_ss(tmem + i * LB_COLS, da, db, idesc, kk > 0);
+            const uint64_t da = da0 + (uint64_t)(i * (2 * LB_A_BLOCK >> 4));
+#pragma unroll
+            for (int kk = 0; kk < KSTEPS; kk++) {
+              const uint64_t ao = (uint64_t)((kk >> 2) * (LB_A_BLOCK >> 4) + (kk & 3) * 2);
+              const uint64_t bo = (uint64_t)((kk >> 2) * (LB_B_BLOCK >> 4) + (kk & 3) * 2);
+              if (kk == 0) mma_ss_first(tmem + i * LB_COLS, da + ao, db + bo, idesc);
+              else mma_ss_acc(tmem + i * LB_COLS, da + ao, db + bo, idesc);
             }
             mma_commit(&acc_full[i]);
             if (t == t1 - 1) mma_commit(&a_empty[i]);
           }
-          for (int kb = 0; kb < kblocks && ok; kb++) mma_commit(&b_empty[(it + kb) % LB_STAGES]);
-          it += kblocks;
+          if (ok) mma_commit(&b_empty[s]);
         }
       }
     }
@@ -146,8 +162,10 @@ labels_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__
       int m, key0, t0, t1;
       unit_of(u, m, key0, t0, t1);
       float mx[2] = {-INFINITY, -INFINITY};
+      int at = t0 % a_tiles;
       for (int t = t0; t < t1; t++, nt++) {
-        const int valid = valid_of(t);
+        const int valid = valid_of(at);
+        if (++at == a_tiles) at = 0;
 #pragma unroll
         for (int i = 0; i < 2; i++) {
           if (ok) ok = mbar_wait(&acc_full[i], nt & 1, abort_flag, p.status);
@@ -247,10 +265,15 @@ extern "C" int locret_cis_labels(const void *q_ans, const void *k_prompt, int32_
   while (h_kv * p.pairs * p.splits < 16 * sms && p.q_tiles / (2 * p.splits) >= 2) p.splits *= 2;
   const long long units = (long long)h_kv * p.pairs * p.splits;
   if (units > 0x7fffffffll) return LOCRET_ERR_INVALID;
-  static PerDeviceFlag attr_set;
-  LCK(allow_dynamic_smem(labels_kernel, LB_SMEM, attr_set));
-  labels_kernel<<<(unsigned)(units < sms ? units : sms), LB_THREADS, LB_SMEM, st>>>(mk, mq, p);
-  LCK(cudaGetLastError());
+  auto launch = [&](auto kernel, PerDeviceFlag &attr_set) -> cudaError_t {
+    if (cudaError_t e = allow_dynamic_smem(kernel, LB_SMEM, attr_set); e != cudaSuccess) return e;
+    kernel<<<(unsigned)(units < sms ? units : sms), LB_THREADS, LB_SMEM, st>>>(mk, mq, p);
+    return cudaGetLastError();
+  };
+  static PerDeviceFlag attr_set[3];
+  if (d == 64) LCK(launch(labels_kernel<64>, attr_set[0]));
+  else if (d == 96) LCK(launch(labels_kernel<96>, attr_set[1]));
+  else LCK(launch(labels_kernel<128>, attr_set[2]));
   int status = 0;
   LCK(cudaMemcpyAsync(&status, p.status, sizeof(int), cudaMemcpyDeviceToHost, st));
   LCK(cudaStreamSynchronize(st));
