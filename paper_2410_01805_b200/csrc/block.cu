@@ -56,24 +56,33 @@ __global__ void __launch_bounds__(256)
 rmsnorm_row_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ gain, bf16 *__restrict__ y, int D, float eps) {
   __shared__ float part[8];
   const int row = blockIdx.x, tid = threadIdx.x;
+  constexpr int V = 4;  // vectors of eight a thread keeps: rows of up to 8192 are read once
   const uint4 *gv = reinterpret_cast<const uint4 *>(gain);
-  uint4 g0 = make_uint4(0, 0, 0, 0);
-  if (tid < D / 8) g0 = gv[tid];   // (the gain depends on nothing before this kernel)
+  uint4 g[V], q[V];
+#pragma unroll
+  for (int i = 0; i < V; i++)
+    if (tid + 256 * i < D / 8) g[i] = __ldg(gv + tid + 256 * i);   // (the gain depends on nothing before this kernel)
   pdl_wait();
   pdl_launch_dependents();
   const uint4 *src = reinterpret_cast<const uint4 *>(x + (size_t)row * D);
   uint4 *dst = reinterpret_cast<uint4 *>(y + (size_t)row * D);
   float ss = 0.f;
-  for (int v = tid; v < D / 8; v += 256) {
-    const uint4 q = src[v];
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+  auto add = [&](const uint4 &v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int e = 0; e < 4; e++) {
       const float a = __uint_as_float(w[e] << 16), b = __uint_as_float(w[e] & 0xffff0000u);
       ss = fmaf(a, a, ss);
       ss = fmaf(b, b, ss);
     }
-  }
+  };
+#pragma unroll
+  for (int i = 0; i < V; i++)
+    if (tid + 256 * i < D / 8) q[i] = src[tid + 256 * i];
+#pragma unroll
+  for (int i = 0; i < V; i++)
+    if (tid + 256 * i < D / 8) add(q[i]);
+  for (int v = tid + 256 * V; v < D / 8; v += 256) add(src[v]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if ((tid & 31) == 0) part[tid >> 5] = ss;
@@ -82,9 +91,8 @@ rmsnorm_row_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ gain, bf
 #pragma unroll
   for (int i = 0; i < 8; i++) t += part[i];
   const float inv = rsqrtf(t / (float)D + eps);
-  for (int v = tid; v < D / 8; v += 256) {
-    const uint4 q = src[v], g = v == tid ? g0 : gv[v];
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w}, gw[4] = {g.x, g.y, g.z, g.w};
+  auto scaled = [&](const uint4 &v, const uint4 &gn) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w}, gw[4] = {gn.x, gn.y, gn.z, gn.w};
     uint32_t o[4];
 #pragma unroll
     for (int e = 0; e < 4; e++) {
@@ -92,8 +100,12 @@ rmsnorm_row_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ gain, bf
       const float b = __uint_as_float(w[e] & 0xffff0000u) * inv * __uint_as_float(gw[e] & 0xffff0000u);
       o[e] = pack_bf16(a, b);
     }
-    dst[v] = make_uint4(o[0], o[1], o[2], o[3]);
-  }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+  };
+#pragma unroll
+  for (int i = 0; i < V; i++)
+    if (tid + 256 * i < D / 8) dst[tid + 256 * i] = scaled(q[i], g[i]);
+  for (int v = tid + 256 * V; v < D / 8; v += 256) dst[v] = scaled(src[v], gv[v]);
 }
 
 cudaError_t launch_rmsnorm(const bf16 *x, const bf16 *gain, bf16 *y, int rows, int D, float eps, cudaStream_t st,

@@ -24,6 +24,7 @@ using namespace tc;
 
 constexpr int SK_THREADS = 128, SK_BK = 64, SK_ROWS = 128;
 constexpr int SK_A_BYTES = SK_ROWS * SK_BK * 2;
+constexpr int SK_MAX_SPLIT = 8;   // portable cluster size
 
 template <int NT>
 struct SkinnyCfg {
@@ -178,11 +179,15 @@ skinny_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
   auto sum4 = [&](int t, int row) {  // rows row .. row + 3 of token t, over the slices of K in order
     const uint32_t a = acc_addr + (uint32_t)(t * SK_ROWS + row) * 4;
     if (S == 1) return *reinterpret_cast<const float4 *>(acc + t * SK_ROWS + row);
-    float4 v = ld_cluster_f4(cluster_map(a, 0));
-    for (int r = 1; r < S; r++) {
-      const float4 w = ld_cluster_f4(cluster_map(a, r));
-      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-    }
+    // (all remote loads in flight before the first is used: one after the other an 8-way sum took 2 us more)
+    float4 w[SK_MAX_SPLIT];
+#pragma unroll
+    for (int r = 0; r < SK_MAX_SPLIT; r++)
+      if (r < S) w[r] = ld_cluster_f4(cluster_map(a, r));
+    float4 v = w[0];
+#pragma unroll
+    for (int r = 1; r < SK_MAX_SPLIT; r++)
+      if (r < S) { v.x += w[r].x; v.y += w[r].y; v.z += w[r].z; v.w += w[r].w; }
     return v;
   };
   const int share = NT / S, t0 = rank * share;
@@ -280,7 +285,7 @@ cudaError_t launch_skinny(const bf16 *X, int ldx, const bf16 *Wt, int ldw, Skinn
   const int ctas = tiles * ((p.n_tok + nt - 1) / nt), slots = 2 * sm_count_of_current_device();
   // the deepest split of K that keeps all CTAs resident at once and gives each at least four K-blocks
   int s = 1;
-  while (s < 8 && ctas * s * 2 <= slots && p.K / SK_BK / (2 * s) >= 4) s *= 2;
+  while (s < SK_MAX_SPLIT && ctas * s * 2 <= slots && p.K / SK_BK / (2 * s) >= 4) s *= 2;
   p.n_split = s;
   switch (nt) {
     case 16: return launch_nt<16, EPI>(X, ldx, Wt, ldw, p, tiles, rows_w, st, pdl);
