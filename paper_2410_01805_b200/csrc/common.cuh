@@ -216,6 +216,8 @@ struct RopeAppendArgs {
   int n_tok, h, h_kv, d, cap, len;
   int64_t seen;
   int per_head;    // the chunk is appended at slot len_m.v[m] + t of KV head m (query heads use their KV head's)
+  bf16 *tok_k, *tok_v;  // one token, 4-bit cache: its rotated key and its value go here, [h_kv][d], in place of k_rot / v
+                        // (null otherwise)
   PerHead len_m;   // (read by rope_append_kernel only: the fused epilogue and the one-token kernel take `len`)
 };
 cudaError_t launch_rope_append(const RopeAppendArgs &a, cudaStream_t st);
@@ -293,31 +295,52 @@ cudaError_t launch_gemv_resid(const bf16 *x, const bf16 *Wt, int N, int K, const
 // act[c] = silu(x . Wg[:, c]) * (x . Wu[:, c]) for one token; Wt [2F x K] in the interleaved
 // layout of launch_gemm_tc_gated
 cudaError_t launch_gemv_gated(const bf16 *x, const bf16 *Wt, int F, int K, bf16 *act, cudaStream_t st);
-// projection + positions + RoPE + cache append of one token (a.staging is not used: `staging` is written)
-cudaError_t launch_gemv_rope(const bf16 *x, const bf16 *Wt, int K, bf16 *staging, const RopeAppendArgs &a,
-                             cudaStream_t st, bool pdl = false);
-// retaining head of one token; the last block sums the per-block partials into
-// score_out[m * score_stride]; counter: one zeroed word, left at zero
+// The three kernels of a one-token step take one layer or a batch of layers with the same input and shape (each kernel is
+// compiled for one layer, whose arguments need no indexing, and for up to DECODE_BATCH).
+constexpr int DECODE_BATCH = 8;
+// projection + positions + RoPE + cache append (a.staging is written, not read); more than one layer if gemv_rope_batched
+template <int N> struct GemvRopeBatchN { const bf16 *Wt[N]; RopeAppendArgs a[N]; };
+typedef GemvRopeBatchN<DECODE_BATCH> GemvRopeBatch;
+bool gemv_rope_batched(int K);
+cudaError_t launch_gemv_rope(const bf16 *x, int K, const GemvRopeBatch &b, int n_layers, cudaStream_t st, bool pdl);
+// retaining head; the last block of a layer sums the per-block partials ([rh_gemv_blocks][h_kv]) into
+// score_out[m * score_stride]; counter: one zeroed word, left at zero.
 // pdl: the kernel is the third of a one-token step's chain (projection, attention, retaining head)
 // launched with programmatic dependent launch; it needs only the projection's output, so it runs beside
 // the attention kernel and waits for that kernel just before it ends (which keeps the chain ordered)
-cudaError_t launch_rh_gemv(const bf16 *z, const bf16 *W1t, const float *W2, float *partial, int d_R, int K,
-                           int h_kv, int act, unsigned *counter, float *score_out, int score_stride,
-                           cudaStream_t st, bool pdl = false);
+struct RhGemvLayer {
+  const bf16 *z, *W1t;
+  const float *W2;
+  float *partial, *score_out;
+  unsigned *counter;
+  int score_stride;
+};
+template <int N> struct RhGemvBatchN { RhGemvLayer l[N]; };
+typedef RhGemvBatchN<DECODE_BATCH> RhGemvBatch;
 int rh_gemv_blocks(int d_R);
-int decode_attn_splits(int h_kv, int n, bool int4);
-// part_o: fp32 [h][n_splits][d]; part_ml: fp32 [h][n_splits][2]; counters: one zeroed word per
+cudaError_t launch_rh_gemv(const RhGemvBatch &b, int n_layers, int d_R, int K, int h_kv, int act, cudaStream_t st, bool pdl);
+// attention.  part_o: fp32 [h][n_splits][d]; part_ml: fp32 [h][n_splits][2]; counters: one zeroed word per
 // (KV head, group of 16 query heads), left at zero (the last split merges the partial results).
-// q4 != nullptr: keys [0, n - 1) are read from the 4-bit cache (expanded and rotated with `cs` on the
-// way into shared memory, at position rank[m * cap + slot] for slot < ranked_len and slot above) and only
-// key n - 1, the token of this step, from k_rot / v.  tok_k / tok_v (4-bit cache only, may be null): the
-// token's pre-RoPE keys and values [h_kv][d], which the kernel quantises into slot n - 1 of the cache.
-struct Int4Half;
-cudaError_t launch_attention_decode(const bf16 *q_rot, const bf16 *k_rot, const bf16 *v, bf16 *out,
-                                    float *part_o, float *part_ml, unsigned *counters, int h, int h_kv, int d,
-                                    int cap, int n, int n_splits, const Int4Half *q4, const float2 *cs,
-                                    const int32_t *rank, int ranked_len, const bf16 *tok_k, const bf16 *tok_v,
-                                    cudaStream_t st, bool pdl = false);
+// q4.kq != nullptr (in all layers of a batch or none): keys [0, n - 1) are read from the 4-bit cache (expanded and rotated
+// with `cs` on the way into shared memory, at position rank[m * cap + slot] for slot < ranked_len and slot above) and only
+// key n - 1, the token of this step, from k_rot / v, which then hold just that unit, [h_kv][d].  tok_k / tok_v (4-bit
+// cache only, may be null): the token's pre-RoPE keys and values [h_kv][d], which the kernel quantises into
+// slot n - 1 of the cache.
+struct DecodeAttnLayer {
+  const bf16 *q_rot, *k_rot, *v;
+  float *part_o, *part_ml;
+  unsigned *counters;
+  bf16 *out;
+  Int4Half q4;
+  const float2 *cs;
+  const int32_t *rank;
+  const bf16 *tok_k, *tok_v;
+  int cap, n, n_splits, ranked_len;
+};
+template <int N> struct DecodeAttnBatchN { DecodeAttnLayer l[N]; };
+typedef DecodeAttnBatchN<DECODE_BATCH> DecodeAttnBatch;
+int decode_attn_splits(int h_kv, int n, bool int4);
+cudaError_t launch_attention_decode(const DecodeAttnBatch &b, int n_layers, int h, int h_kv, int d, cudaStream_t st, bool pdl);
 
 // dst[c][r] = src[r][c]  (weight repack at create)
 cudaError_t launch_transpose_bf16(const bf16 *src, bf16 *dst, int rows, int cols, cudaStream_t st);

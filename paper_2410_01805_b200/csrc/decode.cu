@@ -3,6 +3,8 @@
 // attention.  Plain CUDA cores, 16-byte loads, no tensor cores (there is no contraction to tile).
 #include <stdlib.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace locret {
@@ -39,12 +41,20 @@ constexpr int GV_THREADS = 256;
 // sum_n hidden * W2[n][m] and the block writes one partial score per KV head.
 // The block that finishes last (counted with a wrapping atomic, so the counter is zero again
 // afterwards) adds the per-block partials in block order: deterministic, and no second launch.
-template <int MODE>
+template <int MODE, int NL>
 __global__ void __launch_bounds__(GV_THREADS)
 gemv_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ Wt, int N, int K, bf16 *__restrict__ y,
-            const float *__restrict__ W2, float *__restrict__ partial, int h_kv, int act,
-            unsigned *__restrict__ counter, float *__restrict__ score_out, int score_stride,
-            const bf16 *__restrict__ resid) {
+            const bf16 *__restrict__ resid, int h_kv, int act, const __grid_constant__ RhGemvBatchN<NL> b) {
+  // (MODE 1: blockIdx.y = layer)
+  const float *__restrict__ W2 = nullptr;
+  float *__restrict__ partial = nullptr, *__restrict__ score_out = nullptr;
+  unsigned *__restrict__ counter = nullptr;
+  int score_stride = 0;
+  if (MODE == 1) {
+    const RhGemvLayer &l = b.l[NL == 1 ? 0 : blockIdx.y];
+    x = l.z; Wt = l.W1t; W2 = l.W2; partial = l.partial; score_out = l.score_out; counter = l.counter;
+    score_stride = l.score_stride;
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint4 *sx = reinterpret_cast<uint4 *>(smem_raw);  // K / 8 vectors
   float *swarp = reinterpret_cast<float *>(sx + K / 8);  // [8 warps][32]
@@ -122,6 +132,39 @@ gemv_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ Wt, int N, int 
   }
 }
 
+// Elements i and i + d/2 of head hd of the token's projection: staging, position (= slot), RoPE from the bf16-rounded
+// values (what the pre-RoPE cache stores), append.
+__device__ __forceinline__ void rope_append_pair(const RopeAppendArgs &a, bf16 *staging, int hd, int i, bf16 b0, bf16 b1) {
+  const int half = a.d / 2, n0 = hd * a.d + i, n1 = n0 + half, slot = a.len;
+  staging[n0] = b0;
+  staging[n1] = b1;
+  if (hd < a.h + a.h_kv) {
+    const float2 t = a.cs[(size_t)slot * half + i];
+    const float x0 = __bfloat162float(b0), x1 = __bfloat162float(b1);
+    // lower half: x1 cos − x2 sin ; upper half: x2 cos + x1 sin
+    const bf16 q0 = __float2bfloat16_rn(x0 * t.x - x1 * t.y), q1 = __float2bfloat16_rn(x1 * t.x + x0 * t.y);
+    if (hd < a.h) {
+      a.q_rot[n0] = q0;
+      a.q_rot[n1] = q1;
+    } else {
+      const int m = hd - a.h;
+      const size_t off = ((size_t)m * a.cap + slot) * a.d + i;
+      if (a.k_pre) { a.k_pre[off] = b0; a.k_pre[off + half] = b1; }  // null for a 4-bit cache
+      bf16 *k = a.tok_k ? a.tok_k + (size_t)m * a.d + i : a.k_rot + off;
+      k[0] = q0;
+      k[half] = q1;
+      if (i == 0) a.tid[(size_t)m * a.cap + slot] = a.seen;
+    }
+    if (a.z_post) { a.z_post[n0] = q0; a.z_post[n1] = q1; }
+  } else {
+    const int m = hd - a.h - a.h_kv;
+    bf16 *v = a.tok_v ? a.tok_v + (size_t)m * a.d + i : a.v + ((size_t)m * a.cap + slot) * a.d + i;
+    v[0] = b0;
+    v[half] = b1;
+    if (a.z_post) { a.z_post[n0] = b0; a.z_post[n1] = b1; }
+  }
+}
+
 // Projection of one token with positions, RoPE and cache append: a warp computes the two rows
 // (i, i + d/2) of one head, so it holds a whole rotation pair.  The rotation starts from the
 // bf16-rounded projection, the value the pre-RoPE cache stores.
@@ -151,67 +194,42 @@ gemv_rope_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ Wt, int K,
     }
     s0 = warp_sum(s0);
     s1 = warp_sum(s1);
-    if (lane != 0) continue;
-    const bf16 b0 = __float2bfloat16_rn(s0), b1 = __float2bfloat16_rn(s1);
-    staging[n0] = b0;
-    staging[n1] = b1;
-    const int slot = a.len;
-    if (hd < a.h + a.h_kv) {
-      const float2 t = a.cs[(size_t)slot * half + i];
-      const float x0 = __bfloat162float(b0), x1 = __bfloat162float(b1);
-      // lower half: x1 cos − x2 sin ; upper half: x2 cos + x1 sin
-      const bf16 q0 = __float2bfloat16_rn(x0 * t.x - x1 * t.y), q1 = __float2bfloat16_rn(x1 * t.x + x0 * t.y);
-      if (hd < a.h) {
-        a.q_rot[n0] = q0;
-        a.q_rot[n1] = q1;
-      } else {
-        const int m = hd - a.h;
-        const size_t off = ((size_t)m * a.cap + slot) * a.d + i;
-        if (a.k_pre) { a.k_pre[off] = b0; a.k_pre[off + half] = b1; }  // null for a 4-bit cache
-        a.k_rot[off] = q0;
-        a.k_rot[off + half] = q1;
-        if (i == 0) a.tid[(size_t)m * a.cap + slot] = a.seen;
-      }
-      if (a.z_post) { a.z_post[n0] = q0; a.z_post[n1] = q1; }
-    } else {
-      const int m = hd - a.h - a.h_kv;
-      const size_t off = ((size_t)m * a.cap + slot) * a.d + i;
-      a.v[off] = b0;
-      a.v[off + half] = b1;
-      if (a.z_post) { a.z_post[n0] = b0; a.z_post[n1] = b1; }
-    }
+    if (lane == 0) rope_append_pair(a, staging, hd, i, __float2bfloat16_rn(s0), __float2bfloat16_rn(s1));
   }
 }
 
-// The same projection for K <= 4096 laid out for bandwidth: a block of 512 threads owns a contiguous
-// range of rotation pairs, thread t holds element group t of x in registers (no staging step before
-// the first weight load) and reads group t of both rows of four pairs at a time, so a block has
-// 64 KB of weights in flight and two blocks per SM cover each other's reductions.  The eight
-// partial sums of a batch are reduced with one butterfly that halves the number of values at each
-// step (9 shuffles instead of 40), then across the warps through shared memory.
+// The same projection for K <= 4096 laid out for bandwidth, for one layer or for the layers of a stack that share
+// the input: the rotation pairs of all layers are one range, a block of 512 threads owns a contiguous part of it,
+// thread t holds element group t of x in registers (no staging step before the first weight load) and reads
+// group t of both rows of four pairs at a time, so a block has 64 KB of weights in flight and two blocks per SM
+// cover each other's reductions.  The eight partial sums of a batch are reduced with one butterfly that halves the
+// number of values at each step (9 shuffles instead of 40), then across the warps through shared memory.
 constexpr int GW_THREADS = 512, GW_PB = 4;
 
+template <int NL>
 __global__ void __launch_bounds__(GW_THREADS, 2)
-gemv_rope_wide_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ Wt, int K, bf16 *__restrict__ staging,
-                      RopeAppendArgs a) {
+gemv_rope_wide_kernel(const bf16 *__restrict__ x, int K, int n_layers, const __grid_constant__ GemvRopeBatchN<NL> b) {
   __shared__ float red[2][GW_THREADS / 32][2 * GW_PB];
   __shared__ float res[2][2 * GW_PB];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int kv = K / 8;
   const bool act = tid < kv;
-  const int half = a.d / 2, heads = a.h + 2 * a.h_kv;
-  const int n_pairs = heads * half;
+  const int h = b.a[0].h, h_kv = b.a[0].h_kv, d = b.a[0].d;  // (the same in every layer)
+  const int half = d / 2, heads = h + 2 * h_kv;
+  const int per_layer = heads * half, n_pairs = (NL == 1 ? 1 : n_layers) * per_layer;
   const int p_lo = (int)((long long)blockIdx.x * n_pairs / gridDim.x);
   const int p_hi = (int)((long long)(blockIdx.x + 1) * n_pairs / gridDim.x);
-  const uint4 *W4 = reinterpret_cast<const uint4 *>(Wt);
   // the first batch of weights is requested before x
   uint4 w[2 * GW_PB];
   auto load_batch = [&](int p0) {
 #pragma unroll
     for (int j = 0; j < GW_PB; j++) {
-      const int it = min(p0 + j, n_pairs - 1);
+      int it = min(p0 + j, n_pairs - 1);
+      const int layer = NL == 1 ? 0 : it / per_layer;
+      it -= layer * per_layer;
+      const uint4 *W4 = reinterpret_cast<const uint4 *>(b.Wt[layer]);
       const int hd = it / half, i = it - hd * half;
-      const size_t n0 = (size_t)hd * a.d + i;
+      const size_t n0 = (size_t)hd * d + i;
       w[2 * j] = act ? __ldg(W4 + n0 * kv + tid) : make_uint4(0, 0, 0, 0);
       w[2 * j + 1] = act ? __ldg(W4 + (n0 + half) * kv + tid) : make_uint4(0, 0, 0, 0);
     }
@@ -257,36 +275,11 @@ gemv_rope_wide_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ Wt, i
     }
     __syncthreads();
     if (tid < GW_PB && p0 + tid < p_hi) {
-      const int it = p0 + tid;
-      const int hd = it / half, i = it - hd * half;
-      const int n0 = hd * a.d + i, n1 = n0 + half;
-      const bf16 b0 = __float2bfloat16_rn(res[par][2 * tid]), b1 = __float2bfloat16_rn(res[par][2 * tid + 1]);
-      staging[n0] = b0;
-      staging[n1] = b1;
-      const int slot = a.len;
-      if (hd < a.h + a.h_kv) {
-        const float2 t = a.cs[(size_t)slot * half + i];
-        const float x0 = __bfloat162float(b0), x1 = __bfloat162float(b1);
-        const bf16 q0 = __float2bfloat16_rn(x0 * t.x - x1 * t.y), q1 = __float2bfloat16_rn(x1 * t.x + x0 * t.y);
-        if (hd < a.h) {
-          a.q_rot[n0] = q0;
-          a.q_rot[n1] = q1;
-        } else {
-          const int m = hd - a.h;
-          const size_t off = ((size_t)m * a.cap + slot) * a.d + i;
-          if (a.k_pre) { a.k_pre[off] = b0; a.k_pre[off + half] = b1; }  // null for a 4-bit cache
-          a.k_rot[off] = q0;
-          a.k_rot[off + half] = q1;
-          if (i == 0) a.tid[(size_t)m * a.cap + slot] = a.seen;
-        }
-        if (a.z_post) { a.z_post[n0] = q0; a.z_post[n1] = q1; }
-      } else {
-        const int m = hd - a.h - a.h_kv;
-        const size_t off = ((size_t)m * a.cap + slot) * a.d + i;
-        a.v[off] = b0;
-        a.v[off + half] = b1;
-        if (a.z_post) { a.z_post[n0] = b0; a.z_post[n1] = b1; }
-      }
+      const int layer = NL == 1 ? 0 : (p0 + tid) / per_layer, it = p0 + tid - layer * per_layer;
+      const int hd = it / half;
+      const RopeAppendArgs &a = b.a[layer];
+      rope_append_pair(a, const_cast<bf16 *>(a.staging), hd, it - hd * half, __float2bfloat16_rn(res[par][2 * tid]),
+                       __float2bfloat16_rn(res[par][2 * tid + 1]));
     }
   }
 }
@@ -320,16 +313,20 @@ constexpr int DA_THREADS = 128, DA_G = 16, DA_KT = 64;
 
 // INT4: keys [0, n - 1) come from the 4-bit cache (codes and scales expanded, keys rotated at the
 // unit's position in temporal order, with the arithmetic of the expansion pre-pass, as the tile is brought into shared
-// memory); key n - 1, the token of this step, comes from the bf16 arrays k_rot / v like every key of
-// a bf16 cache.
-template <int D, bool INT4>
-__global__ void __launch_bounds__(DA_THREADS)
-attn_decode_kernel(const bf16 *__restrict__ q_rot, const bf16 *__restrict__ k_rot,
-                   const bf16 *__restrict__ v, float *__restrict__ part_o, float *__restrict__ part_ml,
-                   int h, int h_kv, int cap, int n, int n_splits, float scale_log2,
-                   unsigned *__restrict__ counters, bf16 *__restrict__ out, Int4Half q4,
-                   const float2 *__restrict__ cs, const int32_t *__restrict__ rank, int ranked_len,
-                   const bf16 *__restrict__ tok_k, const bf16 *__restrict__ tok_v) {
+// memory); key n - 1, the token of this step, comes in bf16 from k_rot / v, which then hold that one
+// unit of every head, [h_kv][D].
+template <int D, bool INT4, int NL>
+__global__ void __launch_bounds__(DA_THREADS, INT4 ? 2 : 4)  // (168 registers, for three blocks, cost the 4-bit kernel a third of its speed)
+attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ DecodeAttnBatchN<NL> batch) {
+  const int hgroups = (h / h_kv + DA_G - 1) / DA_G, layer = NL == 1 ? 0 : blockIdx.z / hgroups;
+  const DecodeAttnLayer &a = batch.l[layer];
+  const bf16 *__restrict__ q_rot = a.q_rot, *__restrict__ k_rot = a.k_rot, *__restrict__ v = a.v;
+  float *__restrict__ part_o = a.part_o, *__restrict__ part_ml = a.part_ml;
+  const int cap = a.cap, n = a.n, n_splits = a.n_splits, ranked_len = a.ranked_len;
+  const Int4Half &q4 = a.q4;
+  const float2 *__restrict__ cs = a.cs;
+  const int32_t *__restrict__ rank = a.rank;
+  const bf16 *__restrict__ tok_k = a.tok_k, *__restrict__ tok_v = a.tok_v;
   constexpr int LD = D + 8;
   constexpr int VPR = D / 8;  // 16-byte vectors per row
   extern __shared__ __align__(16) unsigned char da_smem[];
@@ -343,7 +340,8 @@ attn_decode_kernel(const bf16 *__restrict__ q_rot, const bf16 *__restrict__ k_ro
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g4 = lane >> 2, q = lane & 3;
   const int g = h / h_kv;
-  const int m = blockIdx.x, split = blockIdx.y, hg = blockIdx.z;
+  const int m = blockIdx.x, split = blockIdx.y, hg = blockIdx.z - layer * hgroups;
+  if (NL > 1 && split >= n_splits) return;  // (layers of a batch may hold different numbers of keys)
   const int h0 = m * g + hg * DA_G;
   const int gh = min(DA_G, g - hg * DA_G);  // heads handled here
   const int per = (n + n_splits - 1) / n_splits;
@@ -427,7 +425,7 @@ attn_decode_kernel(const bf16 *__restrict__ q_rot, const bf16 *__restrict__ k_ro
         dequant8(pre[i].vw1, pre[i].vs, b);
         va = to_bf16x8(a); vb = to_bf16x8(b);
       } else if (key >= n - 1 && key < k1) {  // the token of this step
-        const size_t off = ((size_t)m * cap + key) * D + c;
+        const size_t off = (size_t)m * D + c;
         ka = *reinterpret_cast<const uint4 *>(k_rot + off); kb = *reinterpret_cast<const uint4 *>(k_rot + off + HALF);
         va = *reinterpret_cast<const uint4 *>(v + off); vb = *reinterpret_cast<const uint4 *>(v + off + HALF);
       }
@@ -591,14 +589,16 @@ attn_decode_kernel(const bf16 *__restrict__ q_rot, const bf16 *__restrict__ k_ro
     lrow[r] += __shfl_xor_sync(0xffffffffu, lrow[r], 2);
     if (q == 0) { wm[warp][g4 + 8 * r] = mrow[r]; wl[warp][g4 + 8 * r] = lrow[r]; }
   }
-  float *fo = reinterpret_cast<float *>(sK);  // [4][16][D] floats = 32 KB at D = 128 <= the tile buffers
+  constexpr int LF = D + 8;                   // (rows of eight lanes then spread over the banks)
+  float *fo = reinterpret_cast<float *>(sK);  // [4][16][LF] floats = 34 KB at D = 128 <= the tile buffers
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < 2; r++)
+    if (g4 + 8 * r < gh) {  // (the rest of the 16 rows is padding)
 #pragma unroll
-    for (int i = 0; i < D / 8; i++) {
-      float2 val = make_float2(o[i][2 * r], o[i][2 * r + 1]);
-      *reinterpret_cast<float2 *>(fo + ((size_t)(warp * DA_G + g4 + 8 * r)) * D + i * 8 + q * 2) = val;
+      for (int i = 0; i < D / 8; i++)
+        *reinterpret_cast<float2 *>(fo + (warp * DA_G + g4 + 8 * r) * LF + i * 8 + q * 2) =
+            make_float2(o[i][2 * r], o[i][2 * r + 1]);
     }
   __syncthreads();
   // partial result of this split: o [h][split][D] (not normalised), (m, l) [h][split][2]
@@ -609,7 +609,7 @@ attn_decode_kernel(const bf16 *__restrict__ q_rot, const bf16 *__restrict__ k_ro
 #pragma unroll
     for (int w = 0; w < 4; w++) {
       const float wgt = (wm[w][i] == -INFINITY) ? 0.f : exp2f(wm[w][i] - mx);
-      acc = fmaf(wgt, fo[((size_t)(w * DA_G + i)) * D + c], acc);
+      acc = fmaf(wgt, fo[(w * DA_G + i) * LF + c], acc);
       l = fmaf(wgt, wl[w][i], l);
     }
     const size_t hs = (size_t)(h0 + i) * n_splits + split;
@@ -620,7 +620,7 @@ attn_decode_kernel(const bf16 *__restrict__ q_rot, const bf16 *__restrict__ k_ro
   // ---- the split that finishes last merges the partial results of all splits
   __threadfence();
   __syncthreads();
-  if (tid == 0) last = atomicInc(&counters[m * gridDim.z + hg], n_splits - 1) == (unsigned)(n_splits - 1);
+  if (tid == 0) last = atomicInc(&a.counters[m * hgroups + hg], n_splits - 1) == (unsigned)(n_splits - 1);
   __syncthreads();
   if (!last) return;
   __threadfence();
@@ -673,7 +673,7 @@ attn_decode_kernel(const bf16 *__restrict__ q_rot, const bf16 *__restrict__ k_ro
     uint2 o2;
     o2.x = pack_bf16(acc.x * inv, acc.y * inv);
     o2.y = pack_bf16(acc.z * inv, acc.w * inv);
-    *reinterpret_cast<uint2 *>(out + (size_t)(h0 + i) * D + c) = o2;
+    *reinterpret_cast<uint2 *>(a.out + (size_t)(h0 + i) * D + c) = o2;
   }
 }
 
@@ -683,8 +683,7 @@ cudaError_t launch_gemv(const bf16 *x, const bf16 *Wt, int N, int K, bf16 *y, cu
   if (K % 8) return cudaErrorInvalidValue;
   const int smem = K * 2 + 8 * 32 * 4;
   const int blocks = min((N + 7) / 8, 148 * 4);
-  gemv_kernel<0><<<blocks, GV_THREADS, smem, st>>>(x, Wt, N, K, y, nullptr, nullptr, 0, 0, nullptr, nullptr, 0,
-                                                   nullptr);
+  gemv_kernel<0, 1><<<blocks, GV_THREADS, smem, st>>>(x, Wt, N, K, y, nullptr, 0, 0, RhGemvBatchN<1>{});
   return cudaGetLastError();
 }
 
@@ -694,7 +693,7 @@ cudaError_t launch_gemv_resid(const bf16 *x, const bf16 *Wt, int N, int K, const
   if (K % 8) return cudaErrorInvalidValue;
   const int smem = K * 2 + 8 * 32 * 4;
   const int blocks = min((N + 7) / 8, 148 * 4);
-  gemv_kernel<0><<<blocks, GV_THREADS, smem, st>>>(x, Wt, N, K, y, nullptr, nullptr, 0, 0, nullptr, nullptr, 0, r);
+  gemv_kernel<0, 1><<<blocks, GV_THREADS, smem, st>>>(x, Wt, N, K, y, r, 0, 0, RhGemvBatchN<1>{});
   return cudaGetLastError();
 }
 
@@ -732,31 +731,38 @@ cudaError_t launch_gemv_gated(const bf16 *x, const bf16 *Wt, int F, int K, bf16 
   return cudaGetLastError();
 }
 
+bool gemv_rope_batched(int K) { return K % 8 == 0 && K / 8 <= GW_THREADS; }
 int rh_gemv_blocks(int d_R) { return min((d_R + 3) / 4, 148 * 4); }
 
-cudaError_t launch_gemv_rope(const bf16 *x, const bf16 *Wt, int K, bf16 *staging, const RopeAppendArgs &a,
-                             cudaStream_t st, bool pdl) {
-  if (K % 8 || a.d % 2) return cudaErrorInvalidValue;
+cudaError_t launch_gemv_rope(const bf16 *x, int K, const GemvRopeBatch &b, int n_layers, cudaStream_t st, bool pdl) {
+  const RopeAppendArgs &a = b.a[0];
+  if (K % 8 || a.d % 2 || n_layers < 1 || n_layers > DECODE_BATCH) return cudaErrorInvalidValue;
   const int items = (a.h + 2 * a.h_kv) * (a.d / 2);
-  if (K / 8 <= GW_THREADS) {
-    const int blocks = min((items + GW_PB - 1) / GW_PB, 148 * 2);
-    return launch_kernel(gemv_rope_wide_kernel, dim3(blocks), dim3(GW_THREADS), 0, st, pdl, x, Wt, K, staging, a);
+  if (gemv_rope_batched(K)) {
+    const int blocks = min((n_layers * items + GW_PB - 1) / GW_PB, 148 * 2);
+    if (n_layers > 1)
+      return launch_kernel(gemv_rope_wide_kernel<DECODE_BATCH>, dim3(blocks), dim3(GW_THREADS), 0, st, pdl, x, K, n_layers, b);
+    GemvRopeBatchN<1> one;
+    one.Wt[0] = b.Wt[0];
+    one.a[0] = a;
+    return launch_kernel(gemv_rope_wide_kernel<1>, dim3(blocks), dim3(GW_THREADS), 0, st, pdl, x, K, 1, one);
   }
+  if (n_layers != 1) return cudaErrorInvalidValue;
   const int blocks = min((items + 7) / 8, 148 * 4);
-  return launch_kernel(gemv_rope_kernel, dim3(blocks), dim3(GV_THREADS), (size_t)K * 2, st, pdl, x, Wt, K, staging, a);
+  return launch_kernel(gemv_rope_kernel, dim3(blocks), dim3(GV_THREADS), (size_t)K * 2, st, pdl, x, b.Wt[0], K,
+                       const_cast<bf16 *>(a.staging), a);
 }
 
-// score_out: where the token's scores go (element m * score_stride for KV head m); counter: one
-// zero-initialised word that the kernel leaves at zero
-cudaError_t launch_rh_gemv(const bf16 *z, const bf16 *W1t, const float *W2, float *partial, int d_R, int K,
-                           int h_kv, int act, unsigned *counter, float *score_out, int score_stride,
-                           cudaStream_t st, bool pdl) {
-  if (K % 16 || h_kv > 32) return cudaErrorInvalidValue;
+cudaError_t launch_rh_gemv(const RhGemvBatch &b, int n_layers, int d_R, int K, int h_kv, int act, cudaStream_t st, bool pdl) {
+  if (K % 16 || h_kv > 32 || n_layers < 1 || n_layers > DECODE_BATCH) return cudaErrorInvalidValue;
   const int smem = K * 2 + 8 * 32 * 4;
-  const int blocks = rh_gemv_blocks(d_R);
-  return launch_kernel(gemv_kernel<1>, dim3(blocks), dim3(GV_THREADS), (size_t)smem, st, pdl, z, W1t, d_R, K,
-                       (bf16 *)nullptr, W2, partial, h_kv, act, counter, score_out, score_stride,
-                       (const bf16 *)nullptr);
+  const dim3 grid(rh_gemv_blocks(d_R), n_layers);
+  const bf16 *none = nullptr;
+  if (n_layers > 1)
+    return launch_kernel(gemv_kernel<1, DECODE_BATCH>, grid, dim3(GV_THREADS), (size_t)smem, st, pdl, none, none, d_R, K,
+                         (bf16 *)nullptr, none, h_kv, act, b);
+  return launch_kernel(gemv_kernel<1, 1>, grid, dim3(GV_THREADS), (size_t)smem, st, pdl, none, none, d_R, K, (bf16 *)nullptr,
+                       none, h_kv, act, RhGemvBatchN<1>{{b.l[0]}});
 }
 
 // Splits of the key range per KV head.  Measured at the Llama shape (8 KV heads, 6000 keys, 256 steps through
@@ -777,33 +783,35 @@ int decode_attn_splits(int h_kv, int n, bool int4) {
   return s < 1 ? 1 : s;
 }
 
-cudaError_t launch_attention_decode(const bf16 *q_rot, const bf16 *k_rot, const bf16 *v, bf16 *out,
-                                    float *part_o, float *part_ml, unsigned *counters, int h, int h_kv, int d,
-                                    int cap, int n, int n_splits, const Int4Half *q4, const float2 *cs,
-                                    const int32_t *rank, int ranked_len, const bf16 *tok_k, const bf16 *tok_v,
-                                    cudaStream_t st, bool pdl) {
-  const int g = h / h_kv;
-  dim3 grid(h_kv, n_splits, (g + DA_G - 1) / DA_G);
-  if ((int)grid.x * (int)grid.z > 32 * 16 || n_splits > 64) return cudaErrorInvalidValue;
+cudaError_t launch_attention_decode(const DecodeAttnBatch &b, int n_layers, int h, int h_kv, int d, cudaStream_t st,
+                                    bool pdl) {
+  const int hgroups = (h / h_kv + DA_G - 1) / DA_G;
+  if (n_layers < 1 || n_layers > DECODE_BATCH || h_kv * hgroups > 32 * 16) return cudaErrorInvalidValue;
+  int splits = 1;
+  for (int i = 0; i < n_layers; i++) splits = b.l[i].n_splits > splits ? b.l[i].n_splits : splits;
+  if (splits > 64) return cudaErrorInvalidValue;
+  const dim3 grid(h_kv, splits, n_layers * hgroups);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)d);
-  const Int4Half qq = q4 ? *q4 : Int4Half{nullptr, nullptr, nullptr, nullptr};
-  auto launch = [&](auto kern, int smem, PerDeviceFlag &attr_set) -> cudaError_t {
-    if (cudaError_t e = allow_dynamic_smem(kern, smem, attr_set); e != cudaSuccess) return e;
-    return launch_kernel(kern, grid, dim3(DA_THREADS), (size_t)smem, st, pdl, q_rot, k_rot, v, part_o, part_ml, h, h_kv,
-                         cap, n, n_splits, scale_log2, counters, out, qq, cs, rank, rank ? ranked_len : 0, tok_k, tok_v);
+  const bool q4 = b.l[0].q4.kq != nullptr;
+  auto run = [&](auto kern1, auto kern_n, PerDeviceFlag (&attr_set)[2]) -> cudaError_t {
+    const size_t smem = (DA_G + 4 * DA_KT) * (d + 8) * 2;
+    if (n_layers > 1) {
+      if (cudaError_t e = allow_dynamic_smem(kern_n, (int)smem, attr_set[1]); e != cudaSuccess) return e;
+      return launch_kernel(kern_n, grid, dim3(DA_THREADS), smem, st, pdl, h, h_kv, scale_log2, b);
+    }
+    if (cudaError_t e = allow_dynamic_smem(kern1, (int)smem, attr_set[0]); e != cudaSuccess) return e;
+    return launch_kernel(kern1, grid, dim3(DA_THREADS), smem, st, pdl, h, h_kv, scale_log2, DecodeAttnBatchN<1>{{b.l[0]}});
   };
-  static PerDeviceFlag set_done[2][3];
-  const int qi = q4 ? 1 : 0;
+  auto launch = [&](auto dim) -> cudaError_t {
+    constexpr int D = decltype(dim)::value;
+    static PerDeviceFlag set_q4[2], set_bf16[2];
+    return q4 ? run(attn_decode_kernel<D, true, 1>, attn_decode_kernel<D, true, DECODE_BATCH>, set_q4)
+              : run(attn_decode_kernel<D, false, 1>, attn_decode_kernel<D, false, DECODE_BATCH>, set_bf16);
+  };
   switch (d) {
-    case 64:
-      return q4 ? launch(attn_decode_kernel<64, true>, (DA_G + 4 * DA_KT) * (64 + 8) * 2, set_done[qi][0])
-                : launch(attn_decode_kernel<64, false>, (DA_G + 4 * DA_KT) * (64 + 8) * 2, set_done[qi][0]);
-    case 96:
-      return q4 ? launch(attn_decode_kernel<96, true>, (DA_G + 4 * DA_KT) * (96 + 8) * 2, set_done[qi][1])
-                : launch(attn_decode_kernel<96, false>, (DA_G + 4 * DA_KT) * (96 + 8) * 2, set_done[qi][1]);
-    case 128:
-      return q4 ? launch(attn_decode_kernel<128, true>, (DA_G + 4 * DA_KT) * (128 + 8) * 2, set_done[qi][2])
-                : launch(attn_decode_kernel<128, false>, (DA_G + 4 * DA_KT) * (128 + 8) * 2, set_done[qi][2]);
+    case 64: return launch(std::integral_constant<int, 64>{});
+    case 96: return launch(std::integral_constant<int, 96>{});
+    case 128: return launch(std::integral_constant<int, 128>{});
   }
   return cudaErrorInvalidValue;
 }

@@ -40,11 +40,21 @@ struct ScratchPool {
   size_t staging_b[2] = {0, 0}, qrot_b = 0, zpost_b[2] = {0, 0}, partial_b = 0, keep_b = 0, kexp_b = 0, vexp_b = 0;
   bf16 *staging[2] = {nullptr, nullptr}, *q_rot = nullptr, *z_post[2] = {nullptr, nullptr};
   bf16 *k_exp = nullptr, *v_exp = nullptr;  // 4-bit caches: bf16 expansion of the layer in flight
-  float *dec_o = nullptr, *dec_ml = nullptr;  // decode attention: per-split partial results
-  size_t deco_b = 0, decml_b = 0;
-  // decode kernels whose last block merges the partial results: zeroed words that each launch
-  // leaves at zero (word 0: retaining head; words 1..: attention, one per KV head x head group)
-  unsigned *dec_cnt = nullptr;
+  // One-token steps: up to DECODE_BATCH layers of a stack go through a launch together, each with a set of its own of the
+  // buffers below (as many sets as layers share the pool, at most DECODE_BATCH; a set has room for the largest of them).
+  struct DecodeSets {
+    int n = 0;
+    size_t o = 0, ml = 0, partial = 0, d_in = 0, hd = 0, kv = 0;  // elements of one set
+    // attention: per-split partial results; retaining head: per-block partial scores
+    float *dec_o = nullptr, *dec_ml = nullptr, *dec_partial = nullptr;
+    // the token's [Q | K | V] before and (retaining-head input variant) after RoPE, its rotated queries, and for 4-bit
+    // caches its rotated key and its value in bf16
+    bf16 *staging = nullptr, *z_post = nullptr, *q_rot = nullptr, *tok_kv = nullptr;
+    size_t o_b = 0, ml_b = 0, partial_b = 0, staging_b = 0, zpost_b = 0, q_b = 0, tok_b = 0;
+    // kernels whose last block merges the partial results: zeroed words that each launch leaves at zero
+    // (word 0: retaining head; words 1..: attention, one per KV head x head group)
+    unsigned *cnt = nullptr;
+  } dec;
   float *partial = nullptr;
   int32_t *keep = nullptr;
   struct CsTable { float theta; int d, cap; float2 *ptr; };
@@ -153,7 +163,9 @@ void release_pool(ScratchPool *p) {
   if (p->ev_exp_free) cudaEventDestroy(p->ev_exp_free);
   if (p->ev_exp_ready) cudaEventDestroy(p->ev_exp_ready);
   if (p->ev_side_idle) cudaEventDestroy(p->ev_side_idle);
-  cudaFree(p->q_rot); cudaFree(p->partial); cudaFree(p->keep); cudaFree(p->dec_o); cudaFree(p->dec_ml); cudaFree(p->dec_cnt);
+  cudaFree(p->q_rot); cudaFree(p->partial); cudaFree(p->keep);
+  cudaFree(p->dec.dec_o); cudaFree(p->dec.dec_ml); cudaFree(p->dec.dec_partial); cudaFree(p->dec.cnt);
+  cudaFree(p->dec.staging); cudaFree(p->dec.z_post); cudaFree(p->dec.q_rot); cudaFree(p->dec.tok_kv);
   cudaFree(p->k_exp); cudaFree(p->v_exp);
   for (auto &t : p->cs) cudaFree(t.ptr);
   g_pools.erase(std::make_pair(p->device, p->st));
@@ -375,9 +387,9 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
             cudaEventCreateWithFlags(&p->ev_exp_ready, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&p->ev_side_idle, cudaEventDisableTiming) == cudaSuccess;
       }
-      if (g && !p->dec_cnt) {
-        g = cudaMalloc(&p->dec_cnt, DEC_CNT_WORDS * sizeof(unsigned)) == cudaSuccess &&
-            cudaMemsetAsync(p->dec_cnt, 0, DEC_CNT_WORDS * sizeof(unsigned), L->st) == cudaSuccess;
+      if (g && !p->dec.cnt) {
+        const size_t bytes = (size_t)DECODE_BATCH * DEC_CNT_WORDS * sizeof(unsigned);
+        g = cudaMalloc(&p->dec.cnt, bytes) == cudaSuccess && cudaMemsetAsync(p->dec.cnt, 0, bytes, L->st) == cudaSuccess;
         if (!g) cudaGetLastError();
       }
       if (p->side) cudaStreamSynchronize(p->side);  // buffers may be replaced below
@@ -390,11 +402,27 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
       {
         int nt = rh_num_tiles(dR) > rh_tc_num_tiles(dR) ? rh_num_tiles(dR) : rh_tc_num_tiles(dR);
         size_t pb = (size_t)nt * chunk * hk * sizeof(float);
-        const size_t pb_dec = (size_t)rh_gemv_blocks(dR) * hk * sizeof(float);
-        if (pb < pb_dec) pb = pb_dec;
         g = g && grow(&p->partial, &p->partial_b, pb, L->st);
-        g = g && grow(&p->dec_o, &p->deco_b, (size_t)h * 64 * d * sizeof(float), L->st);
-        g = g && grow(&p->dec_ml, &p->decml_b, (size_t)h * 64 * 2 * sizeof(float), L->st);
+      }
+      {
+        // (the new sizes count only once every buffer has them)
+        ScratchPool::DecodeSets &ds = p->dec;
+        auto most = [](size_t have, size_t want) { return want > have ? (want + 63) & ~(size_t)63 : have; };
+        const size_t n = p->refs < DECODE_BATCH ? p->refs : DECODE_BATCH;
+        const size_t o = most(ds.o, (size_t)h * 64 * d), ml = most(ds.ml, (size_t)h * 64 * 2),
+                     pt = most(ds.partial, (size_t)rh_gemv_blocks(dR) * hk), din = most(ds.d_in, L->d_in),
+                     qd = most(ds.hd, (size_t)h * d), kvd = most(ds.kv, (size_t)hk * d);
+        g = g && grow(&ds.dec_o, &ds.o_b, n * o * sizeof(float), L->st) &&
+            grow(&ds.dec_ml, &ds.ml_b, n * ml * sizeof(float), L->st) &&
+            grow(&ds.dec_partial, &ds.partial_b, n * pt * sizeof(float), L->st) &&
+            grow(&ds.staging, &ds.staging_b, n * din * sizeof(bf16), L->st) &&
+            grow(&ds.z_post, &ds.zpost_b, n * din * sizeof(bf16), L->st) &&
+            grow(&ds.q_rot, &ds.q_b, n * qd * sizeof(bf16), L->st) &&
+            grow(&ds.tok_kv, &ds.tok_b, n * 2 * kvd * sizeof(bf16), L->st);
+        if (g) {
+          if ((int)n > ds.n) ds.n = (int)n;
+          ds.o = o; ds.ml = ml; ds.partial = pt; ds.d_in = din; ds.hd = qd; ds.kv = kvd;
+        }
       }
       g = g && grow(&p->keep, &p->keep_b, (size_t)hk * budget * sizeof(int32_t), L->st);
       if (L->int4) {
@@ -545,30 +573,123 @@ int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaS
   return LOCRET_OK;
 }
 
+// What a step of n_tok tokens asks of its arguments (the begun half of a divided-heads step is finished first).
+int check_step(const locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t flags, const void *attn_out) {
+  if (!L || !hidden_in || !attn_out) return LOCRET_ERR_INVALID;
+  if (!on_layer_device(L)) return LOCRET_ERR_INVALID;
+  if (L->tp_pending) return LOCRET_ERR_INVALID;
+  if (n_tok < 1 || n_tok > L->chunk) return LOCRET_ERR_INVALID;
+  if (flags & ~(LOCRET_NO_EVICT | LOCRET_LAST_CHUNK)) return LOCRET_ERR_INVALID;
+  if (!aligned16(hidden_in) || !aligned16(attn_out)) return LOCRET_ERR_INVALID;
+  if (L->len + n_tok > L->cap) return LOCRET_ERR_CAPACITY;
+  return LOCRET_OK;
+}
+
+// One token through `count` layers with the same input (checked by the caller; more than one: see stack_batch), a chain of
+// three short kernels on the layers' own stream, overlapped by programmatic dependent launch (an event between them would
+// serialise them again).  Bandwidth-bound kernels of decode.cu.
+int token_step(locret_layer *const *layers, int count, const void *hidden_in, uint32_t flags, void *attn_out,
+               int64_t out_stride) {
+  locret_layer *const L0 = layers[0];
+  ScratchPool *const P = L0->pool;
+  const ScratchPool::DecodeSets &ds = P->dec;
+  const cudaStream_t st = L0->st;
+  const bool pdl = L0->use_pdl && !L0->timing;
+  if (L0->use_side && P->side_dirty) {
+    // the retaining head (and an eviction) run on the layer's own stream here, with scratch other layers' steps may
+    // still be using on the second stream
+    CK(cudaEventRecord(P->ev_side_idle, P->side));
+    CK(cudaStreamWaitEvent(st, P->ev_side_idle, 0));
+    P->side_dirty = false;
+  }
+  GemvRopeBatch qkv;
+  DecodeAttnBatch att;
+  RhGemvBatch rh;
+  for (int i = 0; i < count; i++) {
+    locret_layer *L = layers[i];
+    // this layer's cache is free once its previous selection / compaction has finished
+    if (L->use_side && L->side_pending) CK(cudaStreamWaitEvent(st, L->ev_side, 0));
+    L->side_pending = false;
+    bf16 *const staging = ds.staging + i * ds.d_in, *const q_rot = ds.q_rot + i * ds.hd;
+    bf16 *const z_post = L->cfg.rh_input == 1 ? ds.z_post + i * ds.d_in : nullptr;
+    bf16 *const tok_k = L->int4 ? ds.tok_kv + i * 2 * ds.kv : nullptr, *const tok_v = L->int4 ? tok_k + ds.kv : nullptr;
+    const int n = L->len + 1;
+    RopeAppendArgs &ra = qkv.a[i];
+    ra.staging = staging; ra.q_rot = q_rot; ra.z_post = z_post;
+    ra.k_pre = L->k_pre; ra.k_rot = L->k_rot; ra.v = L->v; ra.tok_k = tok_k; ra.tok_v = tok_v;  // (4-bit: the first three null)
+    ra.tid = L->tid; ra.cs = L->cs;
+    ra.n_tok = 1; ra.h = L->h; ra.h_kv = L->h_kv; ra.d = L->d; ra.cap = L->cap; ra.len = L->len; ra.seen = L->seen;
+    ra.per_head = 0;
+    qkv.Wt[i] = L->wqkv_t;
+    DecodeAttnLayer &al = att.l[i];
+    al.q_rot = q_rot; al.k_rot = L->int4 ? tok_k : L->k_rot; al.v = L->int4 ? tok_v : L->v;
+    al.part_o = ds.dec_o + i * ds.o; al.part_ml = ds.dec_ml + i * ds.ml;
+    al.counters = ds.cnt + i * DEC_CNT_WORDS + 1;
+    al.out = static_cast<bf16 *>(attn_out) + i * out_stride;
+    al.q4 = L->int4 ? L->q4 : Int4Half{nullptr, nullptr, nullptr, nullptr};
+    al.cs = L->cs; al.rank = L->rank[L->rcur]; al.ranked_len = L->ranked_len;
+    al.tok_k = L->int4 ? staging + (size_t)L->h * L->d : nullptr;
+    al.tok_v = L->int4 ? staging + (size_t)(L->h + L->h_kv) * L->d : nullptr;
+    al.cap = L->cap; al.n = n; al.n_splits = decode_attn_splits(L->h_kv, n, L->int4);
+    RhGemvLayer &rl = rh.l[i];
+    rl.z = z_post ? z_post : staging; rl.W1t = L->w1_t; rl.W2 = L->w2f;
+    rl.partial = ds.dec_partial + i * ds.partial; rl.score_out = L->s + L->len; rl.score_stride = L->cap;
+    rl.counter = ds.cnt + i * DEC_CNT_WORDS;
+  }
+  {  // (a) projection, positions, RoPE and append
+    Timed t(L0, LOCRET_K_QKV);
+    CK(launch_gemv_rope((const bf16 *)hidden_in, L0->D, qkv, count, st, pdl));
+  }
+  {  // (b) Eq. 1
+    Timed t(L0, LOCRET_K_ATTN);
+    CK(launch_attention_decode(att, count, L0->h, L0->h_kv, L0->d, st, pdl));
+  }
+  {  // (c) retaining head
+    Timed t(L0, LOCRET_K_RH);
+    CK(launch_rh_gemv(rh, count, L0->d_R, L0->d_in, L0->h_kv, L0->cfg.act, st, pdl));
+  }
+  for (int i = 0; i < count; i++)
+    if (const int rc = evict_and_close(layers[i], 1, flags, false, st); rc != LOCRET_OK) return rc;
+  return LOCRET_OK;
+}
+
+bool takes_token_step(const locret_layer *L) { return L->use_tc && !L->per_head; }
+
+// How many layers from the first on go through one launch per kernel: different layers of one stream with the same shape,
+// none of which would refuse the step.
+int stack_batch(locret_layer *const *layers, int n_layers, const void *hidden_in, const void *attn_out, int64_t out_stride) {
+  const locret_layer *A = layers[0];
+  // (outputs that share memory are written in the layers' order: one launch after the other)
+  if (!A || !takes_token_step(A) || A->timing || out_stride < (int64_t)A->h * A->d || !gemv_rope_batched(A->D)) return 1;
+  const int most = n_layers < A->pool->dec.n ? n_layers : A->pool->dec.n;
+  int k = 0;
+  for (; k < most; k++) {
+    const locret_layer *L = layers[k];
+    if (check_step(L, hidden_in, 1, LOCRET_NO_EVICT, static_cast<const bf16 *>(attn_out) + k * out_stride) != LOCRET_OK) break;
+    if (!takes_token_step(L) || L->timing || L->pool != A->pool || L->use_pdl != A->use_pdl || L->use_side != A->use_side ||
+        L->h != A->h || L->h_kv != A->h_kv || L->d != A->d || L->D != A->D || L->d_R != A->d_R || L->int4 != A->int4 ||
+        L->cfg.act != A->cfg.act)
+      break;
+    bool again = false;
+    for (int j = 0; j < k; j++) again = again || layers[j] == L;
+    if (again) break;
+  }
+  return k > 1 ? k : 1;
+}
+
 // One step.  tp_partial == nullptr: the whole step.  Otherwise the heads of this layer object are
 // one GPU's share: the step stops after attention and this GPU's partial first product of the
 // retaining head (fp32 [n_tok x d_R], written to tp_partial), everything on the layer's stream.
 int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t flags, void *attn_out,
                float *tp_partial, bool tp_peers = false) {
-  if (!L || !hidden_in || !attn_out) return LOCRET_ERR_INVALID;
-  if (!on_layer_device(L)) return LOCRET_ERR_INVALID;
-  if (L->tp_pending) return LOCRET_ERR_INVALID;  // a begun step is finished first
-  if (n_tok < 1 || n_tok > L->chunk) return LOCRET_ERR_INVALID;
-  if (flags & ~(LOCRET_NO_EVICT | LOCRET_LAST_CHUNK)) return LOCRET_ERR_INVALID;
-  if (!aligned16(hidden_in) || !aligned16(attn_out)) return LOCRET_ERR_INVALID;
-  const int n = L->len + n_tok;
-  if (n > L->cap) return LOCRET_ERR_CAPACITY;
+  if (const int rc = check_step(L, hidden_in, n_tok, flags, attn_out); rc != LOCRET_OK) return rc;
   const PerHead *const len_m = L->per_head ? &L->len_m : nullptr;
   ScratchPool *P = L->pool;
   const bool tp = tp_partial != nullptr || tp_peers;
   if (L->per_head && tp) return LOCRET_ERR_INVALID;  // (a budget per head and divided heads are not combined)
-  // one token: bandwidth-bound kernels of decode.cu (with a budget per head a one-token step takes the
-  // chunk's general kernels, which know the heads' own lengths)
-  const bool decode = n_tok == 1 && L->use_tc && !tp && !L->per_head;
-  // (a one-token step is a chain of three short kernels on the layer's own stream, overlapped by
-  // programmatic dependent launch: an event between them would serialise them again)
-  const bool side = L->use_side && !L->serialize && !decode;
-  const bool pdl = decode && L->use_pdl && !L->timing;
+  // (with a budget per head a one-token step takes the chunk's general kernels, which know the heads' own lengths)
+  if (n_tok == 1 && !tp && takes_token_step(L)) return token_step(&L, 1, hidden_in, flags, attn_out, 0);
+  const bool side = L->use_side && !L->serialize;
   cudaStream_t S = side ? P->side : L->st;  // stream of the off-critical-path kernels
   const int sb = P->flip;                    // staging buffer of this call
   P->flip ^= 1;
@@ -604,13 +725,13 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   ra.len_m = L->len_m;
   // with a tensor-core projection whose width is a whole number of tiles the epilogue of the GEMM does the RoPE pass
   // (few tokens: the projection that divides K over a cluster, and the RoPE pass)
-  const bool skinny = !decode && L->use_tc && skinny_use(n_tok, L->d_in, L->D, L->D, L->D);
-  const bool fused_rope = !decode && !skinny && !L->per_head && L->fuse_rope && L->use_tc && n_tok >= 32 &&
+  const bool skinny = L->use_tc && skinny_use(n_tok, L->d_in, L->D, L->D, L->D);
+  const bool fused_rope = !skinny && !L->per_head && L->fuse_rope && L->use_tc && n_tok >= 32 &&
                           qkv_rope_tc_supported(n_tok, L->d_in, L->D, L->D, L->D, L->d);
-  const bool deq = L->int4 && L->len > 0 && !decode;
+  const bool deq = L->int4 && L->len > 0;
   if (deq) {
     // the expansion writes slots [0, len) of the scratch the chunk's units are appended to
-    // (a one-token step reads the codes inside its attention kernel instead).  Only attention
+    //.  Only attention
     // reads it, so it runs on the second stream beside the projection; the scratch is free once
     // the attention kernel that read it last has finished.
     if (side && P->exp_busy) { CK(cudaStreamWaitEvent(S, P->ev_exp_free, 0)); P->exp_busy = false; }
@@ -623,9 +744,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   }
   {  // (a) projections
     Timed t(L, LOCRET_K_QKV);
-    if (decode)  // projection, positions, RoPE and append of the one token in one kernel
-      CK(launch_gemv_rope((const bf16 *)hidden_in, L->wqkv_t, L->D, staging, ra, L->st, pdl));
-    else if (skinny)
+    if (skinny)
       CK(launch_skinny_gemm((const bf16 *)hidden_in, L->D, L->wqkv_t, L->D, staging, L->d_in, n_tok, L->d_in, L->D,
                             nullptr, 0, L->d_status + 1, L->st));
     else if (fused_rope)
@@ -638,7 +757,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
       CK(launch_gemm_bf16((const bf16 *)hidden_in, L->D, L->wqkv_t, L->D, staging, L->d_in, n_tok,
                           L->d_in, L->D, L->st));
   }
-  if (!fused_rope && !decode) {
+  if (!fused_rope) {
     Timed t(L, LOCRET_K_ROPE);
     CK(launch_rope_append(ra, L->st));
   }
@@ -651,7 +770,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   // the codes are read by the compaction of this step and by later steps, never by this step's
   // attention (the chunk attends to its own keys and values in bf16): second stream
   // (a one-token step quantises its token inside the attention kernel)
-  if (L->int4 && !side && !decode) { const int rc = quantize_chunk(L->st); if (rc != LOCRET_OK) return rc; }
+  if (L->int4 && !side) { const int rc = quantize_chunk(L->st); if (rc != LOCRET_OK) return rc; }
   if (side) CK(cudaEventRecord(L->ev_ready, L->st));
   if (side && deq) CK(cudaStreamWaitEvent(L->st, P->ev_exp_ready, 0));
   {  // (b) Eq. 1
@@ -671,18 +790,12 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
                                   (uint64_t)L->h * L->d * 2, 64, 128);
       L->map_q_base = tc_ok ? P->q_rot : nullptr;
     }
-    if (decode)
-      CK(launch_attention_decode(P->q_rot, k_att, v_att, (bf16 *)attn_out, P->dec_o, P->dec_ml, P->dec_cnt + 1,
-                                 L->h, L->h_kv, L->d, L->cap, n, decode_attn_splits(L->h_kv, n, L->int4),
-                                 L->int4 ? &L->q4 : nullptr, L->cs, L->rank[L->rcur], L->ranked_len,
-                                 L->int4 ? staging + (size_t)L->h * L->d : nullptr,
-                                 L->int4 ? staging + (size_t)(L->h + L->h_kv) * L->d : nullptr, L->st, pdl));
     // The CTA-pair kernel is opt-in (LOCRET_ATTN_PAIR=1) and never used in a divided-heads step.  In a test
     // process in which it had run, the projection GEMM of a later divided-heads step (eight shards of the
     // Llama shape on one GPU) reported a device-side time-out in about one full test run in three, also when
     // that step itself used the one-CTA kernel; no run without the pair kernel ever did.  The cause has not
     // been found, so the default is the kernel every earlier run validated.
-    else if (tc_ok && L->attn_pair && !tp && attention_tc2_supported(n_tok, L->h, L->h_kv, L->d))
+    if (tc_ok && L->attn_pair && !tp && attention_tc2_supported(n_tok, L->h, L->h_kv, L->d))
       CK(launch_attention_tc2(&L->map_q, &L->map_k64, &L->map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                               L->d, L->len, L->d_status, L->st, len_m));
     else if (tc_ok)
@@ -744,10 +857,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   {  // (c) retaining head: launched after the attention kernel, so its CTAs fill that kernel's tail
     Timed t(L, LOCRET_K_RH, S);
     const bf16 *z = L->cfg.rh_input == 1 ? z_post : staging;
-    if (decode)
-      CK(launch_rh_gemv(z, L->w1_t, L->w2f, P->partial, L->d_R, L->d_in, L->h_kv, L->cfg.act, P->dec_cnt,
-                        L->s + L->len, L->cap, S, pdl));
-    else if (L->use_tc && skinny_use(n_tok, L->d_R, L->d_in, L->d_in, L->d_in))
+    if (L->use_tc && skinny_use(n_tok, L->d_R, L->d_in, L->d_in, L->d_in))
       CK(launch_skinny_rh(z, L->d_in, L->w1_t, L->w2f, P->partial, n_tok, L->d_R, L->d_in, L->h_kv, L->cfg.act, &n_tiles,
                           L->d_status + 3, S));
     else if (L->use_tc && n_tok >= 32 && gemm_tc_supported(n_tok, L->d_R, L->d_in, L->d_in, L->d_in))
@@ -757,7 +867,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
       CK(launch_rh_gemm(z, L->d_in, L->w1_t, L->w2f, P->partial, n_tok, L->d_R, L->d_in, L->h_kv,
                         L->cfg.act, &n_tiles, S));
   }
-  if (!decode) {  // (the one-token kernel sums its own partial scores)
+  {
     Timed t(L, LOCRET_K_RH_REDUCE, S);
     CK(launch_rh_reduce(P->partial, n_tiles, n_tok, L->h_kv, L->s, L->cap, L->len, S, len_m));
   }
@@ -832,11 +942,14 @@ int locret_decode_step(locret_layer *L, const void *hidden_in, void *attn_out) {
 int locret_decode_step_stack(locret_layer *const *layers, int32_t n_layers, const void *hidden_in, void *attn_out,
                              int64_t out_stride) {
   if (!layers || n_layers < 1 || !attn_out || out_stride < 0 || (out_stride % 8) != 0) return LOCRET_ERR_INVALID;
-  for (int i = 0; i < n_layers; i++) {
+  for (int i = 0; i < n_layers;) {
     if (!layers[i]) return LOCRET_ERR_INVALID;
     bf16 *out = static_cast<bf16 *>(attn_out) + (size_t)i * out_stride;
-    const int rc = locret_prefill_chunk(layers[i], hidden_in, 1, LOCRET_NO_EVICT, out);
+    const int k = stack_batch(layers + i, n_layers - i, hidden_in, out, out_stride);
+    const int rc = k > 1 ? token_step(layers + i, k, hidden_in, LOCRET_NO_EVICT, out, out_stride)
+                         : locret_prefill_chunk(layers[i], hidden_in, 1, LOCRET_NO_EVICT, out);
     if (rc != LOCRET_OK) return rc;
+    i += k;
   }
   return LOCRET_OK;
 }

@@ -1,0 +1,64 @@
+"""One call for a stack of layers puts the layers of a batch through one launch per kernel: the same bits as one call
+per layer, for more layers than a batch holds, for caches of different lengths and ranks, for 4-bit caches, for
+outputs that share memory and for a layer that occurs twice."""
+
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _hidden(n, D, seed):
+    g = np.random.default_rng(8100 + seed)
+    return W.to_bf16_grid(g.standard_normal((n, D)).astype(np.float32))
+
+
+def _run(sh, budgets, order, use_stack, stride_rows=True, steps=3):
+    from paper_2410_01805_b200 import LayerStack, LocretLayer
+    from parity_util import bf16_dev
+    layers = [LocretLayer(sh, *(bf16_dev(a) for a in W.layer_weights(sh, i, seed=W.BASE_SEED + 9)), b, 200, 16, reserve=16)
+              for i, b in enumerate(budgets)]
+    width = sh.n_q_heads * sh.head_dim
+    out = torch.zeros((200, width), dtype=torch.bfloat16, device="cuda")
+    for c in range(2):
+        x = bf16_dev(_hidden(200, sh.d_model, c))
+        for L in layers:
+            L.prefill_chunk(x, out, 0)     # the smaller budgets evict: their slots are out of temporal order
+    picked = [layers[i] for i in order]
+    outs = torch.zeros((steps, len(picked) if stride_rows else 1, width), dtype=torch.bfloat16, device="cuda")
+    stack = LayerStack(picked)
+    for t in range(steps):
+        x = bf16_dev(_hidden(1, sh.d_model, 50 + t))
+        if use_stack:
+            stack.decode_step(x, outs[t], out_stride=width if stride_rows else 0)
+        else:
+            for i, L in enumerate(picked):
+                L.decode_step(x, outs[t, i if stride_rows else 0])
+    assert all(L.sync_status() == 0 for L in layers)
+    states = [L.export_state() for L in layers]
+    got = outs.clone()
+    for L in layers:
+        L.destroy()
+    return got, states
+
+
+@pytest.mark.parametrize("d,h,hk,kw,budgets,order,stride_rows", [
+    (128, 8, 2, {}, [300] * 10, range(10), True),                       # a batch of eight and one of two
+    (64, 4, 2, {}, [300, 390, 150, 400], range(4), True),               # different lengths, ranks and split counts
+    (96, 3, 3, dict(kv_dtype=1), [300, 350, 300], range(3), True),      # 4-bit caches
+    (128, 8, 2, dict(kv_dtype=1), [300, 350, 300], range(3), True),
+    (64, 64, 2, dict(rh_input=1), [300, 300], range(2), True),          # two groups of 16 heads; post-RoPE scores
+    (64, 4, 2, {}, [300, 300, 300], range(3), False),                   # outputs share memory: the last layer's stay
+    (64, 4, 2, {}, [300, 300], [0, 1, 0], True),                        # a layer that occurs twice
+])
+def test_stack_call_equals_calls_per_layer(d, h, hk, kw, budgets, order, stride_rows):
+    sh = W.LayerShape(d_model=256, n_q_heads=h, n_kv_heads=hk, head_dim=d, d_retain=128, rope_theta=500000.0, **kw)
+    a, sa = _run(sh, budgets, list(order), False, stride_rows)
+    b, sb = _run(sh, budgets, list(order), True, stride_rows)
+    assert torch.equal(a, b)
+    for x, y in zip(sa, sb):
+        for key in x:
+            assert np.array_equal(x[key], y[key]), key
