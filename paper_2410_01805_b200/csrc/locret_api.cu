@@ -118,7 +118,8 @@ struct locret_layer {
   bool fuse_rope;  // RoPE + append in the projection's epilogue (LOCRET_UNFUSED_ROPE=1 disables)
   bool use_side;  // off-critical-path kernels go to the pool's second stream (LOCRET_SERIAL=1 disables)
   bool use_pdl;   // one-token steps overlap their kernels by programmatic dependent launch (LOCRET_NO_PDL=1 disables)
-  bool side_pending;
+  bool side_pending;  // work of this layer on the second stream that nothing has waited for yet;
+  bool side_evicts;   //   its last part rewrites the cache (selection and compaction)
   float **d_peers;  // divided heads, fused exchange: device array of the GPUs' sum buffers
   int n_peers;
   float *tp_scratch;  // this GPU's product for shapes the tensor-core GEMM does not take
@@ -336,7 +337,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
     L->attn_pair = ap && ap[0] == '1';
     const char *np = getenv("LOCRET_NO_PDL");
     L->use_pdl = !(np && np[0] == '1');
-    L->side_pending = false;
+    L->side_pending = L->side_evicts = false;
     L->ev_ready = L->ev_attn = L->ev_side = L->ev_tp = nullptr;
   }
 
@@ -568,6 +569,7 @@ int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaS
   if (side) {
     CK(cudaEventRecord(L->ev_side, S));
     L->side_pending = true;
+    L->side_evicts = evicts;
   }
   L->seen += n_tok;
   return LOCRET_OK;
@@ -705,11 +707,15 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   if (side) P->side_dirty = true;
   if (L->use_side) {
     // the staging buffer is free once the retaining head that last read it has run, and this
-    // layer's cache once its previous selection / compaction has finished
+    // layer's cache once its previous selection / compaction has finished.  A step that did not evict left only
+    // scores (and 4-bit codes) pending, which this step touches on the second stream alone: its projection need not
+    // wait for that retaining head (1024 tokens of the Phi-3 shape: 155 us beside attention).
     if (P->stage_busy[sb]) CK(cudaStreamWaitEvent(L->st, P->ev_stage_free[sb], 0));
     P->stage_busy[sb] = false;
-    if (L->side_pending) CK(cudaStreamWaitEvent(L->st, L->ev_side, 0));
-    L->side_pending = false;
+    if (L->side_pending && (L->side_evicts || !side || tp)) {
+      CK(cudaStreamWaitEvent(L->st, L->ev_side, 0));
+      L->side_pending = false;
+    }
   }
 
   // a 4-bit cache is expanded into bf16 scratch first: keys rotated at position = slot
