@@ -107,6 +107,7 @@ __device__ __forceinline__ void rope_pairs8(const uint4 &lo, const uint4 &hi, co
 
 // blockDim.x = d / 16 threads per row, blockDim.y rows per block.
 __global__ void compact_kernel(CompactArgs a) {
+  pdl_wait();
   const int row = blockIdx.x * blockDim.y + threadIdx.y;
   if (row >= a.h_kv * a.src_stride) return;
   const int m = row / a.src_stride, i = row - m * a.src_stride;
@@ -456,6 +457,60 @@ topk_kernel(TopkArgs a, int cache_in_smem) {
   }
 }
 
+// One unit more than the budget, the eviction of a one-token step: the unit that goes is the competing one with
+// the lowest (score, rank), so one pass over the candidates and a block-wide minimum replace the radix select (11 us of a
+// one-token step of the small shape, 1025 candidates, two heads; 4 us this way).  Same results as topk_kernel.
+__global__ void __launch_bounds__(TK_THREADS)
+topk_one_kernel(TopkArgs a) {
+  __shared__ unsigned long long s_best[32];
+  __shared__ int s_slot;
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.x, tid = threadIdx.x, n = a.n, budget = a.budget;
+  const float *sc = a.scores + (size_t)m * a.stride;
+  const int32_t *rk = a.rank[a.rcur] + (size_t)m * a.stride;
+  int32_t *src_of = a.src_of + (size_t)m * a.src_stride;
+  int32_t *rank_new = a.rank[a.rcur ^ 1] + (size_t)m * a.stride;
+  auto rank_at = [&](int i) -> int { return i < a.ranked_len ? rk[i] : i; };
+  unsigned long long best = ~0ull;
+  int slot = -1;
+  for (int i = tid; i < n; i += TK_THREADS) {
+    const int r = rank_at(i);
+    const unsigned long long c = ((unsigned long long)score_key(sc[i]) << 32) | (unsigned)r;
+    if (r >= a.n_pre && r < n - a.n_prot && c < best) { best = c; slot = i; }
+  }
+  unsigned long long w = best;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long y = __shfl_xor_sync(0xffffffffu, w, o);
+    w = y < w ? y : w;
+  }
+  if ((tid & 31) == 0) s_best[tid >> 5] = w;
+  __syncthreads();
+  w = s_best[tid & 31];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long y = __shfl_xor_sync(0xffffffffu, w, o);
+    w = y < w ? y : w;
+  }
+  if (slot >= 0 && best == w) s_slot = slot;  // (ranks are distinct: one thread; at least one unit competes)
+  __syncthreads();
+  const int gone = s_slot, gone_rank = (int)(unsigned)w;
+  int rotated = 0;
+  for (int i = tid; i < budget; i += TK_THREADS) {
+    const int src = i == gone ? budget : i;  // the last unit takes the freed slot
+    const int r = rank_at(src), r_new = r - (r > gone_rank);
+    src_of[i] = src;
+    rank_new[i] = r_new;
+    rotated += src != i || r_new != r;
+  }
+  if (a.counters) {
+    rotated = __reduce_add_sync(0xffffffffu, rotated);
+    if ((tid & 31) == 0 && rotated) atomicAdd(&a.counters[1], (unsigned long long)rotated);
+    if (tid == 0 && gone < budget) atomicAdd(&a.counters[0], 1ull);
+  }
+}
+
 // ---------------------------------------------------------------- utilities
 __global__ void transpose_bf16_kernel(const bf16 *__restrict__ src, bf16 *__restrict__ dst, int rows,
                                       int cols) {
@@ -495,11 +550,10 @@ cudaError_t launch_rope_append(const RopeAppendArgs &a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact(const CompactArgs &a, cudaStream_t st) {
+cudaError_t launch_compact(const CompactArgs &a, cudaStream_t st, bool pdl) {
   const int tpr = a.d / 16, rpb = 256 / tpr;  // threads per row, rows per block
   const int rows = a.h_kv * a.src_stride;
-  compact_kernel<<<(rows + rpb - 1) / rpb, dim3(tpr, rpb), 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(compact_kernel, dim3((rows + rpb - 1) / rpb), dim3(tpr, rpb), 0, st, pdl, a);
 }
 
 cudaError_t launch_rerope(const bf16 *k_pre, bf16 *k_rot, const float2 *cs, int h_kv, int d, int cap,
@@ -517,7 +571,9 @@ size_t topk_smem_bytes(int n, bool cached) {
   return (5 * W + (cached ? 2 * (size_t)n : 0)) * 4;
 }
 
-cudaError_t launch_topk(const TopkArgs &a, int h_kv, cudaStream_t st) {
+cudaError_t launch_topk(const TopkArgs &a, int h_kv, cudaStream_t st, bool pdl) {
+  if (!a.per_head && a.n == a.budget + 1 && a.n <= a.stride)
+    return launch_kernel(topk_one_kernel, dim3(h_kv), dim3(TK_THREADS), 0, st, pdl, a);
   const size_t max_dyn = 200 * 1024;
   static PerDeviceFlag attr_set;
   if (cudaError_t e = allow_dynamic_smem(topk_kernel, (int)max_dyn, attr_set); e != cudaSuccess) return e;

@@ -249,7 +249,8 @@ struct TopkArgs {
   int per_head;
   PerHead n_m, budget_m, nprot_m, ranked_m, rcur_m;
 };
-cudaError_t launch_topk(const TopkArgs &a, int h_kv, cudaStream_t st);
+// (pdl, here and for the compaction: the kernel may be scheduled while the one before it drains)
+cudaError_t launch_topk(const TopkArgs &a, int h_kv, cudaStream_t st, bool pdl = false);
 
 struct CompactArgs {
   bf16 *k, *v, *k_rot;      // [h_kv][cap][d]
@@ -263,7 +264,7 @@ struct CompactArgs {
   int per_head;             // (see TopkArgs) evict_m: 1 where head m evicts in this step
   PerHead budget_m, ranked_m, rcur_m, evict_m;
 };
-cudaError_t launch_compact(const CompactArgs &a, cudaStream_t st);
+cudaError_t launch_compact(const CompactArgs &a, cudaStream_t st, bool pdl = false);
 
 // k_rot[m][i] = RoPE(k_pre[m][i], i) for i < len (used after an import).
 cudaError_t launch_rerope(const bf16 *k_pre, bf16 *k_rot, const float2 *cs, int h_kv, int d, int cap,

@@ -500,7 +500,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
 namespace {
 
 // (d) of the step: protect, top-b, gather; then the bookkeeping that closes the step
-int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaStream_t S) {
+int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaStream_t S, bool pdl = false) {
   ScratchPool *P = L->pool;
   const int n = L->len + n_tok;
   const bool may_evict = !(flags & LOCRET_NO_EVICT);
@@ -527,7 +527,7 @@ int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaS
       a.src_of = P->keep; a.src_stride = L->budget; a.counters = L->d_counters;
       a.per_head = L->per_head ? 1 : 0;
       a.n_m = n_m; a.budget_m = L->budget_m; a.nprot_m = nprot_m; a.ranked_m = L->ranked_m; a.rcur_m = L->rcur_m;
-      CK(launch_topk(a, L->h_kv, S));
+      CK(launch_topk(a, L->h_kv, S, pdl));
     }
     // the gather rewrites keys and values that the attention kernel reads
     if (side) CK(cudaStreamWaitEvent(S, L->ev_attn, 0));
@@ -543,7 +543,7 @@ int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaS
       a.h_kv = L->h_kv; a.d = L->d; a.cap = L->cap; a.budget = L->budget; a.ranked_len = L->ranked_len;
       a.per_head = L->per_head ? 1 : 0;
       a.budget_m = L->budget_m; a.ranked_m = L->ranked_m; a.rcur_m = L->rcur_m; a.evict_m = evict_m;
-      CK(launch_compact(a, S));
+      CK(launch_compact(a, S, pdl));
     }
   }
   if (L->per_head) {
@@ -651,7 +651,7 @@ int token_step(locret_layer *const *layers, int count, const void *hidden_in, ui
     CK(launch_rh_gemv(rh, count, L0->d_R, L0->d_in, L0->h_kv, L0->cfg.act, st, pdl));
   }
   for (int i = 0; i < count; i++)
-    if (const int rc = evict_and_close(layers[i], 1, flags, false, st); rc != LOCRET_OK) return rc;
+    if (const int rc = evict_and_close(layers[i], 1, flags, false, st, pdl); rc != LOCRET_OK) return rc;
   return LOCRET_OK;
 }
 
