@@ -798,9 +798,9 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
     }
     // The CTA-pair kernel is opt-in (LOCRET_ATTN_PAIR=1) and never used in a divided-heads step.  In a test
     // process in which it had run, the projection GEMM of a later divided-heads step (eight shards of the
-    // Llama shape on one GPU) reported a device-side time-out in about one full test run in three, also when
-    // that step itself used the one-CTA kernel; no run without the pair kernel ever did.  The cause has not
-    // been found, so the default is the kernel every earlier run validated.
+    // Llama shape on one GPU) reported a device-side time-out in about one full test run in three.  A cause that
+    // fits has since been mended in that GEMM's launch (its two tensor maps could share a slot of their
+    // cache); the default is still the kernel that every run has validated.
     if (tc_ok && L->attn_pair && !tp && attention_tc2_supported(n_tok, L->h, L->h_kv, L->d))
       CK(launch_attention_tc2(&L->map_q, &L->map_k64, &L->map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                               L->d, L->len, L->d_status, L->st, len_m));

@@ -66,19 +66,21 @@ __global__ void rh_loss_kernel(const float *__restrict__ partial, int n_tiles, c
 //   dpre[t][r] = bf16( (sum_m ds[t][m] W2[r][m]) * silu'(pre[t][r]) )
 //   dW2[r][m] += sum over the slab of silu(pre[t][r]) ds[t][m]
 // The columns' W2 and dW2 stay in registers, ds of the slab in shared memory (heads padded to HK with zeros).
-// Bound by the FMAs (4 HK per pre-activation pair), not by the 6 bytes per element.
+// Bound by instruction issue (about 90 per pair of pre-activations with 8 heads) with four warps per scheduler to hide the
+// latencies, not by the 6 bytes per element: 10240 x 1024, 8 heads, 43 us (64 us with a bound to check per token,
+// which kept the eight tokens' chains from overlapping; the bytes would take 10 us).
 constexpr int DP_THREADS = 128, DP_SLAB = 64;
 
 template <int HK>
 __global__ void __launch_bounds__(DP_THREADS)
 rh_dpre_dw2_kernel(const float *__restrict__ pre, const float *__restrict__ ds, const float *__restrict__ w2,
-                   bf16 *__restrict__ dpre, float *__restrict__ dw2, int n, int d_R, int h_kv) {
+                   bf16 *__restrict__ dpre, float *__restrict__ dw2, int d_R, int h_kv) {
   __shared__ float sds[DP_SLAB][HK];
   const int r = (blockIdx.x * DP_THREADS + threadIdx.x) * 2;
-  const int t0 = blockIdx.y * DP_SLAB, nt = min(DP_SLAB, n - t0);
+  const int t0 = blockIdx.y * DP_SLAB;   // (n is a multiple of 64: slabs are full)
   for (int i = threadIdx.x; i < DP_SLAB * HK; i += DP_THREADS) {
     const int t = i / HK, m = i % HK;
-    sds[t][m] = (t < nt && m < h_kv) ? ds[(size_t)(t0 + t) * h_kv + m] : 0.f;
+    sds[t][m] = m < h_kv ? ds[(size_t)(t0 + t) * h_kv + m] : 0.f;
   }
   __syncthreads();
   if (r >= d_R) return;   // (d_R is even)
@@ -90,22 +92,38 @@ rh_dpre_dw2_kernel(const float *__restrict__ pre, const float *__restrict__ ds, 
       w[e][m] = m < h_kv ? w2[(size_t)(r + e) * h_kv + m] : 0.f;
       acc[e][m] = 0.f;
     }
-#pragma unroll 4
-  for (int t = 0; t < nt; t++) {
-    const float2 p = *reinterpret_cast<const float2 *>(pre + (size_t)(t0 + t) * d_R + r);
-    const float s0 = sigmoidf_(p.x), s1 = sigmoidf_(p.y);
-    const float a0 = p.x * s0, a1 = p.y * s1;
-    float d0 = 0.f, d1 = 0.f;
+  // TB tokens' pre-activations are requested while the TB before them are worked on
+  constexpr int TB = HK > 8 ? 4 : 8;
+  const float *src = pre + (size_t)t0 * d_R + r;
+  bf16 *dst = dpre + (size_t)t0 * d_R + r;
+  float2 next[TB];
 #pragma unroll
-    for (int m = 0; m < HK; m++) {
-      const float g = sds[t][m];
-      d0 = fmaf(g, w[0][m], d0);
-      d1 = fmaf(g, w[1][m], d1);
-      acc[0][m] = fmaf(a0, g, acc[0][m]);
-      acc[1][m] = fmaf(a1, g, acc[1][m]);
+  for (int i = 0; i < TB; i++) next[i] = *reinterpret_cast<const float2 *>(src + (size_t)i * d_R);
+#pragma unroll 1
+  for (int tb = 0; tb < DP_SLAB; tb += TB) {
+    float2 cur[TB];
+#pragma unroll
+    for (int i = 0; i < TB; i++) {
+      cur[i] = next[i];
+      next[i] = *reinterpret_cast<const float2 *>(src + (size_t)min(tb + TB + i, DP_SLAB - 1) * d_R);
     }
-    *reinterpret_cast<uint32_t *>(dpre + (size_t)(t0 + t) * d_R + r) =
-        pack_bf16(d0 * (s0 * (1.0f + p.x * (1.0f - s0))), d1 * (s1 * (1.0f + p.y * (1.0f - s1))));
+#pragma unroll
+    for (int i = 0; i < TB; i++) {
+      const float2 p = cur[i];
+      const float s0 = sigmoidf_(p.x), s1 = sigmoidf_(p.y);
+      const float a0 = p.x * s0, a1 = p.y * s1;
+      float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+      for (int m = 0; m < HK; m++) {
+        const float g = sds[tb + i][m];
+        d0 = fmaf(g, w[0][m], d0);
+        d1 = fmaf(g, w[1][m], d1);
+        acc[0][m] = fmaf(a0, g, acc[0][m]);
+        acc[1][m] = fmaf(a1, g, acc[1][m]);
+      }
+      *reinterpret_cast<uint32_t *>(dst + (size_t)(tb + i) * d_R) =
+          pack_bf16(d0 * (s0 * (1.0f + p.x * (1.0f - s0))), d1 * (s1 * (1.0f + p.y * (1.0f - s1))));
+    }
   }
 #pragma unroll
   for (int e = 0; e < 2; e++)
@@ -172,9 +190,9 @@ extern "C" int locret_rh_loss_grad_ws(const void *z, const float *labels, const 
   TCK(launch_rh_pre_tc((const bf16 *)z, d_in, (const bf16 *)w1, d_R, pre, w2f, partial, n, d_R, d_in, h_kv, d_status, st));
   rh_loss_kernel<<<(n * h_kv + 255) / 256, 256, 0, st>>>(partial, rh_pre_num_tiles(d_R), labels, ds, loss, n, h_kv, alpha);
   TCK(cudaGetLastError());
-  const dim3 grid((d_R / 2 + DP_THREADS - 1) / DP_THREADS, (n + DP_SLAB - 1) / DP_SLAB);
-  if (h_kv <= 8) rh_dpre_dw2_kernel<8><<<grid, DP_THREADS, 0, st>>>(pre, ds, w2f, dpre, d_w2, n, d_R, h_kv);
-  else rh_dpre_dw2_kernel<32><<<grid, DP_THREADS, 0, st>>>(pre, ds, w2f, dpre, d_w2, n, d_R, h_kv);
+  const dim3 grid((d_R / 2 + DP_THREADS - 1) / DP_THREADS, n / DP_SLAB);
+  if (h_kv <= 8) rh_dpre_dw2_kernel<8><<<grid, DP_THREADS, 0, st>>>(pre, ds, w2f, dpre, d_w2, d_R, h_kv);
+  else rh_dpre_dw2_kernel<32><<<grid, DP_THREADS, 0, st>>>(pre, ds, w2f, dpre, d_w2, d_R, h_kv);
   TCK(cudaGetLastError());
   // dW1 [d_in x d_R] = z^T dpre
   TCK(launch_gemm_tn_f32((const bf16 *)z, d_in, dpre, d_R, d_w1, d_R, d_in, d_R, n, d_status, st));
