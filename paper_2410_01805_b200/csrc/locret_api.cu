@@ -50,7 +50,7 @@ struct ScratchPool {
     // the token's [Q | K | V] before and (retaining-head input variant) after RoPE, its rotated queries, and for 4-bit
     // caches its rotated key and its value in bf16
     bf16 *staging = nullptr, *z_post = nullptr, *q_rot = nullptr, *tok_kv = nullptr;
-    size_t o_b = 0, ml_b = 0, partial_b = 0, staging_b = 0, zpost_b = 0, q_b = 0, tok_b = 0;
+    unsigned char *mem = nullptr;  // one allocation holds them all
     // kernels whose last block merges the partial results: zeroed words that each launch leaves at zero
     // (word 0: retaining head; words 1..: attention, one per KV head x head group)
     unsigned *cnt = nullptr;
@@ -165,8 +165,7 @@ void release_pool(ScratchPool *p) {
   if (p->ev_exp_ready) cudaEventDestroy(p->ev_exp_ready);
   if (p->ev_side_idle) cudaEventDestroy(p->ev_side_idle);
   cudaFree(p->q_rot); cudaFree(p->partial); cudaFree(p->keep);
-  cudaFree(p->dec.dec_o); cudaFree(p->dec.dec_ml); cudaFree(p->dec.dec_partial); cudaFree(p->dec.cnt);
-  cudaFree(p->dec.staging); cudaFree(p->dec.z_post); cudaFree(p->dec.q_rot); cudaFree(p->dec.tok_kv);
+  cudaFree(p->dec.mem);
   cudaFree(p->k_exp); cudaFree(p->v_exp);
   for (auto &t : p->cs) cudaFree(t.ptr);
   g_pools.erase(std::make_pair(p->device, p->st));
@@ -227,6 +226,43 @@ bool on_layer_device(const locret_layer *L) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
   return dev == L->device;
+}
+
+// Room in the pool for one-token steps of `L` (as one of p->refs layers): sets for one, two, four or DECODE_BATCH layers, each
+// large enough for every layer of the pool.
+bool grow_decode_sets(ScratchPool *p, const locret_layer *L) {
+  ScratchPool::DecodeSets &ds = p->dec;
+  auto most = [](size_t have, size_t want) { return want > have ? (want + 127) & ~(size_t)127 : have; };
+  int n = 1;
+  while (n < p->refs && n < DECODE_BATCH) n *= 2;
+  if (n < ds.n) n = ds.n;
+  const size_t o = most(ds.o, (size_t)L->h * 64 * L->d), ml = most(ds.ml, (size_t)L->h * 64 * 2),
+               pt = most(ds.partial, (size_t)rh_gemv_blocks(L->d_R) * L->h_kv), din = most(ds.d_in, L->d_in),
+               qd = most(ds.hd, (size_t)L->h * L->d), kvd = most(ds.kv, (size_t)L->h_kv * L->d);
+  if (ds.mem && n == ds.n && o == ds.o && ml == ds.ml && pt == ds.partial && din == ds.d_in && qd == ds.hd && kvd == ds.kv)
+    return true;
+  const size_t cnt_b = (size_t)DECODE_BATCH * DEC_CNT_WORDS * sizeof(unsigned) / 256 * 256 + 256;
+  const size_t bytes = cnt_b + n * ((o + ml + pt) * sizeof(float) + (2 * din + qd + 2 * kvd) * sizeof(bf16));
+  unsigned char *mem = nullptr;
+  if (cudaMalloc(&mem, bytes) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (cudaMemsetAsync(mem, 0, cnt_b, L->st) != cudaSuccess || cudaStreamSynchronize(L->st) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(mem);
+    return false;
+  }
+  cudaFree(ds.mem);  // (nothing enqueued before still runs)
+  ds.mem = mem;
+  ds.n = n;
+  ds.o = o; ds.ml = ml; ds.partial = pt; ds.d_in = din; ds.hd = qd; ds.kv = kvd;
+  ds.cnt = reinterpret_cast<unsigned *>(mem);
+  ds.dec_o = reinterpret_cast<float *>(mem + cnt_b);
+  ds.dec_ml = ds.dec_o + n * o;
+  ds.dec_partial = ds.dec_ml + n * ml;
+  ds.staging = reinterpret_cast<bf16 *>(ds.dec_partial + n * pt);
+  ds.z_post = ds.staging + n * din;
+  ds.q_rot = ds.z_post + n * din;
+  ds.tok_kv = ds.q_rot + n * qd;
+  return true;
 }
 
 // Wait for everything this layer has in flight, on both streams.
@@ -388,11 +424,6 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
             cudaEventCreateWithFlags(&p->ev_exp_ready, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&p->ev_side_idle, cudaEventDisableTiming) == cudaSuccess;
       }
-      if (g && !p->dec.cnt) {
-        const size_t bytes = (size_t)DECODE_BATCH * DEC_CNT_WORDS * sizeof(unsigned);
-        g = cudaMalloc(&p->dec.cnt, bytes) == cudaSuccess && cudaMemsetAsync(p->dec.cnt, 0, bytes, L->st) == cudaSuccess;
-        if (!g) cudaGetLastError();
-      }
       if (p->side) cudaStreamSynchronize(p->side);  // buffers may be replaced below
       for (int i = 0; i < 2; i++) {
         g = g && grow(&p->staging[i], &p->staging_b[i], (size_t)chunk * L->d_in * sizeof(bf16), L->st);
@@ -405,26 +436,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
         size_t pb = (size_t)nt * chunk * hk * sizeof(float);
         g = g && grow(&p->partial, &p->partial_b, pb, L->st);
       }
-      {
-        // (the new sizes count only once every buffer has them)
-        ScratchPool::DecodeSets &ds = p->dec;
-        auto most = [](size_t have, size_t want) { return want > have ? (want + 63) & ~(size_t)63 : have; };
-        const size_t n = p->refs < DECODE_BATCH ? p->refs : DECODE_BATCH;
-        const size_t o = most(ds.o, (size_t)h * 64 * d), ml = most(ds.ml, (size_t)h * 64 * 2),
-                     pt = most(ds.partial, (size_t)rh_gemv_blocks(dR) * hk), din = most(ds.d_in, L->d_in),
-                     qd = most(ds.hd, (size_t)h * d), kvd = most(ds.kv, (size_t)hk * d);
-        g = g && grow(&ds.dec_o, &ds.o_b, n * o * sizeof(float), L->st) &&
-            grow(&ds.dec_ml, &ds.ml_b, n * ml * sizeof(float), L->st) &&
-            grow(&ds.dec_partial, &ds.partial_b, n * pt * sizeof(float), L->st) &&
-            grow(&ds.staging, &ds.staging_b, n * din * sizeof(bf16), L->st) &&
-            grow(&ds.z_post, &ds.zpost_b, n * din * sizeof(bf16), L->st) &&
-            grow(&ds.q_rot, &ds.q_b, n * qd * sizeof(bf16), L->st) &&
-            grow(&ds.tok_kv, &ds.tok_b, n * 2 * kvd * sizeof(bf16), L->st);
-        if (g) {
-          if ((int)n > ds.n) ds.n = (int)n;
-          ds.o = o; ds.ml = ml; ds.partial = pt; ds.d_in = din; ds.hd = qd; ds.kv = kvd;
-        }
-      }
+      g = g && grow_decode_sets(p, L);
       g = g && grow(&p->keep, &p->keep_b, (size_t)hk * budget * sizeof(int32_t), L->st);
       if (L->int4) {
         const size_t before_k = p->kexp_b, before_v = p->vexp_b;
