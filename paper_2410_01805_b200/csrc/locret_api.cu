@@ -120,6 +120,7 @@ struct locret_layer {
   bool use_pdl;   // one-token steps overlap their kernels by programmatic dependent launch (LOCRET_NO_PDL=1 disables)
   bool side_pending;  // work of this layer on the second stream that nothing has waited for yet;
   bool side_evicts;   //   its last part rewrites the cache (selection and compaction)
+  bool codes_on_st;   // 4-bit: a step wrote codes or ranks on the layer's own stream since the second stream last waited for it
   float **d_peers;  // divided heads, fused exchange: device array of the GPUs' sum buffers
   int n_peers;
   float *tp_scratch;  // this GPU's product for shapes the tensor-core GEMM does not take
@@ -373,7 +374,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
     L->attn_pair = ap && ap[0] == '1';
     const char *np = getenv("LOCRET_NO_PDL");
     L->use_pdl = !(np && np[0] == '1');
-    L->side_pending = L->side_evicts = false;
+    L->side_pending = L->side_evicts = L->codes_on_st = false;
     L->ev_ready = L->ev_attn = L->ev_side = L->ev_tp = nullptr;
   }
 
@@ -582,6 +583,8 @@ int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaS
     CK(cudaEventRecord(L->ev_side, S));
     L->side_pending = true;
     L->side_evicts = evicts;
+  } else if (L->int4) {
+    L->codes_on_st = true;
   }
   L->seen += n_tok;
   return LOCRET_OK;
@@ -748,10 +751,15 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
                           qkv_rope_tc_supported(n_tok, L->d_in, L->D, L->D, L->D, L->d);
   const bool deq = L->int4 && L->len > 0;
   if (deq) {
-    // the expansion writes slots [0, len) of the scratch the chunk's units are appended to
-    //.  Only attention
-    // reads it, so it runs on the second stream beside the projection; the scratch is free once
-    // the attention kernel that read it last has finished.
+    // The expansion writes slots [0, len) of the scratch, the chunk's own units are appended behind them.  Only attention
+    // reads it, so it runs on the second stream beside the projection, once the attention kernel that read the scratch
+    // last has finished.  One-token steps do not touch the scratch, but they quantise (and evict) on the layer's own
+    // stream: the expansion waits for those codes and ranks.
+    if (side && L->codes_on_st) {
+      CK(cudaEventRecord(L->ev_ready, L->st));
+      CK(cudaStreamWaitEvent(S, L->ev_ready, 0));
+      L->codes_on_st = false;
+    }
     if (side && P->exp_busy) { CK(cudaStreamWaitEvent(S, P->ev_exp_free, 0)); P->exp_busy = false; }
     {
       Timed t(L, LOCRET_K_DEQUANT, S);
@@ -823,7 +831,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
       CK(launch_attention_mma(P->q_rot, k_att, v_att, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                               L->d, L->cap, L->len, L->st, len_m));
   }
-  if (side && L->int4) {  // the attention kernel just launched is the scratch's last reader (a one-token step reads its own token there)
+  if (side && L->int4) {  // the attention kernel just launched is the scratch's last reader
     CK(cudaEventRecord(P->ev_exp_free, L->st));
     P->exp_busy = true;
   }
