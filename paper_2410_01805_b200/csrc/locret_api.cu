@@ -831,7 +831,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
       CK(launch_attention_mma(P->q_rot, k_att, v_att, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                               L->d, L->cap, L->len, L->st, len_m));
   }
-  if (side && L->int4) {  // the attention kernel just launched is the scratch's last reader
+  if (P->side && L->int4) {  // the attention kernel just launched is the scratch's last reader, whatever stream the next one fills it on
     CK(cudaEventRecord(P->ev_exp_free, L->st));
     P->exp_busy = true;
   }

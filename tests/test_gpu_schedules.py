@@ -74,3 +74,25 @@ def test_four_bit_chunk_after_one_token_steps(how, n_last):
         return out, layers
 
     _both_ways(run)
+
+
+def test_four_bit_chunk_after_a_step_on_one_stream():
+    """A step that keeps every kernel on the layer's stream (timing mode 2) reads the expansion scratch there; the next
+    step, of another layer, fills the scratch on the second stream."""
+    from paper_2410_01805_b200 import NO_EVICT
+    from parity_util import bf16_dev
+
+    def run(wait):
+        sh, layers = _layers(2, 400, 1)
+        x = [bf16_dev(_hidden(300, sh.d_model, 70 + i)) for i in range(3)]
+        out = torch.zeros((2, 300, sh.n_q_heads * sh.head_dim), dtype=torch.bfloat16, device="cuda")
+        for L in layers:
+            L.prefill_chunk(x[0], out[0], NO_EVICT)
+        wait()
+        layers[0].set_timing(2)
+        layers[0].prefill_chunk(x[1], out[0], NO_EVICT)
+        wait()
+        layers[1].prefill_chunk(x[2][:40], out[1, :40], NO_EVICT)
+        return out, layers
+
+    _both_ways(run)
