@@ -45,7 +45,7 @@ constexpr int AT_SMEM = 1024 + 6 * TILE_BYTES + 256 + 2048;  // Q0,Q1,K0,K1,V0,V
 // trigger a rescale (a TMEM round trip on the critical path) at almost every tile that holds one
 // of the workload's 20x-norm outlier keys.
 constexpr float RESCALE_LOG2 = 100.0f;
-constexpr float NO_KEY = -1e30f;  // SPLIT: maximum of a row that has not seen a key yet
+constexpr float LOWEST = -3.402823466e38f;  // SPLIT: maximum of a row that has not seen a key yet (finite: see its use)
 constexpr int PF = 6;       // key tiles prefetched into L2 ahead of the shared-memory pipeline
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -180,8 +180,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   const int n = len + p.n_tok;
   int NK = (len + row0[1] + TILE + TILE - 1) / TILE;
   NK = min(NK, (n + TILE - 1) / TILE);
-  const int tile_lo = SPLIT ? (int)((long long)rank * NK / n_split) : 0;  // (a share may be empty)
-  if (SPLIT) NK = (int)((long long)(rank + 1) * NK / n_split) - tile_lo;
+  const int NK_all = NK;
+  auto share_lo = [&](int k) { return (int)((long long)k * NK_all / n_split); };  // first key tile of share k (a share may be empty)
+  const int tile_lo = SPLIT ? share_lo(rank) : 0;
+  if (SPLIT) NK = share_lo(rank + 1) - tile_lo;
   // The softmax is order independent, so every CTA walks the key tiles that need no mask in its
   // own rotated order: CTAs of one KV head start together, and in a common order they would all
   // ask the L2 for the same K and V lines at the same moment (measured: 1.4x slower).
@@ -378,7 +380,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         xch[(t * 2 + hf) * TILE + r] = tmax;
         pair_sync();
         tmax = fmaxf(tmax, xch[(t * 2 + (hf ^ 1)) * TILE + r]) * c;
-        if (SPLIT) tmax = fmaxf(tmax, NO_KEY);  // a share's first tile may lie wholly behind the causal boundary
+        // a share's first tile may lie wholly behind the causal boundary: -inf less a finite maximum is -inf, not NaN
+        if (SPLIT) tmax = fmaxf(tmax, LOWEST);
 
         if (j == 0) {
           m_used[t] = tmax;
@@ -480,12 +483,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         const int row = row0[t] + (tr & (TILE - 1));
         if (row >= p.n_tok) continue;
         // (unrolled over the largest cluster: every remote load is in flight before the first is used)
+        // Whether a share holds a key that this row sees is told by its key range: a maximum does not tell NaN scores, which
+        // count, from no scores.
         float mk[MAX_SPLIT], lk[MAX_SPLIT], ok4[MAX_SPLIT][4];
-        float mx = NO_KEY;
+        auto has_key = [&](int k) {
+          return k < n_split && share_lo(k) < share_lo(k + 1) && share_lo(k) * TILE <= len + row;
+        };
+        float mx = LOWEST;
 #pragma unroll
         for (int k = 0; k < MAX_SPLIT; k++) {
-          mk[k] = NO_KEY;
-          if (k >= n_split) continue;
+          mk[k] = LOWEST;
+          if (!has_key(k)) continue;
           const uint32_t ma = cluster_map(sm_a, k) + tr * 4;
           const uint32_t oa = cluster_map(so_a, k) + (uint32_t)((t * D + c0) * TILE + (tr & (TILE - 1))) * 4;
           mk[k] = ld_cluster_f1(ma);
@@ -498,7 +506,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         float acc[4] = {0.f, 0.f, 0.f, 0.f}, ls = 0.f;
 #pragma unroll
         for (int k = 0; k < MAX_SPLIT; k++) {
-          if (!(mk[k] > NO_KEY)) continue;  // (a share without a key for this row, or none at all)
+          if (!has_key(k)) continue;
           const float w = exp2f(mk[k] - mx);
           ls = fmaf(w, lk[k], ls);
 #pragma unroll
