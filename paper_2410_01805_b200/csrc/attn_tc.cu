@@ -83,9 +83,9 @@ __device__ __forceinline__ float max_nan(float a, float b) {  // NaN if either i
 }
 // 2^x of two values <= 127 on the FMA pipe: x = n + f with n = rint(x), a polynomial for 2^f (least squares on the relative
 // error over [-1/2, 1/2], reweighted towards its maximum: 9.1e-8, with the fp32 Horner scheme 1.7e-7), and 2^n put
-// together from its exponent.  Below -126 the result is 2^-126 and not 0.
+// together from its exponent; at -127 and below the exponent field is 0 and so is the result (a masked key weighs nothing).
 __device__ __forceinline__ void exp2_poly2(float x0, float x1, float &y0, float &y1) {
-  const uint64_t x = pack_f32x2(max_nan(x0, -126.f), max_nan(x1, -126.f));
+  const uint64_t x = pack_f32x2(max_nan(x0, -127.f), max_nan(x1, -127.f));
   const uint64_t t = add_f32x2(x, pack_f32x2(12582912.f, 12582912.f));  // 1.5 * 2^23: the sum's low bits are rint(x)
   const uint64_t n = add_f32x2(t, pack_f32x2(-12582912.f, -12582912.f));
   const uint64_t f = fma_f32x2(n, pack_f32x2(-1.f, -1.f), x);

@@ -88,3 +88,30 @@ def test_scores_far_below_zero(d, n_tok, cached):
         assert (np.abs(out[r] - ref) <= tol).all(), (r, np.abs(out[r] - ref).max())
     assert gpu.sync_status() == 0
     gpu.destroy()
+
+
+@pytest.mark.parametrize("d", [64, 96, 128])
+@pytest.mark.parametrize("n_tok,cached", [(40, 0), (40, 900), (200, 0), (280, 1500)])
+def test_masked_values_weigh_nothing(d, n_tok, cached):
+    """The values of a later token, however large, leave the rows before it as they are, bit for bit."""
+    g = np.random.default_rng(13)
+
+    def weights(w, sh):   # column 0 of the input reaches the values alone
+        w[0] = 0.0
+        w[0, (sh.n_q_heads + sh.n_kv_heads) * d:] = 1.0
+        return w
+
+    sh, gpu = _layer(d, wqkv=weights, theta=10000.0)
+    x = W.to_bf16_grid(g.standard_normal((n_tok, 128)).astype(np.float32))
+    K, V = (W.to_bf16_grid(g.standard_normal((2, max(cached, 1), d)).astype(np.float32)) for _ in range(2))
+    outs = []
+    for big in (0.0, 2.0 ** 126):
+        x[n_tok // 2:, 0] = big
+        if cached:
+            _import(gpu, sh, K, V)
+        else:
+            gpu.reset()
+        outs.append(_step(gpu, sh, x)[:n_tok // 2])
+    assert np.array_equal(outs[0], outs[1])
+    assert gpu.sync_status() == 0
+    gpu.destroy()
