@@ -181,7 +181,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   int NK = (len + row0[1] + TILE + TILE - 1) / TILE;
   NK = min(NK, (n + TILE - 1) / TILE);
   const int NK_all = NK;
-  auto share_lo = [&](int k) { return (int)((long long)k * NK_all / n_split); };  // first key tile of share k (a share may be empty)
+  auto share_lo = [&](int k) { return k * NK_all / n_split; };  // first key tile of share k (a share may be empty)
   const int tile_lo = SPLIT ? share_lo(rank) : 0;
   if (SPLIT) NK = share_lo(rank + 1) - tile_lo;
   // The softmax is order independent, so every CTA walks the key tiles that need no mask in its
@@ -478,22 +478,23 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       constexpr int G = D / 4;
       const int g_lo = rank * G / n_split, g_hi = (rank + 1) * G / n_split;
       const uint32_t so_a = smem_u32(so), sm_a = smem_u32(sm);
+      // Whether a share holds a key that a row sees is told by its first key: a maximum does not tell NaN scores, which
+      // count, from no scores.
+      int first_key[MAX_SPLIT];
+#pragma unroll
+      for (int k = 0; k < MAX_SPLIT; k++)
+        first_key[k] = k < n_split && share_lo(k) < share_lo(k + 1) ? share_lo(k) * TILE : 0x7fffffff;
       for (int i = threadIdx.x; i < (g_hi - g_lo) * 2 * TILE; i += 256) {
         const int tr = i & (2 * TILE - 1), t = tr >> 7, c0 = (g_lo + i / (2 * TILE)) * 4;
         const int row = row0[t] + (tr & (TILE - 1));
         if (row >= p.n_tok) continue;
         // (unrolled over the largest cluster: every remote load is in flight before the first is used)
-        // Whether a share holds a key that this row sees is told by its key range: a maximum does not tell NaN scores, which
-        // count, from no scores.
         float mk[MAX_SPLIT], lk[MAX_SPLIT], ok4[MAX_SPLIT][4];
-        auto has_key = [&](int k) {
-          return k < n_split && share_lo(k) < share_lo(k + 1) && share_lo(k) * TILE <= len + row;
-        };
         float mx = LOWEST;
 #pragma unroll
         for (int k = 0; k < MAX_SPLIT; k++) {
           mk[k] = LOWEST;
-          if (!has_key(k)) continue;
+          if (first_key[k] > len + row) continue;
           const uint32_t ma = cluster_map(sm_a, k) + tr * 4;
           const uint32_t oa = cluster_map(so_a, k) + (uint32_t)((t * D + c0) * TILE + (tr & (TILE - 1))) * 4;
           mk[k] = ld_cluster_f1(ma);
@@ -506,7 +507,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         float acc[4] = {0.f, 0.f, 0.f, 0.f}, ls = 0.f;
 #pragma unroll
         for (int k = 0; k < MAX_SPLIT; k++) {
-          if (!has_key(k)) continue;
+          if (first_key[k] > len + row) continue;
           const float w = exp2f(mk[k] - mx);
           ls = fmaf(w, lk[k], ls);
 #pragma unroll
