@@ -349,6 +349,20 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         const int limit = len + row;  // last visible key
         const uint32_t s_addr = tmem_base + lane_off + t * TILE;
         const uint32_t o_addr = tmem_base + lane_off + 2 * TILE + t * HD;
+        const int key0 = tile_of(j) * TILE;
+        if (t == 0 && key0 + TILE > n) {
+          // Slots behind the cache's end hold what an earlier request left there, perhaps NaN, which a weight of 0 does
+          // not silence: this warp clears its sixteen rows of V of its half of the keys before it hands over P.
+          if (ok) ok = mbar_wait(&v_full[j & 1], (j >> 1) & 1, abort_flag, p.status);
+          unsigned char *v = sV + (j & 1) * TILE_BYTES;
+          const int r_lo = hf * 64 + quarter * 16;
+          for (int i = lane; i < (D + 63) / 64 * 128; i += 32) {   // 16-byte pieces: column box, row, piece of 128 bytes
+            const int vr = r_lo + ((i >> 3) & 15);
+            if (key0 + vr >= n)
+              *reinterpret_cast<uint4 *>(v + (i >> 7) * HALF_BYTES + vr * 128 + (i & 7) * 16) = make_uint4(0, 0, 0, 0);
+          }
+          fence_proxy_async();
+        }
         if (ok) ok = mbar_wait(&s_full[t], j & 1, abort_flag, p.status);
         tc_fence_after();
         uint32_t s[64];
@@ -356,7 +370,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         tmem_ld32(s_addr + hf * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
         tmem_wait_ld();
 
-        const int key0 = tile_of(j) * TILE;
         float tmax;
         if (key0 + TILE - 1 > len + row0[t]) {  // a tile that crosses the causal boundary
           tmax = -INFINITY;

@@ -443,7 +443,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
         const size_t before_k = p->kexp_b, before_v = p->vexp_b;
         g = g && grow(&p->k_exp, &p->kexp_b, kv_b, L->st);
         g = g && grow(&p->v_exp, &p->vexp_b, kv_b, L->st);
-        // rows past the live range are multiplied by zero probabilities: they must stay finite
+        // the CTA-pair attention kernel multiplies rows past the live range by zero probabilities: they must be finite
         if (g && p->kexp_b != before_k) g = cudaMemsetAsync(p->k_exp, 0, p->kexp_b, L->st) == cudaSuccess;
         if (g && p->vexp_b != before_v) g = cudaMemsetAsync(p->v_exp, 0, p->vexp_b, L->st) == cudaSuccess;
       }

@@ -115,3 +115,31 @@ def test_masked_values_weigh_nothing(d, n_tok, cached):
     assert np.array_equal(outs[0], outs[1])
     assert gpu.sync_status() == 0
     gpu.destroy()
+
+
+@pytest.mark.parametrize("d", [64, 96, 128])
+@pytest.mark.parametrize("kind", ["bf16", "int4", "heads"])
+def test_slots_behind_the_end_do_not_reach_an_output(d, kind):
+    """A request with NaN inputs, a reset, then a short request: the bits of a layer that never saw the first."""
+    g = np.random.default_rng(14)
+    kw = dict(kv_dtype=1) if kind == "int4" else {}
+    sh, used = _layer(d, theta=10000.0, **kw)
+    x = W.to_bf16_grid(g.standard_normal((270, 128)).astype(np.float32))
+    poison = np.full((300, 128), np.nan, np.float32)
+    for sizes in ([1, 20, 1], [2], [63], [64, 1], [130], [200, 45], [270]):
+        outs = []
+        for gpu in (used, _layer(d, theta=10000.0, **kw)[1]):
+            if kind == "heads":
+                gpu.reset()
+                gpu.set_head_budgets([1600, 1500])
+            if gpu is used:
+                _step(gpu, sh, poison)
+                gpu.reset()
+            t = 0
+            for n in sizes:
+                outs.append(_step(gpu, sh, x[t:t + n]))
+                t += n
+            assert gpu.sync_status() == 0
+        half = len(sizes)
+        for a, b in zip(outs[:half], outs[half:]):
+            assert np.isfinite(b).all() and np.array_equal(a, b), sizes
