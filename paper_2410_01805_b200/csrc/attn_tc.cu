@@ -613,14 +613,18 @@ cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, co
   static PerDeviceFlag attr_set, attr_set_split;
   if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, false>, AT_SMEM, attr_set); e != cudaSuccess) return e;
   if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, true>, AT_SMEM, attr_set_split); e != cudaSuccess) return e;
-  // The key tiles are divided when that keeps all CTAs resident at once; the share then takes about two tiles' time
-  // more for the combination.  (With more than one wave of clusters it lost: 1428 tokens over 3072 cached keys of the
-  // Llama shape, 192 CTAs, took 168 us in clusters of two and 104 us undivided.)
+  // The key tiles are divided when that keeps all CTAs resident at once.  (With more than one wave of clusters it lost:
+  // 1428 tokens over 3072 cached keys of the Llama shape, 192 CTAs, took 168 us in clusters of two and 104 us undivided.)
+  // The combination then costs the time of D / 48 + D / (16 s) key tiles (s CTAs share D columns; half a tile less where
+  // half of the rows are padding).  This is a fit over every s at 2 to 1000 tokens and 3 to 36 key tiles of three shapes;
+  // its choice is within 2 us of the best one.  A larger cluster has to be a third of a tile better (its SMs are missing
+  // elsewhere).  300 tokens of the Llama shape, undivided / in clusters of two: 8 tiles 31 / 35 us, 12 tiles 37 / 39,
+  // 16 tiles 45 / 43, 36 tiles 82 / 62; 128 tokens, in clusters of four: 6 tiles 25 / 27, 8 tiles 29 / 27.
   const int nk = (len_max + p.n_tok + TILE - 1) / TILE;
-  int best = 1, best_cost = nk;
+  int best = 1, best_cost = 48 * nk;   // in 1/48 of a tile
   for (int s = 2; s <= MAX_SPLIT && s <= nk && grid * s <= sm_count_of_current_device(); s++) {
-    const int cost = (nk + s - 1) / s + 2;
-    if (cost < best_cost && grid <= resident_clusters<D>(s)) { best = s; best_cost = cost; }
+    const int cost = 48 * ((nk + s - 1) / s) + D + 3 * D / s - (p.n_tok <= TILE / 2 ? 24 : 0);
+    if (cost < best_cost - (best > 1 ? 16 : 0) && grid <= resident_clusters<D>(s)) { best = s; best_cost = cost; }
   }
   p.n_split = best;
   if (best == 1) {
