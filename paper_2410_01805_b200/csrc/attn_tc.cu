@@ -22,8 +22,9 @@
 //                    cover the time one spends polling a barrier.
 // TMEM columns: S0/P0 [0,128), S1/P1 [128,256), O0 [256,384), O1 [384,512).
 // Query row t sees keys [0, len + t]: the retained cache unmasked, the chunk causally.
-#include "tc_common.cuh"
+#include <type_traits>
 
+#include "tc_common.cuh"
 
 namespace locret {
 
@@ -115,8 +116,7 @@ struct AttnParams {
   int n_tok, h, h_kv, d, len, pair_heads;
   float scale_log2;
   int *status;
-  int per_head;   // a budget per head: KV head m holds len_m.v[m] retained units
-  PerHead len_m;
+  PerHead len_m;  // PER_HEAD: KV head m holds len_m.v[m] retained units
   int n_split;    // SPLIT: CTAs of a cluster, each with its share of the key tiles
 };
 
@@ -126,7 +126,8 @@ struct AttnParams {
 // rank r combines its share of the columns over all ranks in rank order.  Bound by latency, not by the key tiles:
 // 45 tokens over 4500 cached keys of the Llama shape take 29 us in 16 clusters of eight (five key tiles each);
 // the mma.sync kernel that took fewer than 64 tokens before needs 124 us (32 CTAs, all keys in sequence).
-template <int D, bool SPLIT>
+// PER_HEAD: a budget per KV head.
+template <int D, bool SPLIT, bool PER_HEAD>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
@@ -176,14 +177,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     head[0] = head[1] = unit % p.h;
   }
   const int kvh = head[0] / g;
-  const int len = p.per_head ? p.len_m.v[kvh] : p.len;   // retained units of this KV head
+  const int len = PER_HEAD ? p.len_m.v[kvh] : p.len;   // retained units of this KV head
   const int n = len + p.n_tok;
   int NK = (len + row0[1] + TILE + TILE - 1) / TILE;
   NK = min(NK, (n + TILE - 1) / TILE);
-  const int NK_all = NK;
-  auto share_lo = [&](int k) { return k * NK_all / n_split; };  // first key tile of share k (a share may be empty)
-  const int tile_lo = SPLIT ? share_lo(rank) : 0;
-  if (SPLIT) NK = share_lo(rank + 1) - tile_lo;
+  const int tile_lo = SPLIT ? rank * NK / n_split : 0;  // (a share may be empty)
+  if (SPLIT) NK = (rank + 1) * NK / n_split - tile_lo;
   // The softmax is order independent, so every CTA walks the key tiles that need no mask in its
   // own rotated order: CTAs of one KV head start together, and in a common order they would all
   // ask the L2 for the same K and V lines at the same moment (measured: 1.4x slower).
@@ -350,19 +349,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         const uint32_t s_addr = tmem_base + lane_off + t * TILE;
         const uint32_t o_addr = tmem_base + lane_off + 2 * TILE + t * HD;
         const int key0 = tile_of(j) * TILE;
-        if (t == 0 && key0 + TILE > n) {
-          // Slots behind the cache's end hold what an earlier request left there, perhaps NaN, which a weight of 0 does
-          // not silence: this warp clears its sixteen rows of V of its half of the keys before it hands over P.
-          if (ok) ok = mbar_wait(&v_full[j & 1], (j >> 1) & 1, abort_flag, p.status);
-          unsigned char *v = sV + (j & 1) * TILE_BYTES;
-          const int r_lo = hf * 64 + quarter * 16;
-          for (int i = lane; i < (D + 63) / 64 * 128; i += 32) {   // 16-byte pieces: column box, row, piece of 128 bytes
-            const int vr = r_lo + ((i >> 3) & 15);
-            if (key0 + vr >= n)
-              *reinterpret_cast<uint4 *>(v + (i >> 7) * HALF_BYTES + vr * 128 + (i & 7) * 16) = make_uint4(0, 0, 0, 0);
-          }
-          fence_proxy_async();
-        }
         if (ok) ok = mbar_wait(&s_full[t], j & 1, abort_flag, p.status);
         tc_fence_after();
         uint32_t s[64];
@@ -452,6 +438,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           unpack_f32x2(lb, b0, b1);
           l[t] += (a0 + a1) + (b0 + b1);
         }
+        if (PER_HEAD && t == 0 && key0 + TILE > n) {
+          // Slots behind the cache's end hold what an earlier request left there, perhaps NaN, which a weight of 0 does
+          // not silence.  map_v ends at the longest head's length, so a shorter head's rows are cleared here: this warp's
+          // sixteen of its half of the keys, before it hands over P.  (Compiled into the
+          // other calls as well it cost their prefill 1 %.)
+          if (ok) ok = mbar_wait(&v_full[j & 1], (j >> 1) & 1, abort_flag, p.status);
+          unsigned char *v = sV + (j & 1) * TILE_BYTES;
+          const int r_lo = hf * 64 + quarter * 16;
+          for (int i = lane; i < (D + 63) / 64 * 128; i += 32) {   // 16-byte pieces: column box, row, piece of 128 bytes
+            const int vr = r_lo + ((i >> 3) & 15);
+            if (key0 + vr >= n)
+              *reinterpret_cast<uint4 *>(v + (i >> 7) * HALF_BYTES + vr * 128 + (i & 7) * 16) = make_uint4(0, 0, 0, 0);
+          }
+          fence_proxy_async();
+        }
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -491,12 +492,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       constexpr int G = D / 4;
       const int g_lo = rank * G / n_split, g_hi = (rank + 1) * G / n_split;
       const uint32_t so_a = smem_u32(so), sm_a = smem_u32(sm);
-      // Whether a share holds a key that a row sees is told by its first key: a maximum does not tell NaN scores, which
-      // count, from no scores.
-      int first_key[MAX_SPLIT];
-#pragma unroll
-      for (int k = 0; k < MAX_SPLIT; k++)
-        first_key[k] = k < n_split && share_lo(k) < share_lo(k + 1) ? share_lo(k) * TILE : 0x7fffffff;
       for (int i = threadIdx.x; i < (g_hi - g_lo) * 2 * TILE; i += 256) {
         const int tr = i & (2 * TILE - 1), t = tr >> 7, c0 = (g_lo + i / (2 * TILE)) * 4;
         const int row = row0[t] + (tr & (TILE - 1));
@@ -507,7 +502,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
 #pragma unroll
         for (int k = 0; k < MAX_SPLIT; k++) {
           mk[k] = LOWEST;
-          if (first_key[k] > len + row) continue;
+          lk[k] = 0.f;
+          if (k >= n_split) continue;
           const uint32_t ma = cluster_map(sm_a, k) + tr * 4;
           const uint32_t oa = cluster_map(so_a, k) + (uint32_t)((t * D + c0) * TILE + (tr & (TILE - 1))) * 4;
           mk[k] = ld_cluster_f1(ma);
@@ -520,7 +516,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         float acc[4] = {0.f, 0.f, 0.f, 0.f}, ls = 0.f;
 #pragma unroll
         for (int k = 0; k < MAX_SPLIT; k++) {
-          if (first_key[k] > len + row) continue;
+          // a share without a key for this row has no weight (its maximum would not do: NaN scores count, and raise none)
+          if (lk[k] == 0.f) continue;
           const float w = exp2f(mk[k] - mx);
           ls = fmaf(w, lk[k], ls);
 #pragma unroll
@@ -600,19 +597,18 @@ int resident_clusters(int size) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, true>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, true, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
     known[dev][size] = n + 1;
   }
   return known[dev][size] - 1;
 }
 
-// map_k / map_v: 3-D maps {d, cap, h_kv} with box {64, 128, 1}; map_q: 2-D {h*d, rows} box {64, 128}.
-template <int D>
+template <int D, bool PER_HEAD>
 cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, const CUtensorMap *map_v, AttnParams &p,
                           int grid, int len_max, cudaStream_t st) {
   static PerDeviceFlag attr_set, attr_set_split;
-  if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, false>, AT_SMEM, attr_set); e != cudaSuccess) return e;
-  if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, true>, AT_SMEM, attr_set_split); e != cudaSuccess) return e;
+  if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, false, PER_HEAD>, AT_SMEM, attr_set); e != cudaSuccess) return e;
+  if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, true, PER_HEAD>, AT_SMEM, attr_set_split); e != cudaSuccess) return e;
   // The key tiles are divided when that keeps all CTAs resident at once.  (With more than one wave of clusters it lost:
   // 1428 tokens over 3072 cached keys of the Llama shape, 192 CTAs, took 168 us in clusters of two and 104 us undivided.)
   // The combination then costs the time of D / 48 + D / (16 s) key tiles (s CTAs share D columns; half a tile less where
@@ -628,7 +624,7 @@ cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, co
   }
   p.n_split = best;
   if (best == 1) {
-    attn_tc_kernel<D, false><<<grid, AT_THREADS, AT_SMEM, st>>>(*map_q, *map_k, *map_v, p);
+    attn_tc_kernel<D, false, PER_HEAD><<<grid, AT_THREADS, AT_SMEM, st>>>(*map_q, *map_k, *map_v, p);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
@@ -641,7 +637,7 @@ cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, co
   attr[0].val.clusterDim.x = best; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, true>, *map_q, *map_k, *map_v, static_cast<const AttnParams>(p));
+  return cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, true, PER_HEAD>, *map_q, *map_k, *map_v, static_cast<const AttnParams>(p));
 }
 
 }  // namespace
@@ -651,7 +647,6 @@ cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map
                                 int len, int *status, cudaStream_t st, const PerHead *len_m) {
   AttnParams p;
   p.out = out; p.n_tok = n_tok; p.h = h; p.h_kv = h_kv; p.d = d; p.len = len;
-  p.per_head = len_m ? 1 : 0;
   p.len_m = len_m ? *len_m : PerHead{};
   p.pair_heads = ((h / h_kv) % 2 == 0) ? 1 : 0;
   p.scale_log2 = 1.4426950408889634f / sqrtf((float)d);
@@ -661,10 +656,15 @@ cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map
   int len_max = len;
   if (len_m)
     for (int m = 0; m < h_kv; m++) len_max = len_m->v[m] > len_max ? len_m->v[m] : len_max;
+  auto launch = [&](auto dim) -> cudaError_t {
+    constexpr int D = decltype(dim)::value;
+    return len_m ? launch_attn_d<D, true>(map_q, map_k, map_v, p, grid, len_max, st)
+                 : launch_attn_d<D, false>(map_q, map_k, map_v, p, grid, len_max, st);
+  };
   switch (d) {
-    case 64: return launch_attn_d<64>(map_q, map_k, map_v, p, grid, len_max, st);
-    case 96: return launch_attn_d<96>(map_q, map_k, map_v, p, grid, len_max, st);
-    case 128: return launch_attn_d<128>(map_q, map_k, map_v, p, grid, len_max, st);
+    case 64: return launch(std::integral_constant<int, 64>{});
+    case 96: return launch(std::integral_constant<int, 96>{});
+    case 128: return launch(std::integral_constant<int, 128>{});
   }
   return cudaErrorInvalidValue;
 }

@@ -129,7 +129,7 @@ struct locret_layer {
   uint32_t tp_flags;
   cudaEvent_t ev_ready, ev_attn, ev_side, ev_tp;  // ev_tp: the divided-heads exchange (both directions)
   bool tc_attn;  // tensor maps for the tcgen05 attention kernel are valid
-  CUtensorMap map_k, map_v, map_q;
+  CUtensorMap map_k, map_q;
   CUtensorMap map_k64;   // keys in boxes of 64 (the CTA-pair attention kernel loads half a key tile per CTA)
   bool attn_pair;
   const void *map_q_base;
@@ -443,7 +443,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
         const size_t before_k = p->kexp_b, before_v = p->vexp_b;
         g = g && grow(&p->k_exp, &p->kexp_b, kv_b, L->st);
         g = g && grow(&p->v_exp, &p->vexp_b, kv_b, L->st);
-        // the CTA-pair attention kernel multiplies rows past the live range by zero probabilities: they must be finite
+        // keys past the live range are read, and masked: no uninitialised memory
         if (g && p->kexp_b != before_k) g = cudaMemsetAsync(p->k_exp, 0, p->kexp_b, L->st) == cudaSuccess;
         if (g && p->vexp_b != before_v) g = cudaMemsetAsync(p->v_exp, 0, p->vexp_b, L->st) == cudaSuccess;
       }
@@ -470,8 +470,6 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
   else
     L->tc_attn = L->use_tc &&
                  tmap_encode_3d_bf16(&L->map_k, L->k_rot, d, L->cap, hk, (uint64_t)d * 2,
-                                     (uint64_t)L->cap * d * 2, 64, 128, 1) &&
-                 tmap_encode_3d_bf16(&L->map_v, L->v, d, L->cap, hk, (uint64_t)d * 2,
                                      (uint64_t)L->cap * d * 2, 64, 128, 1) &&
                  tmap_encode_3d_bf16(&L->map_k64, L->k_rot, d, L->cap, hk, (uint64_t)d * 2,
                                      (uint64_t)L->cap * d * 2, 64, 64, 1);
@@ -805,8 +803,6 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
     if (tc_ok && L->int4 && L->map_kv_base != P->k_exp) {
       tc_ok = tmap_encode_3d_bf16(&L->map_k, P->k_exp, L->d, L->cap, L->h_kv, (uint64_t)L->d * 2,
                                   (uint64_t)L->cap * L->d * 2, 64, 128, 1) &&
-              tmap_encode_3d_bf16(&L->map_v, P->v_exp, L->d, L->cap, L->h_kv, (uint64_t)L->d * 2,
-                                  (uint64_t)L->cap * L->d * 2, 64, 128, 1) &&
               tmap_encode_3d_bf16(&L->map_k64, P->k_exp, L->d, L->cap, L->h_kv, (uint64_t)L->d * 2,
                                   (uint64_t)L->cap * L->d * 2, 64, 64, 1);
       L->map_kv_base = tc_ok ? P->k_exp : nullptr;
@@ -816,16 +812,19 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
                                   (uint64_t)L->h * L->d * 2, 64, 128);
       L->map_q_base = tc_ok ? P->q_rot : nullptr;
     }
+    CUtensorMap map_v;   // of this step: it ends where the cache will (with a budget per head, where its longest head's will)
+    tc_ok = tc_ok && tmap_encode_3d_bf16(&map_v, v_att, L->d, L->len + n_tok, L->h_kv, (uint64_t)L->d * 2,
+                                         (uint64_t)L->cap * L->d * 2, 64, 128, 1);
     // The CTA-pair kernel is opt-in (LOCRET_ATTN_PAIR=1) and never used in a divided-heads step.  In a test
     // process in which it had run, the projection GEMM of a later divided-heads step (eight shards of the
     // Llama shape on one GPU) reported a device-side time-out in about one full test run in three.  A cause that
     // fits has since been mended in that GEMM's launch (its two tensor maps could share a slot of their
     // cache); the default is still the kernel that every run has validated.
     if (tc_ok && L->attn_pair && !tp && attention_tc2_supported(n_tok, L->h, L->h_kv, L->d))
-      CK(launch_attention_tc2(&L->map_q, &L->map_k64, &L->map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
+      CK(launch_attention_tc2(&L->map_q, &L->map_k64, &map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                               L->d, L->len, L->d_status, L->st, len_m));
     else if (tc_ok)
-      CK(launch_attention_tc(&L->map_q, &L->map_k, &L->map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
+      CK(launch_attention_tc(&L->map_q, &L->map_k, &map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                              L->d, L->len, L->d_status, L->st, len_m));
     else
       CK(launch_attention_mma(P->q_rot, k_att, v_att, (bf16 *)attn_out, n_tok, L->h, L->h_kv,

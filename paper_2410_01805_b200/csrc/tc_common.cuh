@@ -281,8 +281,9 @@ bool tmap_encode_3d_bf16(CUtensorMap *map, const void *base, uint64_t d0, uint64
 bool cached_map_k64(CUtensorMap *out, const void *base, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
                     uint32_t box_outer);
 
-// Eq. 1 on tcgen05 (attn_tc.cu).  map_k / map_v: 3-D maps {d, cap, h_kv}, box {64, 128, 1};
-// map_q: 2-D map {h*d, rows}, box {64, 128}.
+// Eq. 1 on tcgen05 (attn_tc.cu).  map_k / map_v: 3-D maps {d, slots, h_kv}, box {64, 128, 1}; map_v has as many slots as
+// the longest head holds units (weights behind the end are 0, and what TMA does not load is 0 and not what an
+// earlier request left there, perhaps NaN).  map_q: 2-D map {h*d, rows}, box {64, 128}.
 bool attention_tc_supported(int n_tok, int h, int h_kv, int d);
 cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map_k,
                                 const CUtensorMap *map_v, bf16 *out, int n_tok, int h, int h_kv, int d,
