@@ -34,6 +34,7 @@ struct ScratchPool {
   // off-critical-path kernels (partial scores, index lists) on the layer's own stream waits for it first
   cudaEvent_t ev_side_idle = nullptr;
   bool side_dirty = false;
+  const locret_layer *last_chunk = nullptr;  // the layer of the last step of more than one token (compared, never read through)
   bool exp_busy = false;  // ev_exp_free recorded and not yet waited for
   bool stage_busy[2] = {false, false};  // recorded and not yet waited for
   int flip = 0;
@@ -722,15 +723,19 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
     // the staging buffer is free once the retaining head that last read it has run, and this
     // layer's cache once its previous selection / compaction has finished.  A step that did not evict left only
     // scores (and 4-bit codes) pending, which this step touches on the second stream alone: its projection need not
-    // wait for that retaining head (1024 tokens of the Phi-3 shape: 155 us beside attention).
+    // wait for that retaining head (1024 tokens of the Phi-3 shape: 155 us beside attention).  It is skipped only where
+    // it would stall: after a step of another layer the staging buffer's event has been waited for and this one is
+    // as good as due, and without it the projection reached the SMs before the retaining head that the step after next
+    // waits for (600 tokens of the Phi-3 shape, four layers in turn: 116 us a step, 107 with the wait).
     if (P->stage_busy[sb]) CK(cudaStreamWaitEvent(L->st, P->ev_stage_free[sb], 0));
     P->stage_busy[sb] = false;
-    if (L->side_pending && (L->side_evicts || !side || tp)) {
+    if (L->side_pending && (L->side_evicts || !side || tp || P->last_chunk != L)) {
       CK(cudaStreamWaitEvent(L->st, L->ev_side, 0));
       L->side_pending = false;
     }
   }
 
+  P->last_chunk = L;
   // a 4-bit cache is expanded into bf16 scratch first: keys rotated at position = slot
   bf16 *const k_att = L->int4 ? P->k_exp : L->k_rot;
   bf16 *const v_att = L->int4 ? P->v_exp : L->v;

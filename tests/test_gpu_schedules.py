@@ -96,3 +96,28 @@ def test_four_bit_chunk_after_a_step_on_one_stream():
         return out, layers
 
     _both_ways(run)
+
+
+@pytest.mark.parametrize("kv_dtype", [0, 1])
+@pytest.mark.parametrize("n_layers", [1, 2])
+def test_chunks_that_evict_and_chunks_that_do_not(kv_dtype, n_layers):
+    """A chunk's projection starts beside its layer's last retaining head if that step did not evict, and after its
+    compaction if it did; one-token steps between them run on the layer's own stream."""
+    from paper_2410_01805_b200 import NO_EVICT
+    from parity_util import bf16_dev
+
+    def run(wait):
+        sh, layers = _layers(n_layers, 500, kv_dtype)
+        sizes = [(300, 0), (150, NO_EVICT), (300, 0), (40, NO_EVICT), (1, 0), (300, 0), (300, 0), (1, NO_EVICT), (64, NO_EVICT),
+                 (200, 0), (130, NO_EVICT), (20, 0)]   # (the third evicts the first 250 of 750 units)
+        out = torch.zeros((n_layers, sum(n for n, _ in sizes), sh.n_q_heads * sh.head_dim), dtype=torch.bfloat16, device="cuda")
+        x = bf16_dev(_hidden(out.shape[1], sh.d_model, 80))
+        t = 0
+        for n, flags in sizes:
+            for i, L in enumerate(layers):
+                wait()
+                L.prefill_chunk(x[t:t + n], out[i, t:t + n], flags)
+            t += n
+        return out, layers
+
+    _both_ways(run)
