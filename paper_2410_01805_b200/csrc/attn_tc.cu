@@ -605,7 +605,7 @@ int resident_clusters(int size) {
 
 template <int D, bool PER_HEAD>
 cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, const CUtensorMap *map_v, AttnParams &p,
-                          int grid, int len_max, cudaStream_t st) {
+                          int grid, int len_max, bool may_divide, cudaStream_t st) {
   static PerDeviceFlag attr_set, attr_set_split;
   if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, false, PER_HEAD>, AT_SMEM, attr_set); e != cudaSuccess) return e;
   if (cudaError_t e = allow_dynamic_smem(attn_tc_kernel<D, true, PER_HEAD>, AT_SMEM, attr_set_split); e != cudaSuccess) return e;
@@ -613,14 +613,14 @@ cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, co
   // 1428 tokens over 3072 cached keys of the Llama shape, 192 CTAs, took 168 us in clusters of two and 104 us undivided.)
   // The combination then costs the time of D / 48 + D / (16 s) key tiles (s CTAs share D columns; half a tile less where
   // half of the rows are padding).  This is a fit over every s at 2 to 1000 tokens and 3 to 36 key tiles of three shapes;
-  // its choice is within 2 us of the best one.  A larger cluster has to be a third of a tile better (its SMs are missing
-  // elsewhere).  300 tokens of the Llama shape, undivided / in clusters of two: 8 tiles 31 / 35 us, 12 tiles 37 / 39,
+  // its choice is within 2 us of the best one.  A larger cluster has to be a third of a tile better, and one
+  // that fills half of the GPU a whole tile: its SMs are missing elsewhere.  300 tokens of the Llama shape, undivided / in clusters of two: 8 tiles 31 / 35 us, 12 tiles 37 / 39,
   // 16 tiles 45 / 43, 36 tiles 82 / 62; 128 tokens, in clusters of four: 6 tiles 25 / 27, 8 tiles 29 / 27.
   const int nk = (len_max + p.n_tok + TILE - 1) / TILE;
   int best = 1, best_cost = 48 * nk;   // in 1/48 of a tile
-  for (int s = 2; s <= MAX_SPLIT && s <= nk && grid * s <= sm_count_of_current_device(); s++) {
+  for (int s = 2; may_divide && s <= MAX_SPLIT && s <= nk && grid * s <= sm_count_of_current_device(); s++) {
     const int cost = 48 * ((nk + s - 1) / s) + D + 3 * D / s - (p.n_tok <= TILE / 2 ? 24 : 0);
-    if (cost < best_cost - (best > 1 ? 16 : 0) && grid <= resident_clusters<D>(s)) { best = s; best_cost = cost; }
+    if (cost < best_cost - (best > 1 ? 16 : 2 * grid * s > sm_count_of_current_device() ? 48 : 0) && grid <= resident_clusters<D>(s)) { best = s; best_cost = cost; }
   }
   p.n_split = best;
   if (best == 1) {
@@ -644,7 +644,7 @@ cudaError_t launch_attn_d(const CUtensorMap *map_q, const CUtensorMap *map_k, co
 
 cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map_k,
                                 const CUtensorMap *map_v, bf16 *out, int n_tok, int h, int h_kv, int d,
-                                int len, int *status, cudaStream_t st, const PerHead *len_m) {
+                                int len, int *status, cudaStream_t st, const PerHead *len_m, bool may_divide) {
   AttnParams p;
   p.out = out; p.n_tok = n_tok; p.h = h; p.h_kv = h_kv; p.d = d; p.len = len;
   p.len_m = len_m ? *len_m : PerHead{};
@@ -658,8 +658,8 @@ cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map
     for (int m = 0; m < h_kv; m++) len_max = len_m->v[m] > len_max ? len_m->v[m] : len_max;
   auto launch = [&](auto dim) -> cudaError_t {
     constexpr int D = decltype(dim)::value;
-    return len_m ? launch_attn_d<D, true>(map_q, map_k, map_v, p, grid, len_max, st)
-                 : launch_attn_d<D, false>(map_q, map_k, map_v, p, grid, len_max, st);
+    return len_m ? launch_attn_d<D, true>(map_q, map_k, map_v, p, grid, len_max, may_divide, st)
+                 : launch_attn_d<D, false>(map_q, map_k, map_v, p, grid, len_max, may_divide, st);
   };
   switch (d) {
     case 64: return launch(std::integral_constant<int, 64>{});

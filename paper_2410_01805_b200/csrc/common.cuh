@@ -191,7 +191,11 @@ int rh_tc_num_tiles(int d_R);
 //   gated: act [n_tok x F] = silu(X Wg) * (X Wu), Wt [2F x K] in the interleaved layout of launch_gemm_tc_gated
 //   rh:    partial[tile][n_tok][h_kv], as launch_rh_gemm_tc, in tiles of 128 rows of W1t
 // use: the rule by which a call takes this path and not the GEMM of gemm_tc.cu
+// use_beside: the same for the retaining head of a layer step (d_model: the K of the step's projection; awaited: the next
+// step waits for it); ctas: how many CTAs it takes
 bool skinny_use(int n_tok, int N, int K, int ldx, int ldw);
+int skinny_ctas(int n_tok, int N, int K);
+bool skinny_use_beside(int n_tok, int N, int K, int ldx, int ldw, int d_model, bool awaited);
 bool skinny_supported(int n_tok, int N, int K, int ldx, int ldw);
 cudaError_t launch_skinny_gemm(const bf16 *X, int ldx, const bf16 *Wt, int ldw, bf16 *Y, int ldy, int n_tok, int N, int K,
                                const bf16 *R, int ldr, int *status, cudaStream_t st, bool pdl = false);

@@ -749,7 +749,11 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   ra.len_m = L->len_m;
   // with a tensor-core projection whose width is a whole number of tiles the epilogue of the GEMM does the RoPE pass
   // (few tokens: the projection that divides K over a cluster, and the RoPE pass)
-  const bool skinny = L->use_tc && skinny_use(n_tok, L->d_in, L->D, L->D, L->D);
+  // Beyond one token tile the projection goes with the retaining head: two CTAs of that kind share an SM with each
+  // other, none does with a wide GEMM's (Llama shape, 256 tokens: 61 us with both wide, 65 with one of each; Phi-3 shape,
+  // 200 tokens: 71 with both narrow, 76 with one of each).
+  const bool skinny_rh = L->use_tc && skinny_use_beside(n_tok, L->d_R, L->d_in, L->d_in, L->d_in, L->D, L->int4);
+  const bool skinny = L->use_tc && (n_tok <= 128 || skinny_rh) && skinny_use(n_tok, L->d_in, L->D, L->D, L->D);
   const bool fused_rope = !skinny && !L->per_head && L->fuse_rope && L->use_tc && n_tok >= 32 &&
                           qkv_rope_tc_supported(n_tok, L->d_in, L->D, L->D, L->D, L->d);
   const bool deq = L->int4 && L->len > 0;
@@ -820,6 +824,10 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
     CUtensorMap map_v;   // of this step: it ends where the cache will (with a budget per head, where its longest head's will)
     tc_ok = tc_ok && tmap_encode_3d_bf16(&map_v, v_att, L->d, L->len + n_tok, L->h_kv, (uint64_t)L->d * 2,
                                          (uint64_t)L->cap * L->d * 2, 64, 128, 1);
+    // (A retaining head that takes most of the GPU for long breaks up the clusters of divided attention: Phi-3 shape, 4-bit
+    // cache of 1000 units, 512 tokens: 147 us a step divided, 128 undivided.)
+    const bool may_divide = !skinny_rh || n_tok <= 256 ||
+                            2 * skinny_ctas(n_tok, L->d_R, L->d_in) <= sm_count_of_current_device();
     // The CTA-pair kernel is opt-in (LOCRET_ATTN_PAIR=1) and never used in a divided-heads step.  In a test
     // process in which it had run, the projection GEMM of a later divided-heads step (eight shards of the
     // Llama shape on one GPU) reported a device-side time-out in about one full test run in three.  A cause that
@@ -830,7 +838,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
                               L->d, L->len, L->d_status, L->st, len_m));
     else if (tc_ok)
       CK(launch_attention_tc(&L->map_q, &L->map_k, &map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
-                             L->d, L->len, L->d_status, L->st, len_m));
+                             L->d, L->len, L->d_status, L->st, len_m, may_divide));
     else
       CK(launch_attention_mma(P->q_rot, k_att, v_att, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                               L->d, L->cap, L->len, L->st, len_m));
@@ -887,7 +895,7 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   {  // (c) retaining head: launched after the attention kernel, so its CTAs fill that kernel's tail
     Timed t(L, LOCRET_K_RH, S);
     const bf16 *z = L->cfg.rh_input == 1 ? z_post : staging;
-    if (L->use_tc && skinny_use(n_tok, L->d_R, L->d_in, L->d_in, L->d_in))
+    if (skinny_rh)
       CK(launch_skinny_rh(z, L->d_in, L->w1_t, L->w2f, P->partial, n_tok, L->d_R, L->d_in, L->h_kv, L->cfg.act, &n_tiles,
                           L->d_status + 3, S));
     else if (L->use_tc && n_tok >= 32 && gemm_tc_supported(n_tok, L->d_R, L->d_in, L->d_in, L->d_in))

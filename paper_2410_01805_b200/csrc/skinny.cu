@@ -277,29 +277,36 @@ cudaError_t launch_nt(const bf16 *X, int ldx, const bf16 *Wt, int ldw, const Ski
   return cudaLaunchKernelEx(&cfg, skinny_kernel<NT, EPI>, mw, mx, p);
 }
 
-template <int EPI>
-cudaError_t launch_skinny(const bf16 *X, int ldx, const bf16 *Wt, int ldw, SkinnyParams p, int rows_w, cudaStream_t st,
-                          bool pdl) {
+struct SkinnyPlan { int tiles, nt, n_split; };   // tiles of 128 weight rows, tokens of a token tile, CTAs that divide K
+
+SkinnyPlan skinny_plan(int n_tok, int rows_w, int K) {
   const int tiles = (rows_w + SK_ROWS - 1) / SK_ROWS;
-  int nt = p.n_tok <= 16 ? 16 : (p.n_tok <= 32 ? 32 : (p.n_tok <= 64 ? 64 : 128));
+  int nt = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : 128));
   // The deepest split of K that keeps all CTAs resident at once and gives each at least four K-blocks; and for small
   // matrices narrower token tiles while not even a third of the SMs has a CTA (the small shape's retaining head at 512
   // tokens: 17.5 us in 16 CTAs, 9.5 us in 64; the Llama shape's at 45 tokens, 64 CTAs, only lost by 128: 38 and 47 us).
   const int sms = sm_count_of_current_device();
   auto split_of = [&](int w) {
-    const int c = tiles * ((p.n_tok + w - 1) / w);
+    const int c = tiles * ((n_tok + w - 1) / w);
     int s = 1;
-    while (s < SK_MAX_SPLIT && c * s * 2 <= 2 * sms && p.K / SK_BK / (2 * s) >= 4) s *= 2;
+    while (s < SK_MAX_SPLIT && c * s * 2 <= 2 * sms && K / SK_BK / (2 * s) >= 4) s *= 2;
     return s;
   };
-  while (nt > 32 && tiles * ((p.n_tok + nt - 1) / nt) * split_of(nt) * 3 <= sms) nt /= 2;
-  p.n_split = split_of(nt);
-  switch (nt) {
-    case 16: return launch_nt<16, EPI>(X, ldx, Wt, ldw, p, tiles, rows_w, st, pdl);
-    case 32: return launch_nt<32, EPI>(X, ldx, Wt, ldw, p, tiles, rows_w, st, pdl);
-    case 64: return launch_nt<64, EPI>(X, ldx, Wt, ldw, p, tiles, rows_w, st, pdl);
+  while (nt > 32 && tiles * ((n_tok + nt - 1) / nt) * split_of(nt) * 3 <= sms) nt /= 2;
+  return {tiles, nt, split_of(nt)};
+}
+
+template <int EPI>
+cudaError_t launch_skinny(const bf16 *X, int ldx, const bf16 *Wt, int ldw, SkinnyParams p, int rows_w, cudaStream_t st,
+                          bool pdl) {
+  const SkinnyPlan plan = skinny_plan(p.n_tok, rows_w, p.K);
+  p.n_split = plan.n_split;
+  switch (plan.nt) {
+    case 16: return launch_nt<16, EPI>(X, ldx, Wt, ldw, p, plan.tiles, rows_w, st, pdl);
+    case 32: return launch_nt<32, EPI>(X, ldx, Wt, ldw, p, plan.tiles, rows_w, st, pdl);
+    case 64: return launch_nt<64, EPI>(X, ldx, Wt, ldw, p, plan.tiles, rows_w, st, pdl);
   }
-  return launch_nt<128, EPI>(X, ldx, Wt, ldw, p, tiles, rows_w, st, pdl);
+  return launch_nt<128, EPI>(X, ldx, Wt, ldw, p, plan.tiles, rows_w, st, pdl);
 }
 
 }  // namespace
@@ -318,6 +325,27 @@ bool skinny_use(int n_tok, int N, int K, int ldx, int ldw) {
   if (n_tok <= 256) return true;
   const int wide_tiles = ((n_tok + 127) / 128) * ((N + 255) / 256);
   return n_tok <= 512 && wide_tiles * 4 <= sm_count_of_current_device();
+}
+
+// The retaining head of a layer step runs beside attention and the next projection.  Up to one token tile its 64 CTAs are
+// little to them.  Beyond, what counts is less its own time than the SMs it takes: at 512 tokens (Phi-3 shape, K = 9216) this
+// path takes 52 us on 128 SMs, the wide GEMM 87 us on 16, and four layers in turn (1000 cached units) took 130 us a step
+// with this one and 100 with that; 384 tokens of the Llama shape, empty cache: 80 / 72.  So beyond 128 tokens it is for
+//   matrices so small that it leaves half of the SMs alone (small shape, 512 tokens: 35 / 42 us a step);
+//   up to 256 tokens a K so long that the wide GEMM's chain of K-blocks outlasts what it runs beside, as it does from about
+//   twice the projection's K on (Phi-3 shape, K = 3 d_model, 200 tokens: 71 / 90; Llama shape, 1.5 d_model: 66 / 61);
+//   and where the next step waits for it (awaited: a 4-bit cache's expansion is enqueued behind it) up to 512 tokens
+//   (Phi-3 shape, 512 tokens, 1000 cached: 128 / 130, 300 tokens 104 / 120).
+int skinny_ctas(int n_tok, int N, int K) {
+  const SkinnyPlan plan = skinny_plan(n_tok, N, K);
+  return plan.tiles * ((n_tok + plan.nt - 1) / plan.nt) * plan.n_split;
+}
+
+bool skinny_use_beside(int n_tok, int N, int K, int ldx, int ldw, int d_model, bool awaited) {
+  if (!skinny_supported(n_tok, N, K, ldx, ldw)) return false;
+  if (n_tok <= 128) return true;
+  if (n_tok <= 512 && 2 * skinny_ctas(n_tok, N, K) <= sm_count_of_current_device()) return true;
+  return n_tok <= (awaited ? 512 : 256) && K > 2 * d_model;
 }
 
 cudaError_t launch_skinny_gemm(const bf16 *X, int ldx, const bf16 *Wt, int ldw, bf16 *Y, int ldy, int n_tok, int N, int K,

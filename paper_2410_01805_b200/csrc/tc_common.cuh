@@ -283,12 +283,12 @@ bool cached_map_k64(CUtensorMap *out, const void *base, uint64_t inner, uint64_t
 
 // Eq. 1 on tcgen05 (attn_tc.cu).  map_k / map_v: 3-D maps {d, slots, h_kv}, box {64, 128, 1}; map_v has as many slots as
 // the longest head holds units (weights behind the end are 0, and what TMA does not load is 0 and not what an
-// earlier request left there, perhaps NaN).  map_q: 2-D map {h*d, rows}, box {64, 128}.
+// earlier request left there, perhaps NaN).  map_q: 2-D map {h*d, rows}, box {64, 128}.  may_divide: few query tiles may
+// divide their keys over clusters, which then need their SMs at the same time.
 bool attention_tc_supported(int n_tok, int h, int h_kv, int d);
 cudaError_t launch_attention_tc(const CUtensorMap *map_q, const CUtensorMap *map_k,
                                 const CUtensorMap *map_v, bf16 *out, int n_tok, int h, int h_kv, int d,
-                                int len, int *status, cudaStream_t st, const PerHead *len_m = nullptr);
-
+                                int len, int *status, cudaStream_t st, const PerHead *len_m, bool may_divide);
 
 // The same on CTA pairs (attn_tc2.cu), head_dim 128.  map_k: box {64, 64, 1}; the others as above.
 bool attention_tc2_supported(int n_tok, int h, int h_kv, int d);

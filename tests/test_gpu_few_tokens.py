@@ -41,3 +41,15 @@ def test_block_steps_of_few_tokens(n_tok):
     ora.attn.prefill_chunk(_hidden(200, 512, 2), 0)
     lockstep_block(ora, gpu, _hidden(n_tok, 512, n_tok), 1, f"block, {n_tok} tokens")
     gpu.destroy()
+
+
+@pytest.mark.parametrize("kv_dtype,n_tok", [(0, 129), (0, 256), (0, 257), (1, 300), (1, 512), (1, 513)])
+def test_retaining_head_of_a_long_k(kv_dtype, n_tok):
+    """K of twelve times d_model: beyond 128 tokens this path up to 256, with a 4-bit cache up to 512, and attention
+    undivided beside its 128 CTAs."""
+    from parity_util import lockstep_chunk, make_pair
+    sh = W.LayerShape(d_model=128, n_q_heads=8, n_kv_heads=2, head_dim=128, d_retain=1024, rope_theta=500000.0, kv_dtype=kv_dtype)
+    ora, gpu = make_pair(sh, W.layer_weights(sh, 0, seed=W.BASE_SEED + 72), budget=1400, chunk=700, n_stab=16)
+    ora.prefill_chunk(_hidden(700, 128, 1), 0)
+    lockstep_chunk(ora, gpu, _hidden(n_tok, 128, n_tok), 1, what=f"{kv_dtype} 700+{n_tok}")
+    gpu.destroy()
