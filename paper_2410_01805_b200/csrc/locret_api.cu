@@ -42,9 +42,9 @@ struct ScratchPool {
   bf16 *staging[2] = {nullptr, nullptr}, *q_rot = nullptr, *z_post[2] = {nullptr, nullptr};
   bf16 *k_exp = nullptr, *v_exp = nullptr;  // 4-bit caches: bf16 expansion of the layer in flight
   // One-token steps: up to DECODE_BATCH layers of a stack go through a launch together, each with a set of its own of the
-  // buffers below (as many sets as layers share the pool, at most DECODE_BATCH; a set has room for the largest of them).
+  // buffers below (a set has room for the largest layer of the pool; a megabyte each for the Llama shape).  All sets from the
+  // first layer on: the buffers stay where they are while layers of the same shape join, as a captured step needs it.
   struct DecodeSets {
-    int n = 0;
     size_t o = 0, ml = 0, partial = 0, d_in = 0, hd = 0, kv = 0;  // elements of one set
     // attention: per-split partial results; retaining head: per-block partial scores
     float *dec_o = nullptr, *dec_ml = nullptr, *dec_partial = nullptr;
@@ -230,18 +230,15 @@ bool on_layer_device(const locret_layer *L) {
   return dev == L->device;
 }
 
-// Room in the pool for one-token steps of `L` (as one of p->refs layers): sets for one, two, four or DECODE_BATCH layers, each
-// large enough for every layer of the pool.
+// Room in the pool for one-token steps of `L`: sets large enough for every layer of the pool.
 bool grow_decode_sets(ScratchPool *p, const locret_layer *L) {
   ScratchPool::DecodeSets &ds = p->dec;
   auto most = [](size_t have, size_t want) { return want > have ? (want + 127) & ~(size_t)127 : have; };
-  int n = 1;
-  while (n < p->refs && n < DECODE_BATCH) n *= 2;
-  if (n < ds.n) n = ds.n;
+  constexpr size_t n = DECODE_BATCH;
   const size_t o = most(ds.o, (size_t)L->h * 64 * L->d), ml = most(ds.ml, (size_t)L->h * 64 * 2),
                pt = most(ds.partial, (size_t)rh_gemv_blocks(L->d_R) * L->h_kv), din = most(ds.d_in, L->d_in),
                qd = most(ds.hd, (size_t)L->h * L->d), kvd = most(ds.kv, (size_t)L->h_kv * L->d);
-  if (ds.mem && n == ds.n && o == ds.o && ml == ds.ml && pt == ds.partial && din == ds.d_in && qd == ds.hd && kvd == ds.kv)
+  if (ds.mem && o == ds.o && ml == ds.ml && pt == ds.partial && din == ds.d_in && qd == ds.hd && kvd == ds.kv)
     return true;
   const size_t cnt_b = (size_t)DECODE_BATCH * DEC_CNT_WORDS * sizeof(unsigned) / 256 * 256 + 256;
   const size_t bytes = cnt_b + n * ((o + ml + pt) * sizeof(float) + (2 * din + qd + 2 * kvd) * sizeof(bf16));
@@ -254,7 +251,6 @@ bool grow_decode_sets(ScratchPool *p, const locret_layer *L) {
   }
   cudaFree(ds.mem);  // (nothing enqueued before still runs)
   ds.mem = mem;
-  ds.n = n;
   ds.o = o; ds.ml = ml; ds.partial = pt; ds.d_in = din; ds.hd = qd; ds.kv = kvd;
   ds.cnt = reinterpret_cast<unsigned *>(mem);
   ds.dec_o = reinterpret_cast<float *>(mem + cnt_b);
@@ -677,9 +673,8 @@ int stack_batch(locret_layer *const *layers, int n_layers, const void *hidden_in
   const locret_layer *A = layers[0];
   // (outputs that share memory are written in the layers' order: one launch after the other)
   if (!A || !takes_token_step(A) || A->timing || out_stride < (int64_t)A->h * A->d || !gemv_rope_batched(A->D)) return 1;
-  const int most = n_layers < A->pool->dec.n ? n_layers : A->pool->dec.n;
   int k = 0;
-  for (; k < most; k++) {
+  for (; k < n_layers && k < DECODE_BATCH; k++) {
     const locret_layer *L = layers[k];
     if (check_step(L, hidden_in, 1, LOCRET_NO_EVICT, static_cast<const bf16 *>(attn_out) + k * out_stride) != LOCRET_OK) break;
     if (!takes_token_step(L) || L->timing || L->pool != A->pool || L->use_pdl != A->use_pdl || L->use_side != A->use_side ||

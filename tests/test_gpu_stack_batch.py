@@ -62,3 +62,42 @@ def test_stack_call_equals_calls_per_layer(d, h, hk, kw, budgets, order, stride_
     for x, y in zip(sa, sb):
         for key in x:
             assert np.array_equal(x[key], y[key]), key
+
+
+@pytest.mark.parametrize("kv_dtype", [0, 1])
+def test_a_captured_step_outlives_the_arrival_of_other_layers(kv_dtype):
+    """A one-token step captured in a CUDA graph, more layers of the same shape on its stream, their steps, then the replay:
+    the output of the same step called directly."""
+    from paper_2410_01805_b200 import LayerStack, LocretLayer
+    from parity_util import bf16_dev
+    sh = W.LayerShape(d_model=256, n_q_heads=8, n_kv_heads=2, head_dim=128, d_retain=128, rope_theta=500000.0, kv_dtype=kv_dtype)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        def layer(i):
+            return LocretLayer(sh, *(bf16_dev(a) for a in W.layer_weights(sh, i, seed=W.BASE_SEED + 9)), 300, 200, 16, reserve=16)
+        x, tok = bf16_dev(_hidden(200, 256, 1)), bf16_dev(_hidden(2, 256, 2))
+        out = torch.zeros((200, 1024), dtype=torch.bfloat16, device="cuda")
+        outs = torch.zeros((9, 1024), dtype=torch.bfloat16, device="cuda")
+        first, twin = layer(0), layer(0)
+        for L in (first, twin):
+            L.prefill_chunk(x, out, 0)
+            L.decode_step(tok[0], outs[0])   # (the chunk's work on the second stream has been waited for)
+        twin.decode_step(tok[1], outs[1])
+        st.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st, capture_error_mode="relaxed"):
+            first.decode_step(tok[1], outs[0])
+        others = [layer(i) for i in range(1, 8)]
+        for L in others:
+            L.prefill_chunk(x, out, 0)
+        LayerStack(others).decode_step(tok[0], outs[2:], out_stride=1024)
+        st.synchronize()
+        for _ in range(2):
+            outs[0] = 0
+            graph.replay()
+            st.synchronize()
+            assert torch.equal(outs[0], outs[1])
+        del graph
+        for L in [first, twin] + others:
+            assert L.sync_status() == 0
+            L.destroy()
