@@ -311,7 +311,8 @@ int locret_import_state_heads(locret_layer *layer, const void *K, const void *V,
 int locret_set_timing(locret_layer *layer, int32_t enable);
 int locret_read_timing(locret_layer *layer, float *ms, int64_t *launches);
 
-/* Total number of this library's kernels launched for the layer since create. */
+/* Total number of this library's kernels launched for the layer since create (one that serves several layers of a stack
+ * counts for each of them). */
 int locret_launch_count(const locret_layer *layer, int64_t *count);
 
 /*

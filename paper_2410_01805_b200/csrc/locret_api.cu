@@ -660,6 +660,7 @@ int token_step(locret_layer *const *layers, int count, const void *hidden_in, ui
     Timed t(L0, LOCRET_K_RH);
     CK(launch_rh_gemv(rh, count, L0->d_R, L0->d_in, L0->h_kv, L0->cfg.act, st, pdl));
   }
+  for (int i = 1; i < count; i++) layers[i]->launches += 3;  // (the first layer's are counted where they are timed)
   for (int i = 0; i < count; i++)
     if (const int rc = evict_and_close(layers[i], 1, flags, false, st, pdl); rc != LOCRET_OK) return rc;
   return LOCRET_OK;

@@ -38,7 +38,7 @@ def _run(sh, budgets, order, use_stack, stride_rows=True, steps=3):
             for i, L in enumerate(picked):
                 L.decode_step(x, outs[t, i if stride_rows else 0])
     assert all(L.sync_status() == 0 for L in layers)
-    states = [L.export_state() for L in layers]
+    states = [dict(L.export_state(), launches=L.launch_count) for L in layers]
     got = outs.clone()
     for L in layers:
         L.destroy()
