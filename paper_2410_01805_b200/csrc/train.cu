@@ -132,20 +132,19 @@ rh_dpre_dw2_kernel(const float *__restrict__ pre, const float *__restrict__ ds, 
       if (m < h_kv) atomicAdd(dw2 + (size_t)(r + e) * h_kv + m, acc[e][m]);
 }
 
-__device__ int g_train_status;
-
 size_t pad256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // The call's workspace in one block: offsets of its arrays.
 struct Workspace {
-  size_t pre, dpre, w2f, partial, ds, bytes;
+  size_t pre, dpre, w2f, partial, ds, status, bytes;   // status: the call's own word, so calls may overlap
   Workspace(size_t n, size_t d_R, size_t h_kv) {
     pre = 0;
     dpre = pre + pad256(n * d_R * sizeof(float));
     w2f = dpre + pad256(n * d_R * sizeof(bf16));
     partial = w2f + pad256(d_R * h_kv * sizeof(float));
     ds = partial + pad256(rh_pre_num_tiles((int)d_R) * n * h_kv * sizeof(float));
-    bytes = ds + pad256(n * h_kv * sizeof(float));
+    status = ds + pad256(n * h_kv * sizeof(float));
+    bytes = status + pad256(sizeof(int));
   }
 };
 
@@ -182,8 +181,7 @@ extern "C" int locret_rh_loss_grad_ws(const void *z, const float *labels, const 
   float *pre = (float *)(base + ws.pre), *w2f = (float *)(base + ws.w2f), *partial = (float *)(base + ws.partial),
         *ds = (float *)(base + ws.ds);
   bf16 *dpre = (bf16 *)(base + ws.dpre);
-  int *d_status = nullptr;
-  TCK(cudaGetSymbolAddress((void **)&d_status, g_train_status));
+  int *d_status = (int *)(base + ws.status);
   rh_clear_kernel<<<(d_R * h_kv + 255) / 256, 256, 0, st>>>((const bf16 *)w2, w2f, d_w2, d_R * h_kv, loss, d_status);
   TCK(cudaGetLastError());
   // pre = z W1 (fp32) and the scores

@@ -32,6 +32,23 @@ def test_loss_and_gradients_at_tile_edges(n, d_in, d_R, hk):
     test_loss_and_gradients_match_the_oracle(n, d_in, d_R, hk)
 
 
+def test_the_training_call_has_its_own_status_word():
+    """Calls may overlap: the word that a timed-out wait writes lies in the call's workspace, cleared by the call."""
+    import ctypes
+    import paper_2410_01805_b200 as P
+    n, d_in, d_R, hk = 64, 64, 32, 2
+    need = ctypes.c_int64()
+    assert P.lib.locret_rh_loss_grad_workspace(n, d_R, hk, ctypes.byref(need)) == 0
+    ws = torch.full((need.value,), 0xFF, dtype=torch.uint8, device="cuda")
+    z, w1, w2 = (torch.zeros(s, dtype=torch.bfloat16, device="cuda") for s in ((n, d_in), (d_in, d_R), (d_R, hk)))
+    lab, loss, g1, g2 = (torch.zeros(s, device="cuda") for s in ((hk, n), (1,), (d_in, d_R), (d_R, hk)))
+    args = [t.data_ptr() for t in (z, lab, w1, w2)] + [n, d_in, d_R, hk, 0.1] + [t.data_ptr() for t in (loss, g1, g2, ws)]
+    st = torch.cuda.current_stream().cuda_stream
+    assert P.lib.locret_rh_loss_grad_ws(*args, need.value, st) == 0
+    assert ws[-256:-252].tolist() == [0, 0, 0, 0] and ws[-252:].eq(0xFF).all()
+    assert P.lib.locret_rh_loss_grad_ws(*args, need.value - 1, st) == -3
+
+
 @pytest.mark.parametrize("n,offset", [(1, 0), (4, 0), (1027, 0), (1024, 1), (1030, 2)])
 def test_adamw_vectors_and_remainder(n, offset):
     from paper_2410_01805_b200 import adamw_step
