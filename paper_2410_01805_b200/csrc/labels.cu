@@ -11,6 +11,9 @@
 // One launch for all heads (a launch of the 128 x 256 GEMM per query head before: two K-blocks per tile, the keys
 // re-read for every head).  131072 keys, 1024 answers, 32 query heads of 8 KV heads of 128: 0.70 ms = 1.57 PFLOP/s
 // (1.45 ms before); the measured burst peak allows 0.64 ms.
+#include <atomic>
+#include <thread>
+
 #include "../../include/locret.h"
 #include "tc_common.cuh"
 
@@ -226,7 +229,31 @@ __global__ void labels_init_kernel(float *labels, size_t n, int *status) {
   if (i < n) labels[i] = -INFINITY;
   if (i == 0) *status = 0;
 }
-__device__ int g_cis_status;
+// The word that a timed-out wait writes, one per call in flight: a call (synchronous, so there are no more of them than host
+// threads) takes a free one of its device for its duration.
+constexpr int STATUS_WORDS = 64;
+__device__ int g_cis_status[STATUS_WORDS];
+std::atomic<unsigned long long> g_cis_taken[MAX_DEVICES];
+
+struct StatusWord {
+  int dev = 0, slot = -1;
+  int *word = nullptr;
+  cudaError_t take() {
+    if (cudaError_t e = current_device_index(&dev); e != cudaSuccess) return e;
+    if (cudaError_t e = cudaGetSymbolAddress((void **)&word, g_cis_status); e != cudaSuccess) return e;
+    unsigned long long taken = g_cis_taken[dev].load();
+    for (;;) {
+      if (~taken == 0) {   // 64 calls are in flight: one of them is about to end
+        std::this_thread::yield();
+        taken = g_cis_taken[dev].load();
+        continue;
+      }
+      const int s = __builtin_ctzll(~taken);
+      if (g_cis_taken[dev].compare_exchange_weak(taken, taken | 1ull << s)) { slot = s; word += s; return cudaSuccess; }
+    }
+  }
+  ~StatusWord() { if (slot >= 0) g_cis_taken[dev].fetch_and(~(1ull << slot)); }
+};
 
 }  // namespace
 
@@ -248,10 +275,6 @@ extern "C" int locret_cis_labels(const void *q_ans, const void *k_prompt, int32_
   p.g = h / h_kv;
   p.gb = 1;
   while (p.g % (2 * p.gb) == 0 && p.gb < 16) p.gb *= 2;
-  LCK(cudaGetSymbolAddress((void **)&p.status, g_cis_status));
-  const size_t n = (size_t)h_kv * n_q;
-  labels_init_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(labels, n, p.status);
-  LCK(cudaGetLastError());
   CUtensorMap mk, mq;
   if (!tmap_encode_3d_bf16(&mk, k_prompt, d, h_kv, n_q, (uint64_t)d * 2, (uint64_t)h_kv * d * 2, 64, 1, LB_ROWS) ||
       !tmap_encode_3d_bf16(&mq, q_ans, d, h, n_a, (uint64_t)d * 2, (uint64_t)h * d * 2, 64, p.gb, LB_COLS / p.gb))
@@ -265,6 +288,12 @@ extern "C" int locret_cis_labels(const void *q_ans, const void *k_prompt, int32_
   while (h_kv * p.pairs * p.splits < 16 * sms && p.q_tiles / (2 * p.splits) >= 2) p.splits *= 2;
   const long long units = (long long)h_kv * p.pairs * p.splits;
   if (units > 0x7fffffffll) return LOCRET_ERR_INVALID;
+  StatusWord own;
+  LCK(own.take());
+  p.status = own.word;
+  const size_t n = (size_t)h_kv * n_q;
+  labels_init_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(labels, n, p.status);
+  LCK(cudaGetLastError());
   auto launch = [&](auto kernel, PerDeviceFlag &attr_set) -> cudaError_t {
     if (cudaError_t e = allow_dynamic_smem(kernel, LB_SMEM, attr_set); e != cudaSuccess) return e;
     kernel<<<(unsigned)(units < sms ? units : sms), LB_THREADS, LB_SMEM, st>>>(mk, mq, p);

@@ -64,3 +64,40 @@ def test_adamw_vectors_and_remainder(n, offset):
     # a dozen fp32 roundings of values of order one, and the update's rounded constants (lr / bias terms: 1e-5 of 5e-4)
     assert (dev[0].cpu().double() - ref).abs().max() <= 16 * 2.0 ** -24 * max(1.0, float(ref.abs().max()))
     assert torch.equal(b16, dev[0].bfloat16())
+
+
+def test_calls_of_several_threads():
+    """Labels and training calls of eight host threads, each on a stream of its own: the results of the same calls alone."""
+    import threading
+    from parity_util import bf16_dev
+    from paper_2410_01805_b200 import cis_labels, rh_loss_grad
+    g = np.random.default_rng(31)
+    work = []
+    for i in range(8):
+        n = 512 + 64 * i
+        q, k = bf16_dev(g.standard_normal((40 + i, 4, 64))), bf16_dev(g.standard_normal((n, 2, 64)))
+        z, w1, w2 = bf16_dev(g.standard_normal((n, 128))), bf16_dev(g.standard_normal((128, 64)) / 11), bf16_dev(g.standard_normal((64, 2)) / 8)
+        labels = cis_labels(q, k)
+        work.append(((q, k), (z, w1, w2), labels, rh_loss_grad(z, labels, w1, w2)))
+    torch.cuda.synchronize()
+    bad = []
+
+    def run(i):
+        (q, k), (z, w1, w2), labels, (loss, d_w1, d_w2) = work[i]
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(20):
+                    assert torch.equal(cis_labels(q, k), labels)
+                    a, b, c = rh_loss_grad(z, labels, w1, w2)
+                    assert torch.equal(b, d_w1)
+                    # loss and dW2 are summed with fp32 atomics: n additions in any order
+                    assert abs(float(a - loss)) <= 1e-5 * abs(float(loss)) and float((c - d_w2).abs().max()) <= 1e-5 * float(d_w2.abs().max())
+        except Exception as e:   # (seen by the thread that waits)
+            bad.append((i, repr(e)))
+
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
