@@ -677,6 +677,9 @@ int stack_batch(locret_layer *const *layers, int n_layers, const void *hidden_in
   int k = 0;
   for (; k < n_layers && k < DECODE_BATCH; k++) {
     const locret_layer *L = layers[k];
+    // (an output that lies over the input is the later layers' input)
+    const uintptr_t in = reinterpret_cast<uintptr_t>(hidden_in), out = reinterpret_cast<uintptr_t>(attn_out) + k * out_stride * sizeof(bf16);
+    if (in < out + (size_t)A->h * A->d * sizeof(bf16) && out < in + (size_t)A->D * sizeof(bf16)) break;
     if (check_step(L, hidden_in, 1, LOCRET_NO_EVICT, static_cast<const bf16 *>(attn_out) + k * out_stride) != LOCRET_OK) break;
     if (!takes_token_step(L) || L->timing || L->pool != A->pool || L->use_pdl != A->use_pdl || L->use_side != A->use_side ||
         L->h != A->h || L->h_kv != A->h_kv || L->d != A->d || L->D != A->D || L->d_R != A->d_R || L->int4 != A->int4 ||

@@ -16,7 +16,7 @@ def _hidden(n, D, seed):
     return W.to_bf16_grid(g.standard_normal((n, D)).astype(np.float32))
 
 
-def _run(sh, budgets, order, use_stack, stride_rows=True, steps=3):
+def _run(sh, budgets, order, use_stack, stride_rows=True, steps=3, over=None):
     from paper_2410_01805_b200 import LayerStack, LocretLayer
     from parity_util import bf16_dev
     layers = [LocretLayer(sh, *(bf16_dev(a) for a in W.layer_weights(sh, i, seed=W.BASE_SEED + 9)), b, 200, 16, reserve=16)
@@ -32,6 +32,9 @@ def _run(sh, budgets, order, use_stack, stride_rows=True, steps=3):
     stack = LayerStack(picked)
     for t in range(steps):
         x = bf16_dev(_hidden(1, sh.d_model, 50 + t))
+        if over is not None:   # the input lies where layer `over` writes
+            outs[t, over] = x[0]
+            x = outs[t, over:over + 1]
         if use_stack:
             stack.decode_step(x, outs[t], out_stride=width if stride_rows else 0)
         else:
@@ -58,6 +61,16 @@ def test_stack_call_equals_calls_per_layer(d, h, hk, kw, budgets, order, stride_
     sh = W.LayerShape(d_model=256, n_q_heads=h, n_kv_heads=hk, head_dim=d, d_retain=128, rope_theta=500000.0, **kw)
     a, sa = _run(sh, budgets, list(order), False, stride_rows)
     b, sb = _run(sh, budgets, list(order), True, stride_rows)
+    assert torch.equal(a, b)
+    for x, y in zip(sa, sb):
+        for key in x:
+            assert np.array_equal(x[key], y[key]), key
+
+
+@pytest.mark.parametrize("over", [0, 1, 3])
+def test_an_output_over_the_input(over):
+    sh = W.LayerShape(d_model=256, n_q_heads=4, n_kv_heads=2, head_dim=64, d_retain=128, rope_theta=500000.0)
+    (a, sa), (b, sb) = (_run(sh, [300] * 4, range(4), use_stack, over=over) for use_stack in (False, True))
     assert torch.equal(a, b)
     for x, y in zip(sa, sb):
         for key in x:
