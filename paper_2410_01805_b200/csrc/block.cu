@@ -339,17 +339,11 @@ int locret_block_prefill_chunk(locret_block *B, const void *x_in, int32_t n_tok,
     swiglu_kernel<<<(unsigned)((n + 255) / 256), 256, 0, B->st>>>(P->gu, P->act, n_tok, F);
     BCK(cudaGetLastError());
   }
-  // y = x1 + act W_down  (d_ff is a multiple of 128, so the fallbacks of W_o are not needed)
-  if (skinny_use(n_tok, D, F, F, F)) {
+  // y = x1 + act W_down  (d_ff is a multiple of 128 and d_model of 32: one of the two takes every call)
+  if (skinny_use(n_tok, D, F, F, F))
     BCK(launch_skinny_gemm(P->act, F, B->wd_t, F, y, D, n_tok, D, F, P->x1, D, B->d_status, B->st, pdl));
-  } else if (tc && gemm_tc_supported(n_tok, D, F, F, F)) {
+  else
     BCK(launch_gemm_tc_resid(P->act, F, B->wd_t, F, y, D, n_tok, D, F, P->x1, D, B->d_status, B->st));
-  } else if (n_tok == 1) {
-    BCK(launch_gemv_resid(P->act, B->wd_t, D, F, P->x1, y, B->st));
-  } else {
-    gemm_resid_naive_kernel<<<dim3((D + 127) / 128, n_tok), 128, 0, B->st>>>(P->act, B->wd_t, P->x1, y, n_tok, D, F);
-    BCK(cudaGetLastError());
-  }
   return LOCRET_OK;
 }
 

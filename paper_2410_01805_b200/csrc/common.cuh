@@ -293,7 +293,6 @@ cudaError_t launch_compact_int4(const Int4Half &q, float *s, int64_t *t, const i
                                 int cap, int budget, cudaStream_t st);
 
 // ---- decoding (decode.cu): one token
-cudaError_t launch_gemv(const bf16 *x, const bf16 *Wt, int N, int K, bf16 *y, cudaStream_t st);
 // y = x Wt^T + r (one token; the residual is added before the one rounding)
 cudaError_t launch_gemv_resid(const bf16 *x, const bf16 *Wt, int N, int K, const bf16 *r, bf16 *y,
                               cudaStream_t st);

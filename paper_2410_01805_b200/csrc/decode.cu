@@ -37,7 +37,7 @@ __device__ __forceinline__ float warp_max(float v) {
 constexpr int GV_THREADS = 256;
 
 // y[n] = sum_k Wt[n][k] x[k]; one warp per output row, rows strided over the grid.
-// MODE 0: bf16 store.  MODE 1 (retaining head): hidden = act(y[n]); every warp keeps
+// MODE 0: bf16 store with a residual.  MODE 1 (retaining head): hidden = act(y[n]); every warp keeps
 // sum_n hidden * W2[n][m] and the block writes one partial score per KV head.
 // The block that finishes last (counted with a wrapping atomic, so the counter is zero again
 // afterwards) adds the per-block partials in block order: deterministic, and no second launch.
@@ -74,7 +74,7 @@ gemv_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ Wt, int N, int 
 #pragma unroll 8
       for (int v = lane; v < K / 8; v += 32) s += dot8(__ldg(row + v), sx[v]);
       s = warp_sum(s);
-      if (lane == 0) y[n] = __float2bfloat16_rn(resid ? s + __bfloat162float(resid[n]) : s);
+      if (lane == 0) y[n] = __float2bfloat16_rn(s + __bfloat162float(resid[n]));
     }
   } else {
     // two warps per row (halves of K), four rows per block at a time: d_R rows are too few to
@@ -678,14 +678,6 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
 }
 
 }  // namespace
-
-cudaError_t launch_gemv(const bf16 *x, const bf16 *Wt, int N, int K, bf16 *y, cudaStream_t st) {
-  if (K % 8) return cudaErrorInvalidValue;
-  const int smem = K * 2 + 8 * 32 * 4;
-  const int blocks = min((N + 7) / 8, 148 * 4);
-  gemv_kernel<0, 1><<<blocks, GV_THREADS, smem, st>>>(x, Wt, N, K, y, nullptr, 0, 0, RhGemvBatchN<1>{});
-  return cudaGetLastError();
-}
 
 // y[n] = x . Wt[n] + r[n]: a projection of one token with its residual connection
 cudaError_t launch_gemv_resid(const bf16 *x, const bf16 *Wt, int N, int K, const bf16 *r, bf16 *y,
