@@ -39,6 +39,7 @@ constexpr int HALF_BYTES = TILE * 128;  // one 64-column swizzled box of 128 row
 constexpr int TILE_BYTES = 2 * HALF_BYTES;
 constexpr int MAX_SPLIT = 8;            // portable cluster size
 constexpr int AT_SMEM = 1024 + 6 * TILE_BYTES + 256 + 2048;  // Q0,Q1,K0,K1,V0,V1 + barriers + softmax exchange
+static_assert(alone_on_an_sm(AT_SMEM), "it takes all 512 columns of tensor memory");
 // The accumulator is rescaled only when a row's maximum has grown by more than 2^100 since the
 // scale in use was fixed.  P is stored as bf16 and O, l accumulate in fp32, both with an 8-bit
 // exponent, so P <= 2^100 and O <= keys * 2^100 * |v| (< 2^122 for 2^14 keys, |v| < 2^8) stay

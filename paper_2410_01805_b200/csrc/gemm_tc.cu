@@ -123,6 +123,9 @@ struct GemmCfg {
   }
 };
 
+static_assert(alone_on_an_sm(GemmCfg<64>::smem_bytes(0)) && alone_on_an_sm(GemmCfg<128>::smem_bytes(0)) &&
+              alone_on_an_sm(GemmCfg<192>::smem_bytes(0)) && alone_on_an_sm(GemmCfg<256>::smem_bytes(0)), "see tc_common.cuh");
+
 // MAJOR: bit 0, A is stored [K x M]; bit 1, B is stored [K x N] (tcgen05 reads such "MN-major" operands as they lie,
 // in swizzled boxes of 64 columns x 64 rows of K).
 template <int BN, int MODE, int HD = 0, int MAJOR = 0>

@@ -30,6 +30,8 @@ constexpr int LB_B_BLOCK = LB_COLS * 128;    // 64 columns of a query tile: 32 K
 constexpr int LB_B_BLOCKS = 4;               // resident: two query tiles of d > 64, four of d = 64
 constexpr int LB_SMEM = 1024 + 4 * LB_A_BLOCK + LB_B_BLOCKS * LB_B_BLOCK + 256;
 
+static_assert(alone_on_an_sm(LB_SMEM), "it takes all 512 columns of tensor memory");
+
 struct LabelParams {
   float *labels;
   int n_q, n_a, h_kv, d, g, gb;  // gb: heads of the group in one query tile (a power of two)

@@ -32,6 +32,7 @@ struct SkinnyCfg {
   static constexpr int STAGE_BYTES = SK_A_BYTES + NT * SK_BK * 2;
   static constexpr int TMEM_COLS = NT < 32 ? 32 : NT;
   static constexpr int SMEM = 1024 + STAGES * STAGE_BYTES + 256;
+  static_assert(SMEM >= SKINNY_MIN_SMEM && TMEM_COLS <= 128, "see tc_common.cuh");
   static_assert(NT * SK_ROWS * 4 <= STAGES * STAGE_BYTES, "the accumulator reuses the stages");
 };
 

@@ -13,6 +13,15 @@ namespace tc {
 constexpr uint32_t WAIT_LIMIT = 1u << 24;
 constexpr int ERR_TIMEOUT = -5;  // LOCRET_ERR_DEVICE_TIMEOUT
 
+// Kernels of different streams share SMs, and a CTA that finds too little tensor memory left waits inside its SM.  CTAs of a
+// cluster wait for one another, so two cluster kernels that wait this way on different SMs could wait for ever.  Shared
+// memory keeps it from coming to that: a CTA that takes more than half of the tensor memory also takes so much shared
+// memory that no CTA of skinny.cu (at most 128 columns, at least this much shared memory) fits beside it, nor another of
+// its own kind.
+constexpr int SKINNY_MIN_SMEM = 96 * 1024;
+constexpr int SM_SMEM = 228 * 1024;
+constexpr bool alone_on_an_sm(int smem) { return smem + SKINNY_MIN_SMEM > SM_SMEM; }
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
