@@ -141,6 +141,9 @@ int locret_decode_step(locret_layer *layer, const void *hidden_in, void *attn_ou
  * alone, where the cost of crossing into the library once per layer is comparable to a layer-step
  * on the device; in a model the caller computes the next layer's input in between and calls
  * locret_decode_step per layer.  Stops at the first layer that returns an error and returns it.
+ * Layers of one stream, shape and kind of cache share their launches, up to eight at a time, with the results of a
+ * call per layer bit for bit; d_model above 4096, a budget per KV head, outputs that share memory with each other or
+ * with the input, and a layer that occurs twice take a launch per layer.
  */
 int locret_decode_step_stack(locret_layer *const *layers, int32_t n_layers, const void *hidden_in,
                              void *attn_out, int64_t out_stride);

@@ -459,7 +459,7 @@ topk_kernel(TopkArgs a, int cache_in_smem) {
 
 // One unit more than the budget, the eviction of a one-token step: the unit that goes is the competing one with
 // the lowest (score, rank), so one pass over the candidates and a block-wide minimum replace the radix select (11 us of a
-// one-token step of the small shape, 1025 candidates, two heads; 4 us this way).  Same results as topk_kernel.
+// one-token step of the small shape, 1025 candidates, two heads; 2.9 us this way).  Same results as topk_kernel.
 __global__ void __launch_bounds__(TK_THREADS)
 topk_one_kernel(TopkArgs a) {
   __shared__ unsigned long long s_best[32];

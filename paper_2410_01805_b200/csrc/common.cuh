@@ -153,21 +153,19 @@ bool gemm_tc_supported(int M, int N, int K, int lda, int ldb);
 // the same GEMM with a residual added before the one rounding: C = A Bt^T + R
 cudaError_t launch_gemm_tc_resid(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M,
                                  int N, int K, const bf16 *R, int ldr, int *status, cudaStream_t st);
-// first half of a gated FFN: C[M x N/2] = silu(A Wg) * (A Wu); Bt [N x K] interleaves, per block of
-// 128 outputs, 128 rows of Wg^T and 128 rows of Wu^T
 // training of the retaining head (operands as they lie, see gemm_tc.cu): pre-activations with partial scores, and A^T B
 int rh_pre_num_tiles(int d_R);
 cudaError_t launch_rh_pre_tc(const bf16 *Z, int ldz, const bf16 *W1, int ldw, float *pre, const float *W2, float *partial,
                              int M, int d_R, int K, int h_kv, int *status, cudaStream_t st);
 cudaError_t launch_gemm_tn_f32(const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int M, int N, int K,
                                int *status, cudaStream_t st);
-// C (fp32, leading dimension ldc in floats) = A Bt^T
 // heads divided over GPUs: this GPU's partial first product of the retaining head (fallback for
 // shapes the tensor-core GEMM does not take), and scores from the summed product
 cudaError_t launch_preact_naive(const bf16 *z, const bf16 *W1t, float *pre, int n_tok, int d_R, int d_in,
                                 cudaStream_t st);
 cudaError_t launch_rh_finish(const float *pre, const float *w2, float *s, int score_stride, int slot0,
                              int n_tok, int d_R, int h_kv, int act, cudaStream_t st);
+// C (fp32, leading dimension ldc in floats) = A Bt^T
 cudaError_t launch_gemm_tc_f32(const bf16 *A, int lda, const bf16 *Bt, int ldb, float *C, int ldc, int M, int N,
                                int K, int *status, cudaStream_t st);
 // the same product ADDED into n_peers fp32 buffers (device array of device pointers; the buffers may be
@@ -176,6 +174,8 @@ cudaError_t launch_gemm_tc_f32_add_peers(const bf16 *A, int lda, const bf16 *Bt,
                                          int n_peers, int ldc, int M, int N, int K, int *status, cudaStream_t st);
 // peers[p][i] += src[i] for i < count (the fallback beside the GEMM above)
 cudaError_t launch_add_to_peers(const float *src, float *const *peers, int n_peers, size_t count, cudaStream_t st);
+// first half of a gated FFN: C[M x N/2] = silu(A Wg) * (A Wu); Bt [N x K] interleaves, per block of
+// 128 outputs, 128 rows of Wg^T and 128 rows of Wu^T
 bool gemm_tc_gated_supported(int M, int N, int K, int lda, int ldb);
 cudaError_t launch_gemm_tc_gated(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M,
                                  int N, int K, int *status, cudaStream_t st);

@@ -9,8 +9,8 @@
 // multiplied.  Eight warps reduce, each thread one row's maximum over half the columns, three-input maxima, all
 // query tiles of a work unit before one atomic maximum per row on the order-preserving integer image.
 // One launch for all heads (a launch of the 128 x 256 GEMM per query head before: two K-blocks per tile, the keys
-// re-read for every head).  131072 keys, 1024 answers, 32 query heads of 8 KV heads of 128: 0.70 ms = 1.57 PFLOP/s
-// (1.45 ms before); the measured burst peak allows 0.64 ms.
+// re-read for every head).  131072 keys, 1024 answers, 32 query heads of 8 KV heads of 128: 0.84 ms a call in a loop, under
+// the power cap, = 1.31 PFLOP/s (1.55 ms before); one call after a pause 0.70 ms; the measured burst peak allows 0.64 ms.
 #include <atomic>
 #include <thread>
 

@@ -801,7 +801,6 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
   };
   // the codes are read by the compaction of this step and by later steps, never by this step's
   // attention (the chunk attends to its own keys and values in bf16): second stream
-  // (a one-token step quantises its token inside the attention kernel)
   if (L->int4 && !side) { const int rc = quantize_chunk(L->st); if (rc != LOCRET_OK) return rc; }
   if (side) CK(cudaEventRecord(L->ev_ready, L->st));
   if (side && deq) CK(cudaStreamWaitEvent(L->st, P->ev_exp_ready, 0));

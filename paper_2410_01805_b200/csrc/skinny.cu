@@ -9,11 +9,11 @@
 // between dependent launches.  The S partial sums meet in distributed shared memory: each CTA
 // leaves its accumulator there as [token][row], and rank r adds the tokens of its share over all ranks
 // in rank order (deterministic, no scratch, no second launch) and runs the epilogue on them:
-// Measured for 20 tokens: W_gate and W_up of the Llama shape (235 MB) 43 us = 5.5 TB/s, W_down (117 MB) 25 us, the
-// QKV projection (50 MB, 45 tokens) 16 us (34 us on 24 tiles of 128 x 256).
 //   EPI 0: bf16 store, with the residual added before the rounding if there is one;
 //   EPI 1: gated FFN, first half: a tile is 64 gate rows and the 64 up rows of the same outputs;
 //   EPI 2: retaining head: activation and the thin product with W2, one partial score per (tile, token, head).
+// Measured for 20 tokens: W_gate and W_up of the Llama shape (235 MB) 43 us = 5.5 TB/s, W_down (117 MB) 25 us, the
+// QKV projection (50 MB, 45 tokens) 16 us (34 us on 24 tiles of 128 x 256).
 #include "tc_common.cuh"
 
 namespace locret {
@@ -317,10 +317,11 @@ bool skinny_supported(int n_tok, int N, int K, int ldx, int ldw) {
 }
 
 // Up to two token tiles the weights stream (almost) once.  Beyond, every further token tile costs about as much as the
-// first, and the GEMM with 128 x 256 tiles wins once its tiles cover a quarter of the SMs.  Microseconds per whole
-// layer step (Llama shape, 4500 cached tokens), this path / that GEMM with nothing else changed: 20 tokens 148 / 206,
-// 45: 152 / 165, 128: 117 / 128; whole blocks over 1000 tokens: 128: 189 / 271, 256: 250 / 300, 384: 355 / 330,
-// 512: 394 / 353.  The small shape (768 and 256 columns) at 512 tokens: 42 / 64.
+// first, and the GEMM with 128 x 256 tiles wins once its tiles cover a quarter of the SMs.  Microseconds, this path / that
+// GEMM with nothing else changed: layer steps of the Llama shape over 4500 units (projection and retaining head), 33
+// tokens: 53 / 67, 45: 54 / 68, 128: 61 / 73; whole blocks over an empty cache (W_o and the FFN), Llama shape, 33: 137 / 220,
+// 128: 159 / 233, 256: 201 / 259, 384: 290 / 293, 512: 339 / 323; Phi-3 shape (its projection of 9216 columns gives up the
+// fused RoPE here), 33: 98 / 159, 128: 112 / 169, 256: 135 / 177, 300: 205 / 202; small shape, 256: 61 / 76, 384: 75 / 82.
 bool skinny_use(int n_tok, int N, int K, int ldx, int ldw) {
   if (!skinny_supported(n_tok, N, K, ldx, ldw)) return false;
   if (n_tok <= 256) return true;
@@ -328,20 +329,20 @@ bool skinny_use(int n_tok, int N, int K, int ldx, int ldw) {
   return n_tok <= 512 && wide_tiles * 4 <= sm_count_of_current_device();
 }
 
-// The retaining head of a layer step runs beside attention and the next projection.  Up to one token tile its 64 CTAs are
-// little to them.  Beyond, what counts is less its own time than the SMs it takes: at 512 tokens (Phi-3 shape, K = 9216) this
-// path takes 52 us on 128 SMs, the wide GEMM 87 us on 16, and four layers in turn (1000 cached units) took 130 us a step
-// with this one and 100 with that; 384 tokens of the Llama shape, empty cache: 80 / 72.  So beyond 128 tokens it is for
-//   matrices so small that it leaves half of the SMs alone (small shape, 512 tokens: 35 / 42 us a step);
-//   up to 256 tokens a K so long that the wide GEMM's chain of K-blocks outlasts what it runs beside, as it does from about
-//   twice the projection's K on (Phi-3 shape, K = 3 d_model, 200 tokens: 71 / 90; Llama shape, 1.5 d_model: 66 / 61);
-//   and where the next step waits for it (awaited: a 4-bit cache's expansion is enqueued behind it) up to 512 tokens
-//   (Phi-3 shape, 512 tokens, 1000 cached: 128 / 130, 300 tokens 104 / 120).
 int skinny_ctas(int n_tok, int N, int K) {
   const SkinnyPlan plan = skinny_plan(n_tok, N, K);
   return plan.tiles * ((n_tok + plan.nt - 1) / plan.nt) * plan.n_split;
 }
 
+// The retaining head of a layer step runs beside attention and the next projection.  Up to one token tile its 64 CTAs are
+// little to them.  Beyond, what counts is less its own time than the SMs it takes: at 512 tokens (Phi-3 shape, K = 9216) this
+// path takes 52 us on 128 SMs, the wide GEMM 87 us on 16, and four layers in turn (1000 cached units) took 130 us a step
+// with this one and 100 with that; 384 tokens of the Llama shape, empty cache: 81 / 73.  So beyond 128 tokens it is for
+//   matrices so small that it leaves half of the SMs alone (small shape, 512 tokens: 35 / 42 us a step);
+//   up to 256 tokens a K so long that the wide GEMM's chain of K-blocks outlasts what it runs beside, as it does from about
+//   twice the projection's K on (Phi-3 shape, K = 3 d_model, 200 tokens: 71 / 90; Llama shape, 1.5 d_model: 66 / 61);
+//   and where the next step waits for it (awaited: a 4-bit cache's expansion is enqueued behind it) up to 512 tokens
+//   (Phi-3 shape, 512 tokens, 1000 cached: 128 / 130, 300 tokens 104 / 120).
 bool skinny_use_beside(int n_tok, int N, int K, int ldx, int ldw, int d_model, bool awaited) {
   if (!skinny_supported(n_tok, N, K, ldx, ldw)) return false;
   if (n_tok <= 128) return true;
