@@ -53,3 +53,15 @@ def test_retaining_head_of_a_long_k(kv_dtype, n_tok):
     ora.prefill_chunk(_hidden(700, 128, 1), 0)
     lockstep_chunk(ora, gpu, _hidden(n_tok, 128, n_tok), 1, what=f"{kv_dtype} 700+{n_tok}")
     gpu.destroy()
+
+
+@pytest.mark.parametrize("kv_dtype", [0, 1])
+@pytest.mark.parametrize("D", [4096, 4608])   # the last width whose layers share a launch, and one beyond
+def test_one_token_of_a_wide_model(D, kv_dtype):
+    from parity_util import lockstep_chunk, make_pair
+    sh = W.LayerShape(d_model=D, n_q_heads=4, n_kv_heads=2, head_dim=64, d_retain=96, rope_theta=500000.0, kv_dtype=kv_dtype)
+    ora, gpu = make_pair(sh, W.layer_weights(sh, 0, seed=W.BASE_SEED + 73), budget=200, chunk=100, n_stab=16)
+    ora.prefill_chunk(_hidden(90, D, 1), 0)
+    for t in range(2):
+        lockstep_chunk(ora, gpu, _hidden(1, D, 60 + t), 1, what=f"{D} token {t}")
+    gpu.destroy()
