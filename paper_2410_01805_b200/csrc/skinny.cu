@@ -343,6 +343,9 @@ int skinny_ctas(int n_tok, int N, int K) {
 //   twice the projection's K on (Phi-3 shape, K = 3 d_model, 200 tokens: 71 / 90; Llama shape, 1.5 d_model: 66 / 61);
 //   and where the next step waits for it (awaited: a 4-bit cache's expansion is enqueued behind it) up to 512 tokens
 //   (Phi-3 shape, 512 tokens, 1000 cached: 128 / 130, 300 tokens 104 / 120).
+// A step that evicts would gain from it as well (Phi-3 shape, budget 700, 300 tokens, four layers: 96 / 118; Llama shape, 200
+// tokens: 71 / 75), but the bits of a step's scores must not depend on its flags, and the same step without an eviction
+// hands over its output later (one layer, 300 tokens: 112 / 78 us until attention is done).
 bool skinny_use_beside(int n_tok, int N, int K, int ldx, int ldw, int d_model, bool awaited) {
   if (!skinny_supported(n_tok, N, K, ldx, ldw)) return false;
   if (n_tok <= 128) return true;
