@@ -1,5 +1,5 @@
 // bf16 GEMM on tcgen05 tensor cores: C[M x N] = A[M x K] · Bt[N x K]^T, fp32 accumulation in
-// tensor memory.  One CTA computes a 128 x BN tile: warp 0 feeds shared memory with TMA
+// tensor memory.  One CTA computes a 128 x BN tile, or a pair of CTAs a 256 x BN tile (PAIR, see GemmCfg): warp 0 feeds shared memory with TMA
 // (128-byte swizzled K-blocks of 64), warp 1 issues tcgen05.mma, warps 2..5 read the
 // accumulator from TMEM and run the epilogue:
 //   MODE 0: bf16 store (the QKV projection);
@@ -109,11 +109,18 @@ __device__ __forceinline__ float fast_act(float x, int act) {
   return apply_act(x, act);
 }
 
-template <int BN>
+// PAIR: a cluster of two CTAs computes a 256-row tile with cta_group::2 instructions: each CTA loads its own 128 rows of A and
+// HALF of the tile's rows of B, and holds its 128 rows of the accumulator.  What a single CTA's K-block of a 128 x 256 tile
+// waits for is its 48 KB from L2 (96 B per cycle and SM at the full MMA rate); here it is 32 KB, which also leaves
+// room for six stages instead of four.  Measured (us, single CTAs / pairs, in the running passes, power cap): QKV projection of 3072
+// tokens with RoPE, Llama shape 118 / 108, Phi-3 shape (192 columns, 1024 tokens) 69.5 / 64.0; gated FFN 487 / 440; W_o and W_down
+// 384 / 338 together; gradients (both operands MN-major) 131 / 120, pre-activations 142 / 136.
+template <int BN, bool PAIR>
 struct GemmCfg {
-  static constexpr int STAGES = BN >= 192 ? 4 : (BN == 128 ? 6 : 8);
+  static constexpr int STAGES = PAIR ? 6 : (BN >= 192 ? 4 : (BN == 128 ? 6 : 8));
   static constexpr int TMEM_COLS = BN == 192 ? 512 : 2 * BN;  // two accumulators; a power of two
-  static constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
+  static constexpr int B_ROWS = PAIR ? BN / 2 : BN;
+  static constexpr int A_BYTES = BM * BK * 2, B_BYTES = B_ROWS * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int W2_BYTES = BN * MAX_HKV * 4;
   static constexpr int EPI_BYTES = 4 * EPI_WARP_BYTES;  // MODE 2: one staged head of 32 rows per warp
@@ -123,12 +130,13 @@ struct GemmCfg {
   }
 };
 
-static_assert(alone_on_an_sm(GemmCfg<64>::smem_bytes(0)) && alone_on_an_sm(GemmCfg<128>::smem_bytes(0)) &&
-              alone_on_an_sm(GemmCfg<192>::smem_bytes(0)) && alone_on_an_sm(GemmCfg<256>::smem_bytes(0)), "see tc_common.cuh");
+static_assert(alone_on_an_sm(GemmCfg<64, false>::smem_bytes(0)) && alone_on_an_sm(GemmCfg<128, false>::smem_bytes(0)) &&
+              alone_on_an_sm(GemmCfg<192, false>::smem_bytes(0)) && alone_on_an_sm(GemmCfg<256, false>::smem_bytes(0)) &&
+              alone_on_an_sm(GemmCfg<192, true>::smem_bytes(0)) && alone_on_an_sm(GemmCfg<256, true>::smem_bytes(0)), "see tc_common.cuh");
 
 // MAJOR: bit 0, A is stored [K x M]; bit 1, B is stored [K x N] (tcgen05 reads such "MN-major" operands as they lie,
 // in swizzled boxes of 64 columns x 64 rows of K).
-template <int BN, int MODE, int HD = 0, int MAJOR = 0>
+template <int BN, int MODE, int HD = 0, int MAJOR = 0, bool PAIR = false>
 __global__ void __launch_bounds__(GT_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                bf16 *__restrict__ C, int ldc, int M, int N, int K, const float *__restrict__ W2,
@@ -137,7 +145,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // Persistent: CTA b computes tiles b, b + gridDim.x, ... (row-block major, so that concurrent
   // CTAs share the A row block in L2).  The accumulator is double-buffered in TMEM: the epilogue
   // of one tile overlaps the main loop of the next.
-  using Cfg = GemmCfg<BN>;
+  using Cfg = GemmCfg<BN, PAIR>;
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
@@ -158,29 +166,33 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // K-blocks of 64; a last partial block reads past the operands' inner extent, where TMA fills zeros
   const int KB = (K + BK - 1) / BK;
   const int tiles_n = (N + BN - 1) / BN;
-  const int tiles_m = (M + BM - 1) / BM;
+  const int tiles_m = (M + BM * (PAIR ? 2 : 1) - 1) / (BM * (PAIR ? 2 : 1));
   const int total = tiles_m * tiles_n;
+  const uint32_t rank = PAIR ? cluster_ctarank() : 0;   // rank 0 issues the pair's MMAs; loads of both are counted on its barriers
+  const int first_tile = PAIR ? blockIdx.x >> 1 : blockIdx.x, tile_step = PAIR ? gridDim.x >> 1 : gridDim.x;
   // tile order: row-block major (concurrent CTAs share the A row block in L2), or, when B is the
   // large operand and does not fit the L2, column-block major (they share the B tile and sweep M)
   auto tile_mn = [&](int tile, int &m0, int &n0) {
     if (n_major) { m0 = (tile % tiles_m) * BM; n0 = (tile / tiles_m) * BN; }
     else { m0 = (tile / tiles_n) * BM; n0 = (tile % tiles_n) * BN; }
+    if (PAIR) m0 = 2 * m0 + (int)rank * BM;
   };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; s++) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int i = 0; i < 2; i++) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4); }
+    for (int i = 0; i < 2; i++) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], PAIR ? 8 : 4); }
     *abort_flag = 0;
     fence_barrier_init();
     prefetch_tmap(&map_a);
     prefetch_tmap(&map_b);
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
-    tmem_relinquish();
+    if (PAIR) { tmem2_alloc(tmem_slot, Cfg::TMEM_COLS); tmem2_relinquish(); }
+    else { tmem_alloc(tmem_slot, Cfg::TMEM_COLS); tmem_relinquish(); }
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync_all();   // the partner's barriers exist before anything is sent to them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -188,7 +200,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
+      for (int tile = first_tile; tile < total && ok; tile += tile_step) {
         int m0, n0;
         tile_mn(tile, m0, n0);
         for (int kb = 0; kb < KB; kb++, it++) {
@@ -196,31 +208,42 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           const uint32_t ph = (it / STAGES) & 1;
           ok = mbar_wait(&empty[s], ph ^ 1, abort_flag, status);
           if (!ok) break;
-          mbar_expect_tx(&full[s], Cfg::STAGE_BYTES);
+          if (!PAIR) mbar_expect_tx(&full[s], Cfg::STAGE_BYTES);
+          else if (rank == 0) mbar_expect_tx(&full[s], 2 * Cfg::STAGE_BYTES);
+          const uint32_t bar0 = PAIR ? map_to_cta(smem_u32(&full[s]), 0) : 0;
+          auto load = [&](unsigned char *dst, const CUtensorMap *map, int c0, int c1) {
+            if (PAIR) tma2_load_2d(dst, map, c0, c1, bar0);
+            else tma_load_2d(dst, map, c0, c1, &full[s]);
+          };
           unsigned char *a_dst = tiles + s * Cfg::STAGE_BYTES;
+          const int nb = n0 + (int)rank * Cfg::B_ROWS;
           if (MAJOR & 1) {
 #pragma unroll
-            for (int i = 0; i < BM / 64; i++) tma_load_2d(a_dst + i * MN_BOX, &map_a, m0 + i * 64, kb * BK, &full[s]);
+            for (int i = 0; i < BM / 64; i++) load(a_dst + i * MN_BOX, &map_a, m0 + i * 64, kb * BK);
           } else {
-            tma_load_2d(a_dst, &map_a, kb * BK, m0, &full[s]);
+            load(a_dst, &map_a, kb * BK, m0);
           }
           if (MAJOR & 2) {
 #pragma unroll
-            for (int i = 0; i < BN / 64; i++)
-              tma_load_2d(a_dst + Cfg::A_BYTES + i * MN_BOX, &map_b, n0 + i * 64, kb * BK, &full[s]);
+            for (int i = 0; i < Cfg::B_ROWS / 64; i++) load(a_dst + Cfg::A_BYTES + i * MN_BOX, &map_b, nb + i * 64, kb * BK);
           } else {
-            tma_load_2d(a_dst + Cfg::A_BYTES, &map_b, kb * BK, n0, &full[s]);
+            load(a_dst + Cfg::A_BYTES, &map_b, kb * BK, nb);
           }
         }
       }
+      // the completions of the last uses of every stage are sent to both CTAs and nobody else waits for them: no CTA ends
+      // while such an arrival is on its way
+      if (PAIR)
+        for (uint32_t i = it > STAGES ? it - STAGES : 0; i < it && ok; i++)
+          ok = mbar_wait(&empty[i % STAGES], (i / STAGES) & 1, abort_flag, status);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16(BM, BN, MAJOR & 1, MAJOR >> 1);
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = idesc_bf16(PAIR ? 2 * BM : BM, BN, MAJOR & 1, MAJOR >> 1);
       constexpr uint64_t a_step = ((MAJOR & 1) ? 16 * 128 : 32) >> 4, b_step = ((MAJOR & 2) ? 16 * 128 : 32) >> 4;
       uint32_t it = 0, lt = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, lt++) {
+      for (int tile = first_tile; tile < total && ok; tile += tile_step, lt++) {
         const uint32_t buf = lt & 1;
         ok = mbar_wait(&acc_empty[buf], ((lt >> 1) & 1) ^ 1, abort_flag, status);
         if (!ok) break;
@@ -238,12 +261,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                                           : desc_kmajor_sw128(a_src + Cfg::A_BYTES);
 #pragma unroll
           for (int k = 0; k < BK / 16; k++) {
-            if (kb == 0 && k == 0) mma_ss_first(d_tmem, da, db, idesc);
+            if (PAIR) mma2_ss(d_tmem, da + (uint64_t)k * a_step, db + (uint64_t)k * b_step, idesc, kb > 0 || k > 0);
+            else if (kb == 0 && k == 0) mma_ss_first(d_tmem, da, db, idesc);
             else mma_ss_acc(d_tmem, da + (uint64_t)k * a_step, db + (uint64_t)k * b_step, idesc);
           }
-          mma_commit(&empty[s]);  // frees the stage once these MMAs have read it
+          // frees the stage once these MMAs have read it
+          if (PAIR) mma2_commit_both(&empty[s]);
+          else mma_commit(&empty[s]);
         }
-        if (ok) mma_commit(&acc_full[buf]);
+        if (ok) {
+          if (PAIR) mma2_commit_both(&acc_full[buf]);
+          else mma_commit(&acc_full[buf]);
+        }
       }
     }
   } else {
@@ -253,7 +282,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     uint32_t lt = 0;
     bool ok = true;
     // (no early exit: after a timed-out wait the warps still meet at the named barrier)
-    for (int tile = blockIdx.x; tile < total; tile += gridDim.x, lt++) {
+    for (int tile = first_tile; tile < total; tile += tile_step, lt++) {
       int m0, n0;
       tile_mn(tile, m0, n0);
       const uint32_t buf = lt & 1;
@@ -551,45 +580,74 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       // every tcgen05.ld of this warp has completed (wait::ld above): the buffer may be reused
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[buf]);
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_remote(map_to_cta(smem_u32(&acc_empty[buf]), 0));
+        else mbar_arrive(&acc_empty[buf]);
+      }
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync_all();   // the partner has read its accumulators and sent what it sends
   tc_fence_after();
   if (warp == 1) {
     __syncwarp();
-    tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
+    if (PAIR) tmem2_dealloc(tmem_base, Cfg::TMEM_COLS);
+    else tmem_dealloc(tmem_base, Cfg::TMEM_COLS);
   }
+  if (PAIR) cluster_sync_all();   // (neither leaves before both have released the pair's tensor memory)
 }
 
-template <int BN, int MODE, int HD = 0, int MAJOR = 0>
-cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M, int N,
-                     int K, const float *W2, float *partial, int h_kv, int act, const RopeAppendArgs &ra,
-                     int *status, cudaStream_t st, const bf16 *resid = nullptr, int ldr = 0) {
-  using Cfg = GemmCfg<BN>;
+template <int BN, int MODE, int HD, int MAJOR, bool PAIR>
+cudaError_t launch_as(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M, int N,
+                      int K, const float *W2, float *partial, int h_kv, int act, const RopeAppendArgs &ra,
+                      int *status, cudaStream_t st, const bf16 *resid, int ldr) {
+  using Cfg = GemmCfg<BN, PAIR>;
+  const auto kernel = gemm_tc_kernel<BN, MODE, HD, MAJOR, PAIR>;
   static PerDeviceFlag attr_set;
-  if (cudaError_t e = allow_dynamic_smem(gemm_tc_kernel<BN, MODE, HD, MAJOR>, Cfg::smem_bytes(MODE), attr_set);
-      e != cudaSuccess)
-    return e;
+  if (cudaError_t e = allow_dynamic_smem(kernel, Cfg::smem_bytes(MODE), attr_set); e != cudaSuccess) return e;
   CUtensorMap ma, mb;
   const bool a_ok = (MAJOR & 1) ? cached_map_k64(&ma, A, M, K, (uint64_t)lda * 2, BK)
                                 : cached_map_k64(&ma, A, K, M, (uint64_t)lda * 2, BM);
   const bool b_ok = (MAJOR & 2) ? cached_map_k64(&mb, Bt, N, K, (uint64_t)ldb * 2, BK)
-                                : cached_map_k64(&mb, Bt, K, N, (uint64_t)ldb * 2, BN);
+                                : cached_map_k64(&mb, Bt, K, N, (uint64_t)ldb * 2, Cfg::B_ROWS);
   if (!a_ok || !b_ok) return cudaErrorInvalidValue;
-  const int num_sms = sm_count_of_current_device();
-  const int total = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-  const int grid = total < num_sms ? total : num_sms;
+  constexpr int CTAS = PAIR ? 2 : 1;
+  const int slots = sm_count_of_current_device() / CTAS;
+  const int total = ((N + BN - 1) / BN) * ((M + BM * CTAS - 1) / (BM * CTAS));
   // B is the larger operand: keep a B tile resident and sweep the rows (each B tile is then read
   // from HBM once; in row-block-major order a B that exceeds the L2 is re-read for every row
   // block, and even one that fits is read about three times)
   const size_t a_bytes = (size_t)M * K * 2, b_bytes = (size_t)N * K * 2;
   const int n_major = MODE != 1 && MODE != 7 && b_bytes > a_bytes;  // (MODE 1 and 7 index their partial sums by column tile either way)
-  gemm_tc_kernel<BN, MODE, HD, MAJOR><<<grid, GT_THREADS, Cfg::smem_bytes(MODE), st>>>(
-      ma, mb, C, ldc, M, N, K, W2, partial, h_kv, act, ra, resid, ldr, n_major, status);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((total < slots ? total : slots) * CTAS);
+  cfg.blockDim = dim3(GT_THREADS);
+  cfg.dynamicSmemBytes = Cfg::smem_bytes(MODE);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CTAS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = PAIR ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, ma, mb, C, ldc, M, N, K, W2, partial, h_kv, act, ra, resid, ldr, n_major, status);
+}
+
+// Pairs of CTAs where they take no more waves than single CTAs do: a wave of either costs the same MMAs, and an odd
+// number of 128-row blocks leaves half of a pair's last tile idle, which only shows in the number of waves.  One
+// block of rows, and the tile widths below 192 that only small matrices take, stay with single CTAs.
+template <int BN, int MODE, int HD = 0, int MAJOR = 0>
+cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M, int N,
+                     int K, const float *W2, float *partial, int h_kv, int act, const RopeAppendArgs &ra,
+                     int *status, cudaStream_t st, const bf16 *resid = nullptr, int ldr = 0) {
+  if constexpr (BN >= 192 && MODE != 6) {
+    const int sms = sm_count_of_current_device(), tn = (N + BN - 1) / BN, blocks = (M + BM - 1) / BM;
+    const int single = (tn * blocks + sms - 1) / sms, pairs = sms / 2, paired = pairs ? (tn * ((blocks + 1) / 2) + pairs - 1) / pairs : 0;
+    if (pairs && blocks > 1 && paired <= single)
+      return launch_as<BN, MODE, HD, MAJOR, true>(A, lda, Bt, ldb, C, ldc, M, N, K, W2, partial, h_kv, act, ra, status, st, resid, ldr);
+  }
+  return launch_as<BN, MODE, HD, MAJOR, false>(A, lda, Bt, ldb, C, ldc, M, N, K, W2, partial, h_kv, act, ra, status, st, resid, ldr);
 }
 
 }  // namespace
