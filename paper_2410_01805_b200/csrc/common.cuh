@@ -302,6 +302,7 @@ cudaError_t launch_gemv_gated(const bf16 *x, const bf16 *Wt, int F, int K, bf16 
 // The three kernels of a one-token step take one layer or a batch of layers with the same input and shape (each kernel is
 // compiled for one layer, whose arguments need no indexing, and for up to DECODE_BATCH).
 constexpr int DECODE_BATCH = 8;
+constexpr int DECODE_HEAD_GROUPS = 32 * 32;   // (KV head, group of query heads) pairs of a layer, at most
 // projection + positions + RoPE + cache append (a.staging is written, not read); more than one layer if gemv_rope_batched
 template <int N> struct GemvRopeBatchN { const bf16 *Wt[N]; RopeAppendArgs a[N]; };
 typedef GemvRopeBatchN<DECODE_BATCH> GemvRopeBatch;
@@ -324,7 +325,7 @@ typedef RhGemvBatchN<DECODE_BATCH> RhGemvBatch;
 int rh_gemv_blocks(int d_R);
 cudaError_t launch_rh_gemv(const RhGemvBatch &b, int n_layers, int d_R, int K, int h_kv, int act, cudaStream_t st, bool pdl);
 // attention.  part_o: fp32 [h][n_splits][d]; part_ml: fp32 [h][n_splits][2]; counters: one zeroed word per
-// (KV head, group of 16 query heads), left at zero (the last split merges the partial results).
+// (KV head, group of 16 query heads; of eight with a 4-bit cache), left at zero (the last split merges the partial results).
 // q4.kq != nullptr (in all layers of a batch or none): keys [0, n - 1) are read from the 4-bit cache (expanded and rotated
 // with `cs` on the way into shared memory, at position rank[m * cap + slot] for slot < ranked_len and slot above) and only
 // key n - 1, the token of this step, from k_rot / v, which then hold just that unit, [h_kv][d].  tok_k / tok_v (4-bit

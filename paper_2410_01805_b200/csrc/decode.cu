@@ -284,23 +284,6 @@ gemv_rope_wide_kernel(const bf16 *__restrict__ x, int K, int n_layers, const __g
   }
 }
 
-// 4-bit codes -> floats, the arithmetic of the cache's expansion pre-pass (two codes per byte, even
-// element in the low nibble, value = code * scale)
-__device__ __forceinline__ void dequant8(uint32_t w, float s, float (&x)[8]) {
-#pragma unroll
-  for (int b = 0; b < 4; b++) {
-    const uint32_t byte = (w >> (8 * b)) & 0xFFu;
-    x[2 * b] = (float)((int)(byte << 28) >> 28) * s;
-    x[2 * b + 1] = (float)((int)(byte << 24) >> 28) * s;
-  }
-}
-__device__ __forceinline__ uint4 to_bf16x8(const float (&x)[8]) {
-  uint4 o;
-  o.x = pack_bf16(x[0], x[1]); o.y = pack_bf16(x[2], x[3]);
-  o.z = pack_bf16(x[4], x[5]); o.w = pack_bf16(x[6], x[7]);
-  return o;
-}
-
 // ---- decode attention on warp-level tensor-core instructions.  grid (h_kv, splits, head groups
 // of <= 16).  The rows of the m16n8k16 tiles are the query heads of one GQA group (all of them read
 // the same keys), padded to 16; keys and values of the split stream through shared memory in
@@ -311,22 +294,14 @@ __device__ __forceinline__ uint4 to_bf16x8(const float (&x)[8]) {
 // order (a wrapping atomic counter, left at zero for the next step).
 constexpr int DA_THREADS = 128, DA_G = 16, DA_KT = 64;
 
-// INT4: keys [0, n - 1) come from the 4-bit cache (codes and scales expanded, keys rotated at the
-// unit's position in temporal order, with the arithmetic of the expansion pre-pass, as the tile is brought into shared
-// memory); key n - 1, the token of this step, comes in bf16 from k_rot / v, which then hold that one
-// unit of every head, [h_kv][D].
-template <int D, bool INT4, int NL>
-__global__ void __launch_bounds__(DA_THREADS, INT4 ? 2 : 4)  // (168 registers, for three blocks, cost the 4-bit kernel a third of its speed)
+template <int D, int NL>
+__global__ void __launch_bounds__(DA_THREADS, 4)
 attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ DecodeAttnBatchN<NL> batch) {
   const int hgroups = (h / h_kv + DA_G - 1) / DA_G, layer = NL == 1 ? 0 : blockIdx.z / hgroups;
   const DecodeAttnLayer &a = batch.l[layer];
   const bf16 *__restrict__ q_rot = a.q_rot, *__restrict__ k_rot = a.k_rot, *__restrict__ v = a.v;
   float *__restrict__ part_o = a.part_o, *__restrict__ part_ml = a.part_ml;
-  const int cap = a.cap, n = a.n, n_splits = a.n_splits, ranked_len = a.ranked_len;
-  const Int4Half &q4 = a.q4;
-  const float2 *__restrict__ cs = a.cs;
-  const int32_t *__restrict__ rank = a.rank;
-  const bf16 *__restrict__ tok_k = a.tok_k, *__restrict__ tok_v = a.tok_v;
+  const int cap = a.cap, n = a.n, n_splits = a.n_splits;
   constexpr int LD = D + 8;
   constexpr int VPR = D / 8;  // 16-byte vectors per row
   extern __shared__ __align__(16) unsigned char da_smem[];
@@ -360,124 +335,17 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
       cp_async16(sV + (buf * DA_KT + r) * LD + c, vbase + off, ok);
     }
   };
-  // 4-bit cache: one thread expands elements [c, c+8) and [c+half, c+half+8) of K and V of one key.
-  // In two steps, so that a tile's codes, scales and ranks are already on their way while the
-  // previous tile is multiplied: fetch_q4 requests them into registers (one tile ahead), expand_q4
-  // reads the (cos, sin) rows of the units' positions, expands, rotates and fills the shared tile.
-  constexpr int Q4_ITER = DA_KT * (D / 16) / DA_THREADS;
-  static_assert(Q4_ITER * DA_THREADS == DA_KT * (D / 16), "whole iterations");
-  struct Q4Pre { uint32_t kw0, kw1, vw0, vw1; float ks, vs; int pos; };  // pos < 0: not a unit of the 4-bit cache
-  Q4Pre pre[INT4 ? Q4_ITER : 1];
-  auto fetch_q4 = [&](int kt) {
-    constexpr int HALF = D / 2, HV = D / 16;
-#pragma unroll
-    for (int i = 0; i < Q4_ITER; i++) {
-      const int x = tid + i * DA_THREADS;
-      const int r = x / HV, c = (x - r * HV) * 8;
-      const int key = k0 + kt * DA_KT + r;
-      pre[i].pos = -1;
-      if (key < n - 1) {
-        const size_t u = (size_t)m * cap + key;
-        const uint8_t *kc = q4.kq + u * HALF, *vc = q4.vq + u * HALF;
-        pre[i].kw0 = *reinterpret_cast<const uint32_t *>(kc + c / 2);
-        pre[i].kw1 = *reinterpret_cast<const uint32_t *>(kc + (c + HALF) / 2);
-        pre[i].vw0 = *reinterpret_cast<const uint32_t *>(vc + c / 2);
-        pre[i].vw1 = *reinterpret_cast<const uint32_t *>(vc + (c + HALF) / 2);
-        pre[i].ks = __half2float(q4.ks[u]);
-        pre[i].vs = __half2float(q4.vs[u]);
-        pre[i].pos = key < ranked_len ? rank[u] : key;  // the unit's place in temporal order
-      }
-    }
-  };
-  auto expand_q4 = [&](int buf, int kt) {
-    constexpr int HALF = D / 2, HV = D / 16;
-    float4 t4[Q4_ITER][4];   // 8 (cos, sin) pairs per item, all requested before any is used
-#pragma unroll
-    for (int i = 0; i < Q4_ITER; i++) {
-      const int x = tid + i * DA_THREADS;
-      const int c = (x - (x / HV) * HV) * 8;
-      if (pre[i].pos >= 0) {
-        const float4 *t = reinterpret_cast<const float4 *>(cs + (size_t)pre[i].pos * HALF + c);
-#pragma unroll
-        for (int e = 0; e < 4; e++) t4[i][e] = __ldg(t + e);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < Q4_ITER; i++) {
-      const int x = tid + i * DA_THREADS;
-      const int r = x / HV, c = (x - r * HV) * 8;
-      const int key = k0 + kt * DA_KT + r;
-      bf16 *kd = sK + (buf * DA_KT + r) * LD, *vd = sV + (buf * DA_KT + r) * LD;
-      uint4 ka = make_uint4(0, 0, 0, 0), kb = ka, va = ka, vb = ka;
-      if (pre[i].pos >= 0) {
-        float a[8], b[8];
-        dequant8(pre[i].kw0, pre[i].ks, a);
-        dequant8(pre[i].kw1, pre[i].ks, b);
-        const float2 *t = reinterpret_cast<const float2 *>(&t4[i][0]);
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-          const float x1 = a[e], x2 = b[e];
-          a[e] = x1 * t[e].x - x2 * t[e].y;
-          b[e] = x2 * t[e].x + x1 * t[e].y;
-        }
-        ka = to_bf16x8(a); kb = to_bf16x8(b);
-        dequant8(pre[i].vw0, pre[i].vs, a);
-        dequant8(pre[i].vw1, pre[i].vs, b);
-        va = to_bf16x8(a); vb = to_bf16x8(b);
-      } else if (key >= n - 1 && key < k1) {  // the token of this step
-        const size_t off = (size_t)m * D + c;
-        ka = *reinterpret_cast<const uint4 *>(k_rot + off); kb = *reinterpret_cast<const uint4 *>(k_rot + off + HALF);
-        va = *reinterpret_cast<const uint4 *>(v + off); vb = *reinterpret_cast<const uint4 *>(v + off + HALF);
-      }
-      *reinterpret_cast<uint4 *>(kd + c) = ka; *reinterpret_cast<uint4 *>(kd + c + HALF) = kb;
-      *reinterpret_cast<uint4 *>(vd + c) = va; *reinterpret_cast<uint4 *>(vd + c + HALF) = vb;
-    }
-  };
   // The retained keys and values were written by earlier steps: a first tile that does not reach
   // the token of this step is requested before the wait for this step's projection.
-  const bool early = !INT4 && NKT > 0 && k0 + DA_KT <= n - 1;
+  const bool early = NKT > 0 && k0 + DA_KT <= n - 1;
   if (early) load_kv(0, 0);
-  if (INT4 && NKT > 0) fetch_q4(0);   // (the token of this step is not among them: it is read in bf16, after the wait)
   pdl_wait();
   pdl_launch_dependents();  // the retaining head reads only what the projection wrote: it may run beside this kernel
-  if (INT4 && tok_k && split == 0 && hg == 0 && warp < 2) {
-    // The token of this step enters the 4-bit cache (this step still reads it in bf16): one warp
-    // quantises its pre-RoPE key, one its value, with the arithmetic of the chunk kernel.
-    const bf16 *src = (warp == 0 ? tok_k : tok_v) + (size_t)m * D;
-    float x0[2], x1[2], amax = 0.f;
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-      const int p = lane + 32 * k;
-      x0[k] = x1[k] = 0.f;
-      if (2 * p < D) {
-        const __nv_bfloat162 v2 = *reinterpret_cast<const __nv_bfloat162 *>(src + 2 * p);
-        x0[k] = __bfloat162float(v2.x);
-        x1[k] = __bfloat162float(v2.y);
-        amax = fmaxf(amax, fmaxf(fabsf(x0[k]), fabsf(x1[k])));
-      }
-    }
-    amax = warp_max(amax);
-    __half sh = __float2half_rn(__fdiv_rn(amax, 7.0f));
-    if (__half2float(sh) == 0.f) sh = __float2half_rn(1.0f);
-    const float sf = __half2float(sh);
-    const size_t u = (size_t)m * cap + (n - 1);
-    uint8_t *dst = (warp == 0 ? q4.kq : q4.vq) + u * (D / 2);
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-      const int p = lane + 32 * k;
-      if (2 * p < D) {
-        const int c0 = (int)fminf(fmaxf(rintf(__fdiv_rn(x0[k], sf)), -8.f), 7.f);
-        const int c1 = (int)fminf(fmaxf(rintf(__fdiv_rn(x1[k], sf)), -8.f), 7.f);
-        dst[p] = (uint8_t)((c0 & 0xF) | ((c1 & 0xF) << 4));
-      }
-    }
-    if (lane == 0) (warp == 0 ? q4.ks : q4.vs)[u] = sh;
-  }
   for (int x = tid; x < DA_G * VPR; x += DA_THREADS) {
     const int r = x / VPR, c = (x - r * VPR) * 8;
     cp_async16(sQ + r * LD + c, q_rot + (size_t)(h0 + min(r, gh - 1)) * D + c, r < gh);
   }
-  if (!INT4 && NKT > 0 && !early) load_kv(0, 0);
+  if (NKT > 0 && !early) load_kv(0, 0);
   cp_async_commit();
 
   uint32_t qf[D / 16][4];
@@ -489,15 +357,9 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
   float mrow[2] = {-INFINITY, -INFINITY}, lrow[2] = {0.f, 0.f};  // heads g4 and g4 + 8
 
   for (int kt = 0; kt < NKT; kt++) {
-    if (INT4) {
-      expand_q4(kt & 1, kt);   // (the other buffer may still be read by a slower warp)
-      if (kt + 1 < NKT) fetch_q4(kt + 1);
-      cp_async_wait<0>();
-    } else {
-      if (kt + 1 < NKT) load_kv((kt + 1) & 1, kt + 1);
-      cp_async_commit();
-      cp_async_wait<1>();
-    }
+    if (kt + 1 < NKT) load_kv((kt + 1) & 1, kt + 1);
+    cp_async_commit();
+    cp_async_wait<1>();
     __syncthreads();
     if (kt == 0) {
 #pragma unroll
@@ -576,9 +438,7 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
       mma_bf16_16816(o[2 * dn], pf, b0, b1);
       mma_bf16_16816(o[2 * dn + 1], pf, b2, b3);
     }
-    // bf16 cache: the next iteration's cp.async refills the buffer read here.  4-bit cache: the next
-    // expansion fills the other buffer, and the one after it comes behind the next iteration's barrier.
-    if (!INT4) __syncthreads();
+    __syncthreads();  // the next iteration's cp.async refills the buffer read here
   }
   cp_async_wait<0>();
 
@@ -674,6 +534,359 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
     o2.x = pack_bf16(acc.x * inv, acc.y * inv);
     o2.y = pack_bf16(acc.z * inv, acc.w * inv);
     *reinterpret_cast<uint2 *>(a.out + (size_t)(h0 + i) * D + c) = o2;
+  }
+}
+
+// ---- the same over a 4-bit cache.  What bounds it is not bytes (8.6 KB for 64 units of a head) but the work on them: codes to
+// floats, the rotation of every key at its own position, and the latency of the (cos, sin) rows that needs.  So nothing
+// passes through shared memory and no warp waits for another inside the loop: a warp takes 16 keys of every tile of 64, and a
+// lane expands and rotates exactly the elements that its operand fragments hold.  For that, keys are the m side of the
+// m16n8k16 tiles and the (up to eight) query heads the n side: S^T = K Q^T, O^T = V^T P^T, with an 8 x 8 transpose of
+// P between them.  The codes, scales and ranks of a warp's next 16 keys are on their way while it works on these.
+//   Which elements a step of a contraction takes, and in which order the keys stand, is free as long as both operands agree:
+// a step takes the lower or the upper elements of 16 rotation pairs (a lane: pairs 2 q, 2 q + 1 and the same + 8, so that
+// the four lanes of a row read whole sectors of its (cos, sin)); row r of S^T is key kr(r), and columns of O are dealt
+// to the lanes in runs of D / 8, so that a lane's value codes lie together.
+// Measured (span of the launch for four Llama layers, 6000 units each): 84 us with tiles expanded into shared memory by
+// threads that each took 16 elements of a key (4150 instructions a warp, conversions among them), 64 us this way.
+constexpr int DQ_G = 8;
+
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
+  uint32_t d;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+  return d;
+}
+// Code J of a word -> 16^J * code: the nibble (its sign bit flipped: code + 8) in the mantissa of 2^23, less 2^23 + 8 * 16^J;
+// exact.  (No conversion instruction: those have a fraction of the rate.)  Times scale / 16^J it is code * scale, rounded once.
+template <int J>
+__device__ __forceinline__ float q4_code(uint32_t w) {
+  return __uint_as_float((w & (0xFu << (4 * J))) ^ (0x4B000000u | (8u << (4 * J)))) - (8388608.f + (float)(8 << (4 * J)));
+}
+// four codes in bits 0-15
+__device__ __forceinline__ void q4_expand4(uint32_t w, float s, float (&x)[4]) {
+  x[0] = q4_code<0>(w) * s;
+  x[1] = q4_code<1>(w) * (s * 0x1p-4f);
+  x[2] = q4_code<2>(w) * (s * 0x1p-8f);
+  x[3] = q4_code<3>(w) * (s * 0x1p-12f);
+}
+
+template <int D, int NL>
+__global__ void __launch_bounds__(DA_THREADS, 2)
+attn_decode_q4_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ DecodeAttnBatchN<NL> batch) {
+  const int hgroups = (h / h_kv + DQ_G - 1) / DQ_G, layer = NL == 1 ? 0 : blockIdx.z / hgroups;
+  const DecodeAttnLayer &a = batch.l[layer];
+  const int cap = a.cap, n = a.n, n_splits = a.n_splits, ranked_len = a.ranked_len;
+  const Int4Half &q4 = a.q4;
+  constexpr int LF = D + 8, NW = D / 16;   // NW: words of a row's lower (or upper) codes
+  __shared__ __align__(16) float fo[4][DQ_G][LF];
+  __shared__ float wm[4][DQ_G], wl[4][DQ_G], sw[DQ_G][64], sinv[DQ_G];
+  __shared__ bool last;
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g4 = lane >> 2, q = lane & 3;
+  const int g = h / h_kv, m = blockIdx.x, split = blockIdx.y, hg = blockIdx.z - layer * hgroups;
+  if (NL > 1 && split >= n_splits) return;  // (layers of a batch may hold different numbers of keys)
+  const int h0 = m * g + hg * DQ_G, gh = min(DQ_G, g - hg * DQ_G);
+  const int per = (n + n_splits - 1) / n_splits, k0 = split * per, k1 = min(n, k0 + per);
+  const int NKT = k1 > k0 ? (k1 - k0 + DA_KT - 1) / DA_KT : 0;
+  // keys of this lane in its warp's 16: two rows of S^T (kr and 8 + kr), four columns of V^T
+  const int kr = (g4 >> 1) + 4 * (g4 & 1);
+
+  struct Tile {
+    uint32_t kw[2][2][NW];   // rows, lower / upper
+    uint32_t vw[4][2];       // (D / 8 codes: 16, 12 or 8)
+    float ks[2], vs[4];
+    int pos[2];
+  };
+  auto fetch = [&](int kt, Tile &t) {   // unit n - 1, the token of this step, is not in the codes
+    const int base = k0 + kt * DA_KT + warp * 16;
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+      const int key = base + 8 * r + kr;
+      const bool ok = key < min(k1, n - 1);
+      const size_t u = (size_t)m * cap + (ok ? key : 0);
+      t.ks[r] = ok ? __half2float(q4.ks[u]) : 0.f;
+      t.pos[r] = !ok ? 0 : (key < ranked_len ? a.rank[u] : key);
+#pragma unroll
+      for (int hf = 0; hf < 2; hf++) {
+        const uint8_t *c = q4.kq + u * (D / 2) + hf * (D / 4);
+        if constexpr (D == 96) {
+#pragma unroll
+          for (int i = 0; i < 3; i++) {
+            const uint2 v = ok ? *reinterpret_cast<const uint2 *>(c + 8 * i) : make_uint2(0, 0);
+            t.kw[r][hf][2 * i] = v.x; t.kw[r][hf][2 * i + 1] = v.y;
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < D / 64; i++) {
+            const uint4 v = ok ? *reinterpret_cast<const uint4 *>(c + 16 * i) : make_uint4(0, 0, 0, 0);
+            t.kw[r][hf][4 * i] = v.x; t.kw[r][hf][4 * i + 1] = v.y; t.kw[r][hf][4 * i + 2] = v.z; t.kw[r][hf][4 * i + 3] = v.w;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++) {   // the keys of S^T rows 2 q, 2 q + 1, 2 q + 8, 2 q + 9
+      const int key = base + q + 4 * i;
+      const bool ok = key < min(k1, n - 1);
+      const size_t u = (size_t)m * cap + (ok ? key : 0);
+      t.vs[i] = ok ? __half2float(q4.vs[u]) : 0.f;
+      const uint8_t *c = q4.vq + u * (D / 2) + (D / 16) * g4;
+      t.vw[i][0] = t.vw[i][1] = 0;
+      if (ok) {
+        if constexpr (D == 128) { const uint2 v = *reinterpret_cast<const uint2 *>(c); t.vw[i][0] = v.x; t.vw[i][1] = v.y; }
+        else if constexpr (D == 64) t.vw[i][0] = *reinterpret_cast<const uint32_t *>(c);
+        else {
+          const uint16_t *p = reinterpret_cast<const uint16_t *>(c);
+          t.vw[i][0] = (uint32_t)p[0] | ((uint32_t)p[1] << 16);
+          t.vw[i][1] = p[2];
+        }
+      }
+    }
+  };
+
+  Tile cur;
+  if (NKT > 0) fetch(0, cur);   // (written by earlier steps)
+  pdl_wait();
+  pdl_launch_dependents();  // the retaining head reads only what the projection wrote: it may run beside this kernel
+  if (a.tok_k && split == 0 && hg == 0 && warp < 2) {
+    // The token of this step enters the 4-bit cache (this step still reads it in bf16): one warp
+    // quantises its pre-RoPE key, one its value, with the arithmetic of the chunk kernel.
+    const bf16 *src = (warp == 0 ? a.tok_k : a.tok_v) + (size_t)m * D;
+    float x0[2], x1[2], amax = 0.f;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const int p = lane + 32 * k;
+      x0[k] = x1[k] = 0.f;
+      if (2 * p < D) {
+        const __nv_bfloat162 v2 = *reinterpret_cast<const __nv_bfloat162 *>(src + 2 * p);
+        x0[k] = __bfloat162float(v2.x);
+        x1[k] = __bfloat162float(v2.y);
+        amax = fmaxf(amax, fmaxf(fabsf(x0[k]), fabsf(x1[k])));
+      }
+    }
+    amax = warp_max(amax);
+    __half sh = __float2half_rn(__fdiv_rn(amax, 7.0f));
+    if (__half2float(sh) == 0.f) sh = __float2half_rn(1.0f);
+    const float sf = __half2float(sh);
+    const size_t u = (size_t)m * cap + (n - 1);
+    uint8_t *dst = (warp == 0 ? q4.kq : q4.vq) + u * (D / 2);
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const int p = lane + 32 * k;
+      if (2 * p < D) {
+        const int c0 = (int)fminf(fmaxf(rintf(__fdiv_rn(x0[k], sf)), -8.f), 7.f);
+        const int c1 = (int)fminf(fmaxf(rintf(__fdiv_rn(x1[k], sf)), -8.f), 7.f);
+        dst[p] = (uint8_t)((c0 & 0xF) | ((c1 & 0xF) << 4));
+      }
+    }
+    if (lane == 0) (warp == 0 ? q4.ks : q4.vs)[u] = sh;
+  }
+  uint32_t qf[D / 16][2];   // head g4
+  {
+    const bf16 *qrow = a.q_rot + (size_t)(h0 + min(g4, gh - 1)) * D + 2 * q;
+#pragma unroll
+    for (int kk = 0; kk < D / 16; kk++) {
+      const bf16 *src = qrow + (kk & 1) * (D / 2) + (kk >> 1) * 16;
+      qf[kk][0] = g4 < gh ? *reinterpret_cast<const uint32_t *>(src) : 0u;
+      qf[kk][1] = g4 < gh ? *reinterpret_cast<const uint32_t *>(src + 8) : 0u;
+    }
+  }
+  float o[D / 16][4];
+#pragma unroll
+  for (int i = 0; i < D / 16; i++)
+#pragma unroll
+    for (int e = 0; e < 4; e++) o[i][e] = 0.f;
+  float mrow[2] = {-INFINITY, -INFINITY}, lrow[2] = {0.f, 0.f};   // heads 2 q and 2 q + 1
+  const uint32_t sel = 0x4440u | (uint32_t)q;   // byte q of a word to bits 0-7, zeros elsewhere
+
+  for (int kt = 0; kt < NKT; kt++) {
+    const int base = k0 + kt * DA_KT + warp * 16;
+    if (base >= k1) break;
+    float4 cs4[2][D / 16];   // pairs 8 e + 2 q and the next
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+      const float4 *c = reinterpret_cast<const float4 *>(a.cs + (size_t)cur.pos[r] * (D / 2)) + q;
+#pragma unroll
+      for (int e = 0; e < D / 16; e++) cs4[r][e] = __ldg(c + 4 * e);
+    }
+    // values while the (cos, sin) rows are on their way: columns (D / 8) g4 + 2 i and the next are rows g4 and g4 + 8 of tile i
+    uint32_t va[D / 16][4];
+#pragma unroll
+    for (int hf = 0; hf < 2; hf++) {
+      float x[2][D / 8];
+#pragma unroll
+      for (int e = 0; e < 2; e++) {
+        const int key = base + q + 4 * (2 * hf + e);
+#pragma unroll
+        for (int b = 0; b < D / 32; b++) {
+          float y[4];
+          q4_expand4(cur.vw[2 * hf + e][b / 2] >> (16 * (b & 1)), cur.vs[2 * hf + e], y);
+#pragma unroll
+          for (int k = 0; k < 4; k++) x[e][4 * b + k] = y[k];
+        }
+        if (key == n - 1) {   // the token of this step
+          const uint32_t *tv = reinterpret_cast<const uint32_t *>(a.v + (size_t)m * D + (D / 8) * g4);
+#pragma unroll
+          for (int k = 0; k < D / 16; k++) {
+            const uint32_t v = tv[k];
+            x[e][2 * k] = __uint_as_float(v << 16);
+            x[e][2 * k + 1] = __uint_as_float(v & 0xffff0000u);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < D / 16; i++) {
+        va[i][2 * hf] = pack_bf16(x[0][2 * i], x[1][2 * i]);
+        va[i][2 * hf + 1] = pack_bf16(x[0][2 * i + 1], x[1][2 * i + 1]);
+      }
+    }
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int b = 0; b < D / 32; b++) {
+      uint32_t lo[4], hi[4];   // fragments of the lower and the upper elements of 16 rotation pairs
+#pragma unroll
+      for (int r = 0; r < 2; r++) {
+        float x1[4], x2[4];
+        const float s0 = cur.ks[r], s1 = s0 * 0x1p-4f;
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+          const uint32_t w1 = __byte_perm(cur.kw[r][0][2 * b + k], 0, sel), w2 = __byte_perm(cur.kw[r][1][2 * b + k], 0, sel);
+          x1[2 * k] = q4_code<0>(w1) * s0; x1[2 * k + 1] = q4_code<1>(w1) * s1;
+          x2[2 * k] = q4_code<0>(w2) * s0; x2[2 * k + 1] = q4_code<1>(w2) * s1;
+        }
+        const float4 c0 = cs4[r][2 * b], c1 = cs4[r][2 * b + 1];
+        const float cc[4] = {c0.x, c0.z, c1.x, c1.z}, sn[4] = {c0.y, c0.w, c1.y, c1.w};
+        float y1[4], y2[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          y1[k] = x1[k] * cc[k] - x2[k] * sn[k];
+          y2[k] = x2[k] * cc[k] + x1[k] * sn[k];
+        }
+        lo[r] = pack_bf16(y1[0], y1[1]); lo[r + 2] = pack_bf16(y1[2], y1[3]);
+        hi[r] = pack_bf16(y2[0], y2[1]); hi[r + 2] = pack_bf16(y2[2], y2[3]);
+        if (base + 8 * r + kr == n - 1) {
+          const uint32_t *tk = reinterpret_cast<const uint32_t *>(a.k_rot + (size_t)m * D + 16 * b + 2 * q);
+          lo[r] = tk[0]; lo[r + 2] = tk[4];
+          hi[r] = tk[D / 4]; hi[r + 2] = tk[D / 4 + 4];
+        }
+      }
+      mma_bf16_16816(s, lo, qf[2 * b][0], qf[2 * b][1]);
+      mma_bf16_16816(s, hi, qf[2 * b + 1][0], qf[2 * b + 1][1]);
+    }
+    if (kt + 1 < NKT) fetch(kt + 1, cur);
+    // online softmax of this warp's 16 keys (the keys past the split's end weigh nothing)
+    float alpha[2];
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      const float v0 = base + kr < k1 ? s[c] * scale_log2 : -INFINITY, v1 = base + 8 + kr < k1 ? s[c + 2] * scale_log2 : -INFINITY;
+      float tmax = fmaxf(v0, v1);
+      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
+      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 8));
+      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
+      const float mnew = fmaxf(mrow[c], tmax), muse = mnew == -INFINITY ? 0.f : mnew;
+      alpha[c] = exp2f(mrow[c] - muse);
+      mrow[c] = mnew;
+      s[c] = exp2f(v0 - muse);
+      s[c + 2] = exp2f(v1 - muse);
+      lrow[c] = lrow[c] * alpha[c] + (s[c] + s[c + 2]);
+    }
+#pragma unroll
+    for (int i = 0; i < D / 16; i++) {
+      o[i][0] *= alpha[0]; o[i][2] *= alpha[0];
+      o[i][1] *= alpha[1]; o[i][3] *= alpha[1];
+    }
+    const uint32_t pb0 = movmatrix_trans(pack_bf16(s[0], s[1])), pb1 = movmatrix_trans(pack_bf16(s[2], s[3]));
+#pragma unroll
+    for (int i = 0; i < D / 16; i++) mma_bf16_16816(o[i], va[i], pb0, pb1);
+  }
+
+  // ---- the four warps' states meet
+#pragma unroll
+  for (int c = 0; c < 2; c++) {
+    lrow[c] += __shfl_xor_sync(0xffffffffu, lrow[c], 4);
+    lrow[c] += __shfl_xor_sync(0xffffffffu, lrow[c], 8);
+    lrow[c] += __shfl_xor_sync(0xffffffffu, lrow[c], 16);
+    const int head = 2 * q + c;
+    if (head < gh) {
+      if (g4 == 0) { wm[warp][head] = mrow[c]; wl[warp][head] = lrow[c]; }
+      float *dst = fo[warp][head] + (D / 8) * g4;
+#pragma unroll
+      for (int i = 0; i < D / 16; i++) *reinterpret_cast<float2 *>(dst + 2 * i) = make_float2(o[i][c], o[i][c + 2]);
+    }
+  }
+  __syncthreads();
+  // partial result of this split: o [h][split][D] (not normalised), (m, l) [h][split][2]
+  for (int idx = tid; idx < gh * (D / 4); idx += DA_THREADS) {
+    const int i = idx / (D / 4), c = (idx - i * (D / 4)) * 4;
+    const float mx = fmaxf(fmaxf(wm[0][i], wm[1][i]), fmaxf(wm[2][i], wm[3][i])), muse = mx == -INFINITY ? 0.f : mx;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float lsum = 0.f;
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+      // (a warp without keys has sum 0; one whose scores are all NaN has no maximum, but a sum that says so)
+      const float wgt = wl[w][i] == 0.f ? 0.f : (wm[w][i] == -INFINITY ? 1.f : exp2f(wm[w][i] - muse));
+      if (wgt != 0.f) {
+        const float4 v = *reinterpret_cast<const float4 *>(&fo[w][i][c]);
+        acc.x = fmaf(wgt, v.x, acc.x); acc.y = fmaf(wgt, v.y, acc.y);
+        acc.z = fmaf(wgt, v.z, acc.z); acc.w = fmaf(wgt, v.w, acc.w);
+        lsum = fmaf(wgt, wl[w][i], lsum);
+      }
+    }
+    const size_t hs = (size_t)(h0 + i) * n_splits + split;
+    *reinterpret_cast<float4 *>(a.part_o + hs * D + c) = acc;
+    if (c == 0) *(reinterpret_cast<float2 *>(a.part_ml) + hs) = make_float2(mx, lsum);
+  }
+
+  // ---- the split that finishes last merges the partial results of all splits, in split order
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicInc(&a.counters[m * hgroups + hg], n_splits - 1) == (unsigned)(n_splits - 1);
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = warp; i < gh; i += 4) {   // weights of the splits, a warp per head
+    float ms[2], ls[2], mx = -INFINITY, lsum = 0.f;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const int s2 = lane + 32 * k;
+      const float2 ml = s2 < n_splits ? __ldcg(reinterpret_cast<const float2 *>(a.part_ml) + (size_t)(h0 + i) * n_splits + s2)
+                                      : make_float2(-INFINITY, 0.f);
+      ms[k] = ml.x; ls[k] = ml.y;
+      mx = fmaxf(mx, ml.x);
+    }
+    mx = warp_max(mx);
+    const float muse = mx == -INFINITY ? 0.f : mx;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const float w = ls[k] == 0.f ? 0.f : (ms[k] == -INFINITY ? 1.f : exp2f(ms[k] - muse));
+      if (w != 0.f) lsum = fmaf(w, ls[k], lsum);
+      sw[i][lane + 32 * k] = w;
+    }
+    lsum = warp_sum(lsum);
+    if (lane == 0) sinv[i] = 1.0f / lsum;
+  }
+  __syncthreads();
+  for (int idx = tid; idx < gh * (D / 4); idx += DA_THREADS) {   // sixteen splits in flight as 16-byte loads
+    const int i = idx / (D / 4), c = (idx - i * (D / 4)) * 4;
+    const float *po = a.part_o + (size_t)(h0 + i) * n_splits * D + c;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s2 = 0; s2 < n_splits; s2 += 16) {
+      float4 v[16];
+#pragma unroll
+      for (int k = 0; k < 16; k++)
+        v[k] = (s2 + k < n_splits) ? __ldcg(reinterpret_cast<const float4 *>(po + (size_t)(s2 + k) * D)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 16; k++) {
+        const float w = s2 + k < n_splits ? sw[i][s2 + k] : 0.f;
+        if (w != 0.f) {
+          acc.x = fmaf(w, v[k].x, acc.x); acc.y = fmaf(w, v[k].y, acc.y);
+          acc.z = fmaf(w, v[k].z, acc.z); acc.w = fmaf(w, v[k].w, acc.w);
+        }
+      }
+    }
+    const float inv = sinv[i];
+    *reinterpret_cast<uint2 *>(a.out + (size_t)(h0 + i) * D + c) =
+        make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
   }
 }
 
@@ -777,16 +990,15 @@ int decode_attn_splits(int h_kv, int n, bool int4) {
 
 cudaError_t launch_attention_decode(const DecodeAttnBatch &b, int n_layers, int h, int h_kv, int d, cudaStream_t st,
                                     bool pdl) {
-  const int hgroups = (h / h_kv + DA_G - 1) / DA_G;
-  if (n_layers < 1 || n_layers > DECODE_BATCH || h_kv * hgroups > 32 * 16) return cudaErrorInvalidValue;
+  const bool q4 = b.l[0].q4.kq != nullptr;
+  const int group = q4 ? DQ_G : DA_G, hgroups = (h / h_kv + group - 1) / group;
+  if (n_layers < 1 || n_layers > DECODE_BATCH || h_kv * hgroups > DECODE_HEAD_GROUPS) return cudaErrorInvalidValue;
   int splits = 1;
   for (int i = 0; i < n_layers; i++) splits = b.l[i].n_splits > splits ? b.l[i].n_splits : splits;
   if (splits > 64) return cudaErrorInvalidValue;
   const dim3 grid(h_kv, splits, n_layers * hgroups);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)d);
-  const bool q4 = b.l[0].q4.kq != nullptr;
-  auto run = [&](auto kern1, auto kern_n, PerDeviceFlag (&attr_set)[2]) -> cudaError_t {
-    const size_t smem = (DA_G + 4 * DA_KT) * (d + 8) * 2;
+  auto run = [&](auto kern1, auto kern_n, size_t smem, PerDeviceFlag (&attr_set)[2]) -> cudaError_t {
     if (n_layers > 1) {
       if (cudaError_t e = allow_dynamic_smem(kern_n, (int)smem, attr_set[1]); e != cudaSuccess) return e;
       return launch_kernel(kern_n, grid, dim3(DA_THREADS), smem, st, pdl, h, h_kv, scale_log2, b);
@@ -797,8 +1009,8 @@ cudaError_t launch_attention_decode(const DecodeAttnBatch &b, int n_layers, int 
   auto launch = [&](auto dim) -> cudaError_t {
     constexpr int D = decltype(dim)::value;
     static PerDeviceFlag set_q4[2], set_bf16[2];
-    return q4 ? run(attn_decode_kernel<D, true, 1>, attn_decode_kernel<D, true, DECODE_BATCH>, set_q4)
-              : run(attn_decode_kernel<D, false, 1>, attn_decode_kernel<D, false, DECODE_BATCH>, set_bf16);
+    return q4 ? run(attn_decode_q4_kernel<D, 1>, attn_decode_q4_kernel<D, DECODE_BATCH>, 0, set_q4)
+              : run(attn_decode_kernel<D, 1>, attn_decode_kernel<D, DECODE_BATCH>, (DA_G + 4 * DA_KT) * (d + 8) * 2, set_bf16);
   };
   switch (d) {
     case 64: return launch(std::integral_constant<int, 64>{});

@@ -78,7 +78,7 @@ bool grow(T **p, size_t *have, size_t want, cudaStream_t st) {
 }
 
 struct TimedEvent { cudaEvent_t a, b; int kind; };
-constexpr int DEC_CNT_WORDS = 1 + 32 * 16;  // retaining head + (KV head, head group) pairs
+constexpr int DEC_CNT_WORDS = 1 + DECODE_HEAD_GROUPS;  // retaining head + (KV head, head group) pairs
 
 }  // namespace
 
