@@ -80,6 +80,8 @@ bool grow(T **p, size_t *have, size_t want, cudaStream_t st) {
 struct TimedEvent { cudaEvent_t a, b; int kind; };
 constexpr int DEC_CNT_WORDS = 1 + DECODE_HEAD_GROUPS;  // retaining head + (KV head, head group) pairs
 
+constexpr size_t LAYER_COUNTER_BYTES = 2 * sizeof(unsigned long long) + 32 * sizeof(unsigned);
+
 }  // namespace
 
 struct locret_layer {
@@ -105,7 +107,7 @@ struct locret_layer {
   // then differ from head to head; `len` is the largest length
   bool per_head;
   PerHead budget_m, len_m, ranked_m, rcur_m;
-  unsigned long long *d_counters;  // [2]: units moved to another slot, rotated keys rewritten
+  unsigned long long *d_counters;  // [2]: units moved to another slot, rotated keys rewritten; behind them a word per KV head (launch_evict_one)
   int device;  // the device that was current at create: every later call must find it current
   const float2 *cs;
   int *d_status;
@@ -399,7 +401,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
   ok = ok && cudaMalloc(&L->s, sc_b) == cudaSuccess;
   ok = ok && cudaMalloc(&L->tid, td_b) == cudaSuccess;
   for (int i = 0; i < 2; i++) ok = ok && cudaMalloc(&L->rank[i], rk_b) == cudaSuccess;
-  ok = ok && cudaMalloc(&L->d_counters, 2 * sizeof(unsigned long long)) == cudaSuccess;
+  ok = ok && cudaMalloc(&L->d_counters, LAYER_COUNTER_BYTES) == cudaSuccess;
   ok = ok && cudaMalloc(&L->d_status, 4 * sizeof(int)) == cudaSuccess;
   if (!ok) { cudaGetLastError(); free_layer_memory(L); delete L; return LOCRET_ERR_ALLOC; }
 
@@ -491,7 +493,7 @@ int locret_create(const locret_layer_cfg *cfg, int32_t budget, int32_t chunk, in
   if (e == cudaSuccess) e = cudaMemsetAsync(L->s, 0, sc_b, L->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(L->tid, 0, td_b, L->st);
   for (int i = 0; i < 2 && e == cudaSuccess; i++) e = cudaMemsetAsync(L->rank[i], 0, rk_b, L->st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L->d_counters, 0, 2 * sizeof(unsigned long long), L->st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L->d_counters, 0, LAYER_COUNTER_BYTES, L->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(L->d_status, 0, 4 * sizeof(int), L->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(L->st);
   if (e != cudaSuccess) {
@@ -525,33 +527,38 @@ int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaS
   }
   if (evicts) {
     const int n_prot = (flags & LOCRET_LAST_CHUNK) ? 0 : (L->n_stab < n ? L->n_stab : n);
-    {
+    // (n_prefix + n_stab <= budget < n, so the prefix never reaches into the protected tail)
+    TopkArgs sel;
+    sel.scores = L->s; sel.rank[0] = L->rank[0]; sel.rank[1] = L->rank[1]; sel.rcur = L->rcur;
+    sel.stride = L->cap; sel.ranked_len = L->ranked_len;
+    sel.n = n; sel.budget = L->budget; sel.n_prot = n_prot; sel.n_pre = L->n_prefix;
+    sel.src_of = P->keep; sel.src_stride = L->budget; sel.counters = L->d_counters;
+    sel.per_head = L->per_head ? 1 : 0;
+    sel.n_m = n_m; sel.budget_m = L->budget_m; sel.nprot_m = nprot_m; sel.ranked_m = L->ranked_m; sel.rcur_m = L->rcur_m;
+    CompactArgs mv;
+    mv.k = L->k_pre; mv.v = L->v; mv.k_rot = L->k_rot; mv.s = L->s; mv.t = L->tid;
+    mv.src_of = P->keep; mv.src_stride = L->budget; mv.rank[0] = L->rank[0]; mv.rank[1] = L->rank[1]; mv.rcur = L->rcur;
+    mv.cs = L->cs;
+    mv.h_kv = L->h_kv; mv.d = L->d; mv.cap = L->cap; mv.budget = L->budget; mv.ranked_len = L->ranked_len;
+    mv.per_head = L->per_head ? 1 : 0;
+    mv.budget_m = L->budget_m; mv.ranked_m = L->ranked_m; mv.rcur_m = L->rcur_m; mv.evict_m = evict_m;
+    // (on the second stream the selection runs beside attention and only the gather waits for it)
+    const bool one = !side && !L->int4 && !L->per_head && n == L->budget + 1;
+    if (one) {
+      Timed t(L, LOCRET_K_COMPACT, S);
+      CK(launch_evict_one(sel, mv, reinterpret_cast<unsigned *>(L->d_counters + 2), S, pdl));
+    } else {
       Timed t(L, LOCRET_K_TOPK, S);
-      // (n_prefix + n_stab <= budget < n, so the prefix never reaches into the protected tail)
-      TopkArgs a;
-      a.scores = L->s; a.rank[0] = L->rank[0]; a.rank[1] = L->rank[1]; a.rcur = L->rcur;
-      a.stride = L->cap; a.ranked_len = L->ranked_len;
-      a.n = n; a.budget = L->budget; a.n_prot = n_prot; a.n_pre = L->n_prefix;
-      a.src_of = P->keep; a.src_stride = L->budget; a.counters = L->d_counters;
-      a.per_head = L->per_head ? 1 : 0;
-      a.n_m = n_m; a.budget_m = L->budget_m; a.nprot_m = nprot_m; a.ranked_m = L->ranked_m; a.rcur_m = L->rcur_m;
-      CK(launch_topk(a, L->h_kv, S, pdl));
+      CK(launch_topk(sel, L->h_kv, S, pdl));
     }
     // the gather rewrites keys and values that the attention kernel reads
     if (side) CK(cudaStreamWaitEvent(S, L->ev_attn, 0));
     if (L->int4) {
       Timed t(L, LOCRET_K_COMPACT, S);
       CK(launch_compact_int4(L->q4, L->s, L->tid, P->keep, L->h_kv, L->d, L->cap, L->budget, S));
-    } else {
+    } else if (!one) {
       Timed t(L, LOCRET_K_COMPACT, S);
-      CompactArgs a;
-      a.k = L->k_pre; a.v = L->v; a.k_rot = L->k_rot; a.s = L->s; a.t = L->tid;
-      a.src_of = P->keep; a.src_stride = L->budget; a.rank[0] = L->rank[0]; a.rank[1] = L->rank[1]; a.rcur = L->rcur;
-      a.cs = L->cs;
-      a.h_kv = L->h_kv; a.d = L->d; a.cap = L->cap; a.budget = L->budget; a.ranked_len = L->ranked_len;
-      a.per_head = L->per_head ? 1 : 0;
-      a.budget_m = L->budget_m; a.ranked_m = L->ranked_m; a.rcur_m = L->rcur_m; a.evict_m = evict_m;
-      CK(launch_compact(a, S, pdl));
+      CK(launch_compact(mv, S, pdl));
     }
   }
   if (L->per_head) {
