@@ -348,7 +348,7 @@ struct DecodeAttnLayer {
 };
 template <int N> struct DecodeAttnBatchN { DecodeAttnLayer l[N]; };
 typedef DecodeAttnBatchN<DECODE_BATCH> DecodeAttnBatch;
-int decode_attn_splits(int h_kv, int n, bool int4);
+int decode_attn_splits(int h_kv, int n);
 cudaError_t launch_attention_decode(const DecodeAttnBatch &b, int n_layers, int h, int h_kv, int d, cudaStream_t st, bool pdl);
 
 // dst[c][r] = src[r][c]  (weight repack at create)

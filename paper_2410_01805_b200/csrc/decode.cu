@@ -985,14 +985,14 @@ cudaError_t launch_rh_gemv(const RhGemvBatch &b, int n_layers, int d_R, int K, i
 // Splits of the key range per KV head.  Measured at the Llama shape (8 KV heads, 6000 keys, 256 steps through
 // 32 layers): with a bf16 cache 64 / 96 / 120 / 148 / 200 / 296 / 444 CTAs in total give 914 / 1058 / 1130 /
 // 1152 / 1224 / 1133 / 1052 tokens/s (more splits shorten each CTA's chain of tiles, but the last split of a
-// head merges them all); a 4-bit cache, whose CTAs also expand and rotate the codes (and load a tile's codes
-// without overlapping the previous tile's arithmetic), wants more: 96 / 148 / 296 / 444 CTAs give 501 / 639 /
-// 825 / 700 tokens/s.
-int decode_attn_splits(int h_kv, int n, bool int4) {
+// head merges them all).  With a 4-bit cache 100 / 148 / 200 / 296 / 400 CTAs take 93.2 / 94.5 / 88.1 / 99.8 / 97.5 us a step of
+// four such layers, 34.7 / 28.5 / 28.4 / 28.0 / 30.7 us of one, and at the Phi-3 shape (32 KV heads of 96) 171 / 187 / 181 / 179 /
+// 177 and 63.7 / 55.5 / 53.5 / 56.2 / 50.9 us.
+int decode_attn_splits(int h_kv, int n) {
   static int forced = -1;
   if (forced < 0) { const char *e = getenv("LOCRET_DEC_CTAS"); forced = e ? atoi(e) : 0; if (forced < 0 || forced > 2048) forced = 0; }
   const int sms = sm_count_of_current_device();
-  const int total = forced ? forced : (int4 ? 2 * sms : (sms * 27) / 20);
+  const int total = forced ? forced : (sms * 27) / 20;
   int s = (total + h_kv - 1) / h_kv;
   const int max_s = (n + 127) / 128;            // at least one 128-key tile per split
   if (s > max_s) s = max_s;

@@ -649,7 +649,7 @@ int token_step(locret_layer *const *layers, int count, const void *hidden_in, ui
     al.cs = L->cs; al.rank = L->rank[L->rcur]; al.ranked_len = L->ranked_len;
     al.tok_k = L->int4 ? staging + (size_t)L->h * L->d : nullptr;
     al.tok_v = L->int4 ? staging + (size_t)(L->h + L->h_kv) * L->d : nullptr;
-    al.cap = L->cap; al.n = n; al.n_splits = decode_attn_splits(L->h_kv, n, L->int4);
+    al.cap = L->cap; al.n = n; al.n_splits = decode_attn_splits(L->h_kv, n);
     RhGemvLayer &rl = rh.l[i];
     rl.z = z_post ? z_post : staging; rl.W1t = L->w1_t; rl.W2 = L->w2f;
     rl.partial = ds.dec_partial + i * ds.partial; rl.score_out = L->s + L->len; rl.score_stride = L->cap;
