@@ -244,20 +244,26 @@ gemv_rope_wide_kernel(const bf16 *__restrict__ x, int K, int n_layers, const __g
   const uint4 xv = act ? __ldg(reinterpret_cast<const uint4 *>(x) + tid) : make_uint4(0, 0, 0, 0);
   int par = 0;
   for (int p0 = p_lo; p0 < p_hi; p0 += GW_PB, par ^= 1) {
-    // Dot products by m16n8k16 tiles: eight groups of four lanes hold eight slices of both rows (rows g and g + 8 of A) and of x
-    // (column g of B), so a slice's sum is on the diagonal, in one lane of its group.  Two instructions for a pair of
-    // rows instead of some fifty: the next batch is requested that much sooner after this one's arrival (four Llama
-    // layers: 48.5 us of launch span, 44.9 this way; a step 82 / 78.5).
+    // dot8 of both rows of a pair at a time: the same rounded sums in half the FMAs, and x is converted once per batch.  What counts
+    // is how soon after a batch's arrival the next one is requested (four Llama layers of 200 units, a step: 59.4 us row by
+    // row, 55.4 in pairs, 55.1 by m16n8k16 tiles; but those truncate their sums, which came out 3e-8 of them too small).
     float v[2 * GW_PB];
+    {
+      uint64_t s[GW_PB] = {};
+      const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
-    for (int j = 0; j < GW_PB; j++) {
-      const uint4 &wa = w[2 * j], &wb = w[2 * j + 1];
-      float c[4] = {0.f, 0.f, 0.f, 0.f};
-      { const uint32_t f[4] = {wa.x, wb.x, wa.y, wb.y}; mma_bf16_16816(c, f, xv.x, xv.y); }
-      { const uint32_t f[4] = {wa.z, wb.z, wa.w, wb.w}; mma_bf16_16816(c, f, xv.z, xv.w); }
-      const bool own = (lane >> 3) == (lane & 3), odd = lane & 4;
-      v[2 * j] = own ? (odd ? c[1] : c[0]) : 0.f;
-      v[2 * j + 1] = own ? (odd ? c[3] : c[2]) : 0.f;
+      for (int i = 0; i < 4; i++) {
+        const float x0 = __uint_as_float(xw[i] << 16), x1 = __uint_as_float(xw[i] & 0xffff0000u);
+        const uint64_t xx0 = pack_f32x2(x0, x0), xx1 = pack_f32x2(x1, x1);
+#pragma unroll
+        for (int j = 0; j < GW_PB; j++) {
+          const uint32_t wa = reinterpret_cast<const uint32_t *>(&w[2 * j])[i], wb = reinterpret_cast<const uint32_t *>(&w[2 * j + 1])[i];
+          s[j] = fma_f32x2(pack_f32x2(__uint_as_float(wa << 16), __uint_as_float(wb << 16)), xx0, s[j]);
+          s[j] = fma_f32x2(pack_f32x2(__uint_as_float(wa & 0xffff0000u), __uint_as_float(wb & 0xffff0000u)), xx1, s[j]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < GW_PB; j++) unpack_f32x2(s[j], v[2 * j], v[2 * j + 1]);
     }
     if (p0 + GW_PB < p_hi) load_batch(p0 + GW_PB);  // in flight during the reduction
     // eight values across 32 lanes: exchange half of them at each of three steps
