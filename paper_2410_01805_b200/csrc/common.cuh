@@ -349,9 +349,9 @@ typedef RhGemvBatchN<DECODE_BATCH> RhGemvBatch;
 int rh_gemv_blocks(int d_R);
 cudaError_t launch_rh_gemv(const RhGemvBatch &b, int n_layers, int d_R, int K, int h_kv, int act, cudaStream_t st, bool pdl);
 // attention.  part_o: fp32 [h][n_splits][d]; part_ml: fp32 [h][n_splits][2]; counters: one zeroed word per
-// (KV head, group of 16 query heads; of eight with a 4-bit cache), left at zero (the last split merges the partial results).
+// (KV head, group of 16 query heads; of eight or 16 with a 4-bit cache), left at zero (the last split merges the partial results).
 // q4.kq != nullptr (in all layers of a batch or none): keys [0, n - 1) are read from the 4-bit cache (expanded and rotated
-// with `cs` on the way into shared memory, at position rank[m * cap + slot] for slot < ranked_len and slot above) and only
+// with `cs` in the operand fragments, at position rank[m * cap + slot] for slot < ranked_len and slot above) and only
 // key n - 1, the token of this step, from k_rot / v, which then hold just that unit, [h_kv][d].  tok_k / tok_v (4-bit
 // cache only, may be null): the token's pre-RoPE keys and values [h_kv][d], which the kernel quantises into
 // slot n - 1 of the cache.

@@ -559,7 +559,7 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
 // floats, the rotation of every key at its own position, and the latency of the (cos, sin) rows that needs.  So nothing
 // passes through shared memory and no warp waits for another inside the loop: a warp takes 16 keys of every tile of 64, and a
 // lane expands and rotates exactly the elements that its operand fragments hold.  For that, keys are the m side of the
-// m16n8k16 tiles and the (up to eight) query heads the n side: S^T = K Q^T, O^T = V^T P^T, with an 8 x 8 transpose of
+// m16n8k16 tiles and the query heads the n side (NT tiles of eight): S^T = K Q^T, O^T = V^T P^T, with an 8 x 8 transpose of
 // P between them.  The codes, scales and ranks of a warp's next 16 keys are on their way while it works on these.
 //   Which elements a step of a contraction takes, and in which order the keys stand, is free as long as both operands agree:
 // a step takes the lower or the upper elements of 16 rotation pairs (a lane: pairs 2 q, 2 q + 1 and the same + 8, so that
@@ -567,8 +567,6 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
 // to the lanes in runs of D / 8, so that a lane's value codes lie together.
 // Measured (span of the launch for four Llama layers, 6000 units each): 84 us with tiles expanded into shared memory by
 // threads that each took 16 elements of a key (4150 instructions a warp, conversions among them), 64 us this way.
-constexpr int DQ_G = 8;
-
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
   uint32_t d;
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
@@ -588,22 +586,24 @@ __device__ __forceinline__ void q4_expand4(uint32_t w, float s, float (&x)[4]) {
   x[3] = q4_code<3>(w) * (s * 0x1p-12f);
 }
 
-template <int D, int NL>
+template <int D, int NL, int NT>
 __global__ void __launch_bounds__(DA_THREADS, 2)
 attn_decode_q4_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ DecodeAttnBatchN<NL> batch) {
-  const int hgroups = (h / h_kv + DQ_G - 1) / DQ_G, layer = NL == 1 ? 0 : blockIdx.z / hgroups;
+  constexpr int G = 8 * NT;
+  const int hgroups = (h / h_kv + G - 1) / G, layer = NL == 1 ? 0 : blockIdx.z / hgroups;
   const DecodeAttnLayer &a = batch.l[layer];
   const int cap = a.cap, n = a.n, n_splits = a.n_splits, ranked_len = a.ranked_len;
   const Int4Half &q4 = a.q4;
   constexpr int LF = D + 8, NW = D / 16;   // NW: words of a row's lower (or upper) codes
-  __shared__ __align__(16) float fo[4][DQ_G][LF];
-  __shared__ float wm[4][DQ_G], wl[4][DQ_G], sw[DQ_G][64], sinv[DQ_G];
+  __shared__ __align__(16) float fo[4][G][LF];
+  __shared__ float wm[4][G], wl[4][G], sw[G][64], sinv[G];
+  __shared__ uint2 sq[NT > 1 ? D / 16 * NT : 1][32];   // two tiles: fragments of the queries, for which no registers are left
   __shared__ bool last;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g4 = lane >> 2, q = lane & 3;
   const int g = h / h_kv, m = blockIdx.x, split = blockIdx.y, hg = blockIdx.z - layer * hgroups;
   if (NL > 1 && split >= n_splits) return;  // (layers of a batch may hold different numbers of keys)
-  const int h0 = m * g + hg * DQ_G, gh = min(DQ_G, g - hg * DQ_G);
+  const int h0 = m * g + hg * G, gh = min(G, g - hg * G);
   const int per = (n + n_splits - 1) / n_splits, k0 = split * per, k1 = min(n, k0 + per);
   const int NKT = k1 > k0 ? (k1 - k0 + DA_KT - 1) / DA_KT : 0;
   // keys of this lane in its warp's 16: two rows of S^T (kr and 8 + kr), four columns of V^T
@@ -699,22 +699,34 @@ attn_decode_q4_kernel(int h, int h_kv, float scale_log2, const __grid_constant__
     }
     if (lane == 0) (warp == 0 ? q4.ks : q4.vs)[u] = sh;
   }
-  uint32_t qf[D / 16][2];   // head g4
-  {
-    const bf16 *qrow = a.q_rot + (size_t)(h0 + min(g4, gh - 1)) * D + 2 * q;
+  uint2 qf[NT > 1 ? 1 : D / 16];   // heads g4, g4 + 8
+  auto load_q = [&](int kk, int t) -> uint2 {
+    const int head = 8 * t + g4;
+    const bf16 *src = a.q_rot + (size_t)(h0 + min(head, gh - 1)) * D + 2 * q + (kk & 1) * (D / 2) + (kk >> 1) * 16;
+    return head < gh ? make_uint2(*reinterpret_cast<const uint32_t *>(src), *reinterpret_cast<const uint32_t *>(src + 8))
+                     : make_uint2(0u, 0u);
+  };
+  if constexpr (NT > 1) {
+    for (int i = warp; i < D / 16 * NT; i += DA_THREADS / 32) sq[i][lane] = load_q(i / NT, i % NT);
+    __syncthreads();
+  } else {
 #pragma unroll
-    for (int kk = 0; kk < D / 16; kk++) {
-      const bf16 *src = qrow + (kk & 1) * (D / 2) + (kk >> 1) * 16;
-      qf[kk][0] = g4 < gh ? *reinterpret_cast<const uint32_t *>(src) : 0u;
-      qf[kk][1] = g4 < gh ? *reinterpret_cast<const uint32_t *>(src + 8) : 0u;
-    }
+    for (int kk = 0; kk < D / 16; kk++) qf[kk] = load_q(kk, 0);
   }
-  float o[D / 16][4];
+  auto q_frag = [&](int kk, int t) -> uint2 {
+    if constexpr (NT > 1) return sq[kk * NT + t][lane];
+    else return qf[kk];
+  };
+  float o[NT][D / 16][4], mrow[NT][2], lrow[NT][2];   // heads 8 t + 2 q and the next
 #pragma unroll
-  for (int i = 0; i < D / 16; i++)
+  for (int t = 0; t < NT; t++) {
 #pragma unroll
-    for (int e = 0; e < 4; e++) o[i][e] = 0.f;
-  float mrow[2] = {-INFINITY, -INFINITY}, lrow[2] = {0.f, 0.f};   // heads 2 q and 2 q + 1
+    for (int i = 0; i < D / 16; i++)
+#pragma unroll
+      for (int e = 0; e < 4; e++) o[t][i][e] = 0.f;
+    mrow[t][0] = mrow[t][1] = -INFINITY;
+    lrow[t][0] = lrow[t][1] = 0.f;
+  }
   const uint32_t sel = 0x4440u | (uint32_t)q;   // byte q of a word to bits 0-7, zeros elsewhere
 
   for (int kt = 0; kt < NKT; kt++) {
@@ -758,7 +770,7 @@ attn_decode_q4_kernel(int h, int h_kv, float scale_log2, const __grid_constant__
         va[i][2 * hf + 1] = pack_bf16(x[0][2 * i + 1], x[1][2 * i + 1]);
       }
     }
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    float s[NT][4] = {};
 #pragma unroll
     for (int b = 0; b < D / 32; b++) {
       uint32_t lo[4], hi[4];   // fragments of the lower and the upper elements of 16 rotation pairs
@@ -788,48 +800,59 @@ attn_decode_q4_kernel(int h, int h_kv, float scale_log2, const __grid_constant__
           hi[r] = tk[D / 4]; hi[r + 2] = tk[D / 4 + 4];
         }
       }
-      mma_bf16_16816(s, lo, qf[2 * b][0], qf[2 * b][1]);
-      mma_bf16_16816(s, hi, qf[2 * b + 1][0], qf[2 * b + 1][1]);
+#pragma unroll
+      for (int t = 0; t < NT; t++) {
+        const uint2 ql = q_frag(2 * b, t), qh = q_frag(2 * b + 1, t);
+        mma_bf16_16816(s[t], lo, ql.x, ql.y);
+        mma_bf16_16816(s[t], hi, qh.x, qh.y);
+      }
     }
     if (kt + 1 < NKT) fetch(kt + 1, cur);
     // online softmax of this warp's 16 keys (the keys past the split's end weigh nothing)
-    float alpha[2];
 #pragma unroll
-    for (int c = 0; c < 2; c++) {
-      const float v0 = base + kr < k1 ? s[c] * scale_log2 : -INFINITY, v1 = base + 8 + kr < k1 ? s[c + 2] * scale_log2 : -INFINITY;
-      float tmax = fmaxf(v0, v1);
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 8));
-      tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
-      const float mnew = fmaxf(mrow[c], tmax), muse = mnew == -INFINITY ? 0.f : mnew;
-      alpha[c] = exp2f(mrow[c] - muse);
-      mrow[c] = mnew;
-      s[c] = exp2f(v0 - muse);
-      s[c + 2] = exp2f(v1 - muse);
-      lrow[c] = lrow[c] * alpha[c] + (s[c] + s[c + 2]);
+    for (int t = 0; t < NT; t++) {
+      float alpha[2];
+#pragma unroll
+      for (int c = 0; c < 2; c++) {
+        const float v0 = base + kr < k1 ? s[t][c] * scale_log2 : -INFINITY, v1 = base + 8 + kr < k1 ? s[t][c + 2] * scale_log2 : -INFINITY;
+        float tmax = fmaxf(v0, v1);
+        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 4));
+        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 8));
+        tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 16));
+        const float mnew = fmaxf(mrow[t][c], tmax), muse = mnew == -INFINITY ? 0.f : mnew;
+        alpha[c] = exp2f(mrow[t][c] - muse);
+        mrow[t][c] = mnew;
+        s[t][c] = exp2f(v0 - muse);
+        s[t][c + 2] = exp2f(v1 - muse);
+        lrow[t][c] = lrow[t][c] * alpha[c] + (s[t][c] + s[t][c + 2]);
+      }
+#pragma unroll
+      for (int i = 0; i < D / 16; i++) {
+        o[t][i][0] *= alpha[0]; o[t][i][2] *= alpha[0];
+        o[t][i][1] *= alpha[1]; o[t][i][3] *= alpha[1];
+      }
+      const uint32_t pb0 = movmatrix_trans(pack_bf16(s[t][0], s[t][1])), pb1 = movmatrix_trans(pack_bf16(s[t][2], s[t][3]));
+#pragma unroll
+      for (int i = 0; i < D / 16; i++) mma_bf16_16816(o[t][i], va[i], pb0, pb1);
     }
-#pragma unroll
-    for (int i = 0; i < D / 16; i++) {
-      o[i][0] *= alpha[0]; o[i][2] *= alpha[0];
-      o[i][1] *= alpha[1]; o[i][3] *= alpha[1];
-    }
-    const uint32_t pb0 = movmatrix_trans(pack_bf16(s[0], s[1])), pb1 = movmatrix_trans(pack_bf16(s[2], s[3]));
-#pragma unroll
-    for (int i = 0; i < D / 16; i++) mma_bf16_16816(o[i], va[i], pb0, pb1);
   }
 
   // ---- the four warps' states meet
 #pragma unroll
-  for (int c = 0; c < 2; c++) {
-    lrow[c] += __shfl_xor_sync(0xffffffffu, lrow[c], 4);
-    lrow[c] += __shfl_xor_sync(0xffffffffu, lrow[c], 8);
-    lrow[c] += __shfl_xor_sync(0xffffffffu, lrow[c], 16);
-    const int head = 2 * q + c;
-    if (head < gh) {
-      if (g4 == 0) { wm[warp][head] = mrow[c]; wl[warp][head] = lrow[c]; }
-      float *dst = fo[warp][head] + (D / 8) * g4;
+  for (int t = 0; t < NT; t++) {
 #pragma unroll
-      for (int i = 0; i < D / 16; i++) *reinterpret_cast<float2 *>(dst + 2 * i) = make_float2(o[i][c], o[i][c + 2]);
+    for (int c = 0; c < 2; c++) {
+      float l = lrow[t][c];
+      l += __shfl_xor_sync(0xffffffffu, l, 4);
+      l += __shfl_xor_sync(0xffffffffu, l, 8);
+      l += __shfl_xor_sync(0xffffffffu, l, 16);
+      const int head = 8 * t + 2 * q + c;
+      if (head < gh) {
+        if (g4 == 0) { wm[warp][head] = mrow[t][c]; wl[warp][head] = l; }
+        float *dst = fo[warp][head] + (D / 8) * g4;
+#pragma unroll
+        for (int i = 0; i < D / 16; i++) *reinterpret_cast<float2 *>(dst + 2 * i) = make_float2(o[t][i][c], o[t][i][c + 2]);
+      }
     }
   }
   __syncthreads();
@@ -1006,13 +1029,31 @@ int decode_attn_splits(int h_kv, int n) {
   return s < 1 ? 1 : s;
 }
 
+// Query heads that a block of the 4-bit kernel serves.  Sixteen: the keys of a larger group are expanded and rotated for half as
+// many blocks; eight: twice the blocks, each with half the heads to merge at the end.  The first pays where the blocks of eight
+// (of which two fit an SM, three of head_dim 64) would take more than one wave and there are keys enough (tiles: 64 units of
+// one KV head, of all layers of the launch).  Measured (us a step, eight / sixteen): 16 heads a KV head, head_dim 128, 6000
+// units, on one KV head 19.2 / 27.7 (94 tiles), on two 55.9 / 59.7 in four layers (752) and 102.3 / 94.6 in eight (1504), on
+// four, 15000 units 46.8 / 45.6 (940), on eight, 16000 units 75.4 / 60.2 (2000); head_dim 64, on four, 15000 units 24.0 / 27.7 (400
+// blocks of eight), on 32 (nine heads each), 2000 units 44.4 / 39.4 (448).
+static int q4_heads_per_block(int g, int d, int tiles, int blocks_of_eight) {
+  const int sms = sm_count_of_current_device();
+  return g > 8 && tiles > 6 * sms && blocks_of_eight > (d == 64 ? 3 : 2) * sms ? 16 : 8;
+}
+
 cudaError_t launch_attention_decode(const DecodeAttnBatch &b, int n_layers, int h, int h_kv, int d, cudaStream_t st,
                                     bool pdl) {
   const bool q4 = b.l[0].q4.kq != nullptr;
-  const int group = q4 ? DQ_G : DA_G, hgroups = (h / h_kv + group - 1) / group;
-  if (n_layers < 1 || n_layers > DECODE_BATCH || h_kv * hgroups > DECODE_HEAD_GROUPS) return cudaErrorInvalidValue;
-  int splits = 1;
-  for (int i = 0; i < n_layers; i++) splits = b.l[i].n_splits > splits ? b.l[i].n_splits : splits;
+  if (n_layers < 1 || n_layers > DECODE_BATCH) return cudaErrorInvalidValue;
+  const int g = h / h_kv;
+  int splits = 1, tiles = 0, blocks_of_eight = 0;
+  for (int i = 0; i < n_layers; i++) {
+    splits = b.l[i].n_splits > splits ? b.l[i].n_splits : splits;
+    tiles += h_kv * ((b.l[i].n + DA_KT - 1) / DA_KT);
+    blocks_of_eight += h_kv * b.l[i].n_splits * ((g + 7) / 8);
+  }
+  const int group = q4 ? q4_heads_per_block(g, d, tiles, blocks_of_eight) : DA_G, hgroups = (g + group - 1) / group;
+  if (h_kv * hgroups > DECODE_HEAD_GROUPS) return cudaErrorInvalidValue;
   if (splits > 64) return cudaErrorInvalidValue;
   const dim3 grid(h_kv, splits, n_layers * hgroups);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)d);
@@ -1026,8 +1067,9 @@ cudaError_t launch_attention_decode(const DecodeAttnBatch &b, int n_layers, int 
   };
   auto launch = [&](auto dim) -> cudaError_t {
     constexpr int D = decltype(dim)::value;
-    static PerDeviceFlag set_q4[2], set_bf16[2];
-    return q4 ? run(attn_decode_q4_kernel<D, 1>, attn_decode_q4_kernel<D, DECODE_BATCH>, 0, set_q4)
+    static PerDeviceFlag set_q4[2], set_q4_two[2], set_bf16[2];
+    if (q4 && group == 8) return run(attn_decode_q4_kernel<D, 1, 1>, attn_decode_q4_kernel<D, DECODE_BATCH, 1>, 0, set_q4);
+    return q4 ? run(attn_decode_q4_kernel<D, 1, 2>, attn_decode_q4_kernel<D, DECODE_BATCH, 2>, 0, set_q4_two)
               : run(attn_decode_kernel<D, 1>, attn_decode_kernel<D, DECODE_BATCH>, (DA_G + 4 * DA_KT) * (d + 8) * 2, set_bf16);
   };
   switch (d) {

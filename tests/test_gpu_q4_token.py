@@ -1,5 +1,6 @@
-"""One token over a 4-bit cache at the edges of its kernel: groups of one to more than eight query heads, caches that end inside
-and at the edge of a warp's 16 keys, of a tile of 64 and of a split, units in and out of temporal order."""
+"""One token over a 4-bit cache at the edges of its kernel: groups of one to more than eight query heads, in blocks of eight and of
+sixteen, caches that end inside and at the edge of a warp's 16 keys, of a tile of 64 and of a split, units in and out of
+temporal order."""
 
 import numpy as np
 import pytest
@@ -51,3 +52,43 @@ def test_tokens_after_an_eviction(h, hk, d):
         check_attention(out[:1].float().cpu().numpy().astype(np.float64), ref, f"token {t}", ora.last_abs_out, ora.last_flip_sens)
     assert gpu.sync_status() == 0
     gpu.destroy()
+
+
+@pytest.mark.parametrize("h,hk,d,first", [(288, 32, 64, 1987), (144, 16, 96, 3584), (80, 8, 128, 7200)])
+def test_one_token_in_blocks_of_sixteen_heads(h, hk, d, first):
+    """More than 6 * 148 tiles of 64 units, the last one with a few, in more blocks of eight than fit the GPU."""
+    from parity_util import lockstep_chunk, make_pair
+    sh = W.LayerShape(d_model=64, n_q_heads=h, n_kv_heads=hk, head_dim=d, d_retain=8, rope_theta=500000.0, kv_dtype=1)
+    ora, gpu = make_pair(sh, W.layer_weights(sh, 0, seed=W.BASE_SEED + 84), budget=8000, chunk=first, n_stab=16)
+    ora.prefill_chunk(_hidden(first, 64, 1), 0, rows=[0])
+    lockstep_chunk(ora, gpu, _hidden(1, 64, 60 + first), 1, what=f"{h} {hk} {d} {first}+1")
+    gpu.destroy()
+
+
+@pytest.mark.parametrize("g,d", [(16, 128), (9, 96), (17, 128)])
+def test_a_stack_in_blocks_of_sixteen_equals_layers_in_blocks_of_eight(g, d):
+    """Eight layers in one launch have enough tiles, one alone has not; the sums are the same."""
+    import torch
+    from paper_2410_01805_b200 import LayerStack, LocretLayer
+    from parity_util import bf16_dev
+    sh = W.LayerShape(d_model=64, n_q_heads=2 * g, n_kv_heads=2, head_dim=d, d_retain=8, rope_theta=500000.0, kv_dtype=1)
+    runs = []
+    for stack in (True, False):
+        layers = [LocretLayer(sh, *(bf16_dev(a) for a in W.layer_weights(sh, i, seed=W.BASE_SEED + 85)), 4000, 1800, 16) for i in range(8)]
+        big = torch.zeros((1800, 2 * g * d), dtype=torch.bfloat16, device="cuda")
+        for c in range(2):
+            for L in layers:
+                L.prefill_chunk(bf16_dev(_hidden(1800, 64, c)), big, 0)
+        outs = torch.zeros((3, 8, 2 * g * d), dtype=torch.bfloat16, device="cuda")
+        for t in range(3):
+            x = bf16_dev(_hidden(1, 64, 90 + t))
+            if stack:
+                LayerStack(layers).decode_step(x, outs[t], out_stride=2 * g * d)
+            else:
+                for i, L in enumerate(layers):
+                    L.decode_step(x, outs[t, i])
+        assert all(L.sync_status() == 0 for L in layers)
+        runs.append(outs.cpu())
+        for L in layers:
+            L.destroy()
+    assert torch.equal(*runs)
