@@ -105,6 +105,24 @@ __device__ __forceinline__ void rope_pairs8(const uint4 &lo, const uint4 &hi, co
   }
 }
 
+// Slot i of head m takes the unit of slot src, which is at `pos` in temporal order: elements [e, e + 8) and their partners.
+__device__ __forceinline__ void move_row(const CompactArgs &a, int m, int src, int i, int pos, int e) {
+  const int half = a.d / 2;
+  const size_t so = ((size_t)m * a.cap + src) * a.d + e, dof = ((size_t)m * a.cap + i) * a.d + e;
+  const uint4 k_lo = *reinterpret_cast<const uint4 *>(a.k + so), k_hi = *reinterpret_cast<const uint4 *>(a.k + so + half);
+  if (src != i) {
+    const uint4 v_lo = *reinterpret_cast<const uint4 *>(a.v + so), v_hi = *reinterpret_cast<const uint4 *>(a.v + so + half);
+    *reinterpret_cast<uint4 *>(a.k + dof) = k_lo;
+    *reinterpret_cast<uint4 *>(a.k + dof + half) = k_hi;
+    *reinterpret_cast<uint4 *>(a.v + dof) = v_lo;
+    *reinterpret_cast<uint4 *>(a.v + dof + half) = v_hi;
+  }
+  uint4 r_lo, r_hi;
+  rope_pairs8(k_lo, k_hi, a.cs + (size_t)pos * half + e, r_lo, r_hi);
+  *reinterpret_cast<uint4 *>(a.k_rot + dof) = r_lo;
+  *reinterpret_cast<uint4 *>(a.k_rot + dof + half) = r_hi;
+}
+
 // blockDim.x = d / 16 threads per row, blockDim.y rows per block.
 __global__ void compact_kernel(CompactArgs a) {
   pdl_wait();
@@ -119,27 +137,11 @@ __global__ void compact_kernel(CompactArgs a) {
   const int pos = a.rank[rcur ^ 1][u];
   const int pos_old = i < ranked_len ? a.rank[rcur][u] : i;
   if (src == i && pos == pos_old) return;  // stays, and stays where it was in the order
-  const int c = threadIdx.x * 8;
-  const int half = a.d / 2;
-  const size_t so = ((size_t)m * a.cap + src) * a.d, dof = u * a.d;
-  const uint4 k_lo = *reinterpret_cast<const uint4 *>(a.k + so + c);
-  const uint4 k_hi = *reinterpret_cast<const uint4 *>(a.k + so + c + half);
-  if (src != i) {
-    const uint4 v_lo = *reinterpret_cast<const uint4 *>(a.v + so + c);
-    const uint4 v_hi = *reinterpret_cast<const uint4 *>(a.v + so + c + half);
-    *reinterpret_cast<uint4 *>(a.k + dof + c) = k_lo;
-    *reinterpret_cast<uint4 *>(a.k + dof + c + half) = k_hi;
-    *reinterpret_cast<uint4 *>(a.v + dof + c) = v_lo;
-    *reinterpret_cast<uint4 *>(a.v + dof + c + half) = v_hi;
-    if (threadIdx.x == 0) {
-      a.s[u] = a.s[(size_t)m * a.cap + src];
-      a.t[u] = a.t[(size_t)m * a.cap + src];
-    }
+  move_row(a, m, src, i, pos, threadIdx.x * 8);
+  if (src != i && threadIdx.x == 0) {
+    a.s[u] = a.s[(size_t)m * a.cap + src];
+    a.t[u] = a.t[(size_t)m * a.cap + src];
   }
-  uint4 r_lo, r_hi;
-  rope_pairs8(k_lo, k_hi, a.cs + (size_t)pos * half + c, r_lo, r_hi);
-  *reinterpret_cast<uint4 *>(a.k_rot + dof + c) = r_lo;
-  *reinterpret_cast<uint4 *>(a.k_rot + dof + c + half) = r_hi;
 }
 
 __global__ void rerope_kernel(const bf16 *k_pre, bf16 *k_rot, const float2 *cs, int h_kv, int d,
@@ -457,84 +459,21 @@ topk_kernel(TopkArgs a, int cache_in_smem) {
   }
 }
 
-// One unit more than the budget, the eviction of a one-token step: the unit that goes is the competing one with
-// the lowest (score, rank), so one pass over the candidates and a block-wide minimum replace the radix select (11 us of a
-// one-token step of the small shape, 1025 candidates, two heads; 2.9 us this way).  Same results as topk_kernel.
-__global__ void __launch_bounds__(TK_THREADS)
-topk_one_kernel(TopkArgs a) {
-  __shared__ unsigned long long s_best[32];
+// ranks before the eviction: rk is head m's row of them
+__device__ __forceinline__ int rank_at(const TopkArgs &a, const int32_t *rk, int i) { return i < a.ranked_len ? rk[i] : i; }
+// The competing unit of head m with the lowest (score, rank), found by the whole block: its slot and its rank.
+template <int THREADS>
+__device__ __forceinline__ int2 lowest_unit(const TopkArgs &a, const int32_t *rk, int m) {
+  constexpr int WARPS = THREADS / 32;
+  __shared__ unsigned long long s_best[WARPS];
   __shared__ int s_slot;
-  pdl_wait();
-  pdl_launch_dependents();
-  const int m = blockIdx.x, tid = threadIdx.x, n = a.n, budget = a.budget;
+  const int tid = threadIdx.x, n = a.n;
   const float *sc = a.scores + (size_t)m * a.stride;
-  const int32_t *rk = a.rank[a.rcur] + (size_t)m * a.stride;
-  int32_t *src_of = a.src_of + (size_t)m * a.src_stride;
-  int32_t *rank_new = a.rank[a.rcur ^ 1] + (size_t)m * a.stride;
-  auto rank_at = [&](int i) -> int { return i < a.ranked_len ? rk[i] : i; };
-  unsigned long long best = ~0ull;
-  int slot = -1;
-  for (int i = tid; i < n; i += TK_THREADS) {
-    const int r = rank_at(i);
-    const unsigned long long c = ((unsigned long long)score_key(sc[i]) << 32) | (unsigned)r;
-    if (r >= a.n_pre && r < n - a.n_prot && c < best) { best = c; slot = i; }
-  }
-  unsigned long long w = best;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long y = __shfl_xor_sync(0xffffffffu, w, o);
-    w = y < w ? y : w;
-  }
-  if ((tid & 31) == 0) s_best[tid >> 5] = w;
-  __syncthreads();
-  w = s_best[tid & 31];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long y = __shfl_xor_sync(0xffffffffu, w, o);
-    w = y < w ? y : w;
-  }
-  if (slot >= 0 && best == w) s_slot = slot;  // (ranks are distinct: one thread; at least one unit competes)
-  __syncthreads();
-  const int gone = s_slot, gone_rank = (int)(unsigned)w;
-  int rotated = 0;
-  for (int i = tid; i < budget; i += TK_THREADS) {
-    const int src = i == gone ? budget : i;  // the last unit takes the freed slot
-    const int r = rank_at(src), r_new = r - (r > gone_rank);
-    src_of[i] = src;
-    rank_new[i] = r_new;
-    rotated += src != i || r_new != r;
-  }
-  if (a.counters) {
-    rotated = __reduce_add_sync(0xffffffffu, rotated);
-    if ((tid & 31) == 0 && rotated) atomicAdd(&a.counters[1], (unsigned long long)rotated);
-    if (tid == 0 && gone < budget) atomicAdd(&a.counters[0], 1ull);
-  }
-}
-
-// The eviction of a one-token step over a bf16 cache in one launch.  What bounds it is latency: selection and gather as two
-// launches took 3.0 + 2.8 us and a hand-over, this one 5.8 us under the profiler, where launches do not overlap, and a step of
-// the small shape 15.25 us with the two, 13.9 with this one.  Every block finds its head's minimum for itself (8 KB of scores
-// and ranks from L2 for 1025 candidates) and gathers its own rows.  Scores and token ids are what other blocks still select
-// by, so the unit that changes its slot brings those along when the last block of its head has selected.
-// grid (blocks per head, heads).
-constexpr int EO_THREADS = 512;
-
-__global__ void __launch_bounds__(EO_THREADS)
-evict_one_kernel(TopkArgs a, CompactArgs c, unsigned *done) {
-  __shared__ unsigned long long s_best[EO_THREADS / 32];
-  __shared__ int s_slot;
-  pdl_wait();
-  pdl_launch_dependents();
-  const int m = blockIdx.y, tid = threadIdx.x, n = a.n, budget = a.budget;
-  const float *sc = a.scores + (size_t)m * a.stride;
-  const int32_t *rk = a.rank[a.rcur] + (size_t)m * a.stride;
-  int32_t *rank_new = a.rank[a.rcur ^ 1] + (size_t)m * a.stride;
-  auto rank_at = [&](int i) -> int { return i < a.ranked_len ? rk[i] : i; };
   unsigned long long best = ~0ull;
   int slot = -1;
 #pragma unroll 4
-  for (int i = tid; i < n; i += EO_THREADS) {
-    const int r = rank_at(i);
+  for (int i = tid; i < n; i += THREADS) {
+    const int r = rank_at(a, rk, i);
     const unsigned long long v = ((unsigned long long)score_key(sc[i]) << 32) | (unsigned)r;
     if (r >= a.n_pre && r < n - a.n_prot && v < best) { best = v; slot = i; }
   }
@@ -546,15 +485,62 @@ evict_one_kernel(TopkArgs a, CompactArgs c, unsigned *done) {
   }
   if ((tid & 31) == 0) s_best[tid >> 5] = w;
   __syncthreads();
-  w = s_best[tid & (EO_THREADS / 32 - 1)];
+  w = s_best[tid & (WARPS - 1)];
 #pragma unroll
-  for (int o = EO_THREADS / 64; o > 0; o >>= 1) {
+  for (int o = WARPS / 2; o > 0; o >>= 1) {
     const unsigned long long y = __shfl_xor_sync(0xffffffffu, w, o);
     w = y < w ? y : w;
   }
   if (slot >= 0 && best == w) s_slot = slot;  // (ranks are distinct: one thread; at least one unit competes)
   __syncthreads();
-  const int gone = s_slot, gone_rank = (int)(unsigned)w;
+  return make_int2(s_slot, (int)(unsigned)w);
+}
+
+// One unit more than the budget, the eviction of a one-token step: the unit that goes is the competing one with
+// the lowest (score, rank), so one pass over the candidates and a block-wide minimum replace the radix select (11 us of a
+// one-token step of the small shape, 1025 candidates, two heads; 2.9 us this way).  Same results as topk_kernel.
+__global__ void __launch_bounds__(TK_THREADS)
+topk_one_kernel(TopkArgs a) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.x, tid = threadIdx.x, budget = a.budget;
+  int32_t *src_of = a.src_of + (size_t)m * a.src_stride;
+  int32_t *rank_new = a.rank[a.rcur ^ 1] + (size_t)m * a.stride;
+  const int32_t *rk = a.rank[a.rcur] + (size_t)m * a.stride;
+  const int2 low = lowest_unit<TK_THREADS>(a, rk, m);
+  const int gone = low.x, gone_rank = low.y;
+  int rotated = 0;
+  for (int i = tid; i < budget; i += TK_THREADS) {
+    const int src = i == gone ? budget : i;  // the last unit takes the freed slot
+    const int r = rank_at(a, rk, src), r_new = r - (r > gone_rank);
+    src_of[i] = src;
+    rank_new[i] = r_new;
+    rotated += src != i || r_new != r;
+  }
+  if (a.counters) {
+    rotated = __reduce_add_sync(0xffffffffu, rotated);
+    if ((tid & 31) == 0 && rotated) atomicAdd(&a.counters[1], (unsigned long long)rotated);
+    if (tid == 0 && gone < budget) atomicAdd(&a.counters[0], 1ull);
+  }
+}
+
+// The eviction of a one-token step over a bf16 cache in one launch, where evicts_one_in_a_launch says so.  What bounds it is
+// latency: selection and gather as two launches took 3.0 + 2.8 us and a hand-over, this one 5.8 us under the profiler, where
+// launches do not overlap, and a step of the small shape 15.25 us with the two, 13.9 with this one.  Every block finds its head's
+// minimum for itself (8 KB of scores and ranks from L2 for 1025 candidates) and gathers its own rows.  Scores and token ids are
+// what other blocks still select by, so the unit that changes its slot brings those along when the last block of its head has
+// selected.  grid (blocks per head, heads).
+constexpr int EO_THREADS = 512;
+
+__global__ void __launch_bounds__(EO_THREADS)
+evict_one_kernel(TopkArgs a, CompactArgs c, unsigned *done) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.y, tid = threadIdx.x, budget = a.budget;
+  int32_t *rank_new = a.rank[a.rcur ^ 1] + (size_t)m * a.stride;
+  const int32_t *rk = a.rank[a.rcur] + (size_t)m * a.stride;
+  const int2 low = lowest_unit<EO_THREADS>(a, rk, m);
+  const int gone = low.x, gone_rank = low.y;
   if (tid == 0 && gone < budget) {
     __threadfence();
     if (atomicInc(&done[m], gridDim.x - 1) == gridDim.x - 1) {
@@ -566,28 +552,16 @@ evict_one_kernel(TopkArgs a, CompactArgs c, unsigned *done) {
     }
   }
   // rows of this block: d / 16 threads each
-  const int tpr = c.d / 16, rpb = EO_THREADS / tpr, half = c.d / 2, e = (tid % tpr) * 8;
+  const int tpr = c.d / 16, rpb = EO_THREADS / tpr, e = (tid % tpr) * 8;
   const int lo = (int)((long long)blockIdx.x * budget / gridDim.x), hi = (int)((long long)(blockIdx.x + 1) * budget / gridDim.x);
   int rotated = 0;
   for (int i = lo + tid / tpr; i < hi && tid < rpb * tpr; i += rpb) {
     const int src = i == gone ? budget : i;  // the last unit takes the freed slot
-    const int r = rank_at(src), r_new = r - (r > gone_rank);
+    const int r = rank_at(a, rk, src), r_new = r - (r > gone_rank);
     if (e == 0) rank_new[i] = r_new;
     if (src == i && r == r_new) continue;
     rotated += e == 0;
-    const size_t so = ((size_t)m * c.cap + src) * c.d, dof = ((size_t)m * c.cap + i) * c.d;
-    const uint4 k_lo = *reinterpret_cast<const uint4 *>(c.k + so + e), k_hi = *reinterpret_cast<const uint4 *>(c.k + so + e + half);
-    if (src != i) {
-      const uint4 v_lo = *reinterpret_cast<const uint4 *>(c.v + so + e), v_hi = *reinterpret_cast<const uint4 *>(c.v + so + e + half);
-      *reinterpret_cast<uint4 *>(c.k + dof + e) = k_lo;
-      *reinterpret_cast<uint4 *>(c.k + dof + e + half) = k_hi;
-      *reinterpret_cast<uint4 *>(c.v + dof + e) = v_lo;
-      *reinterpret_cast<uint4 *>(c.v + dof + e + half) = v_hi;
-    }
-    uint4 r_lo, r_hi;
-    rope_pairs8(k_lo, k_hi, c.cs + (size_t)r_new * half + e, r_lo, r_hi);
-    *reinterpret_cast<uint4 *>(c.k_rot + dof + e) = r_lo;
-    *reinterpret_cast<uint4 *>(c.k_rot + dof + e + half) = r_hi;
+    move_row(c, m, src, i, r_new, e);
   }
   rotated = __reduce_add_sync(0xffffffffu, rotated);
   if ((tid & 31) == 0 && rotated) atomicAdd(&a.counters[1], (unsigned long long)rotated);
@@ -671,11 +645,29 @@ cudaError_t launch_topk(const TopkArgs &a, int h_kv, cudaStream_t st, bool pdl) 
   return cudaGetLastError();
 }
 
-// As many blocks per head as leave a block one pass over its rows, but no more than two for each SM in all.
+static int evict_one_blocks(int d, int budget) {   // per head, as many as leave a block one pass over its rows
+  const int rpb = EO_THREADS / (d / 16);
+  return (budget + rpb - 1) / rpb;
+}
+
+// One launch where every block's search and its passes over its rows cost less than the launch that they save.  Up to 2^23 elements
+// of keys; and with little of that to do for many candidates (512 elements a unit and less, more than 4096 units), only while
+// an SM has no more than one block.  Measured (us a step, two launches / one; first the unit that goes is the oldest, so that every key
+// is rotated, then one of no particular age): 8 heads of 128, 1024 units 18.8 / 18.5 and 18.8 / 17.9, 4096 units 25.2 / 23.7 and
+// 24.5 / 23.2, 8192 units (2^23) 33.2 / 31.7 and 31.6 / 31.4, 16384 units 51.9 / 48.9 and 47.1 / 48.0; 32 heads of 96, 2048 units 31.9 /
+// 30.1 and 30.5 / 29.4, 4096 units 44.7 / 42.6 and 41.1 / 41.4, 16384 units 121 / 122 and 106 / 118; 32 heads of 128, 2048 units 37.2 /
+// 36.6 and 35.5 / 36.0, 16384 units 137 / 136 and 119 / 132; 2 heads of 64, 8192 units (128 blocks) 19.4 / 18.6 and 19.4 / 18.0, 16384 units
+// (256) 24.1 / 24.3 and 23.9 / 24.2; 2 heads of 96, 12288 units (290) 23.9 / 25.7 and 23.6 / 24.1; 8 heads of 64, 12288 units 29.0 /
+// 29.9 and 27.4 / 29.8.
+bool evicts_one_in_a_launch(int h_kv, int d, int budget) {
+  if ((long long)h_kv * d * budget > 1 << 23) return false;
+  return budget <= 4096 || h_kv * d > 512 || h_kv * evict_one_blocks(d, budget) <= sm_count_of_current_device();
+}
+
+// (no more than two blocks for each SM in all)
 cudaError_t launch_evict_one(const TopkArgs &a, const CompactArgs &c, unsigned *done, cudaStream_t st, bool pdl) {
   if (a.per_head || a.n != a.budget + 1 || a.n > a.stride || !a.counters) return cudaErrorInvalidValue;
-  const int rpb = EO_THREADS / (c.d / 16);
-  int blocks = (a.budget + rpb - 1) / rpb;
+  int blocks = evict_one_blocks(c.d, a.budget);
   const int most = 2 * sm_count_of_current_device() / c.h_kv;
   if (blocks > most) blocks = most < 1 ? 1 : most;
   return launch_kernel(evict_one_kernel, dim3(blocks, c.h_kv), dim3(EO_THREADS), 0, st, pdl, a, c, done);

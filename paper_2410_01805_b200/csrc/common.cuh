@@ -291,7 +291,8 @@ struct CompactArgs {
 cudaError_t launch_compact(const CompactArgs &a, cudaStream_t st, bool pdl = false);
 
 // Both in one launch where one unit goes (n == budget + 1, one budget for all heads, bf16 cache; a.counters not null).  a.src_of is
-// not written.  done: a zeroed word per head, left at zero.
+// not written.  done: a zeroed word per head, left at zero.  The first says for which sizes one launch is the faster way.
+bool evicts_one_in_a_launch(int h_kv, int d, int budget);
 cudaError_t launch_evict_one(const TopkArgs &a, const CompactArgs &c, unsigned *done, cudaStream_t st, bool pdl);
 
 // k_rot[m][i] = RoPE(k_pre[m][i], i) for i < len (used after an import).

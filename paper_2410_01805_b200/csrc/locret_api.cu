@@ -543,7 +543,7 @@ int evict_and_close(locret_layer *L, int n_tok, uint32_t flags, bool side, cudaS
     mv.per_head = L->per_head ? 1 : 0;
     mv.budget_m = L->budget_m; mv.ranked_m = L->ranked_m; mv.rcur_m = L->rcur_m; mv.evict_m = evict_m;
     // (on the second stream the selection runs beside attention and only the gather waits for it)
-    const bool one = !side && !L->int4 && !L->per_head && n == L->budget + 1;
+    const bool one = !side && !L->int4 && !L->per_head && n == L->budget + 1 && evicts_one_in_a_launch(L->h_kv, L->d, L->budget);
     if (one) {
       Timed t(L, LOCRET_K_COMPACT, S);
       CK(launch_evict_one(sel, mv, reinterpret_cast<unsigned *>(L->d_counters + 2), S, pdl));
