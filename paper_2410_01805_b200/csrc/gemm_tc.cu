@@ -146,6 +146,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // CTAs share the A row block in L2).  The accumulator is double-buffered in TMEM: the epilogue
   // of one tile overlaps the main loop of the next.
   using Cfg = GemmCfg<BN, PAIR>;
+  static_assert(!(MAJOR & 2) || Cfg::B_ROWS % 64 == 0, "an MN-major B is loaded in boxes of 64 of its columns");
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
@@ -635,8 +636,14 @@ cudaError_t launch_as(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, 
 }
 
 // Pairs of CTAs where they take no more waves than single CTAs do: a wave of either costs the same MMAs, and an odd
-// number of 128-row blocks leaves half of a pair's last tile idle, which only shows in the number of waves.  One
-// block of rows, and the tile widths below 192 that only small matrices take, stay with single CTAs.
+// number of 128-row blocks leaves half of a pair's last tile idle, which mostly shows in the number of waves.  The retaining head,
+// whose SMs others could use, gains as well: 300 tokens of the Phi-3 shape, 16 CTAs in pairs where 12 would do, four layers in
+// turn, 138 us a step, 148 with single CTAs; 129 tokens of the Llama shape (2 blocks) 92.4 / 96.6, 1100 (9 blocks) 165 / 170.  What can
+// lose is a projection of a few odd blocks in two waves beside another layer's retaining head and eviction: 520 tokens of
+// the Phi-3 shape (5 blocks, 48 column tiles), four layers in turn, take 157 us a step in pairs, with single CTAs 147 or, when the two
+// streams fall out of step, 176; one layer alone 180 / 183, whole blocks of that shape 252 / 262.  One block of rows stays with
+// single CTAs, and so do the tile widths below 192, which only small matrices take, and MODE 6, whose sums go to other GPUs (not
+// measured).
 template <int BN, int MODE, int HD = 0, int MAJOR = 0>
 cudaError_t launch_t(const bf16 *A, int lda, const bf16 *Bt, int ldb, bf16 *C, int ldc, int M, int N,
                      int K, const float *W2, float *partial, int h_kv, int act, const RopeAppendArgs &ra,
