@@ -76,9 +76,11 @@ enum {
   LOCRET_K_RH,          /* (c) retaining head GEMM -> activation -> GEMM          */
   LOCRET_K_RH_REDUCE,   /* (c) sum of the retaining head's partial scores (a      */
                         /*     one-token step sums them inside LOCRET_K_RH)        */
-  LOCRET_K_TOPK,        /* (d) per-head selection                                 */
+  LOCRET_K_TOPK,        /* (d) per-head selection, where it is a kernel of its own */
   LOCRET_K_COMPACT,     /* (d) gather in place + re-RoPE of keys whose position   */
-                        /*     changed                                            */
+                        /*     changed; with the selection in the same kernel     */
+                        /*     where a step evicts one unit of a bf16 cache       */
+                        /*     (up to some size)                                  */
   LOCRET_K_DEQUANT,     /* 4-bit cache: expansion of the retained units to bf16   */
   LOCRET_K_QUANT,       /* 4-bit cache: quantisation of the chunk's units         */
   LOCRET_K_COUNT

@@ -161,7 +161,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (warp == 8) {
       // ------------------------------------------------------------ TMA producer (both CTAs)
       if (lane == 0) {
-        const uint32_t q_full0 = map_to_cta(smem_u32(q_full), 0);
+        const uint32_t q_full0 = cluster_map(smem_u32(q_full), 0);
         if (cta == 0) mbar_expect_tx(q_full, 2 * Q_BYTES);
         for (int hh = 0; hh < 2; hh++)
           tma2_load_2d(sQ + hh * QBOX, &map_q, my_head * D + hh * 64, my_row0, q_full0);
@@ -175,7 +175,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           const int s = j % NSTK;
           if (!mbar_wait(&k_empty[s], ((j / NSTK) & 1) ^ 1, abort_flag, p.status)) return false;
           if (cta == 0) mbar_expect_tx(&k_full[s], 2 * K_STAGE);
-          const uint32_t bar0 = map_to_cta(smem_u32(&k_full[s]), 0);
+          const uint32_t bar0 = cluster_map(smem_u32(&k_full[s]), 0);
           for (int hh = 0; hh < 2; hh++)
             tma2_load_3d(sK + s * K_STAGE + hh * KBOX, &map_k, hh * 64, tile_of(j) * TILE + (int)cta * 64, kvh, bar0);
           return true;
@@ -184,7 +184,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           const int s = j % NSTV;
           if (!mbar_wait(&v_empty[s], ((j / NSTV) & 1) ^ 1, abort_flag, p.status)) return false;
           if (cta == 0) mbar_expect_tx(&v_full[s], 2 * V_STAGE);
-          const uint32_t bar0 = map_to_cta(smem_u32(&v_full[s]), 0);
+          const uint32_t bar0 = cluster_map(smem_u32(&v_full[s]), 0);
           tma2_load_3d(sV + s * V_STAGE, &map_v, (int)cta * 64, tile_of(j) * TILE, kvh, bar0);
           return true;
         };
@@ -285,7 +285,7 @@ attn_tc2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const float c = p.scale_log2;
     const int row = my_row0 + r;
     const int limit = len + row;  // last visible key
-    const uint32_t p_half0 = map_to_cta(smem_u32(p_half), 0), p_full0 = map_to_cta(smem_u32(p_full), 0);
+    const uint32_t p_half0 = cluster_map(smem_u32(p_half), 0), p_full0 = cluster_map(smem_u32(p_full), 0);
     float m_mine = -INFINITY, l = 0.f;
     bool ok = true;
 

@@ -1,6 +1,7 @@
-// Decoding (the B = 1 case of Eq. 1): one token per step, so every kernel is bound by the bytes
-// it must read once: the weights for the two projections, the retained keys and values for
-// attention.  Plain CUDA cores, 16-byte loads, no tensor cores (there is no contraction to tile).
+// Decoding (the B = 1 case of Eq. 1): one token per step, so the bytes that a kernel must read once bound it, the weights
+// for the two projections and the retained keys and values for attention, and the latency of its phases.  The projections are
+// dot products on the CUDA cores with 16-byte loads; attention has a small contraction to tile, the query heads of a
+// group (header of each attention kernel); over a 4-bit cache the work on the codes counts more than their bytes.
 #include <stdlib.h>
 
 #include <type_traits>
@@ -566,7 +567,9 @@ attn_decode_kernel(int h, int h_kv, float scale_log2, const __grid_constant__ De
 // the four lanes of a row read whole sectors of its (cos, sin)); row r of S^T is key kr(r), and columns of O are dealt
 // to the lanes in runs of D / 8, so that a lane's value codes lie together.
 // Measured (span of the launch for four Llama layers, 6000 units each): 84 us with tiles expanded into shared memory by
-// threads that each took 16 elements of a key (4150 instructions a warp, conversions among them), 64 us this way.
+// threads that each took 16 elements of a key (4150 instructions a warp, conversions among them), 64 us this way, both with two
+// blocks for each SM.  With the splits of decode_attn_splits a step of four layers with such heads and d_model 1024 takes 71 us,
+// 101 then.
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
   uint32_t d;
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
@@ -1016,7 +1019,9 @@ cudaError_t launch_rh_gemv(const RhGemvBatch &b, int n_layers, int d_R, int K, i
 // 1152 / 1224 / 1133 / 1052 tokens/s (more splits shorten each CTA's chain of tiles, but the last split of a
 // head merges them all).  With a 4-bit cache 100 / 148 / 200 / 296 / 400 CTAs take 93.2 / 94.5 / 88.1 / 99.8 / 97.5 us a step of
 // four such layers, 34.7 / 28.5 / 28.4 / 28.0 / 30.7 us of one, and at the Phi-3 shape (32 KV heads of 96) 171 / 187 / 181 / 179 /
-// 177 and 63.7 / 55.5 / 53.5 / 56.2 / 50.9 us.
+// 177 and 63.7 / 55.5 / 53.5 / 56.2 / 50.9 us: 200 is the best of the first and within 2, 6 and 5 % of the best of the others.
+// Groups of query heads that one block cannot serve multiply the CTAs (a launch of one layer gains from that, see
+// q4_heads_per_block).
 int decode_attn_splits(int h_kv, int n) {
   static int forced = -1;
   if (forced < 0) { const char *e = getenv("LOCRET_DEC_CTAS"); forced = e ? atoi(e) : 0; if (forced < 0 || forced > 2048) forced = 0; }

@@ -211,7 +211,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (!ok) break;
           if (!PAIR) mbar_expect_tx(&full[s], Cfg::STAGE_BYTES);
           else if (rank == 0) mbar_expect_tx(&full[s], 2 * Cfg::STAGE_BYTES);
-          const uint32_t bar0 = PAIR ? map_to_cta(smem_u32(&full[s]), 0) : 0;
+          const uint32_t bar0 = PAIR ? cluster_map(smem_u32(&full[s]), 0) : 0;
           auto load = [&](unsigned char *dst, const CUtensorMap *map, int c0, int c1) {
             if (PAIR) tma2_load_2d(dst, map, c0, c1, bar0);
             else tma_load_2d(dst, map, c0, c1, &full[s]);
@@ -582,7 +582,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        if (PAIR) mbar_arrive_remote(map_to_cta(smem_u32(&acc_empty[buf]), 0));
+        if (PAIR) mbar_arrive_remote(cluster_map(smem_u32(&acc_empty[buf]), 0));
         else mbar_arrive(&acc_empty[buf]);
       }
     }

@@ -833,11 +833,10 @@ int chunk_step(locret_layer *L, const void *hidden_in, int32_t n_tok, uint32_t f
     // cache of 1000 units, 512 tokens: 147 us a step divided, 128 undivided.)
     const bool may_divide = !skinny_rh || n_tok <= 256 ||
                             2 * skinny_ctas(n_tok, L->d_R, L->d_in) <= sm_count_of_current_device();
-    // The CTA-pair kernel is opt-in (LOCRET_ATTN_PAIR=1) and never used in a divided-heads step.  In a test
-    // process in which it had run, the projection GEMM of a later divided-heads step (eight shards of the
-    // Llama shape on one GPU) reported a device-side time-out in about one full test run in three.  A cause that
-    // fits has since been mended in that GEMM's launch (its two tensor maps could share a slot of their
-    // cache); the default is still the kernel that every run has validated.
+    // The CTA-pair kernel is opt-in (LOCRET_ATTN_PAIR=1) and never used in a divided-heads step: its sums are in another order, so
+    // making it the default changes the bits of every prefill.  (The time-outs of a projection GEMM that once came with it were that
+    // GEMM's: its two tensor maps could share a slot of their cache, and A was then loaded in boxes of B, 64 KB a stage
+    // where the barrier expected 48.  The allocation of tensor memory by pairs was suspected too; every wide GEMM does it now.)
     if (tc_ok && L->attn_pair && !tp && attention_tc2_supported(n_tok, L->h, L->h_kv, L->d))
       CK(launch_attention_tc2(&L->map_q, &L->map_k64, &map_v, (bf16 *)attn_out, n_tok, L->h, L->h_kv,
                               L->d, L->len, L->d_status, L->st, len_m));

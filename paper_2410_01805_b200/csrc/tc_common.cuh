@@ -254,12 +254,6 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// address of the same shared-memory object in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t local, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-  return r;
-}
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
   // (no cluster-scope release: what the arrival publishes lives in tensor memory and is ordered by
   // tcgen05.wait::st + tcgen05.fence::before_thread_sync; a cluster-scope fence here cost ~25 % of the kernel)
